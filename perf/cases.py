@@ -281,7 +281,9 @@ def _inputs(case, seed):
         S["weights"] = _randn((A.n_levels, C, C, 27), seed + 14, math.sqrt(1.0 / (27 * C))).to(torch.bfloat16)
     if kind == "cnn":
         S["scale"] = float(np.float32(1.0 / float(A.values.double().mean())))
-        S["weights"] = [_randn((A.n_levels, C, C, 27), seed + 20 + i, math.sqrt(2.0 / (27 * C))).to(torch.bfloat16)
+        # the network's own initial scales: the last layer is a small correction to the residual
+        S["weights"] = [_randn((A.n_levels, C, C, 27), seed + 20 + i,
+                               math.sqrt(2.0 / (27 * C)) * (0.1 if i == N_LAYERS - 1 else 1.0)).to(torch.bfloat16)
                         for i in range(N_LAYERS)]
     return S
 

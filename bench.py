@@ -102,12 +102,11 @@ class ClockSampler:
                 else "warm-up and timed region (timed region shorter than the 50 ms sampling period)"}
 
 
-TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_kernels.cu", "paper_2112_03592_gb300/csrc/apr_device.cuh",
-                   "paper_2112_03592_gb300/csrc/apr_tile.cuh", "paper_2112_03592_gb300/csrc/apr_plan.cu"]
+TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_units.cu", "paper_2112_03592_gb300/csrc/apr_unitplan.cpp",
+                   "paper_2112_03592_gb300/csrc/apr_kernels.cu", "paper_2112_03592_gb300/csrc/apr_device.cuh"]
 
 
-MC_TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_mc.cu", "paper_2112_03592_gb300/csrc/apr_device.cuh",
-                      "paper_2112_03592_gb300/csrc/apr_plan.cu"]
+MC_TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_mc.cu", "paper_2112_03592_gb300/csrc/apr_device.cuh"]
 
 
 def kernel_source_hash(sources=None):
@@ -135,20 +134,6 @@ def recorded_traffic(call, section=None):
     if sha != rec.get("sha1_prefix"):
         return None
     return rec.get("dram_bytes_per_call", {}).get(call)
-
-
-def conv_launches(apr, st_h, k):
-    """Kernels of one apr_convolve (or apr_convolve_adjoint) call on the whole work list: for k = 5
-    with levels below l_max, three when no such level has taps outside the central 3^3 (radius-1
-    launch, persistent radius-2 launch, l_max launch), else two (one launch over all tiles and the
-    hint kernel beside it); otherwise one."""
-    import numpy as np
-    if k != 5 or apr.l_max == apr.l_min:
-        return 1
-    w = np.asarray(st_h, np.float32).reshape(apr.n_levels, 5, 5, 5)[:-1]
-    outer = w.copy()
-    outer[:, 1:4, 1:4, 1:4] = 0
-    return 2 if np.any(outer != 0) else 3
 
 
 def make_replayers(fns, use_graph):
@@ -466,20 +451,15 @@ def run_ours(args, rank, world):
     hbm = float(peaks["hbm_gbs"])
     pix_bytes = float(np.prod(apr.dims)) * 4.0
     # our kernels per step: restriction (one per level holding tree nodes), convolution, convolution
-    # adjoint, push-down (one per level holding tree nodes), stencil-gradient partials, reduction
+    # adjoint (node units, leaf units), push-down (one per level holding tree nodes), stencil-gradient
+    # partials, reduction
     n_tree_levels = len(set(lay.export(G._abi.APR_STRUCT_TREE_ITEMS)[:, 0].tolist()))
-    nc = conv_launches(apr, st_h, K)
-    launches_per_step = n_tree_levels + nc + nc + n_tree_levels + 2
-    # the dominant call of the step: the convolution adjoint (its radius-1 tiles in one launch on the
-    # library's second stream beside the launch over the l_max tiles; the call also clears the two
-    # gradient outputs). Its algorithmic bytes equal the forward's: dL/dout in, dL/dparticles and
-    # dL/dtree out, y indices and row pointers.
+    launches_per_step = n_tree_levels + 1 + 2 + n_tree_levels + 2
+    # the dominant call of the step: the convolution adjoint. Its algorithmic bytes equal the forward's:
+    # dL/dout in, dL/dparticles and dL/dtree out, y indices and row pointers.
     dom_ms, dom_call = (adj_ms, "apr_convolve_adjoint") if adj_ms >= conv_ms else (conv_ms, "apr_convolve")
-    dom_name = dom_call + (": conv_bwd_data_r1_kernel (levels below l_max, radius 1) beside conv_bwd_data_kernel<2> "
-                           "(l_max), conv_bwd_data_r2_pool_kernel after the radius-1 launch"
-                           if dom_call == "apr_convolve_adjoint" else
-                           ": conv_fwd_r1_kernel (levels below l_max, radius 1) beside conv_fwd_kernel<2> (l_max), "
-                           "conv_fwd_r2_pool_kernel after the radius-1 launch")
+    dom_name = dom_call + (": unit_adjoint_kernel<2>, then leaf_adjoint_kernel<2>" if dom_call == "apr_convolve_adjoint"
+                           else ": unit_conv_kernel<2>")
     traffic = recorded_traffic(dom_call)
     rec = {
         "metric": "APR conv Gparticles/s & pixel-equiv GB/s",
@@ -524,8 +504,7 @@ def run_ours(args, rank, world):
                      "traffic": traffic, "traffic_source": "profiles/traffic.json (ncu dram bytes of the call's "
                      "launches, same source)" if traffic else None, "peak_source": src + " (hbm_gbs, copy bandwidth)",
                      "algorithmic_bytes_per_launch": conv_bytes,
-                     "per_launch": "per call: algorithmic bytes of the whole call / the call's event time (its "
-                                   "launches on two streams, joined)",
+                     "per_launch": "per call: algorithmic bytes of the whole call / the call's event time",
                      "convolve_frac": round(conv_bytes / (conv_ms * 1e-3) / 1e9 / hbm, 4)},
         "e2e": {"value": round(world * Np / (e2e * 1e-3) / 1e9, 4), "unit": "Gparticles/s",
                 "h2d_bytes_per_step": T["h2d"], "d2h_bytes_per_step": T["d2h"],
@@ -547,9 +526,8 @@ def run_ours(args, rank, world):
         P = layer_step(args, lay, st_plain, bufs, dev, stream, flush, world)
         pall = [mean(v) for v in P["parts"]]
         pp = pall[:5]
-        p_dom_ms, p_dom = ((pp[2], "conv_bwd_data_kernel<2> (apr_convolve_adjoint: one launch over all tiles)")
-                           if pp[2] >= pp[1] else (pp[1], "conv_fwd_kernel<2> (apr_convolve: one launch over all tiles)"))
-        npc = conv_launches(apr, st_plain.cpu().numpy(), K)
+        p_dom_ms, p_dom = ((pp[2], "unit_adjoint_kernel<2>, then leaf_adjoint_kernel<2> (apr_convolve_adjoint)")
+                           if pp[2] >= pp[1] else (pp[1], "unit_conv_kernel<2> (apr_convolve)"))
         rec["plain5"] = {
             "value": round(world * Np / (P["step_ms"] * 1e-3) / 1e9, 4), "unit": "Gparticles/s",
             "ms_per_step": round(P["step_ms"], 5),
@@ -564,7 +542,7 @@ def run_ours(args, rank, world):
                          "algorithmic_bytes_per_launch": conv_bytes, "peak_source": src + " (hbm_gbs)"},
             "e2e": {"value": round(world * Np / (P["e2e_ms"] * 1e-3) / 1e9, 4), "unit": "Gparticles/s",
                     "h2d_bytes_per_step": P["h2d"], "d2h_bytes_per_step": P["d2h"], "ms_per_step": round(P["e2e_ms"], 4)},
-            "gpu_launches": (2 * n_tree_levels + 2 * npc + 2) * args.steps,
+            "gpu_launches": launches_per_step * args.steps,
         }
     if rank == 0 and not args.no_cpu_baseline:
         rec["cpu_baseline"] = cpu_baseline(apr, st_h, gout.cpu().numpy(), budget_s=args.cpu_budget)
@@ -929,7 +907,7 @@ def run_rl(args, rank, world, full=True):
                      "frac": round(conv_bytes / (conv_ms * 1e-3) / 1e9 / hbm, 4), "traffic": None,
                      "peak_source": src + " (hbm_gbs)", "algorithmic_bytes_per_launch": conv_bytes,
                      "conv_ms": round(conv_ms, 5)},
-        "gpu_launches": RL_ITERS * 2 * (n_tree_levels + conv_launches(apr, st_h, K)) * args.steps,
+        "gpu_launches": RL_ITERS * 2 * (n_tree_levels + 1) * args.steps,
     }
     if not full:
         return rec
@@ -1102,7 +1080,7 @@ def run_surrogate(args, rank, world, pretrained=None):
         # per CNN inference: embedding, 4 x (tree restriction per level, weight layout, convolution;
         # hidden ReLUs fused into the convolution), read-out; per RL run: 2 x (tree + convolution) per iteration
         "gpu_launches": (2 + 4 * (n_tree_levels + 2) +
-                         RL_ITERS * 2 * (n_tree_levels + conv_launches(apr, st.cpu().numpy(), 5))) * args.steps,
+                         RL_ITERS * 2 * (n_tree_levels + 1)) * args.steps,
     }
     return rec
 

@@ -104,20 +104,47 @@ typedef struct {
 #define APR_STRUCT_FWD_PLAN_R2 9
 #define APR_STRUCT_BWD_PLAN_R1 10
 #define APR_STRUCT_BWD_PLAN_R2 11
+/* Convolution units (what the convolution kernels read), host-only handles only (built on the first
+ * request; 0 bytes for a device handle). A parent is the 2 x 2 x 2 block of level-l cells under one cell
+ * of the level-(l-1) grid: a tree node, or for l = l_min a virtual parent (index N_t + i, child maps in
+ * APR_STRUCT_UNIT_MAP, as APR_STRUCT_TREE_NODE_MAP). A unit: 32 bytes {int32 first pure entry, first
+ * node entry, first other entry, first record; int16 pure entries, node entries, coarser particles among
+ * the other entries (first), other entries (the rest are empty slots), records, of which at the grid's
+ * edges (first), l - l_min, 0}. Pure entry: uint32 [4], a slot whose eight cells are level-l particles:
+ * word k = first particle of child row k (28 bits) | bits 4k .. 4k + 3 of the slot number << 28. Node
+ * entry: int32 [8] child map (as APR_STRUCT_TREE_NODE_MAP) and a uint32 info word. Other entry: uint32 [2]
+ * {particle index, info}. info: slot | mirror << 16 | missing << 20 (3-bit axis masks, z 4, x 2, y 1: the
+ * slot lies outside the grid and is its source's octet reversed along the axis; the source's second child
+ * along the axis lies outside the grid). Record: 24 bytes {uint32 node; uint16 edge; uint16 base[9]},
+ * base[3 (dz + 1) + dx + 1] = slot of the parent at (z + dz, x + dx, y - 1), the two after it at y and
+ * y + 1; edge: per axis (z bits 0-2, x, y) bit 0 first parent, bits 1-2 cells from the parent's first one
+ * to the grid's end if at most 3. Leaf units hold the level-(l-1) particles next to nodes: 32 bytes
+ * {uint32 particle; uint32 mask; uint16 edge; uint16 base[9]; uint32 0}, mask bit 3r + j = parent j of row
+ * r is a node; base[r] = the slot of the row's first one. */
+#define APR_STRUCT_UNIT_HDR 12
+#define APR_STRUCT_UNIT_PURE 13
+#define APR_STRUCT_UNIT_NODE 14
+#define APR_STRUCT_UNIT_NODE_INFO 15
+#define APR_STRUCT_UNIT_OTHER 16
+#define APR_STRUCT_UNIT_REC 17
+#define APR_STRUCT_UNIT_MAP 18
+#define APR_STRUCT_LEAF_HDR 19
+#define APR_STRUCT_LEAF_PURE 20
+#define APR_STRUCT_LEAF_NODE 21
+#define APR_STRUCT_LEAF_NODE_INFO 22
+#define APR_STRUCT_LEAF_REC 23
 
 /* Build the device-resident index of an APR (Sec. 3.1 LinearAccess for the particles, Sec. 3.4
  * APR tree structure, and the list of non-empty tiles the kernels are launched on, Sec. 5.2 last
  * paragraph). The tree structure (which nodes exist) is derived from the particle cells; its
- * values are computed later by apr_tree_restrict. y indices are stored as uint16. For every tile
- * the host also lists the non-empty source segments of its staged patch with the prefix of their
- * 8-element packets (tile plans, for stencil radius 1 and 2 and for the multi-channel sub-tiles),
- * so the convolution kernels never evaluate row offsets per call, and for every tree node the indices
- * of its children (32 bytes per node); on a 1024x1024x512 image with 8 M particles the handle holds
- * about 243 MB, plans included (the image itself would be 2.1 GB).
+ * values are computed later by apr_tree_restrict. y indices are stored as uint16. The host also builds
+ * what the kernels read instead of the rows: for every tree node the indices of its children (32 bytes
+ * per node), the convolution units (APR_STRUCT_UNIT_*: groups of parents with the parents around them)
+ * and the source segments of the multi-channel sub-tiles; on a 1024x1024x512 image with 8 M particles
+ * the handle holds about 280 MB, plans included (the image itself would be 2.1 GB).
  * The index is allocated stream-ordered (cudaMallocAsync on `stream`) and uploaded on `stream`;
  * it is ready for work enqueued on `stream` (other streams synchronise with it first). The handle
- * also creates two streams and four events for the concurrent parts of later calls, and 8 bytes of
- * mapped pinned host memory (the radius hint of apr_convolve). Returns
+ * also creates a stream and two events for the concurrent parts of apr_convolve_backward. Returns
  * APR_ERR_INVALID_LAYOUT when the arrays are inconsistent (row sizes, y order and range, and with
  * the flags the partition and the balance), APR_ERR_UNSUPPORTED for more than 2^28 particles or
  * tree nodes, APR_ERR_OOM on allocation failure. *out is NULL on error. */
@@ -172,13 +199,7 @@ apr_status_t apr_tree_restrict(apr_handle_t h, const float *particles, float *tr
  *   k: 3 or 5;  bc: APR_BC_REFLECT or APR_BC_ZERO;  out: device [N_p] float32, overwritten.
  * Requires the 2:1 balance of the APR (checked by APR_REQUIRE_BALANCE at build).
  * A level whose 5^3 stencil is zero outside the central 3^3 (every level below l_max of a restricted
- * stack, Eq. restrict_stenc) is computed with radius 1. For k = 5 the tiles of the levels below l_max
- * run on a second stream that the handle owns, in a launch sized for radius 1, beside the l_max tiles
- * on `stream` (forked from and joined back to `stream` with events: the call stays ordered on
- * `stream` and can be captured into a CUDA graph). When the previous call's stack had taps outside
- * the central 3^3 below l_max (read from a hint that the kernels write, without waiting), one launch
- * over all tiles is taken instead. Either way every output is computed by the same code, so results
- * do not depend on the choice. */
+ * stack, Eq. restrict_stenc) is computed with radius 1. */
 apr_status_t apr_convolve(apr_handle_t h, const float *particles, const float *tree, const float *stencils,
                           int32_t k, int32_t bc, float *out, apr_stream_t stream);
 
@@ -201,8 +222,7 @@ apr_status_t apr_convolve_adjoint_tiles(apr_handle_t h, const float *stencils, i
  * then convolution, Sec. 5.2). workspace: caller-owned device memory of at least
  * apr_convolve_auto_workspace_bytes(h) bytes, 16-byte aligned; it holds the tree values [N_t]
  * afterwards. APR_ERR_INVALID_ARG if it is missing or too small; otherwise as the two calls, with the
- * same results. When the convolution is split by radius (see apr_convolve), its l_max tiles read no
- * tree node, so their launch runs on the handle's second stream beside the restriction. */
+ * same results. */
 size_t apr_convolve_auto_workspace_bytes(apr_handle_t h);
 apr_status_t apr_convolve_auto(apr_handle_t h, const float *particles, const float *stencils, int32_t k, int32_t bc,
                                float *out, void *workspace, size_t workspace_bytes, apr_stream_t stream);
@@ -230,9 +250,8 @@ size_t apr_backward_workspace_bytes(apr_handle_t h, int32_t k);
  * least apr_backward_workspace_bytes(h, k) bytes, 256-byte aligned, contents ignored on entry.
  * Results are deterministic (fixed summation order).
  * When both gradients are requested, the stencil gradient runs on a second stream that the handle
- * owns, forked from `stream` and joined back to it with events, and the data adjoint takes its
- * launches as apr_convolve_adjoint does: the call stays ordered on `stream` (work enqueued after it
- * waits for both gradients) and can be captured into a CUDA graph from `stream`. Concurrent calls on
+ * owns, forked from `stream` and joined back to it with events: the call stays ordered on `stream`
+ * (work enqueued after it waits for both gradients) and can be captured into a CUDA graph from `stream`. Concurrent calls on
  * one handle are serialised while they enqueue. */
 apr_status_t apr_convolve_backward(apr_handle_t h, const float *particles, const float *tree,
                                    const float *stencils, int32_t k, int32_t bc, const float *grad_out,

@@ -155,7 +155,9 @@ class AprLayout:
 
     # ---- structure export (bit-exact checks)
     _EXPORT_DTYPES = {0: np.uint32, 1: np.uint16, 2: np.uint32, 3: np.uint16, 4: np.int32, 5: np.int32, 6: np.int32,
-                      7: np.int32, 8: np.uint32, 9: np.uint32, 10: np.uint32, 11: np.uint32}
+                      7: np.int32, 8: np.uint32, 9: np.uint32, 10: np.uint32, 11: np.uint32, 12: np.int16, 13: np.uint32,
+                      14: np.int32, 15: np.uint32, 16: np.uint32, 17: np.uint16, 18: np.int32, 19: np.int16,
+                      20: np.uint32, 21: np.int32, 22: np.uint32, 23: np.uint16}
 
     def export(self, which: int) -> np.ndarray:
         nbytes = int(self._lib.apr_structure_bytes(self._h, which))
@@ -164,8 +166,17 @@ class AprLayout:
         _abi.check("apr_export_structure",
                    self._lib.apr_export_structure(self._h, which, out.ctypes.data_as(ctypes.c_void_p), nbytes))
         out = out[:nbytes // np.dtype(dt).itemsize]
-        if which == 7:
+        if which in (7, 14, 18, 21):
             return out.reshape(-1, 8)
+        if which in (12, 19):    # unit headers: four int32, then eight int16
+            raw = out.reshape(-1, 16)
+            return np.concatenate([np.ascontiguousarray(raw[:, :8]).view(np.int32), raw[:, 8:].astype(np.int32)], axis=1)
+        if which in (17, 23):
+            return out.reshape(-1, 12 if which == 17 else 16)
+        if which in (13, 20):
+            return out.reshape(-1, 4)
+        if which in (15, 22):
+            return out
         if which >= 8:
             return out.reshape(-1, 2)
         return out.reshape(-1, 4) if which in (4, 5, 6) else out

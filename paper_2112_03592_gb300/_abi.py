@@ -18,6 +18,10 @@ APR_STRUCT_ROW_PTR, APR_STRUCT_Y_IDX, APR_STRUCT_TREE_ROW_PTR, APR_STRUCT_TREE_Y
 APR_STRUCT_FWD_ITEMS, APR_STRUCT_TREE_ITEMS, APR_STRUCT_BWD_ITEMS = 4, 5, 6
 APR_STRUCT_TREE_NODE_MAP = 7
 APR_STRUCT_FWD_PLAN_R1, APR_STRUCT_FWD_PLAN_R2, APR_STRUCT_BWD_PLAN_R1, APR_STRUCT_BWD_PLAN_R2 = 8, 9, 10, 11
+(APR_STRUCT_UNIT_HDR, APR_STRUCT_UNIT_PURE, APR_STRUCT_UNIT_NODE, APR_STRUCT_UNIT_NODE_INFO, APR_STRUCT_UNIT_OTHER,
+ APR_STRUCT_UNIT_REC, APR_STRUCT_UNIT_MAP) = range(12, 19)
+(APR_STRUCT_LEAF_HDR, APR_STRUCT_LEAF_PURE, APR_STRUCT_LEAF_NODE, APR_STRUCT_LEAF_NODE_INFO,
+ APR_STRUCT_LEAF_REC) = range(19, 24)
 APR_TILE_ZX, APR_BLOCK_Y = 8, 64  # work-item geometry, as in include/apr.h
 
 # every function include/apr.h declares, with (restype, argtypes)

@@ -1,6 +1,7 @@
 // C ABI entry points (include/apr.h): handle lifetime, upload of the index, kernel launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -10,27 +11,21 @@
 #include "apr_internal.h"
 
 namespace aprk {
-cudaError_t launch_conv_fwd(int k, const DevLayout &L, const Item *items, int n, const float *vals,
-                            const float *tree, const float *st, int bc, float *out, cudaStream_t s,
-                            int epi_mode = EPI_PLAIN, bool flip = false, const float *aux = nullptr, int tile0 = 0);
 cudaError_t launch_tree_restrict(const TreeNodePlan *np, int node0, int n, const float *vals, float *tree,
                                  cudaStream_t s, int C, int ch, bool pdl);
-cudaError_t launch_gradmag(int k, const DevLayout &L, const Item *items, int n, const float *vals, const float *tree,
-                           const float *st, int bc, float *out, cudaStream_t s);
-cudaError_t launch_bwd_data(int k, const DevLayout &L, const Item *items, int n, const float *st, int bc,
-                            const float *gout, float *gp, float *gt, cudaStream_t s, int tile0 = 0);
-cudaError_t launch_bwd_stencil(int k, const DevLayout &L, const Item *items, int n, const float *vals,
-                               const float *tree, int bc, const float *gout, float *partial, cudaStream_t s);
-cudaError_t launch_stencil_reduce(const float *partial, int n_items, const int64_t *level_begin, int l_min,
-                                  int n_levels, int K3, float *gw, cudaStream_t s);
 cudaError_t launch_tree_pushdown(const TreeNodePlan *np, int node0, int n, float *gp, float *gt, cudaStream_t s,
                                  bool pdl);
-cudaError_t launch_conv_fwd_split(const DevLayout &L, const Item *items, int n_lo, const LevelRanges &lo, int *hint,
-                                  const float *vals, const float *tree, const float *st, int bc, float *out,
-                                  cudaStream_t s, int epi_mode, bool flip, const float *aux);
-cudaError_t launch_bwd_data_split(const DevLayout &L, const Item *items, int n_lo, const LevelRanges &lo, int *hint,
-                                  const float *st, int bc, const float *gout, float *gp, float *gt, cudaStream_t s);
-cudaError_t launch_radius_hint(const DevLayout &L, const LevelRanges &lo, const float *st, int *hint, cudaStream_t s);
+// apr_units.cu
+cudaError_t launch_conv_fwd(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
+                            int bc, float *out, cudaStream_t s, int epi_mode = EPI_PLAIN, bool flip = false,
+                            const float *aux = nullptr, int first_tile = 0, int n_tiles = -1);
+cudaError_t launch_gradmag(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
+                           int n_levels, int bc, float *out, cudaStream_t s);
+cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, const float *gout, float *gp, float *gt,
+                           cudaStream_t s, int first_tile = 0, int n_tiles = -1);
+cudaError_t launch_stencil_grad(int k, const UnitView &U, const int32_t *level_begin, const bool *has, int n_levels,
+                                const float *vals, const float *tree, int bc, const float *gout, float *partial, int stride,
+                                float *gw, cudaStream_t s);
 }  // namespace aprk
 
 using namespace aprk;
@@ -92,117 +87,14 @@ void free_device(apr_handle_s *h) {
 
 bool stencil_k_ok(int32_t k) { return k == 3 || k == 5; }
 
-// Work-item ranges of the levels below l_max (begin: fwd_level_begin or bwd_level_begin).
-LevelRanges lower_levels(const HostIndex &X, const int64_t *begin) {
-    LevelRanges r;
-    r.l0 = X.l_min;
-    r.n = X.l_max - X.l_min;
-    for (int i = 0; i <= r.n; ++i) r.begin[i] = int32_t(begin[X.l_min + i]);
-    return r;
-}
-
-// `side` enqueues work on the handle's split stream, `main` on the caller's stream s: the split
-// stream is forked from s and joined back to it (also when a launch failed, so that a stream capture
-// of s ends joined).
-template <typename Side, typename Main>
-cudaError_t fork_join(apr_handle_t h, cudaStream_t s, Side side, Main main) {
-    std::lock_guard<std::mutex> lock(h->split_mu);
-    cudaError_t e = cudaSuccess;
-    if (!h->split) e = cudaStreamCreateWithFlags(&h->split, cudaStreamNonBlocking);
-    if (e == cudaSuccess && !h->ev_split_fork) e = cudaEventCreateWithFlags(&h->ev_split_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess && !h->ev_split_join) e = cudaEventCreateWithFlags(&h->ev_split_join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(h->ev_split_fork, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->split, h->ev_split_fork, 0);
-    if (e != cudaSuccess) return e;
-    const cudaError_t e_side = side(h->split);
-    const cudaError_t e_main = main(s);
-    e = cudaEventRecord(h->ev_split_join, h->split);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->ev_split_join, 0);
-    return e_side != cudaSuccess ? e_side : e_main != cudaSuccess ? e_main : e;
-}
-
-// Whether the last radius-split or hinted call of kind `which` (0 convolution, 1 data adjoint) saw a
-// level below l_max with taps outside the central 3^3 (read without waiting: it may be older).
-bool outer_taps_seen(apr_handle_t h, int which) {
-    return static_cast<volatile const int *>(h->h_hint)[which] != 0;
-}
-
-// apr_convolve over the whole forward work list (with the Richardson-Lucy epilogues). For k = 5 the
-// levels below l_max run split by radius on the split stream (launch_conv_fwd_split) beside the l_max
-// tiles, unless the last call's stack had taps outside the central 3^3 below l_max: then one launch
-// over all items, with the hint refreshed beside it. Either way every tile is computed the same way.
-cudaError_t conv_fwd_all(apr_handle_t h, int k, const float *vals, const float *tree, const float *st, int bc,
-                         float *out, cudaStream_t s, int epi_mode = EPI_PLAIN, bool flip = false,
-                         const float *aux = nullptr) {
-    const HostIndex &X = h->X;
-    const int n = int(X.fwd_items.size()), n_lo = int(X.fwd_level_begin[X.l_max]);
-    if (k != 5 || n_lo == 0)
-        return launch_conv_fwd(k, h->L, h->d_fwd, n, vals, tree, st, bc, out, s, epi_mode, flip, aux);
-    const LevelRanges lo = lower_levels(X, X.fwd_level_begin);
-    if (outer_taps_seen(h, 0))
-        return fork_join(
-            h, s, [&](cudaStream_t side) { return launch_radius_hint(h->L, lo, st, h->d_hint, side); },
-            [&](cudaStream_t main) { return launch_conv_fwd(k, h->L, h->d_fwd, n, vals, tree, st, bc, out, main, epi_mode, flip, aux); });
-    return fork_join(
-        h, s,
-        [&](cudaStream_t side) {
-            return launch_conv_fwd_split(h->L, h->d_fwd, n_lo, lo, h->d_hint, vals, tree, st, bc, out, side, epi_mode,
-                                         flip, aux);
-        },
-        [&](cudaStream_t main) {
-            return launch_conv_fwd(k, h->L, h->d_fwd, n - n_lo, vals, tree, st, bc, out, main, epi_mode, flip, aux, n_lo);
-        });
-}
-
-// The paper's forward pipeline (Sec. 5.2): the tree restriction of `vals` into `tree`, then
-// conv_fwd_all. When a 5^3 call is split by radius, its l_max tiles read no tree node (the tree ends
-// at level l_max - 1): their launch starts on the split stream beside the restriction, and the
-// levels below l_max follow the restriction on s.
+// The paper's forward pipeline (Sec. 5.2): the tree restriction of `vals` into `tree`, then the
+// convolution over every particle (with the Richardson-Lucy epilogues).
 apr_status_t restrict_then_conv(apr_handle_t h, int k, const float *vals, float *tree, const float *st, int bc,
                                 float *out, cudaStream_t s, int epi_mode = EPI_PLAIN, bool flip = false,
                                 const float *aux = nullptr) {
-    const HostIndex &X = h->X;
-    const int n = int(X.fwd_items.size()), n_lo = int(X.fwd_level_begin[X.l_max]);
-    if (k != 5 || n_lo == 0 || n_lo == n || outer_taps_seen(h, 0)) {
-        const apr_status_t r = apr_tree_restrict(h, vals, tree, 1, s);
-        if (r != APR_OK) return r;
-        return cuda_status(conv_fwd_all(h, k, vals, tree, st, bc, out, s, epi_mode, flip, aux));
-    }
-    const LevelRanges lo = lower_levels(X, X.fwd_level_begin);
-    apr_status_t r = APR_OK;
-    const cudaError_t e = fork_join(
-        h, s,
-        [&](cudaStream_t side) {
-            return launch_conv_fwd(k, h->L, h->d_fwd, n - n_lo, vals, tree, st, bc, out, side, epi_mode, flip, aux, n_lo);
-        },
-        [&](cudaStream_t main) {
-            r = apr_tree_restrict(h, vals, tree, 1, main);
-            if (r != APR_OK) return cudaSuccess;
-            return launch_conv_fwd_split(h->L, h->d_fwd, n_lo, lo, h->d_hint, vals, tree, st, bc, out, main, epi_mode,
-                                         flip, aux);
-        });
+    const apr_status_t r = apr_tree_restrict(h, vals, tree, 1, s);
     if (r != APR_OK) return r;
-    return cuda_status(e);
-}
-
-// The data adjoint over the whole adjoint work list; with `split`, k = 5 chooses its launches like
-// conv_fwd_all.
-cudaError_t bwd_data_all(apr_handle_t h, int k, const float *st, int bc, const float *gout, float *gp, float *gt,
-                         cudaStream_t s, bool split) {
-    const HostIndex &X = h->X;
-    const int n = int(X.bwd_items.size()), n_lo = int(X.bwd_level_begin[X.l_max]);
-    if (!split || k != 5 || n_lo == 0) return launch_bwd_data(k, h->L, h->d_bwd, n, st, bc, gout, gp, gt, s);
-    const LevelRanges lo = lower_levels(X, X.bwd_level_begin);
-    if (outer_taps_seen(h, 1))
-        return fork_join(
-            h, s, [&](cudaStream_t side) { return launch_radius_hint(h->L, lo, st, h->d_hint + 1, side); },
-            [&](cudaStream_t main) { return launch_bwd_data(k, h->L, h->d_bwd, n, st, bc, gout, gp, gt, main); });
-    return fork_join(
-        h, s,
-        [&](cudaStream_t side) {
-            return launch_bwd_data_split(h->L, h->d_bwd, n_lo, lo, h->d_hint + 1, st, bc, gout, gp, gt, side);
-        },
-        [&](cudaStream_t main) { return launch_bwd_data(k, h->L, h->d_bwd, n - n_lo, st, bc, gout, gp, gt, main, n_lo); });
+    return cuda_status(launch_conv_fwd(k, h->U, h->n_fwd_units, vals, tree, st, bc, out, s, epi_mode, flip, aux));
 }
 
 // The tree push-down (apr_tree_restrict_adjoint) of the tree levels [l0, l1] within [l_min, l_max - 1],
@@ -335,13 +227,50 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         if (e == cudaSuccess) e = upload(h, &h->d_fwd, X.fwd_items.data(), X.fwd_items.size());
         if (e == cudaSuccess) e = upload(h, &h->d_bwd, X.bwd_items.data(), X.bwd_items.size());
         if (e == cudaSuccess) e = upload(h, &h->d_tree, X.tree_items.data(), X.tree_items.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_tnplan, X.tnplan.data(), X.tnplan.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_fwd_level_begin, X.fwd_level_begin, size_t(MAXL + 1));
-        for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
-            const HostFPlan &P = i < 2 ? X.fplan[i] : X.bplan[i - 2];
-            e = upload(h, &h->d_fplan_hdr[i], P.hdr.data(), P.hdr.size());
-            if (e == cudaSuccess) e = upload(h, &h->d_fplan_ent[i], P.ent.data(), P.ent.size());
+        // child maps: the tree nodes, then the virtual parents of the cells of l_min
+        if (e == cudaSuccess) {
+            void *p = nullptr;
+            const size_t nb = X.tnplan.size() * sizeof(TreeNodePlan), vb = X.vplan.size() * sizeof(TreeNodePlan);
+            e = dev_alloc(h, &p, std::max<size_t>(nb + vb, sizeof(TreeNodePlan)));
+            h->d_tnplan = static_cast<TreeNodePlan *>(p);
+            const cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
+            if (e == cudaSuccess && nb) e = cudaMemcpyAsync(p, X.tnplan.data(), nb, cudaMemcpyHostToDevice, cs);
+            if (e == cudaSuccess && vb)
+                e = cudaMemcpyAsync(static_cast<char *>(p) + nb, X.vplan.data(), vb, cudaMemcpyHostToDevice, cs);
         }
+        const UnitPlan &UP = X.units;
+        UnitHdr *d_hdr = nullptr, *d_lhdr = nullptr;
+        uint4 *d_pure = nullptr, *d_lpure = nullptr;
+        TreeNodePlan *d_nmap = nullptr, *d_lnmap = nullptr;
+        uint32_t *d_ninfo = nullptr, *d_lninfo = nullptr;
+        uint2 *d_oth = nullptr;
+        NodeRec *d_rec = nullptr;
+        LeafRec *d_lrec = nullptr;
+        int32_t *d_tf = nullptr, *d_tb = nullptr, *d_ltb = nullptr;
+        if (e == cudaSuccess) e = upload(h, &d_hdr, UP.hdr.data(), UP.hdr.size());
+        if (e == cudaSuccess) e = upload(h, &d_lhdr, UP.lhdr.data(), UP.lhdr.size());
+        if (e == cudaSuccess) e = upload(h, &d_pure, UP.pure.data(), UP.pure.size());
+        if (e == cudaSuccess) e = upload(h, &d_lpure, UP.lpure.data(), UP.lpure.size());
+        if (e == cudaSuccess) e = upload(h, &d_nmap, UP.nmap.data(), UP.nmap.size());
+        if (e == cudaSuccess) e = upload(h, &d_lnmap, UP.lnmap.data(), UP.lnmap.size());
+        if (e == cudaSuccess) e = upload(h, &d_ninfo, UP.ninfo.data(), UP.ninfo.size());
+        if (e == cudaSuccess) e = upload(h, &d_lninfo, UP.lninfo.data(), UP.lninfo.size());
+        if (e == cudaSuccess) e = upload(h, &d_oth, UP.oth.data(), UP.oth.size());
+        if (e == cudaSuccess) e = upload(h, &d_rec, UP.rec.data(), UP.rec.size());
+        if (e == cudaSuccess) e = upload(h, &d_lrec, UP.lrec.data(), UP.lrec.size());
+        if (e == cudaSuccess) e = upload(h, &d_tf, UP.tile_f.data(), UP.tile_f.size());
+        if (e == cudaSuccess) e = upload(h, &d_tb, UP.tile_b.data(), UP.tile_b.size());
+        if (e == cudaSuccess) e = upload(h, &d_ltb, UP.ltile_b.data(), UP.ltile_b.size());
+        h->U = UnitView{d_hdr, d_lhdr, d_pure, d_lpure, d_nmap, d_lnmap, d_ninfo, d_lninfo, d_oth, d_rec, d_lrec, d_tf, d_tb, d_ltb, h->d_tnplan,
+                        int32_t(UP.hdr.size()), int32_t(UP.lhdr.size())};
+        h->n_fwd_units = 0;
+        for (int i = X.l_max - X.l_min; i >= 0; --i) {   // finest first
+            const int l = X.l_min + i;
+            h->level_has[i] = X.fwd_level_begin[l + 1] > X.fwd_level_begin[l];
+            h->unit_begin[i] = UP.level_begin[i];
+            if (h->level_has[i]) h->n_fwd_units = i == 0 ? int(UP.hdr.size()) : UP.level_begin[i - 1];
+        }
+        h->complete = UP.complete;
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
             const HostPlan &P = i == 0 ? X.mcfplan : X.mcbplan;
             e = upload(h, &h->d_plan_hdr[i], P.hdr.data(), P.hdr.size());
@@ -381,33 +310,21 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         L.l_min = X.l_min;
         L.l_max = X.l_max;
         for (int l = 0; l < MAXL; ++l) L.geo[l] = X.geo[l];
-        for (int i = 0; i < 2; ++i) {
-            L.fplan[i] = FPlanView{h->d_fplan_hdr[i], h->d_fplan_ent[i]};
-            L.bplan[i] = FPlanView{h->d_fplan_hdr[2 + i], h->d_fplan_ent[2 + i]};
-        }
         L.mcfplan = PlanView{h->d_plan_hdr[0], h->d_plan_ent[0]};
         L.mcbplan = PlanView{h->d_plan_hdr[1], h->d_plan_ent[1]};
         // the plans live on the device now; the host copies are not needed again
-        for (int i = 0; i < 2; ++i) {
-            h->X.fplan[i] = HostFPlan{};
-            h->X.bplan[i] = HostFPlan{};
-        }
         h->X.mcfplan = HostPlan{};
         h->X.mcbplan = HostPlan{};
         h->X.tnplan = std::vector<TreeNodePlan>{};
-        // the second streams of apr_convolve_backward and of the radius split, and their events, are
-        // made here, so that no later call creates them inside a stream capture
+        h->X.vplan = std::vector<TreeNodePlan>{};
+        h->X.vrow_ptr = std::vector<uint32_t>{};
+        h->X.vy = std::vector<uint16_t>{};
+        h->X.units = UnitPlan{};
+        // the second stream of apr_convolve_backward and its events are made here, so that no later call
+        // creates them inside a stream capture
         e = cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->split, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_split_fork, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_split_join, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaHostAlloc(reinterpret_cast<void **>(&h->h_hint), 2 * sizeof(int), cudaHostAllocMapped);
-        if (e == cudaSuccess) {
-            h->h_hint[0] = h->h_hint[1] = 0;
-            e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&h->d_hint), h->h_hint, 0);
-        }
         if (e != cudaSuccess) {
             st = cuda_status(e);
             apr_destroy(h);
@@ -426,10 +343,6 @@ apr_status_t apr_destroy(apr_handle_t h) {
         if (h->ev_fork) cudaEventDestroy(h->ev_fork);
         if (h->ev_join) cudaEventDestroy(h->ev_join);
         if (h->side) cudaStreamDestroy(h->side);
-        if (h->ev_split_fork) cudaEventDestroy(h->ev_split_fork);
-        if (h->ev_split_join) cudaEventDestroy(h->ev_split_join);
-        if (h->split) cudaStreamDestroy(h->split);
-        if (h->h_hint) cudaFreeHost(h->h_hint);
     }
     delete h;
     return APR_OK;
@@ -454,17 +367,60 @@ const HostFPlan *host_plan(apr_handle_t h, int32_t which) {
     if (!h->host_only || which < APR_STRUCT_FWD_PLAN_R1 || which > APR_STRUCT_BWD_PLAN_R2) return nullptr;
     std::lock_guard<std::mutex> lk(h->plan_mu);
     if (!h->host_plans) {
-        if (build_plans(h->X) != APR_OK) return nullptr;
+        if (build_tile_plans(h->X) != APR_OK) return nullptr;
         h->host_plans = true;
     }
     const int i = which - APR_STRUCT_FWD_PLAN_R1;
     return i < 2 ? &h->X.fplan[i] : &h->X.bplan[i - 2];
+}
+
+// One array of the convolution units of a host-only handle (built once, on request).
+bool host_unit_array(apr_handle_t h, int32_t which, const void **src, size_t *bytes) {
+    *src = nullptr;
+    *bytes = 0;
+    if (!h->host_only) return true;
+    {
+        std::lock_guard<std::mutex> lk(h->plan_mu);
+        if (!h->host_units) {
+            try {
+                build_units(h->X);
+            } catch (const std::bad_alloc &) {
+                return false;
+            }
+            h->host_units = true;
+        }
+    }
+    const UnitPlan &U = h->X.units;
+    auto give = [&](const auto &v) {
+        *src = v.data();
+        *bytes = v.size() * sizeof(v[0]);
+    };
+    switch (which) {
+        case APR_STRUCT_UNIT_HDR: give(U.hdr); break;
+        case APR_STRUCT_UNIT_OTHER: give(U.oth); break;
+        case APR_STRUCT_UNIT_REC: give(U.rec); break;
+        case APR_STRUCT_UNIT_MAP: give(h->X.vplan); break;
+        case APR_STRUCT_LEAF_HDR: give(U.lhdr); break;
+        case APR_STRUCT_LEAF_REC: give(U.lrec); break;
+        case APR_STRUCT_UNIT_PURE: give(U.pure); break;
+        case APR_STRUCT_LEAF_PURE: give(U.lpure); break;
+        case APR_STRUCT_UNIT_NODE: give(U.nmap); break;
+        case APR_STRUCT_LEAF_NODE: give(U.lnmap); break;
+        case APR_STRUCT_UNIT_NODE_INFO: give(U.ninfo); break;
+        case APR_STRUCT_LEAF_NODE_INFO: give(U.lninfo); break;
+    }
+    return true;
 }
 }  // namespace
 
 size_t apr_structure_bytes(apr_handle_t h, int32_t which) {
     if (!h) return 0;
     const HostIndex &X = h->X;
+    if (which >= APR_STRUCT_UNIT_HDR && which <= APR_STRUCT_LEAF_REC) {
+        const void *src;
+        size_t n;
+        return host_unit_array(h, which, &src, &n) ? n : 0;
+    }
     if (which >= APR_STRUCT_FWD_PLAN_R1 && which <= APR_STRUCT_BWD_PLAN_R2) {
         const HostFPlan *P = host_plan(h, which);
         return P ? (P->hdr.size() + P->ent.size()) * sizeof(uint2) : 0;
@@ -485,9 +441,16 @@ size_t apr_structure_bytes(apr_handle_t h, int32_t which) {
 apr_status_t apr_export_structure(apr_handle_t h, int32_t which, void *dst, size_t bytes) {
     if (!h || (!dst && bytes)) return APR_ERR_INVALID_ARG;
     const size_t need = apr_structure_bytes(h, which);
-    if (which < APR_STRUCT_ROW_PTR || which > APR_STRUCT_BWD_PLAN_R2) return APR_ERR_INVALID_ARG;
+    if (which < APR_STRUCT_ROW_PTR || which > APR_STRUCT_LEAF_REC) return APR_ERR_INVALID_ARG;
     if (bytes < need) return APR_ERR_INVALID_ARG;
     if (need == 0) return APR_OK;
+    if (which >= APR_STRUCT_UNIT_HDR) {  // host-only handle (need > 0)
+        const void *src;
+        size_t n;
+        if (!host_unit_array(h, which, &src, &n)) return APR_ERR_OOM;
+        memcpy(dst, src, n);
+        return APR_OK;
+    }
     if (which >= APR_STRUCT_FWD_PLAN_R1) {  // host-only handle (need > 0)
         const HostFPlan *P = host_plan(h, which);
         memcpy(dst, P->hdr.data(), P->hdr.size() * sizeof(PlanHdr));
@@ -544,7 +507,7 @@ apr_status_t apr_convolve(apr_handle_t h, const float *particles, const float *t
     if (bc != APR_BC_REFLECT && bc != APR_BC_ZERO) return APR_ERR_INVALID_ARG;
     if (!stencils || (h->X.np && (!particles || !out)) || (h->X.nt && !tree)) return APR_ERR_INVALID_ARG;
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
-    return cuda_status(conv_fwd_all(h, k, particles, tree, stencils, bc, out, stream));
+    return cuda_status(launch_conv_fwd(k, h->U, h->n_fwd_units, particles, tree, stencils, bc, out, stream));
 }
 
 apr_status_t apr_convolve_tiles(apr_handle_t h, const float *particles, const float *tree, const float *stencils,
@@ -557,8 +520,8 @@ apr_status_t apr_convolve_tiles(apr_handle_t h, const float *particles, const fl
     if (first_tile < 0 || n_tiles < 0 || first_tile + n_tiles > nt) return APR_ERR_INVALID_ARG;
     if (!stencils || (h->X.np && (!particles || !out)) || (h->X.nt && !tree)) return APR_ERR_INVALID_ARG;
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
-    return cuda_status(launch_conv_fwd(k, h->L, h->d_fwd, int(n_tiles), particles, tree, stencils, bc, out, stream,
-                                       EPI_PLAIN, false, nullptr, int(first_tile)));
+    return cuda_status(launch_conv_fwd(k, h->U, h->n_fwd_units, particles, tree, stencils, bc, out, stream, EPI_PLAIN, false,
+                                       nullptr, int(first_tile), int(n_tiles)));
 }
 
 apr_status_t apr_convolve_adjoint_tiles(apr_handle_t h, const float *stencils, int32_t k, int32_t bc,
@@ -571,8 +534,8 @@ apr_status_t apr_convolve_adjoint_tiles(apr_handle_t h, const float *stencils, i
     const int64_t nt = int64_t(X.bwd_items.size());
     if (first_tile < 0 || n_tiles < 0 || first_tile + n_tiles > nt) return APR_ERR_INVALID_ARG;
     if (!stencils || (X.np && (!grad_out || !grad_particles)) || (X.nt && !grad_tree)) return APR_ERR_INVALID_ARG;
-    return cuda_status(launch_bwd_data(k, h->L, h->d_bwd, int(n_tiles), stencils, bc, grad_out, grad_particles,
-                                       grad_tree, stream, int(first_tile)));
+    return cuda_status(launch_adjoint(k, h->U, stencils, bc, grad_out, grad_particles, grad_tree, stream, int(first_tile),
+                                      int(n_tiles)));
 }
 
 size_t apr_convolve_auto_workspace_bytes(apr_handle_t h) {
@@ -599,8 +562,8 @@ apr_status_t apr_gradient_magnitude(apr_handle_t h, const float *particles, cons
     if (bc != APR_BC_REFLECT && bc != APR_BC_ZERO) return APR_ERR_INVALID_ARG;
     if (!stencils || (h->X.np && (!particles || !out)) || (h->X.nt && !tree)) return APR_ERR_INVALID_ARG;
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
-    const int n = int(h->X.fwd_items.size());
-    return cuda_status(launch_gradmag(k, h->L, h->d_fwd, n, particles, tree, stencils, bc, out, stream));
+    return cuda_status(launch_gradmag(k, h->U, h->n_fwd_units, particles, tree, stencils, h->X.l_max - h->X.l_min + 1, bc, out,
+                                      stream));
 }
 
 size_t apr_backward_workspace_bytes(apr_handle_t h, int32_t k) {
@@ -611,7 +574,18 @@ size_t apr_backward_workspace_bytes(apr_handle_t h, int32_t k) {
 
 apr_status_t apr_convolve_adjoint(apr_handle_t h, const float *stencils, int32_t k, int32_t bc, const float *grad_out,
                                   float *grad_particles, float *grad_tree, apr_stream_t stream) {
-    return aprk::convolve_adjoint(h, stencils, k, bc, grad_out, grad_particles, grad_tree, stream, true);
+    if (!h || h->host_only) return APR_ERR_INVALID_ARG;
+    if (!stencil_k_ok(k)) return APR_ERR_UNSUPPORTED;
+    if (bc != APR_BC_REFLECT && bc != APR_BC_ZERO) return APR_ERR_INVALID_ARG;
+    const HostIndex &X = h->X;
+    if (!stencils || (X.np && (!grad_out || !grad_particles)) || (X.nt && !grad_tree)) return APR_ERR_INVALID_ARG;
+    // the units store the gradient of every particle and tree node; only in an index in which some have
+    // no record (a layout that was not validated) are the arrays cleared first
+    cudaError_t e = cudaSuccess;
+    if (!h->complete && X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * sizeof(float), stream);
+    if (!h->complete && e == cudaSuccess && X.nt) e = cudaMemsetAsync(grad_tree, 0, size_t(X.nt) * sizeof(float), stream);
+    if (e == cudaSuccess) e = launch_adjoint(k, h->U, stencils, bc, grad_out, grad_particles, grad_tree, stream);
+    return cuda_status(e);
 }
 
 apr_status_t apr_tree_restrict_adjoint(apr_handle_t h, float *grad_tree, float *grad_particles, apr_stream_t stream) {
@@ -641,32 +615,14 @@ apr_status_t apr_convolve_stencil_grad(apr_handle_t h, const float *particles, c
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
     const size_t need = apr_stencil_grad_workspace_bytes(h, k);
     if (need && (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255))) return APR_ERR_INVALID_ARG;
-    const int n = int(X.fwd_items.size());
-    float *partial = static_cast<float *>(workspace);
-    cudaError_t e = launch_bwd_stencil(k, h->L, h->d_fwd, n, particles, tree, bc, grad_out, partial, stream);
-    if (e == cudaSuccess)
-        e = launch_stencil_reduce(partial, n, h->d_fwd_level_begin, X.l_min, X.l_max - X.l_min + 1, k * k * k, grad_stencils, stream);
-    return cuda_status(e);
+    return cuda_status(launch_stencil_grad(k, h->U, h->unit_begin, h->level_has, X.l_max - X.l_min + 1, particles, tree, bc,
+                                           grad_out, static_cast<float *>(workspace), int(X.fwd_items.size()),
+                                           grad_stencils, stream));
 }
 
 }  // extern "C"
 
 namespace aprk {
-apr_status_t convolve_adjoint(apr_handle_t h, const float *stencils, int32_t k, int32_t bc, const float *grad_out,
-                              float *grad_particles, float *grad_tree, apr_stream_t stream, bool split) {
-    if (!h || h->host_only) return APR_ERR_INVALID_ARG;
-    if (!stencil_k_ok(k)) return APR_ERR_UNSUPPORTED;
-    if (bc != APR_BC_REFLECT && bc != APR_BC_ZERO) return APR_ERR_INVALID_ARG;
-    const HostIndex &X = h->X;
-    if (!stencils || (X.np && (!grad_out || !grad_particles)) || (X.nt && !grad_tree)) return APR_ERR_INVALID_ARG;
-    cudaError_t e = cudaSuccess;
-    if (X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * sizeof(float), stream);
-    if (e == cudaSuccess && X.nt) e = cudaMemsetAsync(grad_tree, 0, size_t(X.nt) * sizeof(float), stream);
-    if (e == cudaSuccess)
-        e = bwd_data_all(h, k, stencils, bc, grad_out, grad_particles, grad_tree, stream, split);
-    return cuda_status(e);
-}
-
 apr_status_t convolve_backward(apr_handle_t h, const float *particles, const float *tree, const float *stencils,
                                int32_t k, int32_t bc, const float *grad_out, float *grad_particles,
                                float *grad_stencils, void *workspace, size_t workspace_bytes, apr_stream_t stream,
@@ -698,7 +654,7 @@ apr_status_t convolve_backward(apr_handle_t h, const float *particles, const flo
         if (e != cudaSuccess) return cuda_status(e);
         const apr_status_t sg = apr_convolve_stencil_grad(h, particles, tree, k, bc, grad_out, grad_stencils, partial,
                                                           workspace_bytes - gt_bytes, reinterpret_cast<apr_stream_t>(h->side));
-        st = convolve_adjoint(h, stencils, k, bc, grad_out, grad_particles, gt, stream, true);
+        st = apr_convolve_adjoint(h, stencils, k, bc, grad_out, grad_particles, gt, stream);
         if (st == APR_OK) st = apr_tree_restrict_adjoint(h, gt, grad_particles, stream);
         // always joined, so that a stream capture of the caller's stream ends joined
         e = cudaEventRecord(h->ev_join, h->side);
@@ -708,7 +664,7 @@ apr_status_t convolve_backward(apr_handle_t h, const float *particles, const flo
         return st;
     }
     if (grad_particles) {
-        st = convolve_adjoint(h, stencils, k, bc, grad_out, grad_particles, gt, stream, concurrent);
+        st = apr_convolve_adjoint(h, stencils, k, bc, grad_out, grad_particles, gt, stream);
         if (st == APR_OK) st = apr_tree_restrict_adjoint(h, gt, grad_particles, stream);
     }
     if (st == APR_OK && grad_stencils)

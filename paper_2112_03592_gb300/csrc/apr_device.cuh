@@ -24,12 +24,6 @@ __device__ __forceinline__ void block_sync() {
     __syncthreads();
 }
 
-// Barrier of the two warps 2g and 2g+1 (named barrier 1 + g; barrier 0 is the block barrier).
-__device__ __forceinline__ void pair_sync(int g) {
-    __syncwarp();
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(64) : "memory");
-}
-
 __host__ __device__ __forceinline__ int imax(int a, int b) { return a > b ? a : b; }
 __host__ __device__ __forceinline__ int imin(int a, int b) { return a < b ? a : b; }
 
@@ -100,24 +94,6 @@ __device__ inline void block_scan2(int c0, int c1, int n, int *pre, int *warp_to
     if (tid == 0) pre[n] = warp_tot[NWARP];
     block_sync();
 }
-
-struct SlotYV {
-    int y;
-    float v;
-};
-
-// Loads y and value of element i of segment seg; segments [t0, t1) are tree segments.
-struct YVLoader {
-    using Slot = SlotYV;
-    const uint16_t *py, *ty;
-    const float *pv, *tv;
-    int t0, t1;
-    __device__ __forceinline__ void operator()(int seg, int i, Slot &s) const {
-        const bool t = seg >= t0 && seg < t1;
-        s.y = t ? int(ty[i]) : int(py[i]);
-        s.v = t ? tv[i] : pv[i];
-    }
-};
 
 // Programmatic dependent launch (launch_pdl): pdl_trigger lets the next kernel on the stream start
 // (its blocks run their prologue while this kernel finishes); pdl_wait blocks until the kernel before

@@ -64,13 +64,75 @@ struct HostPlan {
     std::vector<PlanHdr> hdr;
     std::vector<PlanEnt> ent;
 };
-struct FPlanView {     // forward tile plans (apr_tile.cuh: FPlanEnt)
-    const PlanHdr *hdr;
-    const uint2 *ent;
-};
 struct HostFPlan {
     std::vector<PlanHdr> hdr;
     std::vector<uint2> ent;
+};
+
+// Convolution units (built once per APR by build_units, apr_unitplan.cpp): groups of parents ("records")
+// with the list of the parents around them ("slots"), see there. All units of a level are consecutive,
+// the finest level first.
+constexpr int UNIT_RECS = 256;    // most records of a unit
+constexpr int UNIT_SLOTS = 1280;  // most slots of a unit
+struct alignas(16) UnitHdr {
+    int32_t pure0, node0, oth0, rec0;  // first pure, node and other entry, first record
+    int16_t npure;                // slots whose eight cells are particles of the level
+    int16_t nnode;                // the other slots that are nodes
+    int16_t nleaf, noth;          // coarser particles; with the empty slots after them
+    int16_t nrec, nflag;          // records; the first nflag lie at the level grid's edges
+    int16_t lev, pad;             // l - l_min of the child cells
+};
+static_assert(sizeof(UnitHdr) == 32, "unit headers are two 16-byte words");
+// Pure entry: word k = first particle of child row k (28 bits; the second follows it) | 4 bits of the slot
+// number << 28 (bits 4k .. 4k + 3 of it). One 16-byte load gives a slot's eight sources.
+// Node entry: the child map of a slot that is not pure (a copy, so that no load depends on an index), and
+// its info word. Other entry: x = particle index (coarser particles), y = info word.
+// info: slot number (11 bits) | mirror bits << UE_MIRROR | missing bits << UE_MISS, each 3 bits (z 4, x 2,
+// y 1). mirror: the slot lies outside the grid along that axis, its children are the source's in
+// reversed order; missing: the source's second child along that axis lies outside the grid.
+constexpr int UE_MIRROR = 16, UE_MISS = 20;
+constexpr unsigned UE_SLOT = 0x7ffu;
+// A record: a parent whose children are computed, and the slot of the y - 1 neighbour in each of the
+// nine rows (z + dz, x + dx) around it. edge: per axis (z bits 0-2, x 3-5, y 6-8) bit 0 = first parent,
+// bits 1-2 = child cells from the parent's first one to the grid's end if at most 3, else 0.
+struct alignas(8) NodeRec {
+    uint32_t node;
+    uint16_t edge;
+    uint16_t base[9];
+};
+static_assert(sizeof(NodeRec) == 24, "node records are three 8-byte words");
+// A level-(l-1) particle next to nodes, as a coarse source of level l: mask bit 3r + j = neighbour j of
+// row r is a node (a slot); base[r] = slot of the row's first such neighbour.
+struct alignas(16) LeafRec {
+    uint32_t particle, mask;
+    uint16_t edge;
+    uint16_t base[9];
+    uint32_t pad;
+};
+static_assert(sizeof(LeafRec) == 32, "leaf records are two 16-byte words");
+struct UnitPlan {                          // host
+    std::vector<UnitHdr> hdr, lhdr;        // node units, leaf units
+    std::vector<uint4> pure, lpure;        // entries: pure slots, other nodes, the rest
+    std::vector<TreeNodePlan> nmap, lnmap;
+    std::vector<uint32_t> ninfo, lninfo;
+    std::vector<uint2> oth;
+    std::vector<NodeRec> rec;
+    std::vector<LeafRec> lrec;
+    std::vector<int32_t> tile_f, tile_b, ltile_b;  // work item of each record (-1: none): forward, adjoint
+    int32_t level_begin[MAXL + 1] = {};    // first node unit of level l_min + i
+    bool complete = false;                 // every particle and tree node is the child of a record
+};
+struct UnitView {                          // device
+    const UnitHdr *hdr, *lhdr;
+    const uint4 *pure, *lpure;
+    const TreeNodePlan *nmap, *lnmap;
+    const uint32_t *ninfo, *lninfo;
+    const uint2 *oth;
+    const NodeRec *rec;
+    const LeafRec *lrec;
+    const int32_t *tile_f, *tile_b, *ltile_b;
+    const TreeNodePlan *nplan;             // child maps: tree nodes, then virtual parents
+    int32_t n, nl;                         // node units, leaf units
 };
 
 // Everything a kernel needs to walk the index (device pointers).
@@ -85,8 +147,6 @@ struct DevLayout {
     int32_t np, nt;            // particles, tree nodes (value array lengths)
     int32_t l_min, l_max;
     LevelGeo geo[MAXL];
-    FPlanView fplan[2];  // forward tiles (fwd_items), stencil radius 1 and 2
-    FPlanView bplan[2];  // data-adjoint tiles (bwd_items), stencil radius 1 and 2
     PlanView mcfplan;    // multi-channel feature patches of the sub-tiles of fwd_items
     PlanView mcbplan;    // multi-channel data-adjoint sub-tiles of bwd_items
 };
@@ -113,6 +173,10 @@ struct HostIndex {
     HostFPlan bplan[2];                       // data-adjoint tile plans (build_plans), radius 1 and 2
     HostPlan mcfplan, mcbplan;                // multi-channel sub-tile plans (build_mc_plans)
     std::vector<TreeNodePlan> tnplan;         // child maps of the tree nodes (tree_node_plan)
+    std::vector<uint32_t> vrow_ptr;           // virtual parents of the cells of l_min: rows, y, child maps
+    std::vector<uint16_t> vy;
+    std::vector<TreeNodePlan> vplan;
+    UnitPlan units;                           // convolution units (build_units)
 };
 
 // The tree nodes of level l (l_min <= l < l_max): [b, b + n) in tree order.
@@ -122,31 +186,23 @@ inline void tree_level_nodes(const HostIndex &X, int l, int64_t &b, int64_t &n) 
     n = int64_t(X.trow_ptr[size_t(g.trow0) + size_t(g.dz) * size_t(g.dx)]) - b;
 }
 
-// Work items of the consecutive levels l0 .. l0 + n - 1: level l0 + i owns items [begin[i], begin[i + 1])
-// (passed to kernels by value).
-struct LevelRanges {
-    int32_t l0 = 0, n = 0;
-    int32_t begin[MAXL + 1] = {};
-};
-
 // Builds and validates the index from the host layout. Returns APR_OK or an error code; `msg`
 // receives a short reason on failure.
 apr_status_t build_index(const apr_host_layout &L, uint32_t flags, HostIndex &out, const char **msg);
 
-// Builds the tile plans of X's forward and data-adjoint work items (apr_plan.cu) and the
-// multi-channel sub-tile plans. Returns APR_OK, APR_ERR_OOM (host allocation) or
-// APR_ERR_UNSUPPORTED (a tile with 65536 or more staged elements).
+// Builds what a device handle's kernels read (apr_plan.cu): the convolution units, the child maps and
+// the multi-channel sub-tile plans. Returns APR_OK, APR_ERR_OOM (host allocation) or APR_ERR_UNSUPPORTED.
 apr_status_t build_plans(HostIndex &X);
+// Builds the tile plans of X's forward and data-adjoint work items (apr_export_structure).
+apr_status_t build_tile_plans(HostIndex &X);
+// The convolution units of X (after tree_node_plan); throws std::bad_alloc.
+void build_units(HostIndex &X);
 // The multi-channel sub-tile plans (apr_mc.cu); true unless a tile overflows the 16-bit counts.
 bool build_mc_plans(const DevLayout &L, const HostIndex &X, HostPlan &feat, HostPlan &adj);
 // The child map of every tree node (TreeNodePlan), by one merge of each tree row with its child rows.
 // In a complete index every in-grid child cell of a node is a particle or a node of the next level.
 bool tree_node_plan(const DevLayout &L, const HostIndex &X, std::vector<TreeNodePlan> &P);
-// apr_convolve_adjoint; split: a 5^3 stack's levels below l_max on the handle's split stream
-apr_status_t convolve_adjoint(apr_handle_t h, const float *stencils, int32_t k, int32_t bc, const float *grad_out,
-                              float *grad_particles, float *grad_tree, apr_stream_t stream, bool split);
-// apr_convolve_backward; concurrent: the stencil gradient on the handle's second stream and the
-// data adjoint split by radius
+// apr_convolve_backward; concurrent: the stencil gradient on the handle's second stream
 apr_status_t convolve_backward(apr_handle_t h, const float *particles, const float *tree, const float *stencils,
                                int32_t k, int32_t bc, const float *grad_out, float *grad_particles,
                                float *grad_stencils, void *workspace, size_t workspace_bytes, apr_stream_t stream,
@@ -203,7 +259,6 @@ struct apr_handle_s {
     bool host_only = false;
     aprk::DevLayout L{};
     aprk::Item *d_fwd = nullptr, *d_bwd = nullptr, *d_tree = nullptr;
-    int64_t *d_fwd_level_begin = nullptr;
     uint32_t *d_row_ptr = nullptr, *d_trow_ptr = nullptr;
     uint16_t *d_y = nullptr, *d_ty = nullptr, *d_off = nullptr, *d_toff = nullptr;
     unsigned *d_err = nullptr;
@@ -218,23 +273,16 @@ struct apr_handle_s {
     aprk::TreeNodePlan *d_tnplan = nullptr;
     // host-only handles: tile plans built on the first apr_export_structure request for them
     std::mutex plan_mu;
-    bool host_plans = false;
-    aprk::PlanHdr *d_fplan_hdr[4] = {};   // forward radius 1, 2; adjoint radius 1, 2
-    uint2 *d_fplan_ent[4] = {};
+    bool host_plans = false, host_units = false;
+    aprk::UnitView U{};   // convolution units; those of the levels down to the coarsest one with particles
+    int n_fwd_units = 0;
+    int32_t unit_begin[aprk::MAXL + 1] = {};   // first unit of level l_min + i
+    bool level_has[aprk::MAXL + 1] = {};       // whether level l_min + i holds particles
+    bool complete = false;                     // every particle and tree node is the child of a record
     size_t dev_bytes = 0;
     // apr_convolve_backward runs the stencil gradient on a second stream, forked from and joined back
     // to the caller's stream with these events (created on first use; side_mu orders the enqueues)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::mutex side_mu;
-    // a 5^3 convolution or data adjoint over the whole work list runs its radius-1 tiles of the
-    // levels below l_max on this stream, beside the l_max tiles on the caller's stream (split_mu
-    // orders the enqueues; taken after side_mu where both are held)
-    cudaStream_t split = nullptr;
-    cudaEvent_t ev_split_fork = nullptr, ev_split_join = nullptr;
-    std::mutex split_mu;
-    // whether the last such call saw a level below l_max with taps outside the central 3^3 ([0]
-    // convolution, [1] data adjoint): mapped host memory that the kernels write and the host reads to
-    // choose the next call's launches (h_hint host view, d_hint device view)
-    int *h_hint = nullptr, *d_hint = nullptr;
 };

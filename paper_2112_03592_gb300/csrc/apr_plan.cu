@@ -1,9 +1,8 @@
-// Tile plans (host): for every forward and data-adjoint work item and both stencil radii, the
-// non-empty source segments of the item's patch, listed once per APR so that the kernels read them
-// with one coalesced load instead of evaluating every row's offsets (and a block scan) per call.
-// The segments are those of fwd_segment / bwd_segment (apr_tile.cuh), evaluated here on the host
-// copy of the index; forward entries carry the prefix of their 8-element packets. The multi-channel
-// sub-tile plans come from build_mc_plans (apr_mc.cu).
+// Host builders of what the kernels read: the child maps of the tree nodes (tree_node_plan) and, through
+// build_units (apr_unitplan.cpp) and build_mc_plans (apr_mc.cu), the convolution units and the multi-channel
+// sub-tile plans. Also the tile plans that apr_export_structure gives: for every forward and data-adjoint
+// work item and both stencil radii the non-empty source segments of the item's patch (fwd_segment,
+// bwd_segment in apr_tile.cuh), with the prefix of their 8-element packets.
 #include <functional>
 #include <thread>
 #include <vector>
@@ -171,42 +170,56 @@ bool tree_node_plan(const DevLayout &L, const HostIndex &X, std::vector<TreeNode
     return true;
 }
 
-apr_status_t build_plans(HostIndex &X) {
-    const DevLayout L = host_layout_view(X);
-    if (X.np >= FPLAN_MAX_INDEX || X.nt >= FPLAN_MAX_INDEX) return APR_ERR_UNSUPPORTED;
-    apr_status_t st[6] = {APR_OK, APR_OK, APR_OK, APR_OK, APR_OK, APR_OK};
-    auto guarded = [&st](int i, auto f) {
-        return [&st, i, f] {
-            try {
-                if (!f()) st[i] = APR_ERR_UNSUPPORTED;
-            } catch (...) {  // host allocation failure
-                st[i] = APR_ERR_OOM;
-            }
-        };
+namespace {
+
+// Runs the jobs, one thread each (a job whose thread cannot be started runs here).
+apr_status_t run_jobs(std::vector<std::function<bool()>> jobs) {
+    std::vector<apr_status_t> st(jobs.size(), APR_OK);
+    auto guarded = [&](size_t i) {
+        try {
+            if (!jobs[i]()) st[i] = APR_ERR_UNSUPPORTED;
+        } catch (...) {  // host allocation failure
+            st[i] = APR_ERR_OOM;
+        }
     };
-    std::function<void()> jobs[6] = {guarded(0, [&] { return fwd_plan<1>(L, X.fwd_items, X.fplan[0]); }),
-                                     guarded(1, [&] { return fwd_plan<2>(L, X.fwd_items, X.fplan[1]); }),
-                                     guarded(2, [&] { return bwd_plan<1>(L, X.bwd_items, X.bplan[0]); }),
-                                     guarded(3, [&] { return bwd_plan<2>(L, X.bwd_items, X.bplan[1]); }),
-                                     guarded(4, [&] { return build_mc_plans(L, X, X.mcfplan, X.mcbplan); }),
-                                     guarded(5, [&] { return tree_node_plan(L, X, X.tnplan); })};
-    // one thread per plan; a job whose thread cannot be started runs here
     std::vector<std::thread> threads;
     try {
-        threads.reserve(6);
+        threads.reserve(jobs.size());
     } catch (...) {  // the jobs then run here
     }
-    for (auto &job : jobs) {
+    for (size_t i = 0; i < jobs.size(); ++i) {
         try {
-            threads.emplace_back(job);
+            threads.emplace_back(guarded, i);
         } catch (...) {
-            job();
+            guarded(i);
         }
     }
     for (auto &th : threads) th.join();
     for (apr_status_t s : st)
         if (s != APR_OK) return s;
     return APR_OK;
+}
+
+}  // namespace
+
+apr_status_t build_plans(HostIndex &X) {
+    const DevLayout L = host_layout_view(X);
+    if (X.np >= FPLAN_MAX_INDEX || X.nt >= FPLAN_MAX_INDEX) return APR_ERR_UNSUPPORTED;
+    return run_jobs({[&] { return build_mc_plans(L, X, X.mcfplan, X.mcbplan); },
+                     [&] {
+                         if (!tree_node_plan(L, X, X.tnplan)) return false;
+                         build_units(X);
+                         return true;
+                     }});
+}
+
+apr_status_t build_tile_plans(HostIndex &X) {
+    const DevLayout L = host_layout_view(X);
+    if (X.np >= FPLAN_MAX_INDEX || X.nt >= FPLAN_MAX_INDEX) return APR_ERR_UNSUPPORTED;
+    return run_jobs({[&] { return fwd_plan<1>(L, X.fwd_items, X.fplan[0]); },
+                     [&] { return fwd_plan<2>(L, X.fwd_items, X.fplan[1]); },
+                     [&] { return bwd_plan<1>(L, X.bwd_items, X.bplan[0]); },
+                     [&] { return bwd_plan<2>(L, X.bwd_items, X.bplan[1]); }});
 }
 
 }  // namespace aprk

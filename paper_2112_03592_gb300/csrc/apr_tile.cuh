@@ -1,6 +1,5 @@
-// Geometry of a convolution tile and the source segments of its staged patch. Shared by the kernels
-// (apr_kernels.cu) and the host builder of the tile plans (apr_plan.cu): both sides use these
-// definitions, so a plan lists exactly the segments a kernel would compute.
+// Geometry of an 8 x 8 x 64-cell work item and the source segments of its patch, as the tile plans that
+// apr_export_structure gives list them (apr_plan.cu).
 #pragma once
 
 #include "apr_device.cuh"
@@ -9,47 +8,24 @@
 namespace aprk {
 namespace dev {
 
-constexpr int WIN = 8;                 // y cells per compute window
-constexpr int NWIN = BY / WIN;         // windows per interior row
 constexpr int NIR = TZ * TX;           // interior rows of a tile
-constexpr int NIW = NIR * NWIN;        // window slots of a tile
-static_assert(NIW == 2 * NT, "window slots are scanned two per thread");
 
 template <int R>
 struct Geo {
-    static constexpr int K = 2 * R + 1;
-    static constexpr int K3 = K * K * K;
-    static constexpr int NPAIR = K * K;                    // (dz, dx) pairs
     static constexpr int PZ = TZ + 2 * R, PX = TX + 2 * R, PY = BY + 2 * R;
-    static constexpr int PYS = (PY + 3) / 4 * 4;           // row stride, 16-byte multiple
     static constexpr int NROW = PZ * PX;
     static constexpr int NSEG = 3 * NROW;                  // particle, tree, coarser-particle source per row
     static constexpr int NCZ = ((TZ + R - 1) >> 1) + ((R + 1) >> 1) + 1;  // level-(l-1) rows per axis under a patch
     static constexpr int NRSEG = 2 * NIR + NIR / 4;        // backward routing: particles, tree, coarser particles
-    static_assert(WIN + 2 * R <= 12, "a window's taps must fit three 16-byte loads");
-    static_assert((NWIN - 1) * WIN + 12 <= PYS, "window loads stay inside the row");
-    static_assert(NSEG <= 2 * NT && NROW + NRSEG <= 2 * NT, "segments are scanned two per thread");
     static_assert(NCZ * NCZ <= NROW && PZ < 15 && PX < 15, "once-staged coarse rows: segment count, 4-bit row fields");
     static_assert(NROW < 256 && NIR < 127 && NROW + NRSEG < 65536, "meta fields: 8-bit patch row, 7-bit interior row");
 };
 
 // meta of a forward segment of kinds 0-2: patch row | kind << 8, plus META_REFL if the patch row lies
 // outside the grid (the segment holds the reflected row; with zero boundary it is empty); kind 3:
-// (first covered patch row z + 1) | (x + 1) << 4 | 3 << 8. These 11 bits are what a plan stores;
-// with_trow adds (interior row + 1) << 11 for the particle segments of interior rows.
+// (first covered patch row z + 1) | (x + 1) << 4 | 3 << 8. These 11 bits are what a plan stores.
 constexpr int META_REFL = 1 << 10;
 __host__ __device__ __forceinline__ int meta_kind(int meta) { return (meta >> 8) & 3; }
-__host__ __device__ __forceinline__ int meta_trow(int meta) { return ((meta >> 11) & 127) - 1; }
-
-template <int R>
-__host__ __device__ __forceinline__ int with_trow(const LevelGeo &g, const Item &it, int meta) {
-    using G = Geo<R>;
-    if (meta_kind(meta) != 0) return meta;
-    const int pr = meta & 255;
-    const int a = pr / G::PX - R, b = pr % G::PX - R;
-    const bool target = a >= 0 && a < TZ && b >= 0 && b < TX && it.a * TZ + a < g.dz && it.b * TX + b < g.dx;
-    return target ? meta | ((a * TX + b + 1) << 11) : meta;
-}
 
 // Forward tile plans: per work item and stencil radius, the non-empty segments of fwd_segment in
 // segment order, each with the prefix of 8-element packets before it (the packets of segment

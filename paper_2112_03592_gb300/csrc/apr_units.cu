@@ -679,9 +679,9 @@ __device__ __noinline__ void edge_images(const UnitView &U, const UnitHdr &h, Ad
     const int first = before + incl - n;
     S.first[tid] = first;
     __syncthreads();
-    float sum[8];
+    float sum[8], own[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) sum[c] = 0.f;
+    for (int c = 0; c < 8; ++c) sum[c] = own[c] = 0.f;
 #pragma unroll 1
     for (int k0 = 0; k0 < total; k0 += UT) {
         const int k = k0 + tid;
@@ -711,11 +711,20 @@ __device__ __noinline__ void edge_images(const UnitView &U, const UnitHdr &h, Ad
         if (live)
             for (int q = a; q < b; ++q)
 #pragma unroll
-                for (int c = 0; c < 8; ++c) sum[c] += S.H[c][q];
+                for (int c = 0; c < 8; ++c) {
+                    if (ATOMIC && k0 + q == first) own[c] = S.H[c][q];
+                    else sum[c] += S.H[c][q];
+                }
         __syncthreads();
     }
     if (live && n > 0) {
+        // own sums and images are added in the same order either way: the results agree bit for bit
         fold_missing(rec[tid].edge, sum);
+        if (ATOMIC) {
+            fold_missing(rec[tid].edge, own);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sum[c] = own[c] + sum[c];
+        }
         emit_children<ATOMIC>(U, rec[tid].node, sum, !ATOMIC, gp, gt);
     }
 }

@@ -136,6 +136,25 @@ def recorded_traffic(call, section=None):
     return rec.get("dram_bytes_per_call", {}).get(call)
 
 
+def tree_launches(apr, lay, max_levels=4):
+    """Kernels of one tree restriction (or push-down): consecutive levels share a launch, from the coarsest
+    one up, as long as the deepest has at most 2^17 entries (8 per node and level in between)."""
+    rp = lay.export(2)   # APR_STRUCT_TREE_ROW_PTR
+    nodes, r = [], 0
+    for l in range(apr.l_min, apr.l_max):
+        dz, dx, _ = apr.level_dims(l)
+        nodes.append(int(rp[r + dz * dx]) - int(rp[r]))
+        r += dz * dx
+    n, i = 0, 0
+    while i < len(nodes):
+        g = 1
+        while g < max_levels and i + g < len(nodes) and nodes[i] << (3 * g) <= 1 << 17:
+            g += 1
+        n += nodes[i] > 0
+        i += g
+    return n
+
+
 def make_replayers(fns, use_graph):
     """The step's parts as CUDA graphs (one graph per part, replayed on the current stream), so the
     timed region has no host launch gaps; the plain callables when use_graph is false. Each part
@@ -450,11 +469,10 @@ def run_ours(args, rank, world):
     peaks, src = _peaks()
     hbm = float(peaks["hbm_gbs"])
     pix_bytes = float(np.prod(apr.dims)) * 4.0
-    # our kernels per step: restriction (one per level holding tree nodes), convolution, convolution
-    # adjoint (node units, leaf units), push-down (one per level holding tree nodes), stencil-gradient
-    # partials, reduction
-    n_tree_levels = len(set(lay.export(G._abi.APR_STRUCT_TREE_ITEMS)[:, 0].tolist()))
-    launches_per_step = n_tree_levels + 1 + 2 + n_tree_levels + 2
+    # our kernels per step: restriction, convolution, convolution adjoint (node units, leaf units),
+    # push-down, stencil-gradient partials, reduction
+    n_tree = tree_launches(apr, lay)
+    launches_per_step = n_tree + 1 + 2 + n_tree + 2
     # the dominant call of the step: the convolution adjoint. Its algorithmic bytes equal the forward's:
     # dL/dout in, dL/dparticles and dL/dtree out, y indices and row pointers.
     dom_ms, dom_call = (adj_ms, "apr_convolve_adjoint") if adj_ms >= conv_ms else (conv_ms, "apr_convolve")
@@ -683,10 +701,9 @@ def run_mc(args, rank, world, full=True):
     names = ["tree_restrict_bf16", "convolve_mc", "data_adjoint", "weight_grad"]
     dom = max(range(1, 4), key=lambda j: parts[j])
     mc_traffic = recorded_traffic(names[dom], "mc")
-    n_tree_levels = len(set(lay.export(G._abi.APR_STRUCT_TREE_ITEMS)[:, 0].tolist()))
-    # per step: BF16 tree (one launch per level), weight layout + forward, weight layout + data
-    # adjoint, push-down (one per level), weight gradient + its reduction
-    launches_per_step = n_tree_levels + 2 + 2 + n_tree_levels + 2
+    # per step: BF16 tree, weight layout + forward, weight layout + data adjoint, push-down, weight
+    # gradient + its reduction
+    launches_per_step = tree_launches(apr, lay) + 2 + 2 + tree_launches(apr, lay, 3) + 2
     rec = {
         "metric": "APR conv Gparticles/s & pixel-equiv GB/s",
         "value": round(world * Np / (step_ms * 1e-3) / 1e9, 4), "unit": "Gparticles/s",
@@ -885,7 +902,7 @@ def run_rl(args, rank, world, full=True):
     conv_bytes += Np * 4   # the fused epilogue reads one more value per particle
     peaks, src = _peaks()
     hbm = float(peaks["hbm_gbs"])
-    n_tree_levels = len(set(lay.export(G._abi.APR_STRUCT_TREE_ITEMS)[:, 0].tolist()))
+    n_tree = tree_launches(apr, lay)
     pix = float(np.prod(apr.dims))
     rec = {
         "metric": "APR conv Gparticles/s & pixel-equiv GB/s",
@@ -907,7 +924,7 @@ def run_rl(args, rank, world, full=True):
                      "frac": round(conv_bytes / (conv_ms * 1e-3) / 1e9 / hbm, 4), "traffic": None,
                      "peak_source": src + " (hbm_gbs)", "algorithmic_bytes_per_launch": conv_bytes,
                      "conv_ms": round(conv_ms, 5)},
-        "gpu_launches": RL_ITERS * 2 * (n_tree_levels + 1) * args.steps,
+        "gpu_launches": RL_ITERS * 2 * (n_tree + 1) * args.steps,
     }
     if not full:
         return rec
@@ -1056,7 +1073,7 @@ def run_surrogate(args, rank, world, pretrained=None):
 
     rl_ms = timed(run_rl_)
     cnn_ms = timed(run_cnn)
-    n_tree_levels = len(set(lay.export(G._abi.APR_STRUCT_TREE_ITEMS)[:, 0].tolist()))
+    n_tree = tree_launches(apr, lay)
     y = holder[0]
     wts = torch.as_tensor(pixels_per_particle(apr), device=dev)
     ref_clean = torch.as_tensor(clean.values, device=dev)
@@ -1079,8 +1096,8 @@ def run_surrogate(args, rank, world, pretrained=None):
                      "data_s": round(t_data, 1), "train_s": round(t_train, 1)},
         # per CNN inference: embedding, 4 x (tree restriction per level, weight layout, convolution;
         # hidden ReLUs fused into the convolution), read-out; per RL run: 2 x (tree + convolution) per iteration
-        "gpu_launches": (2 + 4 * (n_tree_levels + 2) +
-                         RL_ITERS * 2 * (n_tree_levels + 1)) * args.steps,
+        "gpu_launches": (2 + 4 * (n_tree + 2) +
+                         RL_ITERS * 2 * (n_tree + 1)) * args.steps,
     }
     return rec
 

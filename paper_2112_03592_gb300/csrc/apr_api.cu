@@ -11,10 +11,9 @@
 #include "apr_internal.h"
 
 namespace aprk {
-cudaError_t launch_tree_restrict(const TreeNodePlan *np, int node0, int n, const float *vals, float *tree,
-                                 cudaStream_t s, int C, int ch, bool pdl);
-cudaError_t launch_tree_pushdown(const TreeNodePlan *np, int node0, int n, float *gp, float *gt, cudaStream_t s,
-                                 bool pdl);
+cudaError_t launch_tree_restrict(const TreeNodePlan *np, const TreeGroup &g, const float *vals, float *tree, cudaStream_t s,
+                                 int C, int ch, bool pdl);
+cudaError_t launch_tree_pushdown(const TreeNodePlan *np, const TreeGroup &g, float *gp, float *gt, cudaStream_t s, bool pdl);
 // apr_units.cu
 cudaError_t launch_conv_fwd(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
                             int bc, float *out, cudaStream_t s, int epi_mode = EPI_PLAIN, bool flip = false,
@@ -98,7 +97,7 @@ apr_status_t restrict_then_conv(apr_handle_t h, int k, const float *vals, float 
 }
 
 // The tree push-down (apr_tree_restrict_adjoint) of the tree levels [l0, l1] within [l_min, l_max - 1],
-// coarsest first, one launch per level.
+// coarsest first.
 apr_status_t pushdown_levels(apr_handle_t h, float *grad_tree, float *grad_particles, int l0, int l1,
                              cudaStream_t s) {
     const HostIndex &X = h->X;
@@ -107,11 +106,10 @@ apr_status_t pushdown_levels(apr_handle_t h, float *grad_tree, float *grad_parti
     if (l1 > X.l_max - 1) l1 = X.l_max - 1;
     cudaError_t e = cudaSuccess;
     bool chained = false;   // the launches after the first start early (programmatic dependent launch)
-    for (int l = l0; e == cudaSuccess && l <= l1; ++l) {
-        int64_t b = 0, n = 0;
-        tree_level_nodes(X, l, b, n);
-        e = launch_tree_pushdown(h->d_tnplan, int(b), int(n), grad_particles, grad_tree, s, chained);
-        chained = chained || n > 0;
+    const TreeGroups T = tree_groups(X, l0, l1, 4);
+    for (int i = 0; i < T.n && e == cudaSuccess; ++i) {
+        e = launch_tree_pushdown(h->d_tnplan, T.g[i], grad_particles, grad_tree, s, chained);
+        chained = true;
     }
     return cuda_status(e);
 }
@@ -124,6 +122,19 @@ apr_status_t misaligned() {
 }  // namespace
 
 namespace aprk {
+TreeGroups tree_groups(const HostIndex &X, int l0, int l1, int max_levels) {
+    TreeGroups out;
+    for (int l = l0; l <= l1;) {
+        int64_t b = 0, n = 0;
+        tree_level_nodes(X, l, b, n);
+        int g = 1;
+        while (g < max_levels && l + g <= l1 && (n << (3 * g)) <= tree_group_threads) ++g;
+        if (n > 0) out.g[out.n++] = TreeGroup{int32_t(b), int32_t(n), g};
+        l += g;
+    }
+    return out;
+}
+
 void set_last_message(const char *msg) { snprintf(g_last_msg, sizeof(g_last_msg), "%s", msg); }
 
 cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes) {
@@ -487,13 +498,11 @@ apr_status_t apr_tree_restrict(apr_handle_t h, const float *particles, float *tr
     if ((!particles && h->X.np) || (!tree && h->X.nt)) return APR_ERR_INVALID_ARG;
     const HostIndex &X = h->X;
     bool chained = false;   // the launches after the first start early (programmatic dependent launch)
-    for (int l = X.l_max - 1; l >= X.l_min; --l) {
-        int64_t b = 0, n = 0;
-        tree_level_nodes(X, l, b, n);
+    const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 4);
+    for (int i = T.n - 1; i >= 0; --i) {   // the finest group first
         for (int c = 0; c < channels; ++c) {  // channels-last values: one strided pass per channel
-            cudaError_t e = launch_tree_restrict(h->d_tnplan, int(b), int(n), particles, tree, stream, channels, c,
-                                                 chained);
-            chained = chained || n > 0;
+            const cudaError_t e = launch_tree_restrict(h->d_tnplan, T.g[i], particles, tree, stream, channels, c, chained);
+            chained = true;
             if (e != cudaSuccess) return cuda_status(e);
         }
     }

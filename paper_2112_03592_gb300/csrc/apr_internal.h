@@ -186,6 +186,22 @@ inline void tree_level_nodes(const HostIndex &X, int l, int64_t &b, int64_t &n) 
     n = int64_t(X.trow_ptr[size_t(g.trow0) + size_t(g.dz) * size_t(g.dx)]) - b;
 }
 
+// Consecutive tree levels taken by one launch (apr_kernels.cu): `levels` of them from the coarsest one,
+// whose nodes are [node0, node0 + n).
+struct TreeGroup {
+    int32_t node0, n, levels;
+};
+// The groups of the tree levels [l0, l1] (within [l_min, l_max - 1]), coarsest first: each takes as many
+// levels (at most max_levels) as keep its deepest level at or below tree_group_threads entries.
+// 2^17 entries are less than half of what is resident at once; with 2^20 a group's idle threads cost more than
+// the launches it saves (16-channel restriction of 1 M particles 28 -> 50 us, push-down of 8 M 45 -> 84 us at 2^22).
+constexpr int64_t tree_group_threads = int64_t(1) << 17;
+struct TreeGroups {
+    int n = 0;
+    TreeGroup g[MAXL];
+};
+TreeGroups tree_groups(const HostIndex &X, int l0, int l1, int max_levels);
+
 // Builds and validates the index from the host layout. Returns APR_OK or an error code; `msg`
 // receives a short reason on failure.
 apr_status_t build_index(const apr_host_layout &L, uint32_t flags, HostIndex &out, const char **msg);

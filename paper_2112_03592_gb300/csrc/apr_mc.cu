@@ -26,6 +26,12 @@
 #include "apr_internal.h"
 
 namespace aprk {
+
+// apr_kernels.cu
+cudaError_t launch_tree_restrict_bf16(const TreeNodePlan *np, const TreeGroup &g, const uint16_t *vals, uint16_t *tree,
+                                      cudaStream_t s, bool pdl);
+cudaError_t launch_tree_pushdown16(const TreeNodePlan *np, const TreeGroup &g, float *gp, float *gt, cudaStream_t s, bool pdl);
+
 namespace {
 
 using namespace dev;
@@ -541,111 +547,6 @@ __device__ __forceinline__ void store_weights(const uint4 (&w)[4], unsigned char
     for (int k = 0; k < 4; ++k)
         if (threadIdx.x + k * NT < WV) reinterpret_cast<uint4 *>(wsm)[threadIdx.x + k * NT] = w[k];
     fence_async_smem();
-}
-
-// ---------------------------------------------------------------- BF16 tree restriction
-// One level of the tree restriction for 16 bf16 channels, one thread per (tree node, 8-channel half):
-// the node's children from its child map (TreeNodePlan, apr_internal.h), summed in FP32 in (a, b, e)
-// order, divided by their count in FP32, rounded to bf16 (round to nearest even).
-__global__ void __launch_bounds__(NT) mc_tree_restrict_kernel(const TreeNodePlan *__restrict__ nplan, int node0, int n,
-                                                              const uint4 *__restrict__ vals, uint4 *tree) {
-    pdl_trigger();
-    const int q = int(blockIdx.x) * NT + int(threadIdx.x);
-    const int i = q >> 1, half = q & 1;
-    const bool live = i < n;
-    // the child map is static: read before waiting for the finer level's restriction (the launch
-    // before this one), whose node values this level reads
-    int4 pw = make_int4(0, 0, 0, 0), tw = pw;
-    if (live) {
-        const int4 *m = reinterpret_cast<const int4 *>(nplan + node0 + i);
-        pw = __ldg(m);
-        tw = __ldg(m + 1);
-    }
-    pdl_wait();
-    if (!live) return;
-    const int pv[4] = {pw.x, pw.y, pw.z, pw.w}, tv[4] = {tw.x, tw.y, tw.z, tw.w};
-    uint4 h[8];
-    bool has[8];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const unsigned pm = unsigned(pv[k]) >> 30, tm = unsigned(tv[k]) >> 30;
-        const int pi = int(unsigned(pv[k]) & TNP_INDEX), ti = int(unsigned(tv[k]) & TNP_INDEX);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            // the second child of a kind follows the first of that kind
-            const bool isp = (pm >> e) & 1u, ist = (tm >> e) & 1u;
-            const int ix = isp ? pi + (e ? int(pm & 1u) : 0) : ti + (e ? int(tm & 1u) : 0);
-            has[2 * k + e] = isp || ist;
-            h[2 * k + e] = isp ? vals[2 * size_t(ix) + half] : (ist ? tree[2 * size_t(ix) + half] : make_uint4(0u, 0u, 0u, 0u));
-        }
-    }
-    float acc[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = 0.0f;
-    int cnt = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        if (!has[k]) continue;
-        ++cnt;
-        const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(&h[k]);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float2 f = __bfloat1622float2(p[c]);
-            acc[2 * c] = __fadd_rn(acc[2 * c], f.x);
-            acc[2 * c + 1] = __fadd_rn(acc[2 * c + 1], f.y);
-        }
-    }
-    const float nf = float(cnt ? cnt : 1);
-    uint4 o;
-    __nv_bfloat162 *r = reinterpret_cast<__nv_bfloat162 *>(&o);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) r[c] = __floats2bfloat162_rn(__fdiv_rn(acc[2 * c], nf), __fdiv_rn(acc[2 * c + 1], nf));
-    tree[2 * size_t(node0 + i) + half] = o;
-}
-
-// Transpose of the tree restriction for 16 FP32 gradient channels, one level (coarse to fine), one
-// thread per (tree node, 4-channel group): every child (particle or tree node of level l+1) gets its
-// parent's gradient / #children added. Every child has one parent, so each is written by one thread.
-__global__ void __launch_bounds__(NT) mc_tree_pushdown_kernel(const TreeNodePlan *__restrict__ nplan, int node0, int n,
-                                                              float4 *gp, float4 *gt) {
-    pdl_trigger();
-    const int q = int(blockIdx.x) * NT + int(threadIdx.x);
-    const int i = q >> 2, cg = q & 3;
-    const bool live = i < n;
-    // the child map is static: read before waiting for the coarser level's push-down (the launch
-    // before this one), which writes this level's gradients
-    int4 pw = make_int4(0, 0, 0, 0), tw = pw;
-    if (live) {
-        const int4 *m = reinterpret_cast<const int4 *>(nplan + node0 + i);
-        pw = __ldg(m);
-        tw = __ldg(m + 1);
-    }
-    pdl_wait();
-    if (!live) return;
-    const int pv[4] = {pw.x, pw.y, pw.z, pw.w}, tv[4] = {tw.x, tw.y, tw.z, tw.w};
-    float4 *dst[8];
-    float4 v[8];
-    int cnt = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const unsigned pm = unsigned(pv[k]) >> 30, tm = unsigned(tv[k]) >> 30;
-        const int pi = int(unsigned(pv[k]) & TNP_INDEX), ti = int(unsigned(tv[k]) & TNP_INDEX);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const bool isp = (pm >> e) & 1u, ist = (tm >> e) & 1u;
-            const int ix = isp ? pi + (e ? int(pm & 1u) : 0) : ti + (e ? int(tm & 1u) : 0);
-            dst[2 * k + e] = isp ? gp + size_t(ix) * (MC / 4) + cg : (ist ? gt + size_t(ix) * (MC / 4) + cg : nullptr);
-            cnt += (isp || ist) ? 1 : 0;
-        }
-    }
-    const float4 g = gt[size_t(node0 + i) * (MC / 4) + cg];
-    const float f = float(cnt ? cnt : 1);
-    const float4 s = make_float4(g.x / f, g.y / f, g.z / f, g.w / f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = dst[k] ? *dst[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-        if (dst[k]) *dst[k] = make_float4(v[k].x + s.x, v[k].y + s.y, v[k].z + s.z, v[k].w + s.w);
 }
 
 // ---------------------------------------------------------------- forward
@@ -1378,14 +1279,10 @@ apr_status_t apr_tree_restrict_bf16(apr_handle_t h, const uint16_t *particles, u
     if ((X.np && !particles) || (X.nt && !tree) || !aligned16(particles) || !aligned16(tree)) return APR_ERR_INVALID_ARG;
     cudaError_t e = cudaSuccess;
     bool chained = false;   // the launches after the first start early (programmatic dependent launch)
-    for (int l = X.l_max - 1; e == cudaSuccess && l >= X.l_min; --l) {
-        int64_t b = 0, n = 0;
-        tree_level_nodes(X, l, b, n);
-        if (n > 0)
-            e = launch_pdl(mc_tree_restrict_kernel, dim3(int((2 * n + NT - 1) / NT)), dim3(NT), 0, stream, chained,
-                           h->d_tnplan, int(b), int(n), reinterpret_cast<const uint4 *>(particles),
-                           reinterpret_cast<uint4 *>(tree));
-        chained = chained || n > 0;
+    const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 4);
+    for (int i = T.n - 1; i >= 0 && e == cudaSuccess; --i) {   // the finest group first
+        e = launch_tree_restrict_bf16(h->d_tnplan, T.g[i], particles, tree, stream, chained);
+        chained = true;
     }
     return cuda_status(e);
 }
@@ -1468,14 +1365,10 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
             e = cudaGetLastError();
         }
         bool chained = false;   // the launches after the first start early (programmatic dependent launch)
-        for (int l = X.l_min; e == cudaSuccess && l < X.l_max; ++l) {
-            int64_t b = 0, nt = 0;
-            tree_level_nodes(X, l, b, nt);
-            if (nt > 0)
-                e = launch_pdl(mc_tree_pushdown_kernel, dim3(int((4 * nt + NT - 1) / NT)), dim3(NT), 0, stream, chained,
-                               h->d_tnplan, int(b), int(nt), reinterpret_cast<float4 *>(grad_particles),
-                               reinterpret_cast<float4 *>(gt));
-            chained = chained || nt > 0;
+        const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
+        for (int i = 0; i < T.n && e == cudaSuccess; ++i) {
+            e = launch_tree_pushdown16(h->d_tnplan, T.g[i], grad_particles, gt, stream, chained);
+            chained = true;
         }
     }
     if (e == cudaSuccess && grad_weights) {

@@ -102,11 +102,14 @@ class ClockSampler:
                 else "warm-up and timed region (timed region shorter than the 50 ms sampling period)"}
 
 
-TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_units.cu", "paper_2112_03592_gb300/csrc/apr_unitplan.cpp",
-                   "paper_2112_03592_gb300/csrc/apr_kernels.cu", "paper_2112_03592_gb300/csrc/apr_device.cuh"]
+TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_units.cu", "paper_2112_03592_gb300/csrc/apr_units.cuh",
+                   "paper_2112_03592_gb300/csrc/apr_unitplan.cpp", "paper_2112_03592_gb300/csrc/apr_kernels.cu",
+                   "paper_2112_03592_gb300/csrc/apr_device.cuh"]
 
 
-MC_TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_mc.cu", "paper_2112_03592_gb300/csrc/apr_device.cuh"]
+MC_TRAFFIC_SOURCES = ["paper_2112_03592_gb300/csrc/apr_mc.cu", "paper_2112_03592_gb300/csrc/apr_units.cuh",
+                      "paper_2112_03592_gb300/csrc/apr_unitplan.cpp", "paper_2112_03592_gb300/csrc/apr_kernels.cu",
+                      "paper_2112_03592_gb300/csrc/apr_device.cuh"]
 
 
 def kernel_source_hash(sources=None):
@@ -535,7 +538,7 @@ def run_ours(args, rank, world):
         "clocks": clocks,
         "wall_s_timed_region": round(wall, 4),
         "layout_bytes": lay.layout_bytes(),
-        "layout_build_s": round(t_build, 3),   # once per APR: validation, index, work lists, tile plans, upload
+        "layout_build_s": round(t_build, 3),   # once per APR: validation, index, work lists, convolution units, upload
     }
     # the plain method on the same APR (Sec. 4.1): the 5^3 Gaussian itself at every level (radius 2
     # everywhere), the same step, buffers and timing
@@ -701,9 +704,9 @@ def run_mc(args, rank, world, full=True):
     names = ["tree_restrict_bf16", "convolve_mc", "data_adjoint", "weight_grad"]
     dom = max(range(1, 4), key=lambda j: parts[j])
     mc_traffic = recorded_traffic(names[dom], "mc")
-    # per step: BF16 tree, weight layout + forward, weight layout + data adjoint, push-down, weight
-    # gradient + its reduction
-    launches_per_step = tree_launches(apr, lay) + 2 + 2 + tree_launches(apr, lay, 3) + 2
+    # per step: BF16 tree, weight layout + forward, weight layout + data adjoint (node units, leaf units),
+    # push-down, weight gradient + its reduction
+    launches_per_step = tree_launches(apr, lay) + 2 + 3 + tree_launches(apr, lay, 3) + 2
     rec = {
         "metric": "APR conv Gparticles/s & pixel-equiv GB/s",
         "value": round(world * Np / (step_ms * 1e-3) / 1e9, 4), "unit": "Gparticles/s",
@@ -718,7 +721,7 @@ def run_mc(args, rank, world, full=True):
                    "launch": "CUDA graphs (one per part)" if not args.no_graph else "eager",
                    "parallelism": f"replicas x{world}"},
         "step_ms_parts": {n: round(t, 5) for n, t in zip(names, parts)},
-        "roofline": {"kernel": {1: "mc_fwd_kernel (apr_convolve_mc)", 2: "mc_bwd_data_kernel (+ push-down)",
+        "roofline": {"kernel": {1: "mc_fwd_kernel (apr_convolve_mc)", 2: "mc_adjoint_kernel, mc_leaf_adjoint_kernel (+ push-down)",
                                 3: "mc_wgrad_kernel (+ reduce)"}[dom],
                      "bound": "hbm", "achieved": round(byts / (parts[dom] * 1e-3) / 1e9, 2), "peak": hbm, "unit": "GB/s",
                      "frac": round(byts / (parts[dom] * 1e-3) / 1e9 / hbm, 4), "traffic": mc_traffic,
@@ -918,8 +921,7 @@ def run_rl(args, rank, world, full=True):
                    "l2": "flushed before every step (512 MB write, outside the step events)",
                    "parallelism": f"replicas x{world}"},
         "pixel_equiv_GBps_per_conv": round(pix * 4 * 2 * RL_ITERS / (step_ms * 1e-3) / 1e9, 2),
-        "roofline": {"kernel": "apr_convolve (one call timed alone: conv_fwd_r1_kernel beside conv_fwd_kernel<2>, "
-                               "conv_fwd_r2_pool_kernel)", "bound": "hbm",
+        "roofline": {"kernel": "unit_conv_kernel<2> (one apr_convolve call timed alone)", "bound": "hbm",
                      "achieved": round(conv_bytes / (conv_ms * 1e-3) / 1e9, 2), "peak": hbm, "unit": "GB/s",
                      "frac": round(conv_bytes / (conv_ms * 1e-3) / 1e9 / hbm, 4), "traffic": None,
                      "peak_source": src + " (hbm_gbs)", "algorithmic_bytes_per_launch": conv_bytes,

@@ -22,7 +22,7 @@ cudaError_t launch_gradmag(int k, const UnitView &U, int n_units, const float *v
                            int n_levels, int bc, float *out, cudaStream_t s);
 cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, const float *gout, float *gp, float *gt,
                            cudaStream_t s, int first_tile = 0, int n_tiles = -1);
-cudaError_t launch_stencil_grad(int k, const UnitView &U, const int32_t *level_begin, const bool *has, int n_levels,
+cudaError_t launch_stencil_grad(int k, const UnitView &U, const UnitLevels &W, const UnitRanges &R, int blocks, int n_levels,
                                 const float *vals, const float *tree, int bc, const float *gout, float *partial, int stride,
                                 float *gw, cudaStream_t s);
 }  // namespace aprk
@@ -135,6 +135,36 @@ TreeGroups tree_groups(const HostIndex &X, int l0, int l1, int max_levels) {
     return out;
 }
 
+int unit_levels(apr_handle_t h, int max_blocks, UnitLevels &L, UnitRanges &R) {
+    const int n_levels = h->X.l_max - h->X.l_min + 1;
+    L = UnitLevels{};
+    int lev[MAXL];
+    for (int i = n_levels - 1; i >= 0; --i) {
+        R.first[i] = 0;
+        R.last[i] = -1;
+        const int end = i == 0 ? h->U.n : h->unit_begin[i - 1];
+        if (!h->level_has[i] || end <= h->unit_begin[i]) continue;
+        lev[L.n] = i;
+        L.unit0[L.n] = h->unit_begin[i];
+        L.begin[L.n + 1] = L.begin[L.n] + end - h->unit_begin[i];
+        ++L.n;
+    }
+    const int total = L.begin[L.n];
+    if (total == 0) return 0;
+    const int G = std::max(1, std::min(total, max_blocks));
+    auto block_of = [&](int u) {   // block b with b total / G <= u < (b + 1) total / G
+        int b = int(int64_t(u) * G / total);
+        while (b + 1 < G && int64_t(b + 1) * total / G <= u) ++b;
+        while (b > 0 && int64_t(b) * total / G > u) --b;
+        return b;
+    };
+    for (int i = 0; i < L.n; ++i) {
+        R.first[lev[i]] = block_of(L.begin[i]) + i;
+        R.last[lev[i]] = block_of(L.begin[i + 1] - 1) + i;
+    }
+    return G;
+}
+
 void set_last_message(const char *msg) { snprintf(g_last_msg, sizeof(g_last_msg), "%s", msg); }
 
 cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes) {
@@ -229,15 +259,6 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         }
         const HostIndex &X = h->X;
         cudaError_t e = cudaSuccess;
-        if (e == cudaSuccess) e = upload(h, &h->d_row_ptr, X.row_ptr.data(), X.row_ptr.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_y, X.y.data(), X.y.size(), 8);
-        if (e == cudaSuccess) e = upload(h, &h->d_off, X.off.data(), X.off.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_trow_ptr, X.trow_ptr.data(), X.trow_ptr.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_ty, X.ty.data(), X.ty.size(), 8);
-        if (e == cudaSuccess) e = upload(h, &h->d_toff, X.toff.data(), X.toff.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_fwd, X.fwd_items.data(), X.fwd_items.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_bwd, X.bwd_items.data(), X.bwd_items.size());
-        if (e == cudaSuccess) e = upload(h, &h->d_tree, X.tree_items.data(), X.tree_items.size());
         // child maps: the tree nodes, then the virtual parents of the cells of l_min
         if (e == cudaSuccess) {
             void *p = nullptr;
@@ -282,11 +303,12 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
             if (h->level_has[i]) h->n_fwd_units = i == 0 ? int(UP.hdr.size()) : UP.level_begin[i - 1];
         }
         h->complete = UP.complete;
-        for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-            const HostPlan &P = i == 0 ? X.mcfplan : X.mcbplan;
-            e = upload(h, &h->d_plan_hdr[i], P.hdr.data(), P.hdr.size());
-            if (e == cudaSuccess) e = upload(h, &h->d_plan_ent[i], P.ent.data(), P.ent.size());
-        }
+        h->uncovered = UP.uncovered;
+        h->n_levels_with = 0;
+        for (int i = 0; i <= X.l_max - X.l_min; ++i) h->n_levels_with += h->level_has[i] ? 1 : 0;
+        int dev = 0;
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess) {
             void *p = nullptr;
             e = dev_alloc(h, &p, sizeof(unsigned));
@@ -295,8 +317,8 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         }
 
         if (e == cudaSuccess) {
-            // operand-layout copy of multi-channel weights: [2 (plain, transposed)][levels][27 * 16 * 16]
-            const size_t nb = size_t(2) * size_t(X.l_max - X.l_min + 1) * 27 * 16 * 16 * sizeof(uint16_t);
+            // operand-layout copy of multi-channel weights: [2 (forward, adjoint)][levels][36 * 16 * 16]
+            const size_t nb = size_t(2) * size_t(X.l_max - X.l_min + 1) * 36 * 16 * 16 * sizeof(uint16_t);
             void *p = nullptr;
             e = dev_alloc(h, &p, nb);
             h->d_mcw = static_cast<uint16_t *>(p);
@@ -308,24 +330,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
             delete h;
             return st;
         }
-        DevLayout &L = h->L;
-        L.row_ptr = h->d_row_ptr;
-        L.y = h->d_y;
-        L.off = h->d_off;
-        L.trow_ptr = h->d_trow_ptr;
-        L.ty = h->d_ty;
-        L.toff = h->d_toff;
-        L.err = h->d_err;
-        L.np = int32_t(X.np);
-        L.nt = int32_t(X.nt);
-        L.l_min = X.l_min;
-        L.l_max = X.l_max;
-        for (int l = 0; l < MAXL; ++l) L.geo[l] = X.geo[l];
-        L.mcfplan = PlanView{h->d_plan_hdr[0], h->d_plan_ent[0]};
-        L.mcbplan = PlanView{h->d_plan_hdr[1], h->d_plan_ent[1]};
         // the plans live on the device now; the host copies are not needed again
-        h->X.mcfplan = HostPlan{};
-        h->X.mcbplan = HostPlan{};
         h->X.tnplan = std::vector<TreeNodePlan>{};
         h->X.vplan = std::vector<TreeNodePlan>{};
         h->X.vrow_ptr = std::vector<uint32_t>{};
@@ -469,26 +474,25 @@ apr_status_t apr_export_structure(apr_handle_t h, int32_t which, void *dst, size
         return APR_OK;
     }
     const HostIndex &X = h->X;
-    const void *host_src = nullptr;
-    const void *dev_src = nullptr;
+    if (which == APR_STRUCT_TREE_NODE_MAP && !h->host_only) {
+        // the device copy is the one the kernels read (uploaded on the build stream)
+        cudaError_t e = cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(h->stream));
+        if (e == cudaSuccess) e = cudaMemcpy(dst, h->d_tnplan, need, cudaMemcpyDeviceToHost);
+        return cuda_status(e);
+    }
+    const void *src = nullptr;
     switch (which) {
-        case APR_STRUCT_ROW_PTR: host_src = X.row_ptr.data(); dev_src = h->d_row_ptr; break;
-        case APR_STRUCT_Y_IDX: host_src = X.y.data(); dev_src = h->d_y; break;
-        case APR_STRUCT_TREE_ROW_PTR: host_src = X.trow_ptr.data(); dev_src = h->d_trow_ptr; break;
-        case APR_STRUCT_TREE_Y_IDX: host_src = X.ty.data(); dev_src = h->d_ty; break;
-        case APR_STRUCT_FWD_ITEMS: host_src = X.fwd_items.data(); dev_src = h->d_fwd; break;
-        case APR_STRUCT_TREE_ITEMS: host_src = X.tree_items.data(); dev_src = h->d_tree; break;
-        case APR_STRUCT_TREE_NODE_MAP: host_src = X.tnplan.data(); dev_src = h->d_tnplan; break;
-        case APR_STRUCT_BWD_ITEMS: host_src = X.bwd_items.data(); dev_src = h->d_bwd; break;
+        case APR_STRUCT_ROW_PTR: src = X.row_ptr.data(); break;
+        case APR_STRUCT_Y_IDX: src = X.y.data(); break;
+        case APR_STRUCT_TREE_ROW_PTR: src = X.trow_ptr.data(); break;
+        case APR_STRUCT_TREE_Y_IDX: src = X.ty.data(); break;
+        case APR_STRUCT_FWD_ITEMS: src = X.fwd_items.data(); break;
+        case APR_STRUCT_TREE_ITEMS: src = X.tree_items.data(); break;
+        case APR_STRUCT_TREE_NODE_MAP: src = X.tnplan.data(); break;
+        case APR_STRUCT_BWD_ITEMS: src = X.bwd_items.data(); break;
     }
-    if (h->host_only) {
-        memcpy(dst, host_src, need);
-        return APR_OK;
-    }
-    // the device copy is the one the kernels read (uploaded on the build stream)
-    cudaError_t e = cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(h->stream));
-    if (e == cudaSuccess) e = cudaMemcpy(dst, dev_src, need, cudaMemcpyDeviceToHost);
-    return cuda_status(e);
+    memcpy(dst, src, need);
+    return APR_OK;
 }
 
 apr_status_t apr_tree_restrict(apr_handle_t h, const float *particles, float *tree, int32_t channels,
@@ -624,9 +628,14 @@ apr_status_t apr_convolve_stencil_grad(apr_handle_t h, const float *particles, c
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
     const size_t need = apr_stencil_grad_workspace_bytes(h, k);
     if (need && (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255))) return APR_ERR_INVALID_ARG;
-    return cuda_status(launch_stencil_grad(k, h->U, h->unit_begin, h->level_has, X.l_max - X.l_min + 1, particles, tree, bc,
-                                           grad_out, static_cast<float *>(workspace), int(X.fwd_items.size()),
-                                           grad_stencils, stream));
+    // three blocks per SM are resident; the workspace has a column per forward work item, and a block needs
+    // one per level beyond its first
+    UnitLevels L;
+    UnitRanges R;
+    const int stride = int(X.fwd_items.size());
+    const int blocks = unit_levels(h, std::min(3 * h->sms, stride - h->n_levels_with + 1), L, R);
+    return cuda_status(launch_stencil_grad(k, h->U, L, R, blocks, X.l_max - X.l_min + 1, particles, tree, bc, grad_out,
+                                           static_cast<float *>(workspace), stride, grad_stencils, stream));
 }
 
 }  // extern "C"

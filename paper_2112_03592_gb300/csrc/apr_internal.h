@@ -39,11 +39,6 @@ struct LevelGeo {
 struct PlanHdr {
     int32_t first, count;
 };
-struct PlanEnt {
-    int32_t lo;
-    uint16_t meta, pre;
-};
-static_assert(sizeof(PlanEnt) == 8, "plan entries are 8-byte words");
 // Child map of one tree node (built once per APR; one per node, in tree order): for each of the four
 // child rows k = (a, b) = (k >> 1, k & 1) of level l+1 over the node, p[k] = index of its first
 // particle child there and t[k] = index of its first tree child (bits 0..29), and in bits 30, 31 of
@@ -56,14 +51,6 @@ struct alignas(16) TreeNodePlan {
 };
 static_assert(sizeof(TreeNodePlan) == 32, "node plans are two 16-byte words");
 constexpr uint32_t TNP_INDEX = (1u << 30) - 1u;
-struct PlanView {
-    const PlanHdr *hdr;
-    const PlanEnt *ent;
-};
-struct HostPlan {
-    std::vector<PlanHdr> hdr;
-    std::vector<PlanEnt> ent;
-};
 struct HostFPlan {
     std::vector<PlanHdr> hdr;
     std::vector<uint2> ent;
@@ -73,7 +60,7 @@ struct HostFPlan {
 // with the list of the parents around them ("slots"), see there. All units of a level are consecutive,
 // the finest level first.
 constexpr int UNIT_RECS = 256;    // most records of a unit
-constexpr int UNIT_SLOTS = 1280;  // most slots of a unit
+constexpr int UNIT_SLOTS = 1152;  // most slots of a unit
 struct alignas(16) UnitHdr {
     int32_t pure0, node0, oth0, rec0;  // first pure, node and other entry, first record
     int16_t npure;                // slots whose eight cells are particles of the level
@@ -121,6 +108,17 @@ struct UnitPlan {                          // host
     std::vector<int32_t> tile_f, tile_b, ltile_b;  // work item of each record (-1: none): forward, adjoint
     int32_t level_begin[MAXL + 1] = {};    // first node unit of level l_min + i
     bool complete = false;                 // every particle and tree node is the child of a record
+    bool uncovered = false;                // a cell next to a particle has no source (invalid layout)
+};
+// Blocks of a stencil or weight gradient: a contiguous range of the units of the levels that hold particles
+// each (finest level first); block b writes the sums of its i-th level to partial b + i.
+struct UnitLevels {
+    int n = 0;
+    int unit0[MAXL] = {};          // first unit of the level
+    int begin[MAXL + 1] = {};      // prefix of the levels' unit counts
+};
+struct UnitRanges {                // partials of level l_min + i: first[i] .. last[i] (none if first > last)
+    int first[MAXL], last[MAXL];
 };
 struct UnitView {                          // device
     const UnitHdr *hdr, *lhdr;
@@ -135,7 +133,7 @@ struct UnitView {                          // device
     int32_t n, nl;                         // node units, leaf units
 };
 
-// Everything a kernel needs to walk the index (device pointers).
+// What the host builders need to walk the index.
 struct DevLayout {
     const uint32_t *row_ptr;   // [R+1]
     const uint16_t *y;         // [N_p]
@@ -143,12 +141,9 @@ struct DevLayout {
     const uint32_t *trow_ptr;  // [R_t+1]
     const uint16_t *ty;        // [N_t]
     const uint16_t *toff;
-    unsigned *err;
     int32_t np, nt;            // particles, tree nodes (value array lengths)
     int32_t l_min, l_max;
     LevelGeo geo[MAXL];
-    PlanView mcfplan;    // multi-channel feature patches of the sub-tiles of fwd_items
-    PlanView mcbplan;    // multi-channel data-adjoint sub-tiles of bwd_items
 };
 
 struct Item {  // a work item: level, tile (or row) coordinates, y block
@@ -171,7 +166,6 @@ struct HostIndex {
     int64_t tree_level_begin[MAXL + 1] = {};
     HostFPlan fplan[2];                       // forward tile plans (build_plans), radius 1 and 2
     HostFPlan bplan[2];                       // data-adjoint tile plans (build_plans), radius 1 and 2
-    HostPlan mcfplan, mcbplan;                // multi-channel sub-tile plans (build_mc_plans)
     std::vector<TreeNodePlan> tnplan;         // child maps of the tree nodes (tree_node_plan)
     std::vector<uint32_t> vrow_ptr;           // virtual parents of the cells of l_min: rows, y, child maps
     std::vector<uint16_t> vy;
@@ -206,15 +200,12 @@ TreeGroups tree_groups(const HostIndex &X, int l0, int l1, int max_levels);
 // receives a short reason on failure.
 apr_status_t build_index(const apr_host_layout &L, uint32_t flags, HostIndex &out, const char **msg);
 
-// Builds what a device handle's kernels read (apr_plan.cu): the convolution units, the child maps and
-// the multi-channel sub-tile plans. Returns APR_OK, APR_ERR_OOM (host allocation) or APR_ERR_UNSUPPORTED.
+// Builds what a device handle's kernels read (apr_plan.cu): the child maps and the convolution units. Returns APR_OK, APR_ERR_OOM (host allocation) or APR_ERR_UNSUPPORTED.
 apr_status_t build_plans(HostIndex &X);
 // Builds the tile plans of X's forward and data-adjoint work items (apr_export_structure).
 apr_status_t build_tile_plans(HostIndex &X);
 // The convolution units of X (after tree_node_plan); throws std::bad_alloc.
 void build_units(HostIndex &X);
-// The multi-channel sub-tile plans (apr_mc.cu); true unless a tile overflows the 16-bit counts.
-bool build_mc_plans(const DevLayout &L, const HostIndex &X, HostPlan &feat, HostPlan &adj);
 // The child map of every tree node (TreeNodePlan), by one merge of each tree row with its child rows.
 // In a complete index every in-grid child cell of a node is a particle or a node of the next level.
 bool tree_node_plan(const DevLayout &L, const HostIndex &X, std::vector<TreeNodePlan> &P);
@@ -223,7 +214,9 @@ apr_status_t convolve_backward(apr_handle_t h, const float *particles, const flo
                                int32_t k, int32_t bc, const float *grad_out, float *grad_particles,
                                float *grad_stencils, void *workspace, size_t workspace_bytes, apr_stream_t stream,
                                bool concurrent);
-// DevLayout over the host copy of X's index (for host code that walks it like a kernel).
+// The levels, the ranges and the number of blocks (at most max_blocks; 0 without particles).
+int unit_levels(apr_handle_t h, int max_blocks, UnitLevels &L, UnitRanges &R);
+// DevLayout over X's index.
 DevLayout host_layout_view(const HostIndex &X);
 
 // Record a short reason for the last failure on this thread (read by apr_last_error_message).
@@ -232,7 +225,7 @@ void set_last_message(const char *msg);
 // Epilogues of the convolution kernel (launch_conv_fwd)
 constexpr int EPI_PLAIN = 0, EPI_DIVIDE = 1, EPI_MULTIPLY = 2;
 
-// Bits of the device error word (DevLayout::err), read and cleared by apr_sync_status.
+// Bits of the device error word, read and cleared by apr_sync_status.
 constexpr unsigned ERR_DEVICE_CHECK = 1u;  // a device-side consistency check failed
 constexpr unsigned ERR_TIMEOUT = 2u;       // a bounded wait (tensor-core completion) gave up
 
@@ -273,19 +266,12 @@ inline int64_t level_cells(int64_t D, int l_max, int l) {
 struct apr_handle_s {
     aprk::HostIndex X;
     bool host_only = false;
-    aprk::DevLayout L{};
-    aprk::Item *d_fwd = nullptr, *d_bwd = nullptr, *d_tree = nullptr;
-    uint32_t *d_row_ptr = nullptr, *d_trow_ptr = nullptr;
-    uint16_t *d_y = nullptr, *d_ty = nullptr, *d_off = nullptr, *d_toff = nullptr;
     unsigned *d_err = nullptr;
     uint16_t *d_mcw = nullptr;   // multi-channel weights in the tensor-core operand layout, per level
     apr_stream_t stream = nullptr;                      // the build stream (uploads, stream-ordered allocation)
     apr_allocator alloc{};                              // the caller's allocator, if has_alloc
     bool has_alloc = false;
     std::vector<std::pair<void *, size_t>> blocks;      // every device block of the handle
-    // tile plans: multi-channel feature, adjoint
-    aprk::PlanHdr *d_plan_hdr[2] = {};
-    aprk::PlanEnt *d_plan_ent[2] = {};
     aprk::TreeNodePlan *d_tnplan = nullptr;
     // host-only handles: tile plans built on the first apr_export_structure request for them
     std::mutex plan_mu;
@@ -295,6 +281,8 @@ struct apr_handle_s {
     int32_t unit_begin[aprk::MAXL + 1] = {};   // first unit of level l_min + i
     bool level_has[aprk::MAXL + 1] = {};       // whether level l_min + i holds particles
     bool complete = false;                     // every particle and tree node is the child of a record
+    bool uncovered = false;                    // a cell next to a particle has no source (invalid layout)
+    int n_levels_with = 0, sms = 0;            // levels with particles; multiprocessors of the device
     size_t dev_bytes = 0;
     // apr_convolve_backward runs the stencil gradient on a second stream, forked from and joined back
     // to the caller's stream with these events (created on first use; side_mu orders the enqueues)

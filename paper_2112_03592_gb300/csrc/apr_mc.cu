@@ -1,19 +1,32 @@
-// Multi-channel APR convolution with bfloat16 features and weights on the fifth-generation tensor
-// cores (tcgen05), FP32 accumulation: the per-level filters of an APR CNN layer (Sec. 6), with the
-// isotropic patch of Sec. 3.5 and the per-level convolution of Sec. 4.1 applied per channel pair.
+// Multi-channel APR convolution with bfloat16 features and weights on the fifth-generation tensor cores
+// (tcgen05), FP32 accumulation: the per-level filters of an APR CNN layer (Sec. 6), with the isotropic
+// patch of Sec. 3.5 and the per-level convolution of Sec. 4.1 applied per channel pair.
 //
-// Work decomposition: every convolution work item (an 8 x 8-row, 64-cell tile of one level) is cut
-// into four 4 x 4-row sub-tiles; a CTA takes several consecutive sub-tiles of one item. For each it
-// stages the patch (radius 1) with 16 channels per cell in shared memory from the segments its tile
-// plan lists (built once per APR by build_mc_plans), lists the target cells, and runs the channel
-// mixing as GEMMs:
-//   forward      D[target][co] += sum_e A_e[target][ci] W_e[ci][co]     (A_e gathered per tap)
-//   data adjoint D[row][ci]    += sum_e G(q_row - e)[co] W_e[co][ci]    (one row per pre-image q of a
-//                                  destination; each destination sums its rows afterwards)
-//   weights      D[(e,ci)][co] += sum_t U[t][(e,ci)] g_t[co]             (U: im2col of the targets)
-// The gathered A operand of the first two is written to tensor memory with tcgen05.st (one lane
-// per row, 8 columns per tap), B comes from shared memory, D lives in tensor memory. One thread
-// issues the MMAs; completion is signalled through an mbarrier whose waits are bounded in time.
+// The kernels work on the convolution units (apr_unitplan.cpp). A block takes one unit and builds, from its
+// slot entries, the source row of every cell of every slot (a particle's, a tree node's, or none) in shared
+// memory; no feature is staged per slot. Up to 128 records (parents of 2 x 2 x 2 cells) are the M rows of
+// one accumulator tile:
+//   forward       D[record][child c, co] += sum over the 64 cells around the record of
+//                                           U(cell)[ci] W[tap from child c to cell][ci][co]
+//   data adjoint  the same with dL/dout at the cells and the flipped, transposed weights (children: the
+//                 record's particles and tree nodes; for a coarser particle, the sum over its children)
+//   weights       D[tap row][cell y, ci][e, co] += U(cell)[ci] g(child)[co], summed over the records
+// The A operand of a cell (16 channels = one K step) is loaded from global memory by the row's own threads
+// (lane = record) and written to tensor memory, eight cells per step, while the MMAs of the step before run.
+// One cell serves up to eight children: a cell in reach of both children of an axis takes one MMA of twice the N, so a tile takes
+// 120 MMAs of N = 16 to 64 instead of 27 per 128 children, and gathers 64 cells per record where one row
+// per child gathered 27 per child (216 per record).
+//
+// One warp issues the MMAs; completion is signalled through mbarriers whose waits are bounded in time.
+//
+// Measured (1.0 M particles of a 256^3 image, kernels alone): forward 223 -> 74 us, data adjoint 550 -> 221 us
+// (131 onto the children, 90 onto coarser particles), weight gradient 400 -> 126 us. The kernels before cut
+// 8 x 8 x 64-cell tiles, which particles in thin shells leave mostly empty, into sub-tiles staged in shared
+// memory, and gathered 27 cells per target. Tried on the way here, forward: the A operand in shared memory
+// through 16-byte cp.async 131 us (a wavefront of the L1 pipe per 32-byte sector), with the four cells of a
+// row in one instruction 113 us, MMAs issued by a warp of their own 102 us, through registers into tensor
+// memory with warp-uniform MMA operands 74 us. What bounds it now: the issue of 120 small MMAs and the
+// latency of eight steps of 1000 cycles per tile, at two blocks per SM; DRAM traffic is 66 MB, 10 us.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -21,9 +34,11 @@
 #include <cstddef>
 #include <cstdint>
 #include <mutex>
+#include <utility>
 
 #include "apr_device.cuh"
 #include "apr_internal.h"
+#include "apr_units.cuh"
 
 namespace aprk {
 
@@ -37,33 +52,17 @@ namespace {
 using namespace dev;
 
 constexpr int MC = 16;                      // channels (c_in = c_out)
-constexpr int SZ = 4, SX = 4, SY = BY;      // sub-tile rows (z, x) and cells (y)
-constexpr int PZ = SZ + 2, PX = SX + 2, PY = SY + 2;
-constexpr int NPROW = PZ * PX;              // patch rows
-constexpr int NPC = NPROW * PY;             // patch cells
-constexpr int NIROW = SZ * SX;              // interior rows
-constexpr int MAXT = NIROW * SY;            // interior cells
-constexpr int NSUB_ZX = (TZ / SZ) * (TX / SX);
-constexpr int NSUB = NSUB_ZX * (BY / SY);   // sub-tiles per work item: (z, x) quarters, then y halves
-constexpr int NWY = (PY + 31) / 32;         // 32-bit words of a patch row's cell mask
-constexpr int SPC_F = 4, SPC_B = 2;         // sub-tiles per CTA: forward, data adjoint (measured best)
 constexpr int NTAP = 27;
-constexpr int WTAP = 512;                   // bytes of one tap's 16 x 16 bf16 weight block
-constexpr uint32_t TMEM_COLS = 256;
-constexpr uint32_t TM_A = 0;                // A operand: tap e in columns 8e .. 8e+7
-constexpr uint32_t TM_D = 224;              // accumulator: 16 columns
-constexpr int NSEG_F = 3 * NPROW;           // staging segments of the feature patch
-constexpr int NCZM = ((SZ + 1) >> 1) + 2;   // level-(l-1) rows per axis under a patch (even sub-tile origin)
-constexpr int WG_T = 16;                    // targets per weight-gradient GEMM step (one K step)
-constexpr int WG_MG = 64;                   // M groups of 8 rows allocated (54 used: 27 taps x 2)
-constexpr int WG_ROWS = NTAP * MC;          // 432 rows (e, ci) of the weight gradient
-static_assert(TZ % SZ == 0 && TX % SX == 0 && BY % SY == 0, "sub-tiles must divide the work-item tile");
-static_assert(MAXT % NT == 0, "whole interior cells per thread");
-static_assert(NSUB % SPC_F == 0 && NSUB % SPC_B == 0, "whole sub-tile groups per work item");
-static_assert(SZ % 2 == 0 && SX % 2 == 0, "sub-tiles must be even-aligned (coarse cells)");
-static_assert(TM_A + 8 * NTAP <= TM_D && TM_D + 16 <= TMEM_COLS, "tensor-memory columns");
-static_assert(NPC < 65536 && MAXT <= 1024, "16-bit cell ids");
-static_assert(SZ == SX && NCZM * NCZM <= NPROW, "once-staged coarser rows fit the kind-2 segments");
+constexpr int TILE = 128;                   // records per accumulator tile (M)
+constexpr int WBLK = MC * MC * 2;           // one tap's 16 x 16 weights
+constexpr int NWB = 36;                     // weight blocks of a level (see weight_block)
+constexpr int W_LEVEL = NWB * MC * MC;      // elements of a level's weight blocks
+constexpr uint32_t TMEM_COLS = 256;         // D: child c = 4a + 2b + e in columns 16c .. 16c + 15; then the
+constexpr uint32_t TM_A = 128;              // A operand: two buffers of eight cells of 8 columns
+constexpr int STAGES = 2;
+constexpr int NO_SOURCE = 0x7fffffff;       // source code of an empty cell; tree nodes have bit 31 set
+constexpr int TNT = NT + 32;                // threads of the tile kernels: eight warps gather, the ninth issues the MMAs
+static_assert(NT == 2 * TILE, "two threads per row");
 
 // ---------------------------------------------------------------- PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return uint32_t(__cvta_generic_to_shared(p)); }
@@ -75,9 +74,9 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
            (uint64_t((sbo & 0x3FFFF) >> 4) << 32) | (uint64_t(1) << 46);
 }
 
-// Instruction descriptor of kind::f16: BF16 A and B, FP32 D, M x N, A/B K-major unless *_mn.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? (1u << 15) : 0u) | ((uint32_t(N) >> 3) << 17) |
+// Instruction descriptor of kind::f16: BF16 A and B, FP32 D, M x N, A and B both K-major or both MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool mn) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (3u << 15) : 0u) | ((uint32_t(N) >> 3) << 17) |
            ((uint32_t(M) >> 4) << 24);
 }
 
@@ -107,7 +106,7 @@ __device__ __forceinline__ uint64_t globaltimer() {
 // or 2^24 polls, whichever comes first.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns = 1000000000ull) {
     const uint32_t a = smem_u32(bar);
-    const uint64_t t0 = globaltimer();
+    uint64_t t0 = 0;
     for (uint32_t it = 0; it < (1u << 24); ++it) {
         uint32_t done;
         asm volatile(
@@ -116,16 +115,28 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
             : "r"(a), "r"(parity)
             : "memory");
         if (done) return true;
-        if (globaltimer() - t0 > limit_ns) return false;
+        if ((it & 15u) == 15u) {   // the clock is read at every 16th poll only
+            const uint64_t t = globaltimer();
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > limit_ns) return false;
+        }
     }
     return false;
 }
 
-// D (tensor memory) [+]= A (tensor memory) x B (shared memory descriptor)
-__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
-                 "r"(a), "l"(bdesc), "r"(idesc), "r"(acc)
-                 : "memory");
+// D (tensor memory) [+]= A (tensor memory) x B (shared memory descriptor); executed by a converged warp, issued
+// by the lane with `elected`, so that the operands stay warp-uniform.
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc, uint32_t elected) {
+    asm volatile(
+        "{\n.reg .pred p, e;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 e, %5, 0;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
+        "r"(a), "l"(bdesc), "r"(idesc), "r"(acc), "r"(elected)
+        : "memory");
+}
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t e;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+    return e;
 }
 // D (tensor memory) [+]= A (shared memory descriptor) x B (shared memory descriptor)
 __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
@@ -144,6 +155,12 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint4 &a, const u
                  : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// 32 bytes at a 32-byte aligned address.
+__device__ __forceinline__ void load32(const uint4 *p, uint4 &a, uint4 &b) {
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p));
+}
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
     uint32_t r[16];
@@ -157,10 +174,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void red_add_v4(float *p, float a, float b, float c, float d) {
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
 // Bounded-wait outcome shared by the block: on a timeout every thread leaves through the same path;
@@ -193,1021 +206,821 @@ __global__ void bounded_wait_selftest_kernel(uint64_t limit_ns, unsigned *err) {
     if (__syncthreads_or(!ok) && threadIdx.x == 0) atomicOr(err, ERR_TIMEOUT);
 }
 
-// ---------------------------------------------------------------- geometry
-__device__ __forceinline__ int tap_off(int e) {  // patch-cell offset of tap e = ((dz+1)*3 + dx+1)*3 + dy+1
-    return (e / 9 - 1) * (PX * PY) + ((e / 3) % 3 - 1) * PY + (e % 3 - 1);
+
+// Records that the index does not cover the patch of a particle (a layout that was not validated).
+__global__ void uncovered_kernel(unsigned *err) { atomicOr(err, ERR_DEVICE_CHECK); }
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// A operand rows of taps E0 .. E1-1 (columns TM_A + 8e) for one row: the patch cells at
-// (pz, px, py) + S_ * (tap offset), both 16-byte halves, zero outside the patch or for an invalid row
-// (a warp-collective store, so every lane calls it). The tap offsets are compile-time constants;
-// only rows on the patch edge test them against the patch.
-template <int E0, int E1, int S_>
-__device__ __forceinline__ void store_taps(const uint4 *p0, const uint4 *p1, int pz, int px, int py, bool valid,
-                                           uint32_t taddr) {
-    const bool inner = valid && pz >= 1 && pz <= PZ - 2 && px >= 1 && px <= PX - 2 && py >= 1 && py <= PY - 2;
-    const int cell = (pz * PX + px) * PY + py;
-#pragma unroll
-    for (int e = E0; e < E1; ++e) {
-        const int dz = S_ * (e / 9 - 1), dx = S_ * ((e / 3) % 3 - 1), dy = S_ * (e % 3 - 1);
-        uint4 a = make_uint4(0, 0, 0, 0), b = a;
-        if (inner || (valid && unsigned(pz + dz) < unsigned(PZ) && unsigned(px + dx) < unsigned(PX) &&
-                      unsigned(py + dy) < unsigned(PY))) {
-            const int c = cell + (dz * PX + dx) * PY + dy;
-            a = p0[c];
-            b = p1[c];
-        }
-        tmem_st8(taddr + TM_A + 8 * e, a, b);
-    }
+// ---------------------------------------------------------------- weights
+// Weight blocks of a level: tap (tz, tx, ty) as a K-major B operand block (8-row groups of N at 256 bytes, K
+// chunks of 8 at 128 bytes). A cell reaches, along each axis, child 0 with tap t and child 1 with tap
+// t - 1, so the taps of neighbouring children are laid out one after the other: pair p = 0, 1 of (tz, tx) at
+// blocks 18 p + 2 (3 tz + 2 - tx), holding ty = p + 1 (for child e = 0), then ty = p (e = 1). Two consecutive
+// tx then serve the children b = 0, 1 of one MMA.
+__host__ __device__ constexpr int pair_block(int p, int tz, int tx) { return 18 * p + 2 * (3 * tz + 2 - tx); }
+__device__ __forceinline__ void weight_block(int blk, int &tz, int &tx, int &ty) {
+    const int p = blk / 18, r = (blk % 18) >> 1;
+    ty = p + 1 - (blk & 1);
+    tz = r / 3;
+    tx = 2 - r % 3;
 }
 
-struct Sub {         // a sub-tile: level, interior origin, level grids
-    int l, z0, x0, y0, yb;
-    LevelGeo g, gc;  // level l and level l-1 (gc valid if l > l_min)
-};
-
-__host__ __device__ __forceinline__ bool sub_of(const DevLayout &L, const Item &it, int sub, Sub &s) {
-    s.l = it.l;
-    s.g = L.geo[it.l];
-    s.gc = it.l > L.l_min ? L.geo[it.l - 1] : s.g;
-    const int zx = sub % NSUB_ZX;
-    s.z0 = it.a * TZ + (zx / (TX / SX)) * SZ;
-    s.x0 = it.b * TX + (zx % (TX / SX)) * SX;
-    s.yb = it.yb;
-    s.y0 = it.yb * BY + (sub / NSUB_ZX) * SY;
-    return s.z0 < s.g.dz && s.x0 < s.g.dx && s.y0 < s.g.dy;
-}
-
-// Patch row pr = (iz, ix) covers level cells (z0-1+iz, x0-1+ix). 0: never read, 1: staged from the
-// (reflected) source row, 2: zero (outside the grid with zero boundary).
-__host__ __device__ __forceinline__ int row_mode(const Sub &s, int pr, int bc, int &rz, int &rx) {
-    const int z = s.z0 - 1 + pr / PX, x = s.x0 - 1 + pr % PX;
-    if (z > s.g.dz || x > s.g.dx) return 0;
-    const bool out = z < 0 || z >= s.g.dz || x < 0 || x >= s.g.dx;
-    if (out && bc == APR_BC_ZERO) return 2;
-    rz = reflect_idx(z, s.g.dz);
-    rx = reflect_idx(x, s.g.dx);
-    return 1;
-}
-
-// ---------------------------------------------------------------- feature patch staging
-struct McSlot {
-    int y;
-    uint4 a, b;
-};
-
-// Loads y and the two 16-byte halves of element i of plan entry sg (segment og = meta & MC_SEG;
-// tree segments: [NPROW, 2 NPROW)).
-constexpr int MC_SEG = 255;           // plan meta: segment index; bit 8 = the patch row is outside the grid
-constexpr int MC_REFL = 256;
-struct FeatLoader {
-    using Slot = McSlot;
-    const uint16_t *py, *ty;
-    const uint4 *pv, *tv;
-    const unsigned short *meta;
-    __device__ __forceinline__ void operator()(int sg, int i, Slot &sl) const {
-        const int og = meta[sg] & MC_SEG;
-        const bool t = og >= NPROW && og < 2 * NPROW;
-        sl.y = t ? int(ty[i]) : int(py[i]);
-        const uint4 *v = t ? tv : pv;
-        sl.a = v[2 * size_t(i)];
-        sl.b = v[2 * size_t(i) + 1];
-    }
-};
-
-struct FeatStage {
-    uint4 p0[NPC];  // channels 0-7 of every patch cell
-    uint4 p1[NPC];  // channels 8-15
-    int seg_lo[NSEG_F];
-    int pre[NSEG_F + 1];
-    unsigned short smeta[NSEG_F];  // plan meta of every entry
-    int warp_tot[NWARP + 1];
-    unsigned short segid[SEGID_CAP];
-};
-
-// Staging of the feature patch with u_l (Sec. 3.5) for the cells the sub-tile's targets read:
-// level-l particles, level-l tree nodes and level-(l-1) particles (each covering two cells per
-// axis), reflected or zero outside the grid. Segment s = kind * NPROW + patch row. All patch rows
-// inside the grid: every coarser row is staged once (kind-2 segments then index the NCZM x NCZM
-// level-(l-1) rows under the patch instead of the patch rows).
-__host__ __device__ __forceinline__ bool sub_inner(const Sub &s) {
-    return s.z0 >= 1 && s.x0 >= 1 && s.z0 + SZ + 1 <= s.g.dz && s.x0 + SX + 1 <= s.g.dx;
-}
-
-// Feature segment sg of sub-tile s with the reflecting boundary: index range [lo, hi) of one row's
-// elements; refl: the patch row lies outside the grid (with zero boundary the segment is empty).
-__host__ __device__ inline void feat_segment(const DevLayout &L, const Sub &s, int sg, int &lo, int &hi, bool &refl) {
-    const int ylo = s.y0 - 1;
-    const int ya = imax(ylo, 0), yb = imin(s.y0 + SY + 1, s.g.dy);
-    const bool has_tree = s.l < L.l_max, has_coarse = s.l > L.l_min;
-    const int kind = sg / NPROW, pr = sg - kind * NPROW;
-    lo = 0;
-    hi = 0;
-    refl = false;
-    if (kind == 2 && sub_inner(s)) {
-        // a level-(l-1) row staged once for the (up to) 2 x 2 patch rows it covers
-        if (pr < NCZM * NCZM && has_coarse) {
-            const int cz = ((s.z0 - 1) >> 1) + pr / NCZM, cx = ((s.x0 - 1) >> 1) + pr % NCZM;
-            const int cya = ya >> 1, cyb = imin((yb + 1) >> 1, s.gc.dy);
-            if (cz < s.gc.dz && cx < s.gc.dx)
-                row_range(L.row_ptr, L.off, s.gc.row0, s.gc.off0, s.gc.nb, cz * s.gc.dx + cx, cya, cyb, lo, hi);
-        }
-        return;
-    }
-    int rz = 0, rx = 0;
-    if (row_mode(s, pr, APR_BC_REFLECT, rz, rx) != 1) return;
-    const int z = s.z0 - 1 + pr / PX, x = s.x0 - 1 + pr % PX;
-    refl = z < 0 || z >= s.g.dz || x < 0 || x >= s.g.dx;
-    if (kind == 0) {
-        row_range(L.row_ptr, L.off, s.g.row0, s.g.off0, s.g.nb, rz * s.g.dx + rx, ya, yb, lo, hi);
-    } else if (kind == 1 && has_tree) {
-        row_range(L.trow_ptr, L.toff, s.g.trow0, s.g.toff0, s.g.nb, rz * s.g.dx + rx, ya, yb, lo, hi);
-    } else if (kind == 2 && has_coarse) {
-        const int cya = ya >> 1, cyb = imin((yb + 1) >> 1, s.gc.dy);
-        row_range(L.row_ptr, L.off, s.gc.row0, s.gc.off0, s.gc.nb, (rz >> 1) * s.gc.dx + (rx >> 1), cya, cyb, lo, hi);
-    }
-}
-
-// Reads a sub-tile's plan (entries taken by threads t0, t0 + 1, ...; threads below t0 are free for
-// other loads) into seg_lo / smeta / pre and returns the entry count. drop_refl (zero boundary on a
-// sub-tile with rows outside the grid): the entries flagged MC_REFL are emptied and the counts
-// rescanned by all threads. Ends with a block barrier.
-__device__ __forceinline__ int load_mc_plan(const PlanView &P, int tile, int t0, bool drop_refl, int *seg_lo,
-                                            unsigned short *smeta, int *pre, int *warp_tot) {
-    const int tid = threadIdx.x;
-    const PlanHdr hd = P.hdr[tile];
-    const int n = hd.count;
-    if (tid >= t0)
-        for (int k = tid - t0; k <= n; k += NT - t0) {
-            const PlanEnt e = P.ent[hd.first + k];
-            if (k < n) {
-                seg_lo[k] = e.lo;
-                smeta[k] = e.meta;
-            }
-            if (!drop_refl) pre[k] = e.pre;
-        }
-    if (!drop_refl) {
-        block_sync();
-        return n;
-    }
-    int cnt[2] = {0, 0};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int k = 2 * tid + h;
-        if (k < n) {
-            const PlanEnt e = P.ent[hd.first + k];
-            if (!(e.meta & MC_REFL)) cnt[h] = int(P.ent[hd.first + k + 1].pre) - int(e.pre);
-        }
-    }
-    block_scan2(cnt[0], cnt[1], n, pre, warp_tot);
-    return n;
-}
-
-// Target list of the sub-tile: the level-l particles of its interior, in particle order.
-struct Targets {
-    int idx[MAXT];
-    unsigned short cell[MAXT];
-    int row_lo[NIROW], row_base[NIROW + 1];
-};
-
-// Element loads and patch writes for the nseg plan entries in S (after load_mc_plan); ends with a
-// block barrier. T (optional, its row offsets set): the targets (level-l particles of the in-grid
-// interior rows with y in [y0, y0 + SY), all among the staged elements) are listed as they pass,
-// target j of row r at T->row_base[r] + j.
-__device__ void feature_elements(const DevLayout &L, const Sub &s, const uint4 *vals, const uint4 *tree, int bc,
-                                 int nseg, FeatStage &S, Targets *T = nullptr) {
-    const int tid = threadIdx.x;
-    const int ylo = s.y0 - 1;
-    const int ya = max(ylo, 0), yb = min(s.y0 + SY + 1, s.g.dy);
-    const bool inner = sub_inner(s);
-    const FeatLoader loader{L.y, L.ty, vals, tree, S.smeta};
-    for_each_element(S.seg_lo, S.pre, nseg, S.segid, loader, [&](int sg, int i, const McSlot &sl) {
-        const int og = S.smeta[sg] & MC_SEG;
-        const int kind = og / NPROW, pr = og - kind * NPROW;
-        if (kind < 2) {
-            if (sl.y >= ya && sl.y < yb) {
-                const int c = pr * PY + sl.y - ylo;
-                S.p0[c] = sl.a;
-                S.p1[c] = sl.b;
-                if (T && kind == 0 && sl.y >= s.y0 && sl.y < s.y0 + SY) {
-                    const int iz = pr / PX - 1, ix = pr % PX - 1;
-                    if (unsigned(iz) < unsigned(SZ) && unsigned(ix) < unsigned(SX) && s.z0 + iz < s.g.dz &&
-                        s.x0 + ix < s.g.dx) {
-                        const int r = iz * SX + ix, slot = T->row_base[r] + (i - T->row_lo[r]);
-                        T->idx[slot] = i;
-                        T->cell[slot] = (unsigned short)c;
-                    }
-                }
-            }
-        } else if (!inner) {
-#pragma unroll
-            for (int f = 0; f < 2; ++f) {
-                const int y = 2 * sl.y + f;
-                if (y >= ya && y < yb) {
-                    const int c = pr * PY + y - ylo;
-                    S.p0[c] = sl.a;
-                    S.p1[c] = sl.b;
-                }
-            }
-        } else {
-            const int rz0 = 2 * (((s.z0 - 1) >> 1) + pr / NCZM) - (s.z0 - 1);
-            const int rx0 = 2 * (((s.x0 - 1) >> 1) + pr % NCZM) - (s.x0 - 1);
-#pragma unroll
-            for (int f = 0; f < 2; ++f) {
-                const int y = 2 * sl.y + f;
-                if (y < ya || y >= yb) continue;
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-                        const int pz = rz0 + a, px = rx0 + b;
-                        if (pz < 0 || pz >= PZ || px < 0 || px >= PX) continue;
-                        const int c = (pz * PX + px) * PY + y - ylo;
-                        S.p0[c] = sl.a;
-                        S.p1[c] = sl.b;
-                    }
-            }
-        }
-    });
-    // cells outside the grid (none when the patch lies inside it): the cells y = -1 and y = dy of each
-    // staged row mirror y = 0 and y = dy - 1 (zero with the zero boundary), and with the zero boundary
-    // the rows outside the grid are zero
-    const uint4 z4 = make_uint4(0, 0, 0, 0);
-    if (!inner || ylo < 0 || s.y0 + SY >= s.g.dy) {
-        for (int t = tid; t < 2 * NPROW; t += NT) {
-            const int pr = t >> 1, y = (t & 1) ? s.g.dy : -1, py = y - ylo;
-            int rz, rx;
-            if (py < 0 || py >= PY || row_mode(s, pr, bc, rz, rx) != 1) continue;
-            const int i = pr * PY + py;
-            if (bc == APR_BC_ZERO) {
-                S.p0[i] = z4;
-                S.p1[i] = z4;
-            } else {
-                const int src = pr * PY + reflect_idx(y, s.g.dy) - ylo;  // y = -1 -> 0, y = dy -> dy-1
-                S.p0[i] = S.p0[src];
-                S.p1[i] = S.p1[src];
-            }
-        }
-        if (bc == APR_BC_ZERO && !inner)
-            for (int i = tid; i < NPROW * PY; i += NT) {
-                int rz, rx;
-                if (row_mode(s, i / PY, bc, rz, rx) == 2) {
-                    S.p0[i] = z4;
-                    S.p1[i] = z4;
-                }
-            }
-    }
-    block_sync();
-}
-
-// The whole staging of sub-tile `tile` (index into the feature plan: item * NSUB + sub).
-__device__ void stage_features(const DevLayout &L, const Sub &s, int tile, const uint4 *vals, const uint4 *tree,
-                               int bc, FeatStage &S, Targets *T = nullptr) {
-    const int n = load_mc_plan(L.mcfplan, tile, 0, bc != APR_BC_REFLECT && !sub_inner(s), S.seg_lo, S.smeta, S.pre,
-                               S.warp_tot);
-    feature_elements(L, s, vals, tree, bc, n, S, T);
-}
-
-// Row offsets of the targets (warp 0; no barrier): the sub-tile spans whole y-blocks, so the block
-// offsets give each interior row's level-l particles exactly.
-__device__ __forceinline__ void target_rows(const DevLayout &L, const Sub &s, Targets &T) {
-    static_assert(SY == BY, "sub-tiles span one y-block");
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0) {
-        int lo = 0, cnt = 0;
-        if (lane < NIROW) {
-            const int z = s.z0 + lane / SX, x = s.x0 + lane % SX;
-            if (z < s.g.dz && x < s.g.dx) {
-                const int rr = z * s.g.dx + x;
-                lo = int(pblock(L, s.g, rr, s.yb));
-                cnt = int(pblock(L, s.g, rr, s.yb + 1)) - lo;
-            }
-        }
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        if (lane < NIROW) {
-            T.row_lo[lane] = lo;
-            T.row_base[lane] = incl - cnt;
-        }
-        if (lane == NIROW - 1) T.row_base[NIROW] = incl;
-    }
-}
-
-// Particle index of target j from the row offsets alone (before the list is filled).
-__device__ __forceinline__ int target_index(const Targets &T, int j) {
-    int r = 0;
-#pragma unroll
-    for (int k = 1; k < NIROW; ++k) r = T.row_base[k] <= j ? k : r;
-    return T.row_lo[r] + (j - T.row_base[r]);
-}
-
-// Row offsets of the targets; returns their count (ends with a barrier).
-__device__ int count_targets(const DevLayout &L, const Sub &s, Targets &T) {
-    target_rows(L, s, T);
-    block_sync();
-    return T.row_base[NIROW];
-}
-
-// Weights of every level in the B-operand layout of each tap e: K-major core matrices of 8 rows x 16
-// bytes, N-row group g and K chunk k at (2g + k) * 128 bytes (LBO 128, SBO 256). transpose = 0:
-// N = co, K = ci (forward); transpose = 1: N = ci, K = co (data adjoint). One thread per destination
-// element of out[lev][e * 256 + ...], read from W[lev][co][ci][e].
-__global__ void mc_weight_layout_kernel(const uint16_t *__restrict__ W, int n_levels, int transpose,
+// out[lev][block][...] from W[lev][co][ci][e]. adjoint: N = ci, K = co, taps flipped; else N = co, K = ci.
+__global__ void mc_weight_layout_kernel(const uint16_t *__restrict__ W, int n_levels, int adjoint,
                                         uint16_t *__restrict__ out) {
-    constexpr int PER = MC * MC * NTAP;
-    for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < n_levels * PER; d += gridDim.x * blockDim.x) {
-        const int lev = d / PER, r = d % PER;
-        const int e = r / (MC * MC), q = r % (MC * MC);
+    pdl_trigger();   // the convolution after this one stages its unit meanwhile
+    for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < n_levels * W_LEVEL; d += gridDim.x * blockDim.x) {
+        const int lev = d / W_LEVEL, r = d % W_LEVEL, blk = r / (MC * MC), q = r % (MC * MC);
         const int cm = q / 64, row = (q % 64) / 8, col = q % 8;
         const int n = (cm >> 1) * 8 + row, k = (cm & 1) * 8 + col;
-        const int co = transpose ? k : n, ci = transpose ? n : k;
-        out[d] = W[((size_t(lev) * MC + co) * MC + ci) * NTAP + e];
+        int tz, tx, ty;
+        weight_block(blk, tz, tx, ty);
+        const int e = (tz * 3 + tx) * 3 + ty;
+        const int co = adjoint ? k : n, ci = adjoint ? n : k;
+        out[d] = W[((size_t(lev) * MC + co) * MC + ci) * NTAP + (adjoint ? NTAP - 1 - e : e)];
     }
 }
 
-// One level's operand-layout weights (13 824 contiguous bytes) into shared memory, in two halves: the
-// loads into registers (four 16-byte words per thread) early, the stores into shared memory later,
-// so the loads' latency overlaps other work.
-constexpr int WV = NTAP * WTAP / 16;  // 16-byte words of one level's weights
-static_assert(WV <= 4 * NT, "four weight words per thread");
+// ---------------------------------------------------------------- unit staging
+struct Rows {                         // the tile's rows: row slots of their neighbourhood
+    uint16_t base[9][TILE];
+    uint32_t mask[TILE];              // bit 3r + j: parent j of row r is a slot, at base[r] + the bits before it
+};
 
-__device__ __forceinline__ void preload_weights(const uint16_t *wl, int lev, uint4 (&w)[4]) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(wl + size_t(lev) * MC * MC * NTAP);
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (threadIdx.x + k * NT < WV) w[k] = src[threadIdx.x + k * NT];
-}
-
-__device__ __forceinline__ void store_weights(const uint4 (&w)[4], unsigned char *wsm) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (threadIdx.x + k * NT < WV) reinterpret_cast<uint4 *>(wsm)[threadIdx.x + k * NT] = w[k];
-    fence_async_smem();
-}
-
-// ---------------------------------------------------------------- forward
-struct FwdSmem {
-    FeatStage st;
-    alignas(16) unsigned char w[NTAP * WTAP];
-    Targets tg;
-    uint64_t bar;
+struct McSmem {
+    int code[8][PLANE];               // source of every cell c of every slot
+    Rows rows;
+    alignas(128) float4 sums[TILE * 16];   // image sums (image_chunk)
+    alignas(128) unsigned char W[NWB * WBLK];
+    int first[UNIT_RECS + 1];         // first row of each record (lists of images)
+    int wsum[NWARP];
+    uint64_t bar[STAGES];             // MMAs that read buffer s have completed
     uint32_t tmem;
 };
 
-// out (float32 [N][16]) receives the convolution; if out_bf16 is given instead, it receives
-// bf16(max(conv, 0)), the next layer's input in an APR CNN (the ReLU fused into the write).
-// A CTA takes SPC_F consecutive sub-tiles of one work item (one level): the weights, the mbarrier and
-// the tensor memory are set up once, at its first sub-tile with targets.
-__global__ void __launch_bounds__(NT, 2) mc_fwd_kernel(const DevLayout L, const Item *__restrict__ items,
-                                                       const uint4 *__restrict__ vals, const uint4 *__restrict__ tree,
-                                                       const uint16_t *__restrict__ W, int bc, float *__restrict__ out,
-                                                       uint4 *__restrict__ out_bf16) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    FwdSmem &S = *reinterpret_cast<FwdSmem *>(smraw);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Item it = items[blockIdx.x];
-    // the level's weights are held in registers until the first patch is staged
-    uint4 wreg[4];
-    preload_weights(W, it.l - L.l_min, wreg);
-    const int q = warp & 3;
-    const uint32_t lane_base = uint32_t(32 * q) << 16;
-    constexpr uint32_t idesc = idesc_bf16(128, 16, false);
-    uint32_t phase = 0, tb = 0;
-    bool ready = false, failed = false;  // block-uniform
-    for (int k = 0; k < SPC_F && !failed; ++k) {
-        const int sub = blockIdx.y * SPC_F + k;
-        Sub s;
-        if (!sub_of(L, it, sub, s)) continue;
-        if (k > 0) block_sync();  // the previous sub-tile's readers of S.tg and S.st are done
-        target_rows(L, s, S.tg);  // warp 0, while the other warps read the plan
-        const int nseg = load_mc_plan(L.mcfplan, blockIdx.x * NSUB + sub, 32,
-                                      bc != APR_BC_REFLECT && !sub_inner(s), S.st.seg_lo, S.st.smeta, S.st.pre,
-                                      S.st.warp_tot);
-        const int nt = S.tg.row_base[NIROW];
-        if (nt == 0) continue;
-        feature_elements(L, s, vals, tree, bc, nseg, S.st, &S.tg);
-        if (!ready) {
-            store_weights(wreg, S.w);
-            if (tid == 0) mbar_init(&S.bar);
-            if (warp == 0) tmem_alloc(smem_u32(&S.tmem), TMEM_COLS);
-            ready = true;
-        }
-        fence_async_smem();
-        tc_fence_before();
-        block_sync();
-        tc_fence_after();
-        tb = S.tmem;
-        for (int b0 = 0; b0 < nt; b0 += 128) {
-            const int t = b0 + 32 * q + lane;
-            const int cell = t < nt ? int(S.tg.cell[t]) : 0;
-            const int cz = cell / (PX * PY), cx = (cell / PY) % PX, cy = cell % PY;
-            // rows past the last target are never read back: a warp holding only such rows skips them
-            if (b0 + 32 * q < nt) {
-                if (warp < 4) store_taps<0, 14, 1>(S.st.p0, S.st.p1, cz, cx, cy, t < nt, tb + lane_base);
-                else store_taps<14, NTAP, 1>(S.st.p0, S.st.p1, cz, cx, cy, t < nt, tb + lane_base);
-            }
-            tmem_wait_st();
-            tc_fence_before();
-            block_sync();
-            tc_fence_after();
-            if (tid == 0) {
-                for (int e = 0; e < NTAP; ++e)
-                    mma_ts(tb + TM_D, tb + TM_A + 8 * e, sdesc(smem_u32(S.w + e * WTAP), 128, 256), idesc, e > 0);
-                mma_commit(&S.bar);
-            }
-            if (block_wait_mma(&S.bar, phase, L.err)) {
-                failed = true;
-                break;
-            }
-            phase ^= 1;
-            tc_fence_after();
-            if (warp < 4) {
-                float v[16];
-                tmem_ld16(tb + lane_base + TM_D, v);
-                if (t < nt) {
-                    if (out_bf16) {
-                        uint4 r[2];
-                        __nv_bfloat162 *b2 = reinterpret_cast<__nv_bfloat162 *>(r);
+// Source codes of the unit's slots. VALUES: particles, tree nodes and coarser particles; else the level-l
+// particles only, and nothing outside the grid.
+template <bool VALUES>
+__device__ __forceinline__ void stage_codes(const UnitView &U, const UnitHdr &h, bool leaf, bool reflect, int (*code)[PLANE]) {
+    const int tid = threadIdx.x, nt = int(blockDim.x);
+    const uint4 *pure = (leaf ? U.lpure : U.pure) + h.pure0;
+    const TreeNodePlan *nmap = (leaf ? U.lnmap : U.nmap) + h.node0;
+    const uint32_t *ninfo = (leaf ? U.lninfo : U.ninfo) + h.node0;
+    if (tid < 3)
 #pragma unroll
-                        for (int c = 0; c < MC / 2; ++c) b2[c] = __floats2bfloat162_rn(fmaxf(v[2 * c], 0.f), fmaxf(v[2 * c + 1], 0.f));
-                        out_bf16[2 * size_t(S.tg.idx[t])] = r[0];
-                        out_bf16[2 * size_t(S.tg.idx[t]) + 1] = r[1];
-                    } else {
-                        float4 *o = reinterpret_cast<float4 *>(out + size_t(S.tg.idx[t]) * MC);
+        for (int c = 0; c < 8; ++c) code[c][ZERO_SLOT + tid] = NO_SOURCE;
+    auto put_pure = [&](const uint4 &q) {
+        const unsigned p[4] = {q.x, q.y, q.z, q.w}, s = pure_slot(q);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) o[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-                    }
-                }
-            }
-            tc_fence_before();
-            block_sync();
-            tc_fence_after();
+        for (int k = 0; k < 4; ++k) {
+            code[2 * k][s] = int(p[k] & 0x0fffffffu);
+            code[2 * k + 1][s] = int(p[k] & 0x0fffffffu) + 1;
         }
+    };
+    auto put_node = [&](const int4 &pw, const int4 &tw, unsigned info) {
+        const Octet o(pw, tw);
+        int v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            v[c] = o.kind[c] == 1 ? o.ix[c] : (VALUES && o.kind[c] == 2 ? int(unsigned(o.ix[c]) | 0x80000000u) : NO_SOURCE);
+        if (info >> UE_MIRROR) edge_octet(v, info, VALUES && reflect, NO_SOURCE);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) code[c][info & UE_SLOT] = v[c];
+    };
+    auto put_other = [&](const uint2 &e, int i) {
+        int v[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = VALUES && i < h.nleaf ? int(e.x) : NO_SOURCE;
+        if (e.y >> UE_MIRROR) edge_octet(v, e.y, VALUES && reflect, NO_SOURCE);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) code[c][e.y & UE_SLOT] = v[c];
+    };
+    // the first entries of every kind in flight together, then what is left
+    const uint2 *oth = U.oth + h.oth0;
+    uint4 q[2];
+    uint2 e[2];
+    int4 pw = make_int4(0, 0, 0, 0), tw = pw;
+    unsigned info = 0;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        q[u] = tid + u * nt < h.npure ? __ldg(pure + tid + u * nt) : make_uint4(0, 0, 0, 0);
+        e[u] = tid + u * nt < h.noth ? __ldg(oth + tid + u * nt) : make_uint2(0, 0);
     }
-    if (ready) {
-        tc_fence_before();
-        block_sync();
-        if (warp == 0) tmem_dealloc(tb, TMEM_COLS);
+    if (tid < h.nnode) {
+        const int4 *m = reinterpret_cast<const int4 *>(nmap + tid);
+        pw = __ldg(m);
+        if (VALUES) tw = __ldg(m + 1);
+        info = __ldg(ninfo + tid);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        if (tid + u * nt < h.npure) put_pure(q[u]);
+        if (tid + u * nt < h.noth) put_other(e[u], tid + u * nt);
+    }
+    if (tid < h.nnode) put_node(pw, tw, info);
+    for (int i = tid + 2 * nt; i < h.npure; i += nt) put_pure(__ldg(pure + i));
+    for (int i = tid + 2 * nt; i < h.noth; i += nt) put_other(__ldg(oth + i), i);
+    for (int i = tid + nt; i < h.nnode; i += nt) {
+        const int4 *m = reinterpret_cast<const int4 *>(nmap + i);
+        put_node(__ldg(m), VALUES ? __ldg(m + 1) : make_int4(0, 0, 0, 0), __ldg(ninfo + i));
     }
 }
 
-// ---------------------------------------------------------------- data adjoint
-constexpr int NSEG_B = NPROW + 3 * NIROW;  // gradient rows, then interior particle / tree / coarse rows
-// Row groups of the data adjoint: a destination with q pre-images that a gradient reaches takes an
-// aligned group of rows, one pre-image per row: class 0 (33..64 pre-images, 32 rows, two passes),
-// class c = 1..6 (2^(6-c) rows for up to that many pre-images). Classes are laid out in order, so
-// every group starts at a multiple of its size and stays inside one warp's 32 rows.
-constexpr int NCLS = 7;
-__device__ __forceinline__ int group_rows(int c) { return min(32, 64 >> c); }
-__device__ __forceinline__ int group_class(int q) { return q > 32 ? 0 : 6 - (q > 1 ? 32 - __clz(q - 1) : 0); }
-constexpr unsigned char SRC_NONE = 0xFF, SRC_P = 0, SRC_T = 1, SRC_C = 2;  // source kinds of a patch cell
-static_assert(SRC_P == 0 && SRC_T == 1, "interior particle / tree segments store their kind index");
+// Row r of the tile: record `rec` of a node unit at its own place (one set of loads: nine dependent ones
+// would cost more than the row's sums), ...
+__device__ __forceinline__ void put_node_row(Rows &R, int r, const NodeRec *rec) {
+    const uint2 *q = reinterpret_cast<const uint2 *>(rec);
+    const uint2 r0 = __ldg(q), r1 = __ldg(q + 1), r2 = __ldg(q + 2);
+    unsigned b[9];
+    unpack_bases(r0.y, r1, r2, b);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) R.base[k][r] = uint16_t(b[k]);
+    R.mask[r] = 0x7ffffffu;
+}
+// ... at the image of shift t (edge_shifts; 0: its own place), ...
+__device__ __forceinline__ void put_image_row(Rows &R, int r, const NodeRec *rec, int t) {
+    const int iz = t >> 4, ix = (t >> 2) & 3, iy = t & 3, dy = iy == 1 ? -1 : (iy == 0 ? 0 : iy - 1);
+    unsigned mask = 0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const int oz = image_layer(iz, q / 3), ox = image_layer(ix, q % 3);
+        if (oz >= 0 && ox >= 0) {
+            R.base[q][r] = uint16_t(int(rec->base[3 * oz + ox]) + dy);
+            mask |= 7u << (3 * q);
+        }
+    }
+    R.mask[r] = mask;
+}
+// ... of a leaf unit.
+__device__ __forceinline__ void put_leaf_row(Rows &R, int r, const LeafRec *rec, int t) {
+    const int iz = t >> 4, ix = (t >> 2) & 3, iy = t & 3;
+    const unsigned all = rec->mask;
+    unsigned mask = 0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const int oz = image_layer(iz, q / 3), ox = image_layer(ix, q % 3), o = 3 * oz + ox;
+        if (oz >= 0 && ox >= 0) {
+            const unsigned m = (all >> (3 * o)) & 7u;
+            R.base[q][r] = uint16_t(rec->base[o] + (iy == 0 ? 0 : __popc(m & (iy == 3 ? 3u : 1u))));
+            mask |= (iy == 0 ? m : (iy == 1 ? (m << 1) & 4u : (m >> (iy - 1)) & 1u)) << (3 * q);
+        }
+    }
+    R.mask[r] = mask;
+}
 
-struct BwdSmem {
-    uint4 g0[NPC];  // bf16 gradient of the targets, channels 0-7 (zero elsewhere)
-    uint4 g1[NPC];
-    alignas(16) unsigned char w[NTAP * WTAP];
-    int srci[MAXT];                 // source of each interior cell: index ...
-    unsigned char srck[MAXT];       // ... and kind (particle, tree, coarse particle)
-    unsigned short dorder[MAXT];    // candidate cells, then the destinations grouped by row-group class in slot order
-    unsigned tmask[NPROW][NWY];     // cells holding a target, per patch row (bits along y)
-    unsigned hot[NPROW][NWY];       // cells within distance 1 of a target
-    int seg_lo[NSEG_B];
-    int pre[NSEG_B + 1];
-    unsigned short smeta[NSEG_B];  // plan meta (segment index) of every entry
-    int warp_tot[NWARP + 1];
-    unsigned short segid[SEGID_CAP];
-    int ccnt[NCLS];                 // destinations per row-group class
-    int coff[NCLS + 1];             // first destination (in dorder) of each class
-    int rbase[NCLS + 1];            // first row of each class
-    uint64_t bar;
-    uint32_t tmem;
+// Source code of cell (iz, ix, iy) (0..3 per axis, from one before the parent's first cell) of row r.
+__device__ __forceinline__ int cell_code(const int (*code)[PLANE], unsigned m, unsigned base, int c0, int iy) {
+    const int j = (iy + 1) >> 1;
+    return (m >> j) & 1u ? code[c0 + ((iy + 1) & 1)][base + __popc(m & ((1u << j) - 1u))] : NO_SOURCE;
+}
+
+__device__ __forceinline__ const uint4 *source_row(const uint4 *vals, const uint4 *tree, int code) {
+    return (code < 0 ? tree : vals) + 2 * size_t(code == NO_SOURCE ? 0 : code & 0x7fffffff);
+}
+
+// ---------------------------------------------------------------- the tile GEMM
+// Step k: the cell rows (iz, ix = x0) and (iz, x0 + 1), iz and x0 from the order below (the first step's rows
+// both reach both z children, and its second row all eight children; see issue_row).
+__device__ __forceinline__ int step_z(int k) { return k < 2 ? 1 : (k < 4 ? 0 : k >> 1); }
+__device__ __forceinline__ int step_x(int k) { return 2 * (k & 1); }
+
+// The four cells of row (iz, ix) of tile row r: up to 128 contiguous bytes. wide: 32-byte aligned features,
+// one load per cell (lane = record touches 16 lines per load either way; 16-byte loads touch them twice).
+struct CellRow {
+    uint4 v[4][2];
+    __device__ __forceinline__ void load(const int (*code)[PLANE], const Rows &rows, int r, int iz, int ix,
+                                         const uint4 *__restrict__ vals, const uint4 *__restrict__ tree, bool wide) {
+        const int q = ((iz + 1) >> 1) * 3 + ((ix + 1) >> 1), c0 = ((iz + 1) & 1) * 4 + ((ix + 1) & 1) * 2;
+        const unsigned m = (rows.mask[r] >> (3 * q)) & 7u, base = rows.base[q][r];
+        int src[4];
+#pragma unroll
+        for (int iy = 0; iy < 4; ++iy) src[iy] = cell_code(code, m, base, c0, iy);
+#pragma unroll
+        for (int iy = 0; iy < 4; ++iy) {
+            v[iy][0] = v[iy][1] = make_uint4(0, 0, 0, 0);
+            if (src[iy] != NO_SOURCE) {
+                const uint4 *p = source_row(vals, tree, src[iy]);
+                if (wide) {
+                    load32(p, v[iy][0], v[iy][1]);
+                } else {
+                    v[iy][0] = __ldg(p);
+                    v[iy][1] = __ldg(p + 1);
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ void store(uint32_t a) const {
+#pragma unroll
+        for (int iy = 0; iy < 4; ++iy) tmem_st8(a + 8 * iy, v[iy][0], v[iy][1]);
+    }
 };
 
-// Segment sg of the data-adjoint sub-tile s: [0, NPROW) the targets of the patch rows (inside the
-// grid only; y in the patch window), then per interior row the level-l particles, the level-l tree
-// nodes and the level-(l-1) particles over the interior y range.
-__host__ __device__ inline void adj_segment(const DevLayout &L, const Sub &s, int sg, int &lo, int &hi) {
-    const int ylo = s.y0 - 1;
-    const int ya = imax(ylo, 0), yb = imin(s.y0 + SY + 1, s.g.dy);
-    const int yia = s.y0, yib = imin(s.y0 + SY, s.g.dy);
-    const bool has_tree = s.l < L.l_max, has_coarse = s.l > L.l_min;
-    lo = 0;
-    hi = 0;
-    if (sg < NPROW) {
-        const int z = s.z0 - 1 + sg / PX, x = s.x0 - 1 + sg % PX;
-        if (z >= 0 && z < s.g.dz && x >= 0 && x < s.g.dx)
-            row_range(L.row_ptr, L.off, s.g.row0, s.g.off0, s.g.nb, z * s.g.dx + x, ya, yb, lo, hi);
-        return;
-    }
-    const int k = (sg - NPROW) / NIROW, r = (sg - NPROW) % NIROW;
-    const int z = s.z0 + r / SX, x = s.x0 + r % SX;
-    if (z >= s.g.dz || x >= s.g.dx) return;
-    if (k == 0)
-        row_range(L.row_ptr, L.off, s.g.row0, s.g.off0, s.g.nb, z * s.g.dx + x, yia, yib, lo, hi);
-    else if (k == 1 && has_tree)
-        row_range(L.trow_ptr, L.toff, s.g.trow0, s.g.toff0, s.g.nb, z * s.g.dx + x, yia, yib, lo, hi);
-    else if (k == 2 && has_coarse)
-        row_range(L.row_ptr, L.off, s.gc.row0, s.gc.off0, s.gc.nb, (z >> 1) * s.gc.dx + (x >> 1), yia >> 1,
-                  imin((yib + 1) >> 1, s.gc.dy), lo, hi);
-}
-
-__device__ __forceinline__ bool hot_at(const BwdSmem &S, int pz, int px, int py) {
-    return (S.hot[pz * PX + px][py >> 5] >> (py & 31)) & 1u;
-}
-
-// Pre-images along one axis of a destination whose first fine coordinate is u: its in-grid fine
-// cells (one, or two for a coarse particle) and the out-of-grid cells that reflect onto them, as
-// patch coordinates (position - base, base = the patch's first position) packed 8 bits each into
-// *w (registers, no local array). Returns the count (at most 4).
-__device__ __forceinline__ int axis_pre(int u, bool coarse, int d, bool reflect, int base, uint32_t *w) {
-    uint32_t v = uint32_t(u - base);
-    int n = 1;
-    if (coarse && u + 1 < d) v |= uint32_t(u + 1 - base) << (8 * n++);
-    if (reflect) {
-        if (u == 0) v |= uint32_t(-1 - base) << (8 * n++);
-        if ((coarse ? min(u + 1, d - 1) : u) == d - 1) v |= uint32_t(d - base) << (8 * n++);
-    }
-    *w = v;
-    return n;
-}
-__device__ __forceinline__ int pre_at(uint32_t w, int a) { return int((w >> (8 * a)) & 255u); }
-
-__global__ void __launch_bounds__(NT, 2) mc_bwd_data_kernel(const DevLayout L, const Item *__restrict__ items,
-                                                            const uint16_t *__restrict__ W, int bc,
-                                                            const uint4 *__restrict__ gout, float *__restrict__ gp,
-                                                            float *__restrict__ gt) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    BwdSmem &S = *reinterpret_cast<BwdSmem *>(smraw);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Item it = items[blockIdx.x];
-    // the level's (transposed) weights are loaded now and held in registers until the first
-    // destination list is known, so their latency overlaps the staging
-    uint4 wreg[4];
-    preload_weights(W, it.l - L.l_min, wreg);
-    const bool reflect = bc == APR_BC_REFLECT;
-    const int q = warp & 3;
-    const uint32_t lane_base = uint32_t(32 * q) << 16;
-    constexpr uint32_t idesc = idesc_bf16(128, 16, false);
-    uint32_t phase = 0, tb = 0;
-    bool ready = false, stop = false;  // block-uniform
-    // SPC_B consecutive sub-tiles of the work item; the weights, the mbarrier and the tensor memory
-    // are set up once, at the first sub-tile with destinations
-    for (int kk = 0; kk < SPC_B && !stop; ++kk) {
-        const int sub = blockIdx.y * SPC_B + kk;
-        Sub s;
-        if (!sub_of(L, it, sub, s)) continue;
-        if (kk > 0) block_sync();  // the previous sub-tile's readers of the shared tables are done
-        const int ylo = s.y0 - 1;
-        const int ya = max(ylo, 0), yb = min(s.y0 + SY + 1, s.g.dy);  // gradient rows: y range of the patch
-        const int yia = s.y0, yib = min(s.y0 + SY, s.g.dy);            // interior y range
-        const uint4 z4 = make_uint4(0, 0, 0, 0);
-        for (int i = tid; i < NPC; i += NT) {
-            S.g0[i] = z4;
-            S.g1[i] = z4;
-        }
-        for (int i = tid; i < MAXT; i += NT) S.srck[i] = SRC_NONE;
-        for (int i = tid; i < NPROW * NWY; i += NT) (&S.tmask[0][0])[i] = 0;
-        const int nseg = load_mc_plan(L.mcbplan, blockIdx.x * NSUB + sub, 0, false, S.seg_lo, S.smeta, S.pre,
-                                      S.warp_tot);
-
-        struct Loader {
-            using Slot = McSlot;
-            const DevLayout *L;
-            const uint4 *gout;
-            const unsigned short *meta;
-            __device__ void operator()(int k, int i, Slot &sl) const {
-                const int sg = meta[k];
-                const bool t = sg >= NPROW + NIROW && sg < NPROW + 2 * NIROW;
-                sl.y = t ? int(L->ty[i]) : int(L->y[i]);
-                if (sg < NPROW) {
-                    sl.a = gout[2 * size_t(i)];
-                    sl.b = gout[2 * size_t(i) + 1];
-                }
-            }
-        } loader{&L, gout, S.smeta};
-        for_each_element(S.seg_lo, S.pre, nseg, S.segid, loader, [&](int ent, int i, const McSlot &sl) {
-            const int sg = S.smeta[ent];
-            if (sg < NPROW) {
-                if (sl.y >= ya && sl.y < yb) {
-                    const int py = sl.y - ylo;
-                    S.g0[sg * PY + py] = sl.a;
-                    S.g1[sg * PY + py] = sl.b;
-                    atomicOr(&S.tmask[sg][py >> 5], 1u << (py & 31));
-                }
-                return;
-            }
-            const int k = (sg - NPROW) / NIROW, r = (sg - NPROW) % NIROW;
-            if (k < 2) {
-                if (sl.y >= yia && sl.y < yib) {
-                    S.srck[r * SY + sl.y - s.y0] = (unsigned char)k;
-                    S.srci[r * SY + sl.y - s.y0] = i;
-                }
+// MMAs of cell row (iz, ix) (one warp), all operands constants away from the bases: built at run time they
+// cost more than the MMAs take. INIT: the first MMAs of the tile; cell (1, 1, 1) reaches all eight children
+// and overwrites D.
+template <int iz, int ix, bool INIT>
+__device__ __forceinline__ void issue_row(uint32_t D, uint32_t A, uint64_t W, uint32_t el) {
+    constexpr int b0 = ix == 3 ? 1 : 0, nb = ix == 0 || ix == 3 ? 1 : 2;
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        const int iy = o == 0 ? 1 : (o == 1 ? 2 : (o == 2 ? 0 : 3));
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const int tz = iz - a;
+            if (tz < 0 || tz > 2) continue;
+            if (iy == 1 || iy == 2) {
+                mma_ts(D + 64 * a + 32 * b0, A + 8 * iy, W + pair_block(iy - 1, tz, ix - b0) * (WBLK >> 4), idesc_bf16(128, 32 * nb, false),
+                       INIT && o == 0 ? 0u : 1u, el);
             } else {
 #pragma unroll
-                for (int f = 0; f < 2; ++f) {
-                    const int y = 2 * sl.y + f;
-                    if (y >= yia && y < yib) {
-                        S.srck[r * SY + y - s.y0] = SRC_C;
-                        S.srci[r * SY + y - s.y0] = i;
-                    }
-                }
+                for (int b = b0; b < b0 + nb; ++b)   // ty = 0 for child e = 0, ty = 2 for e = 1
+                    mma_ts(D + 64 * a + 32 * b + (iy == 3 ? 16 : 0), A + 8 * iy,
+                           W + (iy == 0 ? pair_block(0, tz, ix - b) + 1 : pair_block(1, tz, ix - b)) * (WBLK >> 4),
+                           idesc_bf16(128, 16, false), 1u, el);
             }
-        });
-        // cells within distance 1 of a target: y dilation of each row, OR over the 3 x 3 neighbour rows
-        if (tid < NPROW) {
-            const int pz = tid / PX, px = tid % PX;
-            unsigned h[NWY] = {};
-            for (int dz = -1; dz <= 1; ++dz)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int qz = pz + dz, qx = px + dx;
-                    if (qz < 0 || qz >= PZ || qx < 0 || qx >= PX) continue;
-                    const unsigned *m = S.tmask[qz * PX + qx];
-#pragma unroll
-                    for (int w = 0; w < NWY; ++w)
-                        h[w] |= m[w] | (m[w] << 1) | (m[w] >> 1) | (w + 1 < NWY ? m[w + 1] << 31 : 0u) |
-                                (w > 0 ? m[w - 1] >> 31 : 0u);
-                }
-#pragma unroll
-            for (int w = 0; w < NWY; ++w) S.hot[tid][w] = h[w];
-        }
-        block_sync();
-        // destinations: every particle / tree node of the interior, and every coarse particle (anchored
-        // at its first fine cell), with q > 0 pre-images within distance 1 of a target (the others add
-        // exact zeros). Each takes a slot in its row-group class. First the candidates (interior cells
-        // holding a particle, a tree node or a coarse particle's first cell) are listed in cell order
-        // (warp w: cells [w CPT 32, (w + 1) CPT 32)), in dorder's space; an uncovered cell next to a
-        // target means an invalid layout.
-        constexpr int CPT = MAXT / NT;  // interior cells per thread
-        if (tid < NCLS) S.ccnt[tid] = 0;
-        unsigned bal[CPT];
-        int wcnt = 0;
-#pragma unroll
-        for (int u = 0; u < CPT; ++u) {
-            const int ic = (warp * CPT + u) * 32 + lane;
-            const int r = ic / SY, iy = ic % SY;
-            const int z = s.z0 + r / SX, x = s.x0 + r % SX, y = s.y0 + iy;
-            bool cand = false;
-            if (z < s.g.dz && x < s.g.dx && y < s.g.dy) {
-                const int k = S.srck[ic];
-                if (k == SRC_NONE) {
-                    if (hot_at(S, r / SX + 1, r % SX + 1, iy + 1)) atomicOr(L.err, ERR_DEVICE_CHECK);
-                } else {
-                    cand = k != SRC_C || !((z | x | y) & 1);
-                }
-            }
-            bal[u] = __ballot_sync(0xffffffffu, cand);
-            wcnt += __popc(bal[u]);
-        }
-        if (lane == 0) S.warp_tot[warp] = wcnt;
-        block_sync();
-        int ncand = 0, cbase = 0;
-#pragma unroll
-        for (int w = 0; w < NWARP; ++w) {
-            cbase += w < warp ? S.warp_tot[w] : 0;
-            ncand += S.warp_tot[w];
-        }
-        const unsigned below = (1u << lane) - 1u;
-#pragma unroll
-        for (int u = 0; u < CPT; ++u) {
-            if ((bal[u] >> lane) & 1u) S.dorder[cbase + __popc(bal[u] & below)] = (unsigned short)((warp * CPT + u) * 32 + lane);
-            cbase += __popc(bal[u]);
-        }
-        block_sync();
-        // class of candidate cell ic as a destination (-1: no pre-image within reach of a target)
-        auto dest_class = [&](int ic) -> int {
-            const int r = ic / SY, iy = ic % SY;
-            const int z = s.z0 + r / SX, x = s.x0 + r % SX, y = s.y0 + iy;
-            const bool coarse = S.srck[ic] == SRC_C;
-            uint32_t wz, wx, wy;
-            const int nz = axis_pre(z, coarse, s.g.dz, reflect, s.z0 - 1, &wz);
-            const int nx = axis_pre(x, coarse, s.g.dx, reflect, s.x0 - 1, &wx);
-            const int ny = axis_pre(y, coarse, s.g.dy, reflect, ylo, &wy);
-            int q = 0;
-            for (int a = 0; a < nz; ++a)
-                for (int b = 0; b < nx; ++b)
-                    for (int c = 0; c < ny; ++c) q += hot_at(S, pre_at(wz, a), pre_at(wx, b), pre_at(wy, c));
-            return q == 0 ? -1 : group_class(q);
-        };
-        int my_ic[CPT], my_c[CPT], my_slot[CPT];
-#pragma unroll
-        for (int u = 0; u < CPT; ++u) {
-            const int jc = tid + u * NT;
-            my_ic[u] = 0;
-            my_c[u] = -1;
-            my_slot[u] = 0;
-            if (jc < ncand) {
-                my_ic[u] = S.dorder[jc];
-                my_c[u] = dest_class(my_ic[u]);
-                if (my_c[u] >= 0) my_slot[u] = atomicAdd(&S.ccnt[my_c[u]], 1);
-            }
-        }
-        block_sync();
-        if (tid == 0) {
-            int d = 0, rw = 0;
-            for (int c = 0; c < NCLS; ++c) {
-                S.coff[c] = d;
-                S.rbase[c] = rw;
-                d += S.ccnt[c];
-                rw += S.ccnt[c] * group_rows(c);
-            }
-            S.coff[NCLS] = d;
-            S.rbase[NCLS] = rw;
-        }
-        block_sync();
-#pragma unroll
-        for (int u = 0; u < CPT; ++u)
-            if (my_c[u] >= 0) S.dorder[S.coff[my_c[u]] + my_slot[u]] = (unsigned short)my_ic[u];
-        const int nrows = S.rbase[NCLS], rows2 = S.rbase[1];  // rows2: the two-pass rows come first
-        if (nrows == 0) continue;
-        if (!ready) {
-            store_weights(wreg, S.w);
-            if (tid == 0) mbar_init(&S.bar);
-            if (warp == 0) tmem_alloc(smem_u32(&S.tmem), TMEM_COLS);
-            ready = true;
-        }
-        fence_async_smem();
-        tc_fence_before();
-        block_sync();
-        tc_fence_after();
-        tb = S.tmem;
-        for (int b0 = 0; b0 < nrows; b0 += 128) {
-            // this thread's row: destination ic, its j-th pre-image (j + 32 in the second pass)
-            const int row = b0 + 32 * q + lane;
-            int ic = -1, j = 0, gr = 0;
-            if (row < nrows) {
-                int c = 0;
-                while (row >= S.rbase[c + 1]) ++c;
-                gr = group_rows(c);
-                const int off = row - S.rbase[c];
-                ic = S.dorder[S.coff[c] + off / gr];
-                j = off % gr;
-            }
-            uint32_t wz = 0, wx = 0, wy = 0;
-            int nz = 0, nx = 0, ny = 0;
-            if (ic >= 0) {
-                const int r = ic / SY;
-                const bool coarse = S.srck[ic] == SRC_C;
-                nz = axis_pre(s.z0 + r / SX, coarse, s.g.dz, reflect, s.z0 - 1, &wz);
-                nx = axis_pre(s.x0 + r % SX, coarse, s.g.dx, reflect, s.x0 - 1, &wx);
-                ny = axis_pre(s.y0 + ic % SY, coarse, s.g.dy, reflect, ylo, &wy);
-            }
-            const int npass = b0 < rows2 ? 2 : 1;
-            bool failed = false;
-            for (int pass = 0; pass < npass; ++pass) {
-                // the (j + 32 pass)-th pre-image within distance 1 of a target, in (z, x, y) order
-                int pz = -100, px = 0, py = 0, want = j + 32 * pass;
-                for (int a = 0; a < nz && pz < -1; ++a)
-                    for (int bb = 0; bb < nx && pz < -1; ++bb)
-                        for (int c = 0; c < ny; ++c) {
-                            const int tz = pre_at(wz, a), tx = pre_at(wx, bb), ty = pre_at(wy, c);
-                            if (!hot_at(S, tz, tx, ty)) continue;
-                            if (want-- == 0) {
-                                pz = tz;
-                                px = tx;
-                                py = ty;
-                                break;
-                            }
-                        }
-                // rows past the last one are never read back: a warp holding only such rows skips them;
-                // the adjoint reads G at q - e (the flipped stencil)
-                if (b0 + 32 * q < nrows) {
-                    if (warp < 4) store_taps<0, 14, -1>(S.g0, S.g1, pz, px, py, pz >= 0, tb + lane_base);
-                    else store_taps<14, NTAP, -1>(S.g0, S.g1, pz, px, py, pz >= 0, tb + lane_base);
-                }
-                tmem_wait_st();
-                tc_fence_before();
-                block_sync();
-                tc_fence_after();
-                if (tid == 0) {
-                    for (int e = 0; e < NTAP; ++e)
-                        mma_ts(tb + TM_D, tb + TM_A + 8 * e, sdesc(smem_u32(S.w + e * WTAP), 128, 256),
-                               idesc, (pass > 0 || e > 0) ? 1u : 0u);
-                    mma_commit(&S.bar);
-                }
-                if (block_wait_mma(&S.bar, phase, L.err)) {
-                    failed = true;
-                    break;
-                }
-                phase ^= 1;
-                tc_fence_after();
-            }
-            if (failed) {
-                stop = true;
-                break;
-            }
-            if (warp < 4) {
-                float v[16];
-                tmem_ld16(tb + lane_base + TM_D, v);
-                // sum over the row group in a fixed butterfly order (every lane of a group gets the same sum)
-                const int gmax = __reduce_max_sync(0xffffffffu, gr);
-                for (int w = 1; w < gmax; w <<= 1) {
-#pragma unroll
-                    for (int c = 0; c < MC; ++c) {
-                        const float o = __shfl_xor_sync(0xffffffffu, v[c], w);
-                        if (w < gr) v[c] += o;
-                    }
-                }
-                if (ic >= 0 && j == 0) {
-                    const int k = S.srck[ic];
-                    const size_t idx = size_t(S.srci[ic]);
-                    if (k == SRC_T) {
-                        float4 *o = reinterpret_cast<float4 *>(gt + idx * MC);
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) o[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) red_add_v4(gp + idx * MC + 4 * c, v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-                    }
-                }
-            }
-            tc_fence_before();
-            block_sync();
-            tc_fence_after();
         }
     }
-    if (ready) {
-        tc_fence_before();
-        block_sync();
-        if (warp == 0) tmem_dealloc(tb, TMEM_COLS);
+}
+__device__ __forceinline__ void issue_step(uint32_t D, uint32_t A, uint64_t W, int k, uint32_t el) {
+    switch (k) {
+        case 0: issue_row<1, 1, true>(D, A + 32, W, el); issue_row<1, 0, false>(D, A, W, el); break;
+        case 1: issue_row<1, 2, false>(D, A, W, el); issue_row<1, 3, false>(D, A + 32, W, el); break;
+        case 2: issue_row<0, 0, false>(D, A, W, el); issue_row<0, 1, false>(D, A + 32, W, el); break;
+        case 3: issue_row<0, 2, false>(D, A, W, el); issue_row<0, 3, false>(D, A + 32, W, el); break;
+        case 4: issue_row<2, 0, false>(D, A, W, el); issue_row<2, 1, false>(D, A + 32, W, el); break;
+        case 5: issue_row<2, 2, false>(D, A, W, el); issue_row<2, 3, false>(D, A + 32, W, el); break;
+        case 6: issue_row<3, 0, false>(D, A, W, el); issue_row<3, 1, false>(D, A + 32, W, el); break;
+        default: issue_row<3, 2, false>(D, A, W, el); issue_row<3, 3, false>(D, A + 32, W, el); break;
     }
 }
 
-// ---------------------------------------------------------------- weight gradient
-struct WgradSmem {
-    FeatStage st;
-    Targets tg;
-    alignas(16) unsigned char u[WG_MG * WG_T * 16];  // im2col of WG_T targets: group mg = 2e + h, target t at mg*256 + t*16
-    alignas(16) unsigned char gtile[2 * (WG_T / 8) * 128];  // g^T: co group g, target chunk k at (2g + k) * 128
-    uint64_t bar;
-    uint32_t tmem;
-};
+// D = the tile's sums (S.rows, S.code, S.W and the tensor memory are set up, with a barrier since). Eight
+// warps load: warps q and q + 4 the rows 32 q .. 32 q + 31, one cell row each; the loads of step k + 1 are in
+// flight while step k is written to tensor memory and handed to the ninth warp, which issues the MMAs. A
+// buffer is written again once the MMAs of two steps before have completed. phase: one bit per buffer.
+// True on a timeout.
+__device__ __forceinline__ bool tile_gemm(McSmem &S, const uint4 *__restrict__ vals, const uint4 *__restrict__ tree, bool wide,
+                                          uint32_t D, uint32_t &phase, unsigned *err) {
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int q = warp & 3, half = warp >> 2, r = 32 * q + lane;
+    const uint64_t W = sdesc(smem_u32(S.W), 128, 256);
+    bool ok = true;
+    if (warp < NWARP) {
+        const uint32_t a0 = D + TM_A + (uint32_t(32 * q) << 16) + 32 * half;
+        CellRow c;
+        c.load(S.code, S.rows, r, step_z(0), step_x(0) + half, vals, tree, wide);
+#pragma unroll 1
+        for (int k = 0; k < 8; ++k) {
+            if (k >= 2) ok = mbar_wait(&S.bar[k & 1], (phase >> (k & 1)) & 1u);
+            if (k >= 2) phase ^= 1u << (k & 1);
+            __syncwarp();
+            tc_fence_after();
+            c.store(a0 + 64 * (k & 1));
+            tmem_wait_st();
+            tc_fence_before();
+            if (k + 1 < 8) c.load(S.code, S.rows, r, step_z(k + 1), step_x(k + 1) + half, vals, tree, wide);
+            if (__syncthreads_or(!ok)) break;
+        }
+    } else {
+        const uint32_t el = elect_one();
+#pragma unroll 1
+        for (int k = 0; k < 8; ++k) {
+            if (k >= 2) phase ^= 1u << (k & 1);
+            if (__syncthreads_or(false)) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            issue_step(D, D + TM_A + 64 * (k & 1), W, k, el);
+            if (el) mma_commit(&S.bar[k & 1]);
+            __syncwarp();
+        }
+    }
+    // the last two steps
+    if (ok) ok = mbar_wait(&S.bar[0], phase & 1u) && mbar_wait(&S.bar[1], (phase >> 1) & 1u);
+    const bool bad = block_timed_out(ok, &S.bar[1], (phase >> 1) & 1u, err);
+    phase ^= 3u;
+    tc_fence_after();
+    return bad;
+}
 
-struct WgradPlan {
-    int first[MAXL], last[MAXL];  // CTAs whose unit range meets each level (inclusive), -1 if none
-};
-
-// Persistent: CTA i handles units [i*U/G, (i+1)*U/G) (unit = work item x sub-tile, ordered by level)
-// and keeps one FP32 accumulator per level in tensor memory, flushed to partial[i + level index].
-__global__ void __launch_bounds__(NT, 2) mc_wgrad_kernel(const DevLayout L, const Item *__restrict__ items, int n_units,
-                                                         const uint4 *__restrict__ vals, const uint4 *__restrict__ tree,
-                                                         int bc, const uint4 *__restrict__ gout,
-                                                         float *__restrict__ partial) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    WgradSmem &S = *reinterpret_cast<WgradSmem *>(smraw);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int G = gridDim.x;
-    const int u0 = int((int64_t(blockIdx.x) * n_units) / G), u1 = int((int64_t(blockIdx.x + 1) * n_units) / G);
-    if (u0 >= u1) return;
-    if (tid == 0) mbar_init(&S.bar);
-    for (int i = tid; i < int(sizeof(S.u) / 16); i += NT) reinterpret_cast<uint4 *>(S.u)[i] = make_uint4(0, 0, 0, 0);
-    if (warp == 0) tmem_alloc(smem_u32(&S.tmem), TMEM_COLS);
+// Block set-up shared by the tile kernels: tensor memory, mbarrier, the level's weights (cp.async, waited
+// for by the caller's first cp_wait<0>). The caller's next barrier publishes S.tmem.
+__device__ __forceinline__ void tile_setup(McSmem &S, const uint16_t *wl, int lev) {
+    const int tid = threadIdx.x;
+    if (tid < STAGES) mbar_init(&S.bar[tid]);
+    __syncwarp();
+    if ((tid >> 5) == 0) tmem_alloc(smem_u32(&S.tmem), TMEM_COLS);
+    const uint4 *src = reinterpret_cast<const uint4 *>(wl + size_t(lev) * W_LEVEL);
+    for (int i = tid; i < NWB * WBLK / 16; i += TNT) cp_async16(smem_u32(S.W) + i * 16, src + i, true);
+    cp_commit();
+}
+// Ends the set-up: weights landed and visible to the tensor cores, rows and codes visible to the block.
+__device__ __forceinline__ void tile_ready() {
+    cp_wait<0>();
+    fence_async_smem();
     tc_fence_before();
     block_sync();
     tc_fence_after();
-    const uint32_t tb = S.tmem;
-    const int q = warp & 3;
-    const uint32_t lane_base = uint32_t(32 * q) << 16;
-    constexpr uint32_t idesc = idesc_bf16(128, 16, true);
-    uint32_t phase = 0;
-    // this thread's im2col share, the same in every K step: target it_t, taps ie0 and ie1 (both halves)
-    static_assert(NT == WG_T * 16 && NTAP <= 32, "one target and two taps per thread");
-    const int it_t = tid % WG_T, ie0 = tid / WG_T, ie1 = ie0 + 16;
-    const int off0 = tap_off(ie0), off1 = ie1 < NTAP ? tap_off(ie1) : 0;
-    int cur_l = items[u0 / NSUB].l;
-    bool dirty = false, failed = false;
-    // writes the level's accumulator (zeros if nothing was accumulated) to partial[cta + level index];
-    // D block mb (rows 128 mb .. +127 of (e, ci)) lives in columns 16 mb .. 16 mb + 15
-    auto flush = [&]() {
-        if (warp < 4) {
-            float *dst = partial + size_t(blockIdx.x + cur_l - L.l_min) * WG_ROWS * MC;
-            for (int mb = 0; mb < 4; ++mb) {
-                float v[16];
-                tmem_ld16(tb + lane_base + 16 * mb, v);
-                const int row = 128 * mb + 32 * q + lane;
-                if (row < WG_ROWS) {
-                    float4 *o = reinterpret_cast<float4 *>(dst + size_t(row) * MC);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        o[c] = dirty ? make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3])
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-        }
-        tc_fence_before();
-        block_sync();
-        tc_fence_after();
-    };
-    for (int u = u0; u < u1 && !failed; ++u) {
-        Sub s;
-        const Item it = items[u / NSUB];
-        if (it.l != cur_l) {
-            flush();
-            cur_l = it.l;
-            dirty = false;
-        }
-        if (!sub_of(L, it, u % NSUB, s)) continue;
-        const int nt = count_targets(L, s, S.tg);
-        if (nt == 0) continue;
-        // dL/dout of the first step's targets, loaded while the patch is staged; each step then loads
-        // the next step's while its MMAs run (threads 0 .. 2 WG_T - 1: target tid / 2, half tid % 2)
-        uint4 gnext = make_uint4(0, 0, 0, 0);
-        if (tid < 2 * WG_T && (tid >> 1) < nt) gnext = gout[2 * size_t(target_index(S.tg, tid >> 1)) + (tid & 1)];
-        stage_features(L, s, u, vals, tree, bc, S.st, &S.tg);
-        for (int t0 = 0; t0 < nt; t0 += WG_T) {
-            // im2col: entry (mg, t) = channels 8h .. 8h+7 of tap e = mg / 2 at target t0 + t; this
-            // thread copies both halves of taps ie0 and ie1 for target it_t
-            {
-                const bool live = t0 + it_t < nt;
-                const int cell = live ? int(S.tg.cell[t0 + it_t]) : 0;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int e = h ? ie1 : ie0;
-                    if (e < NTAP) {
-                        uint4 a = make_uint4(0, 0, 0, 0), b = a;
-                        if (live) {
-                            const int c = cell + (h ? off1 : off0);
-                            a = S.st.p0[c];
-                            b = S.st.p1[c];
-                        }
-                        *reinterpret_cast<uint4 *>(S.u + (2 * e) * (WG_T * 16) + it_t * 16) = a;
-                        *reinterpret_cast<uint4 *>(S.u + (2 * e + 1) * (WG_T * 16) + it_t * 16) = b;
-                    }
-                }
-            }
-            // g^T (N = co rows, K = targets), K-major core matrices
-            if (tid < 2 * WG_T) {
-                const int tt = tid >> 1, h = tid & 1, tn = t0 + WG_T + tt;
-                const uint4 v = gnext;
-                gnext = tn < nt ? gout[2 * size_t(S.tg.idx[tn]) + h] : make_uint4(0, 0, 0, 0);
-                const uint16_t *p = reinterpret_cast<const uint16_t *>(&v);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)  // co = 8h + j
-                    *reinterpret_cast<uint16_t *>(S.gtile + (h * (WG_T / 8) + (tt >> 3)) * 128 + j * 16 + (tt & 7) * 2) = p[j];
-            }
-            fence_async_smem();
-            tc_fence_before();
-            block_sync();
-            tc_fence_after();
-            if (tid == 0) {
-                const uint64_t bd = sdesc(smem_u32(S.gtile), 128, (WG_T / 8) * 128);
-                for (int mb = 0; mb < 4; ++mb) {
-                    const uint64_t ad = sdesc(smem_u32(S.u + mb * 16 * (WG_T * 16)), 128, WG_T * 16);
-                    mma_ss(tb + 16 * mb, ad, bd, idesc, dirty ? 1u : 0u);
-                }
-                mma_commit(&S.bar);
-            }
-            if (block_wait_mma(&S.bar, phase, L.err)) {
-                failed = true;
-                break;
-            }
-            phase ^= 1;
-            dirty = true;
-            tc_fence_after();
-        }
-    }
-    if (!failed) flush();
+}
+__device__ __forceinline__ void tile_teardown(const McSmem &S) {
     tc_fence_before();
     block_sync();
-    if (warp == 0) tmem_dealloc(tb, TMEM_COLS);
+    if ((threadIdx.x >> 5) == 0) tmem_dealloc(S.tmem, TMEM_COLS);
 }
 
-// grad_weights[lev][co][ci][e] = sum over the level's CTAs (in order) of partial[cta + lev][16e + ci][co]
-__global__ void mc_wgrad_reduce_kernel(const float *__restrict__ partial, WgradPlan plan, int n_levels,
+// Orders the tile's tensor-memory reads before the next tile's MMAs.
+__device__ __forceinline__ void tile_done() {
+    tc_fence_before();
+    block_sync();
+    tc_fence_after();
+}
+
+// ---------------------------------------------------------------- forward
+// out (float32 [N][16]) receives the convolution; if out_bf16 is given instead, it receives
+// bf16(max(conv, 0)), the next layer's input in an APR CNN (the ReLU fused into the write).
+__global__ void __launch_bounds__(TNT, 2) mc_fwd_kernel(const UnitView U, const uint4 *__restrict__ vals,
+                                                       const uint4 *__restrict__ tree, const uint16_t *__restrict__ W, int bc,
+                                                       float *__restrict__ out, uint4 *__restrict__ out_bf16, unsigned *err) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    McSmem &S = *reinterpret_cast<McSmem *>(smraw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const UnitHdr h = U.hdr[blockIdx.x];
+    stage_codes<true>(U, h, false, bc == APR_BC_REFLECT, S.code);
+    pdl_wait();   // the weight layout and the tree are written by the launches before this one
+    tile_setup(S, W, h.lev);
+    const bool wide = ((reinterpret_cast<uintptr_t>(vals) | reinterpret_cast<uintptr_t>(tree)) & 31u) == 0;
+    uint32_t phase = 0;
+    const int q = warp & 3, a = warp >> 2;
+    for (int t0 = 0; t0 < h.nrec; t0 += TILE) {
+        if (tid < TILE) {
+            if (t0 + tid < h.nrec) put_node_row(S.rows, tid, U.rec + h.rec0 + t0 + tid);
+            else S.rows.mask[tid] = 0;
+        }
+        tile_ready();
+        const uint32_t D = S.tmem;
+        if (tile_gemm(S, vals, tree, wide, D, phase, err)) break;
+        // lane = record, this warp's half of the children (a): the particles' outputs
+        const int r = t0 + 32 * q + lane;
+        int2 pw = make_int2(0, 0);
+        if (warp < NWARP && r < h.nrec) pw = __ldg(reinterpret_cast<const int2 *>(U.nplan[U.rec[h.rec0 + r].node].p + 2 * a));
+        if (warp < NWARP)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float v[16];
+            tmem_ld16(D + (uint32_t(32 * q) << 16) + 64 * a + 16 * c, v);
+            const unsigned w = unsigned(c < 2 ? pw.x : pw.y), pm = w >> 30;
+            if ((pm >> (c & 1)) & 1u) {
+                const size_t p = (w & TNP_INDEX) + (c & 1 ? pm & 1u : 0u);
+                if (out_bf16) {
+                    uint4 o[2];
+                    __nv_bfloat162 *b2 = reinterpret_cast<__nv_bfloat162 *>(o);
+#pragma unroll
+                    for (int k = 0; k < MC / 2; ++k) b2[k] = __floats2bfloat162_rn(fmaxf(v[2 * k], 0.f), fmaxf(v[2 * k + 1], 0.f));
+                    out_bf16[2 * p] = o[0];
+                    out_bf16[2 * p + 1] = o[1];
+                } else {
+                    float4 *o = reinterpret_cast<float4 *>(out + p * MC);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) o[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                }
+            }
+        }
+        tile_done();
+    }
+    tile_teardown(S);
+}
+
+// ---------------------------------------------------------------- data adjoint
+// 4 channels at p, added.
+__device__ __forceinline__ void add4(float *p, const float4 &s) {
+    float4 *q = reinterpret_cast<float4 *>(p);
+    float4 v = *q;
+    v.x += s.x;
+    v.y += s.y;
+    v.z += s.z;
+    v.w += s.w;
+    *q = v;
+}
+
+// Exclusive prefix of n (one value of each of the first NT threads) into first[0 .. NT]. Ends with a barrier.
+__device__ __forceinline__ int prefix_rows(McSmem &S, int n) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31 && warp < NWARP) S.wsum[warp] = incl;
+    block_sync();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < NWARP; ++w) {
+        before += w < warp ? S.wsum[w] : 0;
+        total += S.wsum[w];
+    }
+    if (tid < NT) S.first[tid] = before + incl - n;
+    if (tid == 0) S.first[NT] = total;
+    block_sync();
+    return total;
+}
+// The record (of n) that owns row k.
+__device__ __forceinline__ int row_owner(const McSmem &S, int n, int k) {
+    int a = 0, b = n;
+    while (b - a > 1) {
+        const int m = (a + b) / 2;
+        if (S.first[m] <= k) a = m;
+        else b = m;
+    }
+    return a;
+}
+// The n-th set bit of m (n < its population count).
+__device__ __forceinline__ int nth_bit(unsigned long long m, int n) {
+    for (; n > 0; --n) m &= m - 1ull;
+    return __ffsll((long long)m) - 1;
+}
+// Images of an edge record (edge_shifts<1> without its own place), after them one row that repeats its own
+// place if it has missing children (their sums belong to their siblings).
+__device__ __forceinline__ int image_rows(unsigned edge) {
+    return __popcll(edge_shifts<1>(edge)) - 1 + (missing_children(edge) ? 1 : 0);
+}
+__device__ __forceinline__ int image_row(unsigned edge, int j) {
+    const unsigned long long m = edge_shifts<1>(edge) & ~1ull;
+    return j < __popcll(m) ? nth_bit(m, j) : 0;
+}
+
+// Float4 chunk k (0..15) of row r in the 128 x 64-float staging of the image sums (16-byte chunks swizzled by
+// the row: conflict-free for lane = row).
+__device__ __forceinline__ float4 *image_chunk(McSmem &S, int r, int k) {
+    return S.sums + r * 16 + (k ^ (r & 15));
+}
+
+// Data adjoint onto the children of every record: particles (gp) and tree nodes (gt) are stored, then, with
+// reflection, the images of the edge records are added.
+__global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, const uint16_t *__restrict__ W, int bc,
+                                                           const uint4 *__restrict__ gout, float *__restrict__ gp,
+                                                           float *__restrict__ gt, unsigned *err) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    McSmem &S = *reinterpret_cast<McSmem *>(smraw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const UnitHdr h = U.hdr[blockIdx.x];
+    const NodeRec *rec = U.rec + h.rec0;
+    stage_codes<false>(U, h, false, false, S.code);
+    pdl_wait();   // the weight layout is written by the launch before this one
+    tile_setup(S, W, h.lev);
+    const bool wide = (reinterpret_cast<uintptr_t>(gout) & 31u) == 0;
+    uint32_t phase = 0;
+    const int q = warp & 3, a = warp >> 2;
+    bool failed = false;
+    for (int t0 = 0; t0 < h.nrec && !failed; t0 += TILE) {
+        if (tid < TILE) {
+            if (t0 + tid < h.nrec) put_node_row(S.rows, tid, rec + t0 + tid);
+            else S.rows.mask[tid] = 0;
+        }
+        tile_ready();
+        const uint32_t D = S.tmem;
+        failed = tile_gemm(S, gout, gout, wide, D, phase, err);
+        if (failed) break;
+        const int r = t0 + 32 * q + lane;
+        int4 pw = make_int4(0, 0, 0, 0), tw = pw;
+        if (warp < NWARP && r < h.nrec) {
+            const int4 *m = reinterpret_cast<const int4 *>(U.nplan + rec[r].node);
+            pw = __ldg(m);
+            tw = __ldg(m + 1);
+        }
+        const int pk[2] = {a ? pw.z : pw.x, a ? pw.w : pw.y}, tk[2] = {a ? tw.z : tw.x, a ? tw.w : tw.y};
+        if (warp < NWARP)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float v[16];
+            tmem_ld16(D + (uint32_t(32 * q) << 16) + 64 * a + 16 * c, v);
+            const unsigned p = unsigned(pk[c >> 1]), t = unsigned(tk[c >> 1]), pm = p >> 30, tm = t >> 30;
+            const int e = c & 1;
+            float *dst = nullptr;
+            if ((pm >> e) & 1u) dst = gp + (size_t(p & TNP_INDEX) + (e ? pm & 1u : 0u)) * MC;
+            else if ((tm >> e) & 1u) dst = gt + (size_t(t & TNP_INDEX) + (e ? tm & 1u : 0u)) * MC;
+            if (dst)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    reinterpret_cast<float4 *>(dst)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+        }
+        tile_done();
+    }
+    if (!failed && bc == APR_BC_REFLECT && h.nflag > 0) {
+        const int total = prefix_rows(S, tid < h.nflag ? image_rows(rec[tid].edge) : 0);
+        for (int k0 = 0; k0 < total && !failed; k0 += TILE) {
+            if (tid < TILE) {
+                const int k = k0 + tid;
+                if (k < total) {
+                    const int i = row_owner(S, h.nflag, k);
+                    put_image_row(S.rows, tid, rec + i, image_row(rec[i].edge, k - S.first[i]));
+                } else {
+                    S.rows.mask[tid] = 0;
+                }
+            }
+            tile_ready();
+            const uint32_t D = S.tmem;
+            failed = tile_gemm(S, gout, gout, wide, D, phase, err);
+            if (failed) break;
+            // source children of half a (64 columns) through shared memory; one
+            // thread per (record, child place (b, e), four channels) adds the rows' sums in order
+            const int i0 = row_owner(S, h.nflag, k0), i1 = row_owner(S, h.nflag, min(k0 + TILE, total) - 1);
+            for (int half = 0; half < 2; ++half) {
+                if (warp < NWARP)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    float v[16];
+                    const int col = 32 * a + 16 * c, r = 32 * q + lane;
+                    tmem_ld16(D + (uint32_t(32 * q) << 16) + 64 * half + col, v);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        *image_chunk(S, r, col / 4 + k) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                }
+                block_sync();
+                for (int w = tid; w < (i1 - i0 + 1) * 16; w += TNT) {
+                    const int i = i0 + (w >> 4), place = (w >> 2) & 3, ch = w & 3;
+                    const unsigned edge = rec[i].edge, miss = missing_children(edge);
+                    const TreeNodePlan &m = U.nplan[rec[i].node];
+                    for (int k = max(S.first[i], k0); k < min(S.first[i + 1], k0 + TILE); ++k) {
+                        const int t = image_row(edge, k - S.first[i]);
+                        const unsigned mir = (t >> 4 ? 4u : 0u) | ((t >> 2) & 3 ? 2u : 0u) | (t & 3 ? 1u : 0u);
+                        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+                        unsigned to = 8u;   // the target child (the same for every source found)
+                        for (int src = 0; src < 4; ++src) {
+                            const unsigned full = (4u * half + src) ^ mir;   // before a missing child is folded
+                            if ((t == 0 && !(full & miss)) || int((full & ~miss) & 3u) != place) continue;
+                            to = full & ~miss;
+                            const float4 v = *image_chunk(S, k - k0, src * 4 + ch);
+                            s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
+                        }
+                        if (to == 8u) continue;
+                        const unsigned p = unsigned(m.p[to >> 1]), tt = unsigned(m.t[to >> 1]), pm = p >> 30, tm = tt >> 30;
+                        const int e = int(to & 1u);
+                        if ((pm >> e) & 1u) add4(gp + (size_t(p & TNP_INDEX) + (e ? pm & 1u : 0u)) * MC + 4 * ch, s);
+                        else if ((tm >> e) & 1u) add4(gt + (size_t(tt & TNP_INDEX) + (e ? tm & 1u : 0u)) * MC + 4 * ch, s);
+                    }
+                }
+                block_sync();
+            }
+            tile_done();
+        }
+    }
+    tile_teardown(S);
+}
+
+// Data adjoint onto the coarser particles next to nodes: the sums over their eight cells, added to gp
+// (after mc_adjoint_kernel). Rows: every record at its own place and, with reflection, at its images.
+__global__ void __launch_bounds__(TNT, 2) mc_leaf_adjoint_kernel(const UnitView U, const uint16_t *__restrict__ W, int bc,
+                                                                const uint4 *__restrict__ gout, float *__restrict__ gp,
+                                                                unsigned *err) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    McSmem &S = *reinterpret_cast<McSmem *>(smraw);
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const UnitHdr h = U.lhdr[blockIdx.x];
+    const LeafRec *rec = U.lrec + h.rec0;
+    const bool reflect = bc == APR_BC_REFLECT;
+    stage_codes<false>(U, h, true, false, S.code);
+    tile_setup(S, W, h.lev);
+    const bool wide = (reinterpret_cast<uintptr_t>(gout) & 31u) == 0;
+    uint32_t phase = 0;
+    const int total = prefix_rows(S, tid < h.nrec ? (reflect ? __popcll(edge_shifts<1>(rec[tid].edge)) : 1) : 0);
+    for (int k0 = 0; k0 < total; k0 += TILE) {
+        unsigned skip = 0;   // cells outside the grid are no part of the source (zero boundary)
+        if (tid < TILE) {
+            const int k = k0 + tid;
+            if (k < total) {
+                const int i = row_owner(S, h.nrec, k);
+                put_leaf_row(S.rows, tid, rec + i, reflect ? nth_bit(edge_shifts<1>(rec[i].edge), k - S.first[i]) : 0);
+                if (!reflect) skip = missing_children(rec[i].edge);
+            } else {
+                S.rows.mask[tid] = 0;
+            }
+        }
+        tile_ready();
+        const uint32_t D = S.tmem;
+        if (tile_gemm(S, gout, gout, wide, D, phase, err)) break;
+        if (warp < 4) {   // thread = row
+            float s[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) s[k] = 0.f;
+            for (unsigned c = 0; c < 8; ++c) {
+                float v[16];
+                tmem_ld16(D + (uint32_t(32 * warp) << 16) + 16 * c, v);
+                if (!(c & skip))
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) s[k] += v[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) *image_chunk(S, tid, k) = make_float4(s[4 * k], s[4 * k + 1], s[4 * k + 2], s[4 * k + 3]);
+        }
+        block_sync();
+        const int i0 = row_owner(S, h.nrec, k0), i1 = row_owner(S, h.nrec, min(k0 + TILE, total) - 1);
+        for (int w = tid; w < (i1 - i0 + 1) * 4; w += TNT) {
+            const int i = i0 + (w >> 2), ch = w & 3;
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = max(S.first[i], k0); k < min(S.first[i + 1], k0 + TILE); ++k) {
+                const float4 v = *image_chunk(S, k - k0, ch);
+                s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
+            }
+            add4(gp + size_t(rec[i].particle) * MC + 4 * ch, s);
+        }
+        tile_done();
+    }
+    tile_teardown(S);
+}
+
+// ---------------------------------------------------------------- weight gradient
+// One block per SM takes a contiguous range of the units of the levels that hold particles. Per tile of 128
+// records, the four planes iz of cells are gathered one after the other (16 cells, two buffers), and for
+// every child row (a, b) the taps tz = iz - a and tx = 0..2 take MMAs over K = the records:
+//   D[tz][tx block][(tx, iy, ci)][(e, co)] += U(cell (iz, b + tx, iy))[ci] g(child (a, b, e))[co]
+// with M = 128 = two rows of four cells x 16 channels (the second block's second half is not used: it reads
+// the next row or past the plane, inside the block's shared memory). The tap along y is iy - e. After
+// every tile D is added to FP32 registers (96 per thread), so that the tensor cores' accumulation chains stay
+// at 32 MMAs; a level's sums are written to the level's partial of the block and reduced in order.
+constexpr int WG_SBO = 2048 + 16;           // 8 channels of a cell for 128 records, padded: eight lanes write
+                                            // eight pieces of one record without bank conflicts
+constexpr int WG_CELL = 2 * WG_SBO;
+constexpr int PLANE_BYTES = 16 * WG_CELL;
+constexpr uint32_t WG_TMEM = 256;           // D: block (tz, tx block) in columns 32 (2 tz + block), 192 used
+constexpr int WG_OUT = NTAP * MC * MC;      // floats of one partial: [tap][ci][co]
+struct WgradSmem {
+    int code[8][PLANE];
+    Rows rows;
+    alignas(128) unsigned char A[2][PLANE_BYTES];   // cell-major: (2 cell + h) WG_SBO + (r / 8) 128 + (r % 8) 16
+    alignas(128) unsigned char g[8 * WG_CELL];      // the same for the eight children
+    uint64_t bar;
+    uint32_t tmem;
+};
+
+__device__ __forceinline__ void gather_plane(const WgradSmem &S, const uint4 *__restrict__ vals, const uint4 *__restrict__ tree,
+                                             int iz, uint32_t A) {
+    const int lane = threadIdx.x & 31, iy = (lane >> 1) & 3, h = lane & 1;   // eight lanes per row
+    const uint32_t dst = A + uint32_t((2 * iy + h) * WG_SBO);
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+        const int r = (threadIdx.x >> 5) * 16 + 4 * j + (lane >> 3);
+        const unsigned mask = S.rows.mask[r];
+#pragma unroll
+        for (int ix = 0; ix < 4; ++ix) {
+            const int q = ((iz + 1) >> 1) * 3 + ((ix + 1) >> 1), c0 = ((iz + 1) & 1) * 4 + ((ix + 1) & 1) * 2;
+            const int code = cell_code(S.code, (mask >> (3 * q)) & 7u, S.rows.base[q][r], c0, iy);
+            cp_async16(dst + 4 * ix * WG_CELL + (r >> 3) * 128 + (r & 7) * 16, source_row(vals, tree, code) + h, code != NO_SOURCE);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const UnitLevels L, const uint4 *__restrict__ vals,
+                                                         const uint4 *__restrict__ tree, int bc,
+                                                         const uint4 *__restrict__ gout, float *__restrict__ partial,
+                                                         unsigned *err) {
+    extern __shared__ __align__(128) unsigned char smraw[];
+    WgradSmem &S = *reinterpret_cast<WgradSmem *>(smraw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = warp & 3, half = warp >> 2;
+    const int total = L.begin[L.n];
+    const int u0 = int(int64_t(blockIdx.x) * total / gridDim.x), u1 = int(int64_t(blockIdx.x + 1) * total / gridDim.x);
+    if (tid == 0) mbar_init(&S.bar);
+    if (warp == 0) tmem_alloc(smem_u32(&S.tmem), WG_TMEM);
+    tile_done();
+    const uint32_t D = S.tmem, A = smem_u32(S.A[0]), G = smem_u32(S.g);
+    constexpr uint32_t idesc = idesc_bf16(128, 32, true);
+    uint32_t phase = 0;
+    bool failed = false;
+    for (int i = 0; i < L.n && !failed; ++i) {
+        const int ua = max(u0, L.begin[i]), ub = min(u1, L.begin[i + 1]);
+        if (ua >= ub) continue;
+        float acc[96];
+#pragma unroll
+        for (int k = 0; k < 96; ++k) acc[k] = 0.f;
+        for (int u = ua; u < ub && !failed; ++u) {
+            const UnitHdr h = U.hdr[L.unit0[i] + u - L.begin[i]];
+            stage_codes<true>(U, h, false, bc == APR_BC_REFLECT, S.code);
+            for (int t0 = 0; t0 < h.nrec && !failed; t0 += TILE) {
+                if (tid < TILE) {
+                    if (t0 + tid < h.nrec) put_node_row(S.rows, tid, U.rec + h.rec0 + t0 + tid);
+                    else S.rows.mask[tid] = 0;
+                }
+                block_sync();
+                {
+                    // dL/dout of the records' children (zero where the child is no particle)
+                    const int be = (lane >> 1) & 3, hh = lane & 1;   // eight lanes per row: child (b, e), half
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int r = warp * 16 + 4 * j + (lane >> 3);
+                        int4 pw = make_int4(0, 0, 0, 0);
+                        if (t0 + r < h.nrec) pw = child_particles(U, U.rec[h.rec0 + t0 + r].node);
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) {
+                            const unsigned w = unsigned(be < 2 ? (a ? pw.z : pw.x) : (a ? pw.w : pw.y)), pm = w >> 30;
+                            const size_t p = (w & TNP_INDEX) + (be & 1 ? pm & 1u : 0u);
+                            cp_async16(G + uint32_t((2 * (4 * a + be) + hh) * WG_SBO + (r >> 3) * 128 + (r & 7) * 16),
+                                       gout + 2 * p + hh, (pm >> (be & 1)) & 1u);
+                        }
+                    }
+                }
+                gather_plane(S, vals, tree, 0, A);
+                cp_commit();
+                gather_plane(S, vals, tree, 1, A + PLANE_BYTES);
+                cp_commit();
+#pragma unroll 1
+                for (int iz = 0; iz < 4; ++iz) {
+                    cp_wait<1>();
+                    fence_async_smem();
+                    tile_done();
+                    if (tid == 0) {
+                        const uint64_t P = sdesc(A + (iz & 1) * PLANE_BYTES, 128, WG_SBO), B = sdesc(G, 128, WG_SBO);
+                        for (int a = 0; a < 2; ++a) {
+                            const int tz = iz - a;
+                            if (tz < 0 || tz > 2) continue;
+#pragma unroll
+                            for (int b = 0; b < 2; ++b)
+#pragma unroll
+                                for (int blk = 0; blk < 2; ++blk)
+#pragma unroll
+                                    for (int ks = 0; ks < TILE / 16; ++ks)
+                                        mma_ss(D + 64 * tz + 32 * blk, P + (((b + 2 * blk) * 4 * WG_CELL + ks * 256) >> 4),
+                                               B + uint32_t(a * 4 * WG_CELL >> 4) + ((2 * b * WG_CELL + ks * 256) >> 4), idesc,
+                                               b + ks > 0 ? 1u : (a > 0 ? 1u : 0u));
+                        }
+                        mma_commit(&S.bar);
+                    }
+                    if (block_wait_mma(&S.bar, phase, err)) {
+                        failed = true;
+                        break;
+                    }
+                    phase ^= 1;
+                    if (iz + 2 < 4) gather_plane(S, vals, tree, iz + 2, A + (iz & 1) * PLANE_BYTES);
+                    cp_commit();
+                }
+                cp_wait<0>();
+                if (failed) break;
+                tc_fence_after();
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    float v[16];
+                    tmem_ld16(D + (uint32_t(32 * q) << 16) + 96 * half + 16 * k, v);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) acc[16 * k + c] += v[c];
+                }
+                tile_done();
+            }
+        }
+        if (failed) break;
+        // sums of the level: thread (row 32 q + lane, columns 96 half ..) to shared memory, block by block of
+        // 32 columns, then tap (tz, tx, ty), ci, co = its two children e of rows (tx, iy = ty + e, ci)
+        float *stage = reinterpret_cast<float *>(S.A[0]);   // [128][33]
+        float *dst = partial + size_t(blockIdx.x + i) * WG_OUT;
+#pragma unroll
+        for (int blk = 0; blk < 6; ++blk) {                 // (tz, tx block)
+            block_sync();
+            if (half == blk / 3)
+#pragma unroll
+                for (int c = 0; c < 32; ++c) stage[(32 * q + lane) * 33 + c] = acc[32 * (blk % 3) + c];
+            block_sync();
+            const int ntx = blk & 1 ? 1 : 2;
+            for (int o = tid; o < ntx * 3 * MC * MC; o += NT) {
+                const int co = o % MC, ci = (o / MC) % MC, ty = (o / (MC * MC)) % 3, txo = o / (3 * MC * MC);
+                const float *s = stage + ((txo * 4 + ty) * MC + ci) * 33 + co;
+                const int tap = ((blk >> 1) * 3 + 2 * (blk & 1) + txo) * 3 + ty;
+                dst[(tap * MC + ci) * MC + co] = s[0] + s[MC * 33 + 16];   // e = 0: iy = ty; e = 1: iy = ty + 1
+            }
+        }
+        block_sync();
+    }
+    tile_done();
+    if (warp == 0) tmem_dealloc(D, WG_TMEM);
+}
+
+// grad_weights[lev][co][ci][e] = sum over the level's partials, in order; zero for a level without particles.
+__global__ void mc_wgrad_reduce_kernel(const float *__restrict__ partial, const UnitRanges R, int n_levels,
                                        float *__restrict__ gw) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_levels * WG_ROWS * MC) return;
-    const int lev = i / (WG_ROWS * MC), r = i % (WG_ROWS * MC);
-    const int row = r / MC, co = r % MC;
-    float acc = 0.0f;
-    if (plan.first[lev] >= 0)
-        for (int c = plan.first[lev]; c <= plan.last[lev]; ++c) acc += partial[(size_t(c) + lev) * WG_ROWS * MC + r];
-    const int e = row / MC, ci = row % MC;
-    gw[((size_t(lev) * MC + co) * MC + ci) * NTAP + e] = acc;
+    if (i >= n_levels * WG_OUT) return;
+    const int lev = i / WG_OUT, r = i % WG_OUT;
+    float s = 0.f;
+    for (int c = R.first[lev]; c <= R.last[lev]; ++c) s += partial[size_t(c) * WG_OUT + r];
+    const int co = r % MC, ci = (r / MC) % MC, e = r / (MC * MC);
+    gw[((size_t(lev) * MC + co) * MC + ci) * NTAP + e] = s;
 }
 
-// Each CTA of the tensor-core kernels holds 256 of the SM's 512 tensor-memory columns, so their
-// shared memory must admit exactly two CTAs per SM (228 KB per SM, 1 KB reserved per CTA).
-constexpr size_t kTwoPerSmMin = 76 * 1024, kTwoPerSmMax = 112 * 1024;
-static_assert(sizeof(FwdSmem) > kTwoPerSmMin && sizeof(FwdSmem) <= kTwoPerSmMax, "forward: two CTAs per SM");
-static_assert(sizeof(BwdSmem) > kTwoPerSmMin && sizeof(BwdSmem) <= kTwoPerSmMax, "data adjoint: two CTAs per SM");
-static_assert(sizeof(WgradSmem) > kTwoPerSmMin && sizeof(WgradSmem) <= kTwoPerSmMax, "weight gradient: two CTAs per SM");
-// operands of tensor-core descriptors and 16-byte vector accesses start on 16-byte boundaries
-static_assert(offsetof(FwdSmem, w) % 16 == 0 && offsetof(BwdSmem, w) % 16 == 0, "weights alignment");
-static_assert(offsetof(WgradSmem, u) % 16 == 0 && offsetof(WgradSmem, gtile) % 16 == 0, "operand alignment");
-static_assert(offsetof(BwdSmem, g1) % 16 == 0 && offsetof(FeatStage, p1) % 16 == 0, "patch alignment");
-static_assert(offsetof(FwdSmem, bar) % 8 == 0 && offsetof(BwdSmem, bar) % 8 == 0 && offsetof(WgradSmem, bar) % 8 == 0,
-              "mbarrier alignment");
+// The tile kernels' shared memory admits two blocks per SM (228 KB per SM, 1 KB reserved per block), each
+// with half of the SM's 512 tensor-memory columns; the weight gradient takes an SM to itself.
+static_assert(2 * (sizeof(McSmem) + 1024) <= 228 * 1024, "tile kernels: two blocks per SM");
+static_assert(sizeof(WgradSmem) <= 227 * 1024, "weight gradient: one block per SM");
+static_assert(offsetof(McSmem, W) % 128 == 0 && offsetof(McSmem, bar) % 8 == 0, "alignment");
+static_assert(offsetof(WgradSmem, A) % 128 == 0 && offsetof(WgradSmem, g) % 128 == 0 && offsetof(WgradSmem, bar) % 8 == 0, "alignment");
+static_assert(PLANE_BYTES >= 128 * 33 * 4, "sums staged in an A buffer");
 
-cudaError_t set_smem(const void *fn, size_t bytes) { return set_max_dynamic_smem(fn, bytes); }
-
-// CTAs of the weight-gradient kernel: 8 per SM (2 resident at a time), so each CTA accumulates a
-// short chain of tensor-core MMAs (about 1/8 of an SM's share of the units) before its partial sum
-// is written; the fixed-order reduction then adds the partials in FP32.
+// Partials the workspace of the weight gradient holds (without the levels): the blocks are at most as many.
 int wgrad_ctas(int n_units) {
     static int sms = 0;
     static std::once_flag once;
@@ -1219,45 +1032,23 @@ int wgrad_ctas(int n_units) {
     return std::max(1, std::min(n_units, 8 * sms));
 }
 
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl, Args &&...args) {
+    if (grid <= 0) return cudaSuccess;
+    const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void *>(kernel), smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kernel, dim3(grid), dim3(block), smem, s, pdl, std::forward<Args>(args)...);
+}
+
+cudaError_t layout_weights(const uint16_t *W, int n_levels, int adjoint, uint16_t *out, cudaStream_t s) {
+    mc_weight_layout_kernel<<<(n_levels * W_LEVEL + 255) / 256, 256, 0, s>>>(W, n_levels, adjoint, out);
+    return cudaGetLastError();
+}
+
 bool mc_args_ok(int32_t c_in, int32_t c_out, int32_t k) { return c_in == MC && c_out == MC && k == 3; }
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
-
-// Multi-channel sub-tile plans (host): for every sub-tile (item * NSUB + sub) the non-empty feature
-// segments (fwd_items; meta = segment index | MC_REFL for rows outside the grid) and the non-empty
-// data-adjoint segments (bwd_items; meta = segment index). Entries as in the single-channel plans.
-bool build_mc_plans(const DevLayout &L, const HostIndex &X, HostPlan &feat, HostPlan &adj) {
-    bool ok = true;
-    auto build = [&](const std::vector<Item> &items, HostPlan &P, bool features) {
-        P.hdr.assign(items.size() * NSUB, PlanHdr{0, 0});
-        P.ent.clear();
-        for (size_t t = 0; t < items.size(); ++t)
-            for (int sub = 0; sub < NSUB; ++sub) {
-                const int first = int(P.ent.size());
-                int total = 0;
-                Sub s;
-                if (sub_of(L, items[t], sub, s)) {
-                    const int nseg = features ? NSEG_F : NSEG_B;
-                    for (int sg = 0; sg < nseg; ++sg) {
-                        int lo = 0, hi = 0;
-                        bool refl = false;
-                        if (features) feat_segment(L, s, sg, lo, hi, refl);
-                        else adj_segment(L, s, sg, lo, hi);
-                        if (hi <= lo) continue;
-                        P.ent.push_back(PlanEnt{lo, uint16_t(sg | (refl ? MC_REFL : 0)), uint16_t(total)});
-                        total += hi - lo;
-                        if (total > 65535) ok = false;
-                    }
-                }
-                P.hdr[t * NSUB + sub] = PlanHdr{first, int(P.ent.size()) - first};
-                P.ent.push_back(PlanEnt{0, 0, uint16_t(total)});
-            }
-    };
-    build(X.fwd_items, feat, true);
-    build(X.bwd_items, adj, false);
-    return ok;
-}
 
 }  // namespace aprk
 
@@ -1296,16 +1087,13 @@ static apr_status_t convolve_mc(apr_handle_t h, const uint16_t *particles, const
     const HostIndex &X = h->X;
     if (!weights || (X.np && (!particles || (!out && !out_bf16))) || (X.nt && !tree)) return APR_ERR_INVALID_ARG;
     if (!aligned16(particles) || !aligned16(tree) || !aligned16(out) || !aligned16(out_bf16)) return APR_ERR_INVALID_ARG;
-    const size_t sm = sizeof(FwdSmem);
-    cudaError_t e = set_smem(reinterpret_cast<const void *>(mc_fwd_kernel), sm);
-    const int n = int(X.fwd_items.size());
     const int nl = X.l_max - X.l_min + 1;
-    if (e == cudaSuccess && n > 0) {
-        mc_weight_layout_kernel<<<(nl * MC * MC * NTAP + 255) / 256, 256, 0, stream>>>(weights, nl, 0, h->d_mcw);
-        mc_fwd_kernel<<<dim3(n, NSUB / SPC_F), NT, sm, stream>>>(h->L, h->d_fwd, reinterpret_cast<const uint4 *>(particles),
-                                                          reinterpret_cast<const uint4 *>(tree), h->d_mcw, bc, out,
-                                                          reinterpret_cast<uint4 *>(out_bf16));
-        e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (h->n_fwd_units > 0) {
+        e = layout_weights(weights, nl, 0, h->d_mcw, stream);
+        if (e == cudaSuccess)
+            e = launch(mc_fwd_kernel, h->n_fwd_units, TNT, sizeof(McSmem), stream, true, h->U, reinterpret_cast<const uint4 *>(particles),
+                       reinterpret_cast<const uint4 *>(tree), h->d_mcw, bc, out, reinterpret_cast<uint4 *>(out_bf16), h->d_err);
     }
     return cuda_status(e);
 }
@@ -1326,9 +1114,9 @@ apr_status_t apr_convolve_mc_relu_bf16(apr_handle_t h, const uint16_t *particles
 size_t apr_mc_backward_workspace_bytes(apr_handle_t h, int32_t c_in, int32_t c_out, int32_t k) {
     if (!h || !mc_args_ok(c_in, c_out, k)) return 0;
     const int L = h->X.l_max - h->X.l_min + 1;
-    const int units = int(h->X.fwd_items.size()) * NSUB;
+    const int units = int(h->X.fwd_items.size()) * 4;
     const size_t gt = (size_t(h->X.nt) * MC * sizeof(float) + 255) / 256 * 256;
-    return gt + size_t(wgrad_ctas(units) + L) * WG_ROWS * MC * sizeof(float);
+    return gt + size_t(wgrad_ctas(units) + L) * WG_OUT * sizeof(float);
 }
 
 apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles, const uint16_t *tree,
@@ -1352,18 +1140,18 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
     const int n_levels = X.l_max - X.l_min + 1;
     cudaError_t e = cudaSuccess;
     if (grad_particles) {
-        if (X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * MC * sizeof(float), stream);
-        if (e == cudaSuccess && X.nt) e = cudaMemsetAsync(gt, 0, size_t(X.nt) * MC * sizeof(float), stream);
-        if (e == cudaSuccess) e = set_smem(reinterpret_cast<const void *>(mc_bwd_data_kernel), sizeof(BwdSmem));
-        const int n = int(X.bwd_items.size());
-        const uint16_t *wt = h->d_mcw + size_t(n_levels) * MC * MC * NTAP;
-        if (e == cudaSuccess && n > 0) {
-            mc_weight_layout_kernel<<<(n_levels * MC * MC * NTAP + 255) / 256, 256, 0, stream>>>(
-                weights, n_levels, 1, h->d_mcw + size_t(n_levels) * MC * MC * NTAP);
-            mc_bwd_data_kernel<<<dim3(n, NSUB / SPC_B), NT, sizeof(BwdSmem), stream>>>(
-                h->L, h->d_bwd, wt, bc, reinterpret_cast<const uint4 *>(grad_out), grad_particles, gt);
-            e = cudaGetLastError();
-        }
+        // every particle and tree node is the child of one record, which stores its gradient; only in an
+        // index in which some have no record (a layout that was not validated) are the arrays cleared first
+        if (!h->complete && X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * MC * sizeof(float), stream);
+        if (!h->complete && e == cudaSuccess && X.nt) e = cudaMemsetAsync(gt, 0, size_t(X.nt) * MC * sizeof(float), stream);
+        if (h->uncovered) uncovered_kernel<<<1, 1, 0, stream>>>(h->d_err);
+        uint16_t *wt = h->d_mcw + size_t(n_levels) * W_LEVEL;
+        const uint4 *g4 = reinterpret_cast<const uint4 *>(grad_out);
+        if (e == cudaSuccess) e = layout_weights(weights, n_levels, 1, wt, stream);
+        if (e == cudaSuccess)
+            e = launch(mc_adjoint_kernel, h->U.n, TNT, sizeof(McSmem), stream, true, h->U, wt, bc, g4, grad_particles, gt, h->d_err);
+        if (e == cudaSuccess)
+            e = launch(mc_leaf_adjoint_kernel, h->U.nl, TNT, sizeof(McSmem), stream, false, h->U, wt, bc, g4, grad_particles, h->d_err);
         bool chained = false;   // the launches after the first start early (programmatic dependent launch)
         const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
         for (int i = 0; i < T.n && e == cudaSuccess; ++i) {
@@ -1372,33 +1160,16 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
         }
     }
     if (e == cudaSuccess && grad_weights) {
-        const int units = int(X.fwd_items.size()) * NSUB;
-        const int G = wgrad_ctas(units);
-        WgradPlan plan;
-        for (int i = 0; i < MAXL; ++i) plan.first[i] = plan.last[i] = -1;
-        auto cta_of = [&](int64_t u) {  // CTA c with c*units/G <= u < (c+1)*units/G
-            int c = int((u * G) / units);
-            while (c + 1 < G && (int64_t(c + 1) * units) / G <= u) ++c;
-            while (c > 0 && (int64_t(c) * units) / G > u) --c;
-            return c;
-        };
-        for (int lv = 0; lv < n_levels; ++lv) {
-            const int64_t ua = X.fwd_level_begin[X.l_min + lv] * NSUB, ub = X.fwd_level_begin[X.l_min + lv + 1] * NSUB;
-            if (ua >= ub) continue;
-            plan.first[lv] = cta_of(ua);
-            plan.last[lv] = cta_of(ub - 1);
-        }
-        e = set_smem(reinterpret_cast<const void *>(mc_wgrad_kernel), sizeof(WgradSmem));
-        if (e == cudaSuccess && units > 0) {
-            mc_wgrad_kernel<<<G, NT, sizeof(WgradSmem), stream>>>(h->L, h->d_fwd, units,
-                                                                  reinterpret_cast<const uint4 *>(particles),
-                                                                  reinterpret_cast<const uint4 *>(tree), bc,
-                                                                  reinterpret_cast<const uint4 *>(grad_out), partial);
-            e = cudaGetLastError();
-        }
+        UnitLevels L;
+        UnitRanges R;
+        const int slots = wgrad_ctas(int(X.fwd_items.size()) * 4);
+        const int G = unit_levels(h, std::min(slots, (wgrad_ctas(1 << 30) + 7) / 8), L, R);
+        if (G > 0)
+            e = launch(mc_wgrad_kernel, G, NT, sizeof(WgradSmem), stream, false, h->U, L, reinterpret_cast<const uint4 *>(particles),
+                       reinterpret_cast<const uint4 *>(tree), bc, reinterpret_cast<const uint4 *>(grad_out), partial, h->d_err);
         if (e == cudaSuccess) {
-            const int tot = n_levels * WG_ROWS * MC;
-            mc_wgrad_reduce_kernel<<<(tot + 255) / 256, 256, 0, stream>>>(partial, plan, n_levels, grad_weights);
+            const int tot = n_levels * WG_OUT;
+            mc_wgrad_reduce_kernel<<<(tot + 255) / 256, 256, 0, stream>>>(partial, R, n_levels, grad_weights);
             e = cudaGetLastError();
         }
     }

@@ -1,6 +1,5 @@
 // Host builders of what the kernels read: the child maps of the tree nodes (tree_node_plan) and, through
-// build_units (apr_unitplan.cpp) and build_mc_plans (apr_mc.cu), the convolution units and the multi-channel
-// sub-tile plans. Also the tile plans that apr_export_structure gives: for every forward and data-adjoint
+// build_units (apr_unitplan.cpp), the convolution units. Also the tile plans that apr_export_structure gives: for every forward and data-adjoint
 // work item and both stencil radii the non-empty source segments of the item's patch (fwd_segment,
 // bwd_segment in apr_tile.cuh), with the prefix of their 8-element packets.
 #include <functional>
@@ -205,12 +204,13 @@ apr_status_t run_jobs(std::vector<std::function<bool()>> jobs) {
 apr_status_t build_plans(HostIndex &X) {
     const DevLayout L = host_layout_view(X);
     if (X.np >= FPLAN_MAX_INDEX || X.nt >= FPLAN_MAX_INDEX) return APR_ERR_UNSUPPORTED;
-    return run_jobs({[&] { return build_mc_plans(L, X, X.mcfplan, X.mcbplan); },
-                     [&] {
-                         if (!tree_node_plan(L, X, X.tnplan)) return false;
-                         build_units(X);
-                         return true;
-                     }});
+    try {
+        if (!tree_node_plan(L, X, X.tnplan)) return APR_ERR_UNSUPPORTED;
+        build_units(X);
+    } catch (...) {  // host allocation failure
+        return APR_ERR_OOM;
+    }
+    return APR_OK;
 }
 
 apr_status_t build_tile_plans(HostIndex &X) {

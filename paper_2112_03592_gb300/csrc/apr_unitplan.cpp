@@ -73,6 +73,7 @@ struct JobOut {
     std::vector<NodeRec> rec;
     std::vector<LeafRec> lrec;
     std::vector<int32_t> tf, tb, ltb;
+    bool uncovered = false;
 };
 
 class BlockJob {
@@ -136,9 +137,12 @@ class BlockJob {
         }
     }
 
+    // The unit under construction lies in rows [za_, zb_] x [xa_, xb_] (records); slots one row further.
     void reset() {
-        memset(T_, 0, sizeof(T_));
-        memset(D_, 0, sizeof(D_));
+        for (int z = std::max(za_ - 1, 0); z <= zb_ + 1; ++z)
+            for (int x = std::max(xa_ - 1, 0); x <= xb_ + 1; ++x) T_[z][x] = D_[z][x] = 0;
+        za_ = xa_ = UW;
+        zb_ = xb_ = -2;
         nrec_ = nslot_ = 0;
     }
 
@@ -180,14 +184,18 @@ class BlockJob {
                 D_[z + dz][x + dx] |= w;
             }
         T_[z][x] |= 1ull << j;
+        za_ = std::min(za_, z);
+        zb_ = std::max(zb_, z);
+        xa_ = std::min(xa_, x);
+        xb_ = std::max(xb_, x);
         ++nrec_;
     }
 
     int rank(int z, int x, int j) const { return pre_[z][x] + popc(D_[z][x] & ((1ull << j) - 1ull)); }
     void prefix() {
         int n = 0;
-        for (int z = 0; z < UW; ++z)
-            for (int x = 0; x < UW; ++x) {
+        for (int z = za_ - 1; z <= zb_ + 1; ++z)
+            for (int x = xa_ - 1; x <= xb_ + 1; ++x) {
                 pre_[z][x] = n;
                 n += popc(D_[z][x]);
             }
@@ -200,8 +208,8 @@ class BlockJob {
     int records(F f) {
         int nflag = 0;
         for (int pass = 0; pass < 2; ++pass)
-            for (int z = 1; z <= UB; ++z)
-                for (int x = 1; x <= UB; ++x) {
+            for (int z = za_; z <= zb_; ++z)
+                for (int x = xa_; x <= xb_; ++x) {
                     uint64_t w = T_[z][x];
                     while (w) {
                         const int j = __builtin_ctzll(w);
@@ -241,9 +249,40 @@ class BlockJob {
         pure.push_back(uint4{w[0], w[1], w[2], w[3]});
     }
 
+    // Whether child cell c of in-grid parent (z, x, j) has a source.
+    bool covered(int z, int x, int j, int c) const {
+        const uint64_t bit = 1ull << j;
+        if (!(K_.N[z][x] & bit)) return (K_.L[z][x] & bit) != 0;
+        const TreeNodePlan &m = P_.maps[K_.n0[z][x] + popc(K_.N[z][x] & (bit - 1ull))];
+        return ((uint32_t(m.p[c >> 1]) | uint32_t(m.t[c >> 1])) >> (30 + (c & 1))) & 1u;
+    }
+    // Whether a cell next to a particle of the unit's records lies in the grid and has no source (possible
+    // only in a layout that was not validated).
+    bool any_uncovered() const {
+        for (int z = za_; z <= zb_; ++z)
+            for (int x = xa_; x <= xb_; ++x)
+                for (uint64_t w = T_[z][x]; w; w &= w - 1) {
+                    const int j = __builtin_ctzll(w);
+                    const TreeNodePlan &m = P_.maps[K_.n0[z][x] + popc(K_.N[z][x] & ((1ull << j) - 1ull))];
+                    for (int c = 0; c < 8; ++c) {
+                        if (!((uint32_t(m.p[c >> 1]) >> (30 + (c & 1))) & 1u)) continue;
+                        for (int t = 0; t < 27; ++t) {
+                            const int cz = 2 * (z0_ - 1 + z) + (c >> 2) + t / 9 - 1, cx = 2 * (x0_ - 1 + x) + ((c >> 1) & 1) + (t / 3) % 3 - 1,
+                                      cy = 2 * (y0_ - Y0 + j) + (c & 1) + t % 3 - 1;
+                            if (cz < 0 || cx < 0 || cy < 0 || cz >= P_.dz || cx >= P_.dx || cy >= P_.dy) continue;
+                            if (!covered((cz >> 1) - (z0_ - 1), (cx >> 1) - (x0_ - 1), (cy >> 1) - (y0_ - Y0),
+                                         4 * (cz & 1) + 2 * (cx & 1) + (cy & 1)))
+                                return true;
+                        }
+                    }
+                }
+        return false;
+    }
+
     void close_nodes() {
         if (!nrec_) return;
         prefix();
+        bool holes = false;   // in-grid slots or children without a source
         UnitHdr h{};
         h.pure0 = int32_t(o_.pure.size());
         h.node0 = int32_t(o_.nmap.size());
@@ -253,8 +292,8 @@ class BlockJob {
         std::vector<uint2> &leaf = tmp_leaf_, &zero = tmp_zero_;
         leaf.clear();
         zero.clear();
-        for (int z = 0; z < UW; ++z)
-            for (int x = 0; x < UW; ++x) {
+        for (int z = za_ - 1; z <= zb_ + 1; ++z)
+            for (int x = xa_ - 1; x <= xb_ + 1; ++x) {
                 uint64_t w = D_[z][x];
                 unsigned pos = unsigned(pre_[z][x]);
                 for (; w; w &= w - 1, ++pos) {
@@ -273,10 +312,15 @@ class BlockJob {
                     const unsigned mir = (mz ? 4u : 0u) | (mx ? 2u : 0u) | (my ? 1u : 0u);
                     unsigned info = pos | (mir << UE_MIRROR) | (miss << UE_MISS);
                     if (K_.N[wz][wx] & bit) {
+                        const TreeNodePlan &m = P_.maps[K_.n0[wz][wx] + popc(K_.N[wz][wx] & below)];
+                        int kids = 0;
+                        for (int k = 0; k < 4; ++k) kids += popc((uint32_t(m.p[k]) | uint32_t(m.t[k])) >> 30);
+                        holes = holes || kids != 8 >> popc(miss);
                         put_node(uint32_t(K_.n0[wz][wx] + popc(K_.N[wz][wx] & below)), info, o_.pure, o_.nmap, o_.ninfo);
                     } else if (K_.L[wz][wx] & bit) {
                         leaf.push_back(uint2{uint32_t(K_.l0[wz][wx] + popc(K_.L[wz][wx] & below)), info});
                     } else {
+                        holes = true;
                         zero.push_back(uint2{0u, info});
                     }
                 }
@@ -299,6 +343,7 @@ class BlockJob {
             o_.tb.push_back(b);
         }));
         h.nrec = int16_t(nrec_);
+        if (holes && any_uncovered()) o_.uncovered = true;
         o_.hdr.push_back(h);
     }
 
@@ -316,8 +361,8 @@ class BlockJob {
         h.node0 = int32_t(o_.lnmap.size());
         h.rec0 = int32_t(o_.lrec.size());
         h.lev = int16_t(lev_);
-        for (int z = 0; z < UW; ++z)
-            for (int x = 0; x < UW; ++x) {
+        for (int z = za_ - 1; z <= zb_ + 1; ++z)
+            for (int x = xa_ - 1; x <= xb_ + 1; ++x) {
                 uint64_t w = D_[z][x];
                 unsigned pos = unsigned(pre_[z][x]);
                 for (; w; w &= w - 1, ++pos) {
@@ -367,6 +412,7 @@ class BlockJob {
     int ntx_, nty_;
     JobOut &o_;
     int z0_ = 0, x0_ = 0, y0_ = 0, nrec_ = 0, nslot_ = 0;
+    int za_ = 1, zb_ = UB, xa_ = 1, xb_ = UB;   // (the first reset clears everything)
     Block K_;
     uint64_t T_[UW][UW], D_[UW][UW];
     int pre_[UW][UW];
@@ -506,7 +552,7 @@ void build_units(HostIndex &X) {
             failed = true;
         }
     };
-    const unsigned nth = unsigned(std::min<size_t>(std::max(1u, std::min(16u, std::thread::hardware_concurrency())), jobs.size() / 8 + 1));
+    const unsigned nth = unsigned(std::min<size_t>(std::max(1u, std::min(16u, std::thread::hardware_concurrency())), jobs.size()));
     std::vector<std::thread> threads;
     for (unsigned t = 1; t < nth; ++t) {
         try {
@@ -557,6 +603,7 @@ void build_units(HostIndex &X) {
                 h.rec0 += int32_t(U.lrec.size());
                 U.lhdr.push_back(h);
             }
+            U.uncovered = U.uncovered || o.uncovered;
             append(U.pure, o.pure);
             append(U.lpure, o.lpure);
             append(U.nmap, o.nmap);

@@ -28,6 +28,7 @@
 
 #include "apr_device.cuh"
 #include "apr_internal.h"
+#include "apr_units.cuh"
 
 namespace aprk {
 
@@ -52,11 +53,6 @@ template <int R>
 __device__ __forceinline__ float tap(const float *w, int row, int t) {
     return R == 1 ? w[row * 4 + (t < 2 ? t : 3)] : w[row * 8 + (t < 4 ? t : 7)];
 }
-
-// Slots of a plane: the unit's, then three that stay zero (ZERO_SLOT: the neighbours of an image outside
-// the grid).
-constexpr int PLANE = UNIT_SLOTS + 4;
-constexpr unsigned ZERO_SLOT = UNIT_SLOTS;
 
 // The staged octets (see above); SC: one plane per cell.
 struct Planes {
@@ -135,64 +131,6 @@ struct Taps {
     }
 };
 
-// The children of a parent from its child map: child c = 2k + e (k = (a, b) the child row, e the child's y
-// parity) is a particle (kind 1) or a tree node (kind 2) at index ix[c], or absent (kind 0).
-struct Octet {
-    int ix[8];
-    int kind[8];
-    __device__ __forceinline__ Octet(const int4 &pw, const int4 &tw) {
-        const int pv[4] = {pw.x, pw.y, pw.z, pw.w}, tv[4] = {tw.x, tw.y, tw.z, tw.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const unsigned pm = unsigned(pv[k]) >> 30, tm = unsigned(tv[k]) >> 30;
-            const int pi = int(unsigned(pv[k]) & TNP_INDEX), ti = int(unsigned(tv[k]) & TNP_INDEX);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const bool isp = (pm >> e) & 1u, ist = (tm >> e) & 1u;
-                kind[2 * k + e] = isp ? 1 : (ist ? 2 : 0);
-                ix[2 * k + e] = isp ? pi + (e ? int(pm & 1u) : 0) : ti + (e ? int(tm & 1u) : 0);
-            }
-        }
-    }
-};
-
-// An octet at or outside the grid's edge: with reflection a missing child takes its sibling's value and
-// a mirrored octet is reversed along the mirrored axes; with the zero boundary the missing children and
-// every slot outside the grid are zero.
-__device__ __forceinline__ void edge_octet(float (&v)[8], unsigned info, bool reflect) {
-    const unsigned mir = (info >> UE_MIRROR) & 7u, miss = (info >> UE_MISS) & 7u;
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-        const int m = 1 << ax;
-        if (miss & m) {
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c & m) v[c] = reflect ? v[c ^ m] : 0.f;
-        }
-    }
-    if (mir && !reflect) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[c] = 0.f;
-    }
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-        const int m = 1 << ax;
-        if (mir & m) {
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c & m) {
-                    const float t = v[c];
-                    v[c] = v[c ^ m];
-                    v[c ^ m] = t;
-                }
-        }
-    }
-}
-
-__device__ __forceinline__ unsigned pure_slot(const uint4 &q) {
-    return (q.x >> 28) | ((q.y >> 28) << 4) | ((q.z >> 28) << 8);
-}
-
 // Staging of a unit's slots. issue(): loads the entries, then the values of the first slots of every kind
 // (2 pure, 1 other node and 2 remaining ones per thread: nearly all of a unit), all in flight together;
 // commit(): writes them to shared memory and takes what is left in loops. The chain is header -> entry ->
@@ -269,7 +207,7 @@ struct Staging {
     }
     template <bool SC>
     __device__ __forceinline__ void put(Planes &pl, unsigned info, float (&v)[8], bool reflect) const {
-        if (info >> UE_MIRROR) edge_octet(v, info, reflect);
+        if (info >> UE_MIRROR) edge_octet(v, info, reflect, 0.f);
         pl.store<SC>(info & UE_SLOT, v);
     }
     template <bool SC>
@@ -334,18 +272,6 @@ __device__ __forceinline__ Staging<false> gradient_staging(const UnitView &U, co
     return s;
 }
 
-// Nine row slots in the words of a record.
-__device__ __forceinline__ void unpack_bases(unsigned w1, const uint2 &r1, const uint2 &r2, unsigned (&b)[9]) {
-    b[0] = w1 >> 16;
-    b[1] = r1.x & 0xffffu;
-    b[2] = r1.x >> 16;
-    b[3] = r1.y & 0xffffu;
-    b[4] = r1.y >> 16;
-    b[5] = r2.x & 0xffffu;
-    b[6] = r2.x >> 16;
-    b[7] = r2.y & 0xffffu;
-    b[8] = r2.y >> 16;
-}
 // A record, loaded ahead of the staging: its row slots go to shared memory, node and edge word stay.
 struct Rec {
     uint2 r0, r1, r2;
@@ -484,22 +410,6 @@ struct TileRange {
     }
 };
 
-__device__ __forceinline__ int4 child_particles(const UnitView &U, unsigned node) {
-    return __ldg(reinterpret_cast<const int4 *>(U.nplan + node));
-}
-// f(particle, c) for the particles among the children.
-template <typename F>
-__device__ __forceinline__ void for_child_particles(const int4 &pw, F f) {
-    const int pv[4] = {pw.x, pw.y, pw.z, pw.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const unsigned pm = unsigned(pv[k]) >> 30;
-        const int pi = int(unsigned(pv[k]) & TNP_INDEX);
-        if (pm & 1u) f(pi, 2 * k);
-        if (pm & 2u) f(pi + int(pm & 1u), 2 * k + 1);
-    }
-}
-
 // ------------------------------------------------------------------------------------------------
 // APR convolution (Sec. 4.1).
 // ------------------------------------------------------------------------------------------------
@@ -582,41 +492,6 @@ __global__ void __launch_bounds__(UT, 3) unit_gradmag_kernel(const UnitView U, c
 // record's children) or the level-(l-1) particle over c (leaf_adjoint_kernel, launched after it, adds the
 // sum over the particle's eight cells). A particle gets at most these two terms, in this order.
 // ------------------------------------------------------------------------------------------------
-// Images. With reflection, out-of-grid cells c' within R of the grid add to H of the cell they reflect
-// onto. Those cells are the children of parents outside the grid, so their sums are those of a record
-// there: the same sums over a neighbourhood shifted along the axis (one layer of it inside the grid, the
-// others zero), with the children mirrored. Per axis, from the 3-bit edge code, the shifts that occur:
-// bit 0 none, bit 1 by -1 (first parent), bit 2 by +1 (the grid ends with this parent's second child, or
-// the grid is a single cell), bit 3 by +2 (an odd grid ends with the next parent's first child; only
-// radius 2 reaches back). A missing second child (an odd grid's last parent) is itself the image of its
-// sibling.
-template <int R>
-__device__ __forceinline__ unsigned axis_shifts(unsigned code) {
-    const unsigned left = code >> 1;
-    return 1u | ((code & 1u) ? 2u : 0u) | (left == 2u || code == 3u ? 4u : 0u) | (R == 2 && left == 3u ? 8u : 0u);
-}
-// All shift triples of an edge word: bit 16 iz + 4 ix + iy.
-template <int R>
-__device__ __forceinline__ unsigned long long edge_shifts(unsigned edge) {
-    const unsigned z = axis_shifts<R>(edge & 7u), x = axis_shifts<R>((edge >> 3) & 7u), y = axis_shifts<R>((edge >> 6) & 7u);
-    unsigned xy = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) xy |= ((x >> i) & 1u) ? y << (4 * i) : 0u;
-    unsigned long long m = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) m |= ((z >> i) & 1u) ? (unsigned long long)xy << (16 * i) : 0ull;
-    return m;
-}
-// Layer of the record's neighbourhood that layer d of the image with shift index i reads (-1: zero).
-__device__ __forceinline__ int image_layer(int i, int d) {
-    if (i == 0) return d;
-    return d == (i == 1 ? 2 : 0) ? (i == 3 ? 2 : 1) : -1;
-}
-__device__ __forceinline__ unsigned missing_children(unsigned edge) {   // axis mask z 4, x 2, y 1
-    return ((edge >> 1) & 3u) == 1u ? (((edge >> 4) & 3u) == 1u ? 6u : 4u) | (((edge >> 7) & 3u) == 1u ? 1u : 0u)
-                                    : (((edge >> 4) & 3u) == 1u ? 2u : 0u) | (((edge >> 7) & 3u) == 1u ? 1u : 0u);
-}
-
 // A missing child's sum belongs to its sibling.
 __device__ __forceinline__ void fold_missing(unsigned edge, float (&v)[8]) {
     const unsigned miss = missing_children(edge);
@@ -914,13 +789,6 @@ __global__ void __launch_bounds__(UT, 4) leaf_adjoint_kernel(const UnitView U, c
 // register per lane and chains stay short. At a level's end the warps' sums are written to the level's
 // partial of this block, and stencil_grad_reduce_kernel adds the blocks in order.
 // ------------------------------------------------------------------------------------------------
-struct WgradLevels {           // levels with particles, finest first
-    int n;
-    int lev[MAXL];             // l - l_min
-    int unit0[MAXL];           // first unit of the level
-    int begin[MAXL + 1];       // prefix of the levels' unit counts
-};
-
 template <int R>
 struct WgradSmem {
     static constexpr int K = 2 * R + 1, Q = R == 1 ? 4 : 2, NT = K * Q * 32;
@@ -952,7 +820,7 @@ __device__ __forceinline__ float lane_sums(const float (&v)[N]) {
 }
 
 template <int R>
-__global__ void __launch_bounds__(WgradSmem<R>::NT, R == 1 ? 2 : 3) unit_wgrad_kernel(const UnitView U, const WgradLevels W,
+__global__ void __launch_bounds__(WgradSmem<R>::NT, R == 1 ? 2 : 3) unit_wgrad_kernel(const UnitView U, const UnitLevels W,
                                                                       const float *__restrict__ vals,
                                                                       const float *__restrict__ tree, int bc,
                                                                       const float *__restrict__ gout,
@@ -1044,11 +912,8 @@ __global__ void __launch_bounds__(WgradSmem<R>::NT, R == 1 ? 2 : 3) unit_wgrad_k
 
 // grad_w[lev][e] = sum of the level's block partials (partial[e][block + i], blocks first .. last for the
 // i-th level), in a fixed order; zero for a level without particles.
-struct WgradRanges {
-    int first[MAXL], last[MAXL];   // by l - l_min: range of partials, empty if first > last
-};
 __global__ void __launch_bounds__(128) stencil_grad_reduce_kernel(const float *__restrict__ partial, int stride,
-                                                                  const WgradRanges rg, int K3,
+                                                                  const UnitRanges rg, int K3,
                                                                   float *__restrict__ gw) {
     __shared__ float red[4];
     const int lev = blockIdx.y, e = blockIdx.x, tid = threadIdx.x;
@@ -1117,52 +982,16 @@ cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, co
     return k == 3 ? launch_adjoint_t<1>(U, st, bc, gout, gp, gt, s, tr) : launch_adjoint_t<2>(U, st, bc, gout, gp, gt, s, tr);
 }
 
-// The stencil gradient into gw [n_levels][k^3]. partial: k^3 x stride floats. level_begin: first unit of
-// level l_min + i (the finest level first); has: whether level l_min + i holds particles. The blocks and
-// levels fit the stride: block b writes its i-th level to column b + i.
-cudaError_t launch_stencil_grad(int k, const UnitView &U, const int32_t *level_begin, const bool *has, int n_levels,
+// The stencil gradient into gw [n_levels][k^3], on the blocks of W, R (unit_levels). partial: k^3 x stride
+// floats; block b writes its i-th level to column b + i.
+cudaError_t launch_stencil_grad(int k, const UnitView &U, const UnitLevels &W, const UnitRanges &R, int blocks, int n_levels,
                                 const float *vals, const float *tree, int bc, const float *gout, float *partial, int stride,
                                 float *gw, cudaStream_t s) {
-    if (n_levels <= 0) return cudaSuccess;
-    WgradLevels W{};
-    WgradRanges rg{};
-    for (int lev = n_levels - 1; lev >= 0; --lev) {
-        rg.first[lev] = 0;
-        rg.last[lev] = -1;
-        const int end = lev == 0 ? U.n : level_begin[lev - 1];
-        if (!has[lev] || end <= level_begin[lev]) continue;
-        W.lev[W.n] = lev;
-        W.unit0[W.n] = level_begin[lev];
-        W.begin[W.n + 1] = W.begin[W.n] + end - level_begin[lev];
-        ++W.n;
-    }
-    const int total = W.begin[W.n];
-    if (total > 0) {
-        // three blocks per SM are resident; at most one column per block and level
-        static int sms = 0;
-        static std::once_flag once;
-        std::call_once(once, [] {
-            int dev = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-                sms = 152;
-        });
-        const int G = std::max(1, std::min({total, 3 * sms, stride - W.n + 1}));
-        auto block_of = [&](int u) {   // block b with b total / G <= u < (b + 1) total / G
-            int b = int(int64_t(u) * G / total);
-            while (b + 1 < G && int64_t(b + 1) * total / G <= u) ++b;
-            while (b > 0 && int64_t(b) * total / G > u) --b;
-            return b;
-        };
-        for (int i = 0; i < W.n; ++i) {
-            rg.first[W.lev[i]] = block_of(W.begin[i]) + i;
-            rg.last[W.lev[i]] = block_of(W.begin[i + 1] - 1) + i;
-        }
-        const cudaError_t e =
-            k == 3 ? launch(unit_wgrad_kernel<1>, G, WgradSmem<1>::NT, sizeof(WgradSmem<1>), s, U, W, vals, tree, bc, gout, partial, stride)
-                   : launch(unit_wgrad_kernel<2>, G, WgradSmem<2>::NT, sizeof(WgradSmem<2>), s, U, W, vals, tree, bc, gout, partial, stride);
-        if (e != cudaSuccess) return e;
-    }
-    stencil_grad_reduce_kernel<<<dim3(k * k * k, n_levels), 128, 0, s>>>(partial, stride, rg, k * k * k, gw);
+    const cudaError_t e =
+        k == 3 ? launch(unit_wgrad_kernel<1>, blocks, WgradSmem<1>::NT, sizeof(WgradSmem<1>), s, U, W, vals, tree, bc, gout, partial, stride)
+               : launch(unit_wgrad_kernel<2>, blocks, WgradSmem<2>::NT, sizeof(WgradSmem<2>), s, U, W, vals, tree, bc, gout, partial, stride);
+    if (e != cudaSuccess) return e;
+    stencil_grad_reduce_kernel<<<dim3(k * k * k, n_levels), 128, 0, s>>>(partial, stride, R, k * k * k, gw);
     return cudaGetLastError();
 }
 

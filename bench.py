@@ -1096,9 +1096,9 @@ def run_surrogate(args, rank, world, pretrained=None):
                     "weighting": "pixels covered by each particle (pixel-equivalent)"},
         "training": {"loss_first": round(float(np.mean(hist[:10])), 6), "loss_last": round(float(np.mean(hist[-10:])), 6),
                      "data_s": round(t_data, 1), "train_s": round(t_train, 1)},
-        # per CNN inference: embedding, 4 x (tree restriction per level, weight layout, convolution;
-        # hidden ReLUs fused into the convolution), read-out; per RL run: 2 x (tree + convolution) per iteration
-        "gpu_launches": (2 + 4 * (n_tree + 2) +
+        # per CNN inference: embedding, 4 x (tree restriction, weight layout, convolution; hidden
+        # ReLUs and the read-out fused into the convolution); per RL run: 2 x (tree + convolution) per iteration
+        "gpu_launches": (1 + 4 * (n_tree + 2) +
                          RL_ITERS * 2 * (n_tree + 1)) * args.steps,
     }
     return rec

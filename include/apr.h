@@ -362,6 +362,13 @@ apr_status_t apr_convolve_mc_relu_bf16(apr_handle_t h, const uint16_t *particles
                                        const uint16_t *weights, int32_t c_in, int32_t c_out, int32_t k, int32_t bc,
                                        uint16_t *out, apr_stream_t stream);
 
+/* apr_convolve_mc with the last layer's read-out fused into the write: y[p] = x[p] + inv_scale * conv[p][0]
+ * (device [N_p] float32; as apr_mc_readout of the float32 result, which is not written). x and y may be the
+ * same buffer. For inference. */
+apr_status_t apr_convolve_mc_readout(apr_handle_t h, const uint16_t *particles, const uint16_t *tree,
+                                     const uint16_t *weights, int32_t c_in, int32_t c_out, int32_t k, int32_t bc,
+                                     const float *x, float inv_scale, float *y, apr_stream_t stream);
+
 /* Scratch bytes of apr_convolve_mc_backward (tree gradient and per-block weight-gradient partials). */
 size_t apr_mc_backward_workspace_bytes(apr_handle_t h, int32_t c_in, int32_t c_out, int32_t k);
 

@@ -36,7 +36,7 @@ from ._abi import (APR_BC_REFLECT, APR_BC_ZERO, APR_HOST_ONLY, APR_REQUIRE_BALAN
 __all__ = ["AprLayout", "AprConv", "apr_build_device", "apr_tree_restrict", "apr_convolve", "apr_convolve_auto",
            "apr_convolve_backward", "apr_convolve_adjoint", "apr_tree_restrict_adjoint",
            "apr_tree_restrict_adjoint_levels",
-           "apr_convolve_stencil_grad", "apr_gradient_magnitude", "sobel_stencils", "apr_richardson_lucy", "apr_tree_restrict_bf16", "apr_convolve_mc", "apr_convolve_mc_relu_bf16", "apr_convolve_mc_backward",
+           "apr_convolve_stencil_grad", "apr_gradient_magnitude", "sobel_stencils", "apr_richardson_lucy", "apr_tree_restrict_bf16", "apr_convolve_mc", "apr_convolve_mc_relu_bf16", "apr_convolve_mc_readout", "apr_convolve_mc_backward",
            "apr_mc_embed_bf16", "apr_mc_relu_bf16", "apr_mc_relu_backward_bf16", "apr_mc_readout",
            "apr_mc_readout_backward_bf16", "apr_restrict_stencil", "apr_rescale_stencil", "apr_dense_convolve", "apr_convolve_tiles",
            "apr_convolve_adjoint_tiles", "AprError",
@@ -480,6 +480,25 @@ def apr_convolve_mc_relu_bf16(layout: AprLayout, particles, tree, weights, bc=AP
     _abi.check("apr_convolve_mc_relu_bf16", layout._lib.apr_convolve_mc_relu_bf16(
         layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
         ctypes.c_void_p(weights.data_ptr()), C, C, k, int(bc), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+    return out
+
+
+def apr_convolve_mc_readout(layout: AprLayout, particles, tree, weights, x, inv_scale, bc=APR_BC_REFLECT, out=None, stream=None):
+    """x + inv_scale * apr_convolve_mc(...)[:, 0] (float32 [N_p]): the last CNN layer with the read-out fused (inference)."""
+    import torch
+    C = MC_CHANNELS
+    k = 3
+    _dev_ptr(particles, "particles", layout.n_particles * C, torch.bfloat16)
+    _dev_ptr(tree, "tree", layout.n_tree * C, torch.bfloat16)
+    _dev_ptr(weights, "weights", layout.n_levels * C * C * k ** 3, torch.bfloat16)
+    _dev_ptr(x, "x", layout.n_particles, torch.float32)
+    if out is None:
+        out = torch.empty(layout.n_particles, dtype=torch.float32, device=particles.device)
+    _dev_ptr(out, "y", layout.n_particles, torch.float32)
+    _abi.check("apr_convolve_mc_readout", layout._lib.apr_convolve_mc_readout(
+        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
+        ctypes.c_void_p(weights.data_ptr()), C, C, k, int(bc), ctypes.c_void_p(x.data_ptr()), float(inv_scale),
+        ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
     return out
 
 

@@ -13,7 +13,7 @@ from __future__ import annotations
 
 import math
 
-from . import (apr_convolve_mc, apr_convolve_mc_backward, apr_convolve_mc_relu_bf16, apr_mc_embed_bf16, apr_mc_readout,
+from . import (apr_convolve_mc, apr_convolve_mc_backward, apr_convolve_mc_readout, apr_convolve_mc_relu_bf16, apr_mc_embed_bf16, apr_mc_readout,
                apr_mc_readout_backward_bf16, apr_mc_relu_backward_bf16, apr_mc_relu_bf16, apr_tree_restrict_bf16)
 
 C = 16
@@ -55,6 +55,8 @@ class AprCnn:
             if not keep and i + 1 < self.n_layers:
                 h = apr_convolve_mc_relu_bf16(layout, h, tree, Wb[i])   # inference: ReLU fused into the write
                 continue
+            if not keep:
+                return apr_convolve_mc_readout(layout, h, tree, Wb[i], x, 1.0 / scale)
             c = apr_convolve_mc(layout, h, tree, Wb[i])
             if keep:
                 saved.append((h, tree, c))

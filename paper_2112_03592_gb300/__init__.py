@@ -45,9 +45,9 @@ __all__ = ["AprLayout", "AprConv", "apr_build_device", "apr_tree_restrict", "apr
 
 
 def _stream_ptr(stream=None):
+    """cudaStream_t of `stream`, or of the current stream (read without building a Stream object, which costs 3 us)."""
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def _dev_ptr(t, name, numel=None, dtype=None):
@@ -60,7 +60,7 @@ def _dev_ptr(t, name, numel=None, dtype=None):
         raise TypeError(f"{name} must be {dtype}")
     if numel is not None and t.numel() != numel:
         raise ValueError(f"{name} must have {numel} elements, has {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _torch_allocator():
@@ -104,7 +104,7 @@ class AprLayout:
         L.y_idx = self._y_idx.ctypes.data_as(ctypes.c_void_p)
         L.n_particles = int(self._y_idx.size)
         h = ctypes.c_void_p()
-        stream = ctypes.c_void_p(0)
+        stream = None
         if not (flags & APR_HOST_ONLY):
             stream = _stream_ptr()
         self._alloc_keep = None
@@ -124,7 +124,7 @@ class AprLayout:
         self.n_particles = int(lib.apr_num_particles(h))
         self.n_tree = int(lib.apr_num_tree(h))
         self.host_only = bool(flags & APR_HOST_ONLY)
-        self._ws = {}
+        self._ws, self._ws_bytes = {}, {}
 
     @classmethod
     def from_apr(cls, apr, flags=APR_VALIDATE | APR_REQUIRE_BALANCE, allocator=None):
@@ -181,14 +181,23 @@ class AprLayout:
             return out.reshape(-1, 2)
         return out.reshape(-1, 4) if which in (4, 5, 6) else out
 
-    def workspace(self, k):
-        import torch
-        nbytes = int(self._lib.apr_backward_workspace_bytes(self._h, k))
-        ws = self._ws.get(k)
+    def _bytes(self, key, fn, *args):
+        """fn(handle, *args), a constant of the layout, asked once."""
+        n = self._ws_bytes.get(key)
+        if n is None:
+            n = self._ws_bytes[key] = int(fn(self._h, *args))
+        return n
+
+    def _scratch(self, key, nbytes, device):
+        ws = self._ws.get(key)
         if ws is None or ws.numel() < nbytes:
-            ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device="cuda")
-            self._ws[k] = ws
-        return ws, nbytes
+            import torch
+            ws = self._ws[key] = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+        return ws
+
+    def workspace(self, k):
+        nbytes = self._bytes(k, self._lib.apr_backward_workspace_bytes, k)
+        return self._scratch(k, nbytes, "cuda"), nbytes
 
     def sync_status(self, stream=None):
         _abi.check("apr_sync_status", self._lib.apr_sync_status(self._h, _stream_ptr(stream)))
@@ -207,9 +216,10 @@ def apr_tree_restrict(layout: AprLayout, particles, tree=None, stream=None):
     _dev_ptr(particles, "particles", layout.n_particles * C, torch.float32)
     if tree is None:
         tree = torch.empty((layout.n_tree,) if C == 1 else (layout.n_tree, C), dtype=torch.float32, device=particles.device)
-    _dev_ptr(tree, "tree", layout.n_tree * C, torch.float32)
+    else:
+        _dev_ptr(tree, "tree", layout.n_tree * C, torch.float32)
     _abi.check("apr_tree_restrict", layout._lib.apr_tree_restrict(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()), C, _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(), C, _stream_ptr(stream)))
     return tree
 
 
@@ -220,10 +230,11 @@ def apr_convolve(layout: AprLayout, particles, tree, stencils, k, bc=APR_BC_REFL
     _dev_ptr(stencils, "stencils", layout.n_levels * k ** 3, torch.float32)
     if out is None:
         out = torch.empty(layout.n_particles, dtype=torch.float32, device=particles.device)
-    _dev_ptr(out, "out", layout.n_particles, torch.float32)
+    else:
+        _dev_ptr(out, "out", layout.n_particles, torch.float32)
     _abi.check("apr_convolve", layout._lib.apr_convolve(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
-        ctypes.c_void_p(stencils.data_ptr()), int(k), int(bc), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(),
+        stencils.data_ptr(), int(k), int(bc), out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -236,14 +247,14 @@ def apr_convolve_auto(layout: AprLayout, particles, stencils, k, bc=APR_BC_REFLE
     _dev_ptr(stencils, "stencils", layout.n_levels * k ** 3, torch.float32)
     if out is None:
         out = torch.empty(layout.n_particles, dtype=torch.float32, device=particles.device)
-    _dev_ptr(out, "out", layout.n_particles, torch.float32)
-    nbytes = int(layout._lib.apr_convolve_auto_workspace_bytes(layout.handle))
+    else:
+        _dev_ptr(out, "out", layout.n_particles, torch.float32)
     if workspace is None:
+        nbytes = layout._bytes("auto", layout._lib.apr_convolve_auto_workspace_bytes)
         workspace = torch.empty(nbytes, dtype=torch.uint8, device=particles.device)
     _abi.check("apr_convolve_auto", layout._lib.apr_convolve_auto(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(stencils.data_ptr()), int(k), int(bc),
-        ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(workspace.data_ptr()), ctypes.c_size_t(workspace.numel() *
-                                                                                         workspace.element_size()),
+        layout.handle, particles.data_ptr(), stencils.data_ptr(), int(k), int(bc),
+        out.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
         _stream_ptr(stream)))
     return out
 
@@ -257,10 +268,11 @@ def apr_gradient_magnitude(layout: AprLayout, particles, tree, stencils3, k, bc=
     _dev_ptr(stencils3, "stencils3", 3 * layout.n_levels * k ** 3, torch.float32)
     if out is None:
         out = torch.empty(layout.n_particles, dtype=torch.float32, device=particles.device)
-    _dev_ptr(out, "out", layout.n_particles, torch.float32)
+    else:
+        _dev_ptr(out, "out", layout.n_particles, torch.float32)
     _abi.check("apr_gradient_magnitude", layout._lib.apr_gradient_magnitude(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
-        ctypes.c_void_p(stencils3.data_ptr()), int(k), int(bc), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(),
+        stencils3.data_ptr(), int(k), int(bc), out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -330,7 +342,7 @@ def apr_convolve_backward(layout: AprLayout, particles, tree, stencils, k, grad_
     import torch
     _dev_ptr(grad_out, "grad_out", layout.n_particles, torch.float32)
     _dev_ptr(stencils, "stencils", layout.n_levels * k ** 3, torch.float32)
-    gp_ptr = gw_ptr = ctypes.c_void_p(0)
+    gp_ptr = gw_ptr = None
     if need_particles:
         if grad_particles is None:
             grad_particles = torch.empty(layout.n_particles, dtype=torch.float32, device=grad_out.device)
@@ -343,10 +355,10 @@ def apr_convolve_backward(layout: AprLayout, particles, tree, stencils, k, grad_
         gw_ptr = _dev_ptr(grad_stencils, "grad_stencils", layout.n_levels * k ** 3, torch.float32)
     ws, nbytes = layout.workspace(k)
     _abi.check("apr_convolve_backward", layout._lib.apr_convolve_backward(
-        layout.handle, ctypes.c_void_p(particles.data_ptr() if particles is not None else 0),
-        ctypes.c_void_p(tree.data_ptr() if tree is not None else 0), ctypes.c_void_p(stencils.data_ptr()),
-        int(k), int(bc), ctypes.c_void_p(grad_out.data_ptr()), gp_ptr, gw_ptr,
-        ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(ws.numel()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr() if particles is not None else None,
+        tree.data_ptr() if tree is not None else None, stencils.data_ptr(),
+        int(k), int(bc), grad_out.data_ptr(), gp_ptr, gw_ptr,
+        ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return (grad_particles if need_particles else None), (grad_stencils if need_stencils else None)
 
 
@@ -394,18 +406,14 @@ def apr_convolve_stencil_grad(layout: AprLayout, particles, tree, k, grad_out, b
     import torch
     if grad_stencils is None:
         grad_stencils = torch.empty((layout.n_levels, k ** 3), dtype=torch.float32, device=grad_out.device)
-    nbytes = int(layout._lib.apr_stencil_grad_workspace_bytes(layout.handle, k))
     key = ("sg", k)
-    ws = layout._ws.get(key)
-    if ws is None or ws.numel() < nbytes:
-        ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=grad_out.device)
-        layout._ws[key] = ws
+    ws = layout._scratch(key, layout._bytes(key, layout._lib.apr_stencil_grad_workspace_bytes, k), grad_out.device)
     _abi.check("apr_convolve_stencil_grad", layout._lib.apr_convolve_stencil_grad(
         layout.handle, _dev_ptr(particles, "particles", layout.n_particles, torch.float32),
         _dev_ptr(tree, "tree", layout.n_tree, torch.float32), int(k), int(bc),
         _dev_ptr(grad_out, "grad_out", layout.n_particles, torch.float32),
         _dev_ptr(grad_stencils, "grad_stencils", layout.n_levels * k ** 3, torch.float32),
-        ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(ws.numel()), _stream_ptr(stream)))
+        ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return grad_stencils
 
 
@@ -419,15 +427,11 @@ def apr_richardson_lucy(layout: AprLayout, observed, stencils, k, n_iter, bc=APR
     if estimate is None:
         estimate = observed.clone()
     _dev_ptr(estimate, "estimate", layout.n_particles, torch.float32)
-    nbytes = int(layout._lib.apr_rl_workspace_bytes(layout.handle))
-    key = ("rl",)
-    ws = layout._ws.get(key)
-    if ws is None or ws.numel() < nbytes:
-        ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=observed.device)
-        layout._ws[key] = ws
+    key = "rl"
+    ws = layout._scratch(key, layout._bytes(key, layout._lib.apr_rl_workspace_bytes), observed.device)
     _abi.check("apr_richardson_lucy", layout._lib.apr_richardson_lucy(
-        layout.handle, ctypes.c_void_p(observed.data_ptr()), ctypes.c_void_p(stencils.data_ptr()), int(k), int(bc),
-        int(n_iter), ctypes.c_void_p(estimate.data_ptr()), ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(ws.numel()),
+        layout.handle, observed.data_ptr(), stencils.data_ptr(), int(k), int(bc),
+        int(n_iter), estimate.data_ptr(), ws.data_ptr(), ws.numel(),
         _stream_ptr(stream)))
     return estimate
 
@@ -443,9 +447,10 @@ def apr_tree_restrict_bf16(layout: AprLayout, particles, tree=None, stream=None)
     _dev_ptr(particles, "particles", layout.n_particles * C, torch.bfloat16)
     if tree is None:
         tree = torch.empty((layout.n_tree, C), dtype=torch.bfloat16, device=particles.device)
-    _dev_ptr(tree, "tree", layout.n_tree * C, torch.bfloat16)
+    else:
+        _dev_ptr(tree, "tree", layout.n_tree * C, torch.bfloat16)
     _abi.check("apr_tree_restrict_bf16", layout._lib.apr_tree_restrict_bf16(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()), C, _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(), C, _stream_ptr(stream)))
     return tree
 
 
@@ -459,10 +464,11 @@ def apr_convolve_mc(layout: AprLayout, particles, tree, weights, bc=APR_BC_REFLE
     _dev_ptr(weights, "weights", layout.n_levels * C * C * k ** 3, torch.bfloat16)
     if out is None:
         out = torch.empty((layout.n_particles, C), dtype=torch.float32, device=particles.device)
-    _dev_ptr(out, "out", layout.n_particles * C, torch.float32)
+    else:
+        _dev_ptr(out, "out", layout.n_particles * C, torch.float32)
     _abi.check("apr_convolve_mc", layout._lib.apr_convolve_mc(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
-        ctypes.c_void_p(weights.data_ptr()), C, C, k, int(bc), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(),
+        weights.data_ptr(), C, C, k, int(bc), out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -476,10 +482,11 @@ def apr_convolve_mc_relu_bf16(layout: AprLayout, particles, tree, weights, bc=AP
     _dev_ptr(weights, "weights", layout.n_levels * C * C * k ** 3, torch.bfloat16)
     if out is None:
         out = torch.empty((layout.n_particles, C), dtype=torch.bfloat16, device=particles.device)
-    _dev_ptr(out, "out", layout.n_particles * C, torch.bfloat16)
+    else:
+        _dev_ptr(out, "out", layout.n_particles * C, torch.bfloat16)
     _abi.check("apr_convolve_mc_relu_bf16", layout._lib.apr_convolve_mc_relu_bf16(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
-        ctypes.c_void_p(weights.data_ptr()), C, C, k, int(bc), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(),
+        weights.data_ptr(), C, C, k, int(bc), out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -494,11 +501,12 @@ def apr_convolve_mc_readout(layout: AprLayout, particles, tree, weights, x, inv_
     _dev_ptr(x, "x", layout.n_particles, torch.float32)
     if out is None:
         out = torch.empty(layout.n_particles, dtype=torch.float32, device=particles.device)
-    _dev_ptr(out, "y", layout.n_particles, torch.float32)
+    else:
+        _dev_ptr(out, "y", layout.n_particles, torch.float32)
     _abi.check("apr_convolve_mc_readout", layout._lib.apr_convolve_mc_readout(
-        layout.handle, ctypes.c_void_p(particles.data_ptr()), ctypes.c_void_p(tree.data_ptr()),
-        ctypes.c_void_p(weights.data_ptr()), C, C, k, int(bc), ctypes.c_void_p(x.data_ptr()), float(inv_scale),
-        ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr(), tree.data_ptr(),
+        weights.data_ptr(), C, C, k, int(bc), x.data_ptr(), float(inv_scale),
+        out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -511,7 +519,7 @@ def apr_convolve_mc_backward(layout: AprLayout, particles, tree, weights, grad_o
     k = 3
     _dev_ptr(grad_out, "grad_out", layout.n_particles * C, torch.bfloat16)
     _dev_ptr(weights, "weights", layout.n_levels * C * C * k ** 3, torch.bfloat16)
-    gp_ptr = gw_ptr = ctypes.c_void_p(0)
+    gp_ptr = gw_ptr = None
     if need_particles:
         if grad_particles is None:
             grad_particles = torch.empty((layout.n_particles, C), dtype=torch.float32, device=grad_out.device)
@@ -522,17 +530,13 @@ def apr_convolve_mc_backward(layout: AprLayout, particles, tree, weights, grad_o
         if grad_weights is None:
             grad_weights = torch.empty((layout.n_levels, C, C, k ** 3), dtype=torch.float32, device=grad_out.device)
         gw_ptr = _dev_ptr(grad_weights, "grad_weights", layout.n_levels * C * C * k ** 3, torch.float32)
-    nbytes = int(layout._lib.apr_mc_backward_workspace_bytes(layout.handle, C, C, k))
     key = ("mc", k)
-    ws = layout._ws.get(key)
-    if ws is None or ws.numel() < nbytes:
-        ws = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=grad_out.device)
-        layout._ws[key] = ws
+    ws = layout._scratch(key, layout._bytes(key, layout._lib.apr_mc_backward_workspace_bytes, C, C, k), grad_out.device)
     _abi.check("apr_convolve_mc_backward", layout._lib.apr_convolve_mc_backward(
-        layout.handle, ctypes.c_void_p(particles.data_ptr() if particles is not None else 0),
-        ctypes.c_void_p(tree.data_ptr() if tree is not None else 0), ctypes.c_void_p(weights.data_ptr()),
-        C, C, k, int(bc), ctypes.c_void_p(grad_out.data_ptr()), gp_ptr, gw_ptr,
-        ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(ws.numel()), _stream_ptr(stream)))
+        layout.handle, particles.data_ptr() if particles is not None else None,
+        tree.data_ptr() if tree is not None else None, weights.data_ptr(),
+        C, C, k, int(bc), grad_out.data_ptr(), gp_ptr, gw_ptr,
+        ws.data_ptr(), ws.numel(), _stream_ptr(stream)))
     return (grad_particles if need_particles else None), (grad_weights if need_weights else None)
 
 
@@ -543,9 +547,10 @@ def apr_mc_embed_bf16(x, scale, out=None, stream=None):
     _dev_ptr(x, "x", n, torch.float32)
     if out is None:
         out = torch.empty((n, MC_CHANNELS), dtype=torch.bfloat16, device=x.device)
-    _dev_ptr(out, "out", n * MC_CHANNELS, torch.bfloat16)
+    else:
+        _dev_ptr(out, "out", n * MC_CHANNELS, torch.bfloat16)
     _abi.check("apr_mc_embed_bf16", _abi.load().apr_mc_embed_bf16(
-        ctypes.c_void_p(x.data_ptr()), n, float(scale), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        x.data_ptr(), n, float(scale), out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -555,9 +560,10 @@ def apr_mc_relu_bf16(inp, out=None, stream=None):
     _dev_ptr(inp, "in", n, torch.float32)
     if out is None:
         out = torch.empty(inp.shape, dtype=torch.bfloat16, device=inp.device)
-    _dev_ptr(out, "out", n, torch.bfloat16)
+    else:
+        _dev_ptr(out, "out", n, torch.bfloat16)
     _abi.check("apr_mc_relu_bf16", _abi.load().apr_mc_relu_bf16(
-        ctypes.c_void_p(inp.data_ptr()), n, ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        inp.data_ptr(), n, out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -568,9 +574,10 @@ def apr_mc_relu_backward_bf16(pre, grad_post, out=None, stream=None):
     _dev_ptr(grad_post, "grad_post", n, torch.float32)
     if out is None:
         out = torch.empty(pre.shape, dtype=torch.bfloat16, device=pre.device)
-    _dev_ptr(out, "grad_pre", n, torch.bfloat16)
+    else:
+        _dev_ptr(out, "grad_pre", n, torch.bfloat16)
     _abi.check("apr_mc_relu_backward_bf16", _abi.load().apr_mc_relu_backward_bf16(
-        ctypes.c_void_p(pre.data_ptr()), ctypes.c_void_p(grad_post.data_ptr()), n, ctypes.c_void_p(out.data_ptr()),
+        pre.data_ptr(), grad_post.data_ptr(), n, out.data_ptr(),
         _stream_ptr(stream)))
     return out
 
@@ -582,10 +589,11 @@ def apr_mc_readout(conv, x, inv_scale, out=None, stream=None):
     _dev_ptr(x, "x", n, torch.float32)
     if out is None:
         out = torch.empty(n, dtype=torch.float32, device=x.device)
-    _dev_ptr(out, "y", n, torch.float32)
+    else:
+        _dev_ptr(out, "y", n, torch.float32)
     _abi.check("apr_mc_readout", _abi.load().apr_mc_readout(
-        ctypes.c_void_p(conv.data_ptr()), ctypes.c_void_p(x.data_ptr()), n, float(inv_scale),
-        ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        conv.data_ptr(), x.data_ptr(), n, float(inv_scale),
+        out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -595,9 +603,10 @@ def apr_mc_readout_backward_bf16(grad_y, inv_scale, out=None, stream=None):
     _dev_ptr(grad_y, "grad_y", n, torch.float32)
     if out is None:
         out = torch.empty((n, MC_CHANNELS), dtype=torch.bfloat16, device=grad_y.device)
-    _dev_ptr(out, "grad_conv", n * MC_CHANNELS, torch.bfloat16)
+    else:
+        _dev_ptr(out, "grad_conv", n * MC_CHANNELS, torch.bfloat16)
     _abi.check("apr_mc_readout_backward_bf16", _abi.load().apr_mc_readout_backward_bf16(
-        ctypes.c_void_p(grad_y.data_ptr()), n, float(inv_scale), ctypes.c_void_p(out.data_ptr()), _stream_ptr(stream)))
+        grad_y.data_ptr(), n, float(inv_scale), out.data_ptr(), _stream_ptr(stream)))
     return out
 
 
@@ -634,8 +643,10 @@ def _autograd_function():
         def forward(ctx, particles, stencils, layout, k, bc):
             particles = particles.contiguous()
             stencils = stencils.contiguous()
-            tree = apr_tree_restrict(layout, particles)
-            out = apr_convolve(layout, particles, tree, stencils, k, bc)
+            n_t = layout.n_tree   # restriction and convolution in one call; its workspace is the tree
+            tree = torch.empty(max(n_t, 1), dtype=torch.float32, device=particles.device)
+            out = apr_convolve_auto(layout, particles, stencils, k, bc, workspace=tree)
+            tree = tree[:n_t] if n_t == 0 else tree
             ctx.save_for_backward(particles, tree, stencils)
             ctx.layout, ctx.k, ctx.bc = layout, k, bc
             return out

@@ -98,7 +98,9 @@ struct alignas(16) LeafRec {
 };
 static_assert(sizeof(LeafRec) == 32, "leaf records are two 16-byte words");
 struct UnitPlan {                          // host
-    std::vector<UnitHdr> hdr, lhdr;        // node units, leaf units
+    std::vector<UnitHdr> hdr, lhdr;        // node units (finest level first), leaf units (longest first)
+    std::vector<UnitHdr> work;             // the node units again: those of the forward pass, then the rest, longest first
+    int32_t n_forward = 0;                 // node units of the levels down to the coarsest that holds particles
     std::vector<uint4> pure, lpure;        // entries: pure slots, other nodes, the rest
     std::vector<TreeNodePlan> nmap, lnmap;
     std::vector<uint32_t> ninfo, lninfo;
@@ -121,7 +123,7 @@ struct UnitRanges {                // partials of level l_min + i: first[i] .. l
     int first[MAXL], last[MAXL];
 };
 struct UnitView {                          // device
-    const UnitHdr *hdr, *lhdr;
+    const UnitHdr *hdr, *lhdr, *work;
     const uint4 *pure, *lpure;
     const TreeNodePlan *nmap, *lnmap;
     const uint32_t *ninfo, *lninfo;

@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_fwd_kernel(const UnitView U, const 
     extern __shared__ __align__(128) unsigned char smraw[];
     McSmem &S = *reinterpret_cast<McSmem *>(smraw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const UnitHdr h = U.hdr[blockIdx.x];
+    const UnitHdr h = U.work[blockIdx.x];
     stage_codes<true>(U, h, false, bc == APR_BC_REFLECT, S.code);
     pdl_wait();   // the weight layout and the tree are written by the launches before this one
     tile_setup(S, W, h.lev);
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
     extern __shared__ __align__(128) unsigned char smraw[];
     McSmem &S = *reinterpret_cast<McSmem *>(smraw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const UnitHdr h = U.hdr[blockIdx.x];
+    const UnitHdr h = U.work[blockIdx.x];
     const NodeRec *rec = U.rec + h.rec0;
     stage_codes<false>(U, h, false, false, S.code);
     pdl_wait();   // the weight layout is written by the launch before this one

@@ -476,6 +476,18 @@ void virtual_parents(HostIndex &X) {
     X.vrow_ptr[size_t(pz) * px] = uint32_t(X.vy.size());
 }
 
+// The units of a launch in descending order of their work (a record's sums cost about as much as staging four
+// pure slots or two others), so that its last wave consists of short ones. In the order they are built (finest
+// level first, along the curve) the long blocks of the second finest level still start in the last of two or
+// three waves. Measured: 20 Richardson-Lucy iterations of 2.8 M particles (3 waves) 2717 -> 2506 us, gradient
+// magnitude of 1.2 M 39 -> 35 us, 16-channel leaf adjoint of 1 M 90 -> 75 us and of the FP32 one of 8 M 84 -> 72 us.
+// The lost neighbourhood of units that run together costs up to 5 us of the 8 M particles' 124 us node adjoint.
+template <typename It>
+void sort_by_work(It first, It last) {
+    auto work = [](const UnitHdr &h) { return 4 * int(h.nrec) + int(h.npure) + 2 * (int(h.nnode) + int(h.noth)); };
+    std::stable_sort(first, last, [&](const UnitHdr &a, const UnitHdr &b) { return work(a) > work(b); });
+}
+
 }  // namespace
 
 void build_units(HostIndex &X) {
@@ -619,6 +631,14 @@ void build_units(HostIndex &X) {
             o = JobOut{};
         }
     }
+    sort_by_work(U.lhdr.begin(), U.lhdr.end());
+    U.work = U.hdr;
+    for (int l = X.l_max; l >= X.l_min; --l)
+        if (X.fwd_level_begin[l + 1] > X.fwd_level_begin[l])
+            U.n_forward = l == X.l_min ? int32_t(U.hdr.size()) : U.level_begin[l - 1 - X.l_min];
+    const auto forward = U.work.begin() + U.n_forward;
+    sort_by_work(U.work.begin(), forward);
+    sort_by_work(forward, U.work.end());
     // whether every particle and tree node is some parent's child (each then has its own gradient
     // written by exactly one record)
     int64_t child_p = 0, child_t = 0;

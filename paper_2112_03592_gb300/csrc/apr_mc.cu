@@ -272,20 +272,42 @@ __global__ void mc_weight_layout_kernel(const uint16_t *__restrict__ W, int n_le
 }
 
 // ---------------------------------------------------------------- unit staging
-struct Rows {                         // the tile's rows: row slots of their neighbourhood
-    uint16_t base[9][TILE];
+struct Rows {                         // row slots of the unit's records, then of a tile's image or leaf rows
+    uint16_t base[9][UNIT_RECS + TILE];
     uint32_t mask[TILE];              // bit 3r + j: parent j of row r is a slot, at base[r] + the bits before it
 };
 
+// What every tile kernel keeps in shared memory. The gather reads every cell about eight times and lives on the L1
+// cache, which is what two blocks leave of 256 KB: nothing else belongs here (forward of 1 M particles with 28 KB
+// of L1 82 to 86 us, with 60 KB 66 us, with 92 KB 60 us).
 struct McSmem {
     int code[8][PLANE];               // source of every cell c of every slot
     Rows rows;
-    alignas(128) float4 sums[TILE * 16];   // image sums (image_chunk)
     alignas(128) unsigned char W[NWB * WBLK];
-    int first[UNIT_RECS + 1];         // first row of each record (lists of images)
-    int wsum[NWARP];
+    int4 children[UNIT_RECS];         // the records' child particles (TreeNodePlan::p)
     uint64_t bar[STAGES];             // MMAs that read buffer s have completed
     uint32_t tmem;
+};
+constexpr int IMAGE_ROWS = TILE / 2;   // image rows of a tile
+struct McRowLists {                   // rows of several images per record
+    int first[UNIT_RECS + 1];         // first row of each record
+    int wsum[NWARP];
+};
+struct McAdjSmem {
+    McSmem s;
+    alignas(16) float4 sums[IMAGE_ROWS * 32];   // image sums (image_chunk)
+    int4 nodes[UNIT_RECS];            // the records' tree-node children (TreeNodePlan::t)
+    uint16_t edge[UNIT_RECS];         // their edge words
+    McRowLists list;
+};
+struct McLeafSmem {
+    McSmem s;
+    alignas(16) float4 sums[2][TILE * 4];   // a row's sums over the four cells of one z plane
+    uint32_t mask[UNIT_RECS];         // of the records
+    int particle[UNIT_RECS];
+    uint16_t edge[UNIT_RECS];
+    uint8_t skip[TILE];               // cells of a row outside the grid: no part of the source (zero boundary)
+    McRowLists list;
 };
 
 // Source codes of the unit's slots. VALUES: particles, tree nodes and coarser particles; else the level-l
@@ -356,8 +378,42 @@ __device__ __forceinline__ void stage_codes(const UnitView &U, const UnitHdr &h,
     }
 }
 
-// Row r of the tile: record `rec` of a node unit at its own place (one set of loads: nine dependent ones
-// would cost more than the row's sums), ...
+// Record `rec` of a node unit at its own place: all 27 parents are slots (one set of loads: nine dependent
+// ones would cost more than the row's sums). Thread r keeps record r of the unit from its header to the staging,
+// so that neither the rows nor the children of any tile wait for another chain of loads (record by record per tile:
+// forward of 1 M particles 66 us, data adjoint 108 us, leaf adjoint 76 us; so 60, 96 and 71 us, the last two with the
+// images' sums below).
+struct NodeRow {
+    uint2 r0, r1, r2;
+    int4 pw, tw;
+    __device__ __forceinline__ void load(const UnitView &U, const UnitHdr &h, bool nodes) {
+        if (int(threadIdx.x) >= h.nrec) return;
+        const uint2 *q = reinterpret_cast<const uint2 *>(U.rec + h.rec0 + threadIdx.x);
+        r0 = __ldg(q);
+        r1 = __ldg(q + 1);
+        r2 = __ldg(q + 2);
+        const int4 *m = reinterpret_cast<const int4 *>(U.nplan + r0.x);
+        pw = __ldg(m);
+        if (nodes) tw = __ldg(m + 1);
+    }
+    // Rows past the unit's records read the empty slots.
+    __device__ __forceinline__ void put(McSmem &S, const UnitHdr &h) const {
+        const int r = threadIdx.x;
+        if (r >= UNIT_RECS) return;
+        unsigned b[9];
+        unpack_bases(r0.y, r1, r2, b);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) S.rows.base[k][r] = uint16_t(r < h.nrec ? b[k] : ZERO_SLOT);
+        S.children[r] = r < h.nrec ? pw : make_int4(0, 0, 0, 0);
+    }
+    __device__ __forceinline__ void put_nodes(McAdjSmem &A, const UnitHdr &h) const {
+        const int r = threadIdx.x;
+        if (r >= UNIT_RECS) return;
+        A.nodes[r] = r < h.nrec ? tw : make_int4(0, 0, 0, 0);
+        A.edge[r] = uint16_t(r < h.nrec ? r0.y & 0xffffu : 0u);
+    }
+};
+// Row r of the tile in the weight gradient: a record at its own place, ...
 __device__ __forceinline__ void put_node_row(Rows &R, int r, const NodeRec *rec) {
     const uint2 *q = reinterpret_cast<const uint2 *>(rec);
     const uint2 r0 = __ldg(q), r1 = __ldg(q + 1), r2 = __ldg(q + 2);
@@ -367,31 +423,30 @@ __device__ __forceinline__ void put_node_row(Rows &R, int r, const NodeRec *rec)
     for (int k = 0; k < 9; ++k) R.base[k][r] = uint16_t(b[k]);
     R.mask[r] = 0x7ffffffu;
 }
-// ... at the image of shift t (edge_shifts; 0: its own place), ...
-__device__ __forceinline__ void put_image_row(Rows &R, int r, const NodeRec *rec, int t) {
+// ... in the adjoint record i of the unit at the image of shift t (edge_shifts; 0: its own place), ...
+__device__ __forceinline__ void put_image_row(Rows &R, int r, int i, int t) {
     const int iz = t >> 4, ix = (t >> 2) & 3, iy = t & 3, dy = iy == 1 ? -1 : (iy == 0 ? 0 : iy - 1);
     unsigned mask = 0;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const int oz = image_layer(iz, q / 3), ox = image_layer(ix, q % 3);
         if (oz >= 0 && ox >= 0) {
-            R.base[q][r] = uint16_t(int(rec->base[3 * oz + ox]) + dy);
+            R.base[q][UNIT_RECS + r] = uint16_t(int(R.base[3 * oz + ox][i]) + dy);
             mask |= 7u << (3 * q);
         }
     }
     R.mask[r] = mask;
 }
-// ... of a leaf unit.
-__device__ __forceinline__ void put_leaf_row(Rows &R, int r, const LeafRec *rec, int t) {
+// ... record i, with slots `all`, of a leaf unit.
+__device__ __forceinline__ void put_leaf_row(Rows &R, int r, int i, unsigned all, int t) {
     const int iz = t >> 4, ix = (t >> 2) & 3, iy = t & 3;
-    const unsigned all = rec->mask;
     unsigned mask = 0;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const int oz = image_layer(iz, q / 3), ox = image_layer(ix, q % 3), o = 3 * oz + ox;
         if (oz >= 0 && ox >= 0) {
             const unsigned m = (all >> (3 * o)) & 7u;
-            R.base[q][r] = uint16_t(rec->base[o] + (iy == 0 ? 0 : __popc(m & (iy == 3 ? 3u : 1u))));
+            R.base[q][UNIT_RECS + r] = uint16_t(R.base[o][i] + (iy == 0 ? 0 : __popc(m & (iy == 3 ? 3u : 1u))));
             mask |= (iy == 0 ? m : (iy == 1 ? (m << 1) & 4u : (m >> (iy - 1)) & 1u)) << (3 * q);
         }
     }
@@ -416,15 +471,18 @@ __device__ __forceinline__ int step_x(int k) { return 2 * (k & 1); }
 
 // The four cells of row (iz, ix) of tile row r: up to 128 contiguous bytes. wide: 32-byte aligned features,
 // one load per cell (lane = record touches 16 lines per load either way; 16-byte loads touch them twice).
+// FULL: node records at their own place (no mask: all 27 parents are slots).
+template <bool FULL>
 struct CellRow {
     uint4 v[4][2];
     __device__ __forceinline__ void load(const int (*code)[PLANE], const Rows &rows, int r, int iz, int ix,
                                          const uint4 *__restrict__ vals, const uint4 *__restrict__ tree, bool wide) {
         const int q = ((iz + 1) >> 1) * 3 + ((ix + 1) >> 1), c0 = ((iz + 1) & 1) * 4 + ((ix + 1) & 1) * 2;
-        const unsigned m = (rows.mask[r] >> (3 * q)) & 7u, base = rows.base[q][r];
+        const unsigned m = FULL ? 7u : (rows.mask[r - UNIT_RECS] >> (3 * q)) & 7u, base = rows.base[q][r];
         int src[4];
 #pragma unroll
-        for (int iy = 0; iy < 4; ++iy) src[iy] = cell_code(code, m, base, c0, iy);
+        for (int iy = 0; iy < 4; ++iy)
+            src[iy] = FULL ? code[c0 + ((iy + 1) & 1)][base + ((iy + 1) >> 1)] : cell_code(code, m, base, c0, iy);
 #pragma unroll
         for (int iy = 0; iy < 4; ++iy) {
             v[iy][0] = v[iy][1] = make_uint4(0, 0, 0, 0);
@@ -488,16 +546,17 @@ __device__ __forceinline__ void issue_step(uint32_t D, uint32_t A, uint64_t W, i
 // warps load: warps q and q + 4 the rows 32 q .. 32 q + 31, one cell row each; the loads of step k + 1 are in
 // flight while step k is written to tensor memory and handed to the ninth warp, which issues the MMAs. A
 // buffer is written again once the MMAs of two steps before have completed. phase: one bit per buffer.
-// True on a timeout.
-__device__ __forceinline__ bool tile_gemm(McSmem &S, const uint4 *__restrict__ vals, const uint4 *__restrict__ tree, bool wide,
+// True on a timeout. FULL: rows row0 .. of the unit's records; else the tile's rows.
+template <bool FULL>
+__device__ __forceinline__ bool tile_gemm(McSmem &S, int row0, const uint4 *__restrict__ vals, const uint4 *__restrict__ tree, bool wide,
                                           uint32_t D, uint32_t &phase, unsigned *err) {
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    const int q = warp & 3, half = warp >> 2, r = 32 * q + lane;
+    const int q = warp & 3, half = warp >> 2, r = (FULL ? row0 : UNIT_RECS) + 32 * q + lane;
     const uint64_t W = sdesc(smem_u32(S.W), 128, 256);
     bool ok = true;
     if (warp < NWARP) {
         const uint32_t a0 = D + TM_A + (uint32_t(32 * q) << 16) + 32 * half;
-        CellRow c;
+        CellRow<FULL> c;
         c.load(S.code, S.rows, r, step_z(0), step_x(0) + half, vals, tree, wide);
 #pragma unroll 1
         for (int k = 0; k < 8; ++k) {
@@ -585,25 +644,23 @@ __global__ void __launch_bounds__(TNT, 2) mc_fwd_kernel(const UnitView U, const 
     McSmem &S = *reinterpret_cast<McSmem *>(smraw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.work[blockIdx.x];
+    NodeRow row;
+    row.load(U, h, false);
     stage_codes<true>(U, h, false, bc == APR_BC_REFLECT, S.code);
+    row.put(S, h);
     pdl_wait();   // the weight layout and the tree are written by the launches before this one
     tile_setup(S, W, h.lev);
+    tile_ready();
+    const uint32_t D = S.tmem;
     const bool wide = ((reinterpret_cast<uintptr_t>(vals) | reinterpret_cast<uintptr_t>(tree)) & 31u) == 0;
     const bool wide_out = ((reinterpret_cast<uintptr_t>(o.out) | reinterpret_cast<uintptr_t>(o.out_bf16)) & 31u) == 0;
     uint32_t phase = 0;
     const int q = warp & 3, a = warp >> 2;
     for (int t0 = 0; t0 < h.nrec; t0 += TILE) {
-        if (tid < TILE) {
-            if (t0 + tid < h.nrec) put_node_row(S.rows, tid, U.rec + h.rec0 + t0 + tid);
-            else S.rows.mask[tid] = 0;
-        }
-        tile_ready();
-        const uint32_t D = S.tmem;
-        if (tile_gemm(S, vals, tree, wide, D, phase, err)) break;
+        if (tile_gemm<true>(S, t0, vals, tree, wide, D, phase, err)) break;
         // lane = record, this warp's half of the children (a): the particles' outputs
-        const int r = t0 + 32 * q + lane;
         int2 pw = make_int2(0, 0);
-        if (warp < NWARP && r < h.nrec) pw = __ldg(reinterpret_cast<const int2 *>(U.nplan[U.rec[h.rec0 + r].node].p + 2 * a));
+        if (warp < NWARP) pw = reinterpret_cast<const int2 *>(S.children + t0 + 32 * q + lane)[a];
         if (warp < NWARP)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -648,7 +705,7 @@ __device__ __forceinline__ void add4(float *p, const float4 &s) {
 }
 
 // Exclusive prefix of n (one value of each of the first NT threads) into first[0 .. NT]. Ends with a barrier.
-__device__ __forceinline__ int prefix_rows(McSmem &S, int n) {
+__device__ __forceinline__ int prefix_rows(McRowLists &S, int n) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int incl = n;
 #pragma unroll
@@ -670,7 +727,7 @@ __device__ __forceinline__ int prefix_rows(McSmem &S, int n) {
     return total;
 }
 // The record (of n) that owns row k.
-__device__ __forceinline__ int row_owner(const McSmem &S, int n, int k) {
+__device__ __forceinline__ int row_owner(const McRowLists &S, int n, int k) {
     int a = 0, b = n;
     while (b - a > 1) {
         const int m = (a + b) / 2;
@@ -694,10 +751,10 @@ __device__ __forceinline__ int image_row(unsigned edge, int j) {
     return j < __popcll(m) ? nth_bit(m, j) : 0;
 }
 
-// Float4 chunk k (0..15) of row r in the 128 x 64-float staging of the image sums (16-byte chunks swizzled by
+// Float4 chunk k (0..31) of row r in the 64 x 128-float staging of the image sums (16-byte chunks swizzled by
 // the row: conflict-free for lane = row).
-__device__ __forceinline__ float4 *image_chunk(McSmem &S, int r, int k) {
-    return S.sums + r * 16 + (k ^ (r & 15));
+__device__ __forceinline__ float4 *image_chunk(McAdjSmem &S, int r, int k) {
+    return S.sums + r * 32 + (k ^ (r & 31));
 }
 
 // Data adjoint onto the children of every record: particles (gp) and tree nodes (gt) are stored, then, with
@@ -706,35 +763,37 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
                                                            const uint4 *__restrict__ gout, float *__restrict__ gp,
                                                            float *__restrict__ gt, unsigned *err) {
     extern __shared__ __align__(128) unsigned char smraw[];
-    McSmem &S = *reinterpret_cast<McSmem *>(smraw);
+    McAdjSmem &M = *reinterpret_cast<McAdjSmem *>(smraw);
+    McSmem &S = M.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.work[blockIdx.x];
     const NodeRec *rec = U.rec + h.rec0;
+    NodeRow row;
+    row.load(U, h, true);
     stage_codes<false>(U, h, false, false, S.code);
+    row.put(S, h);
+    row.put_nodes(M, h);
     pdl_wait();   // the weight layout is written by the launch before this one
     tile_setup(S, W, h.lev);
+    tile_ready();
+    const uint32_t D = S.tmem;
     const bool wide = (reinterpret_cast<uintptr_t>(gout) & 31u) == 0;
     const bool wide_out = ((reinterpret_cast<uintptr_t>(gp) | reinterpret_cast<uintptr_t>(gt)) & 31u) == 0;
     uint32_t phase = 0;
     const int q = warp & 3, a = warp >> 2;
     bool failed = false;
     for (int t0 = 0; t0 < h.nrec && !failed; t0 += TILE) {
-        if (tid < TILE) {
-            if (t0 + tid < h.nrec) put_node_row(S.rows, tid, rec + t0 + tid);
-            else S.rows.mask[tid] = 0;
-        }
-        tile_ready();
-        const uint32_t D = S.tmem;
-        failed = tile_gemm(S, gout, gout, wide, D, phase, err);
+        failed = tile_gemm<true>(S, t0, gout, gout, wide, D, phase, err);
         if (failed) break;
-        const int r = t0 + 32 * q + lane;
-        int4 pw = make_int4(0, 0, 0, 0), tw = pw;
-        if (warp < NWARP && r < h.nrec) {
-            const int4 *m = reinterpret_cast<const int4 *>(U.nplan + rec[r].node);
-            pw = __ldg(m);
-            tw = __ldg(m + 1);
+        int pk[2] = {}, tk[2] = {};
+        if (warp < NWARP) {
+            const int2 p = reinterpret_cast<const int2 *>(S.children + t0 + 32 * q + lane)[a];
+            const int2 t = reinterpret_cast<const int2 *>(M.nodes + t0 + 32 * q + lane)[a];
+            pk[0] = p.x;
+            pk[1] = p.y;
+            tk[0] = t.x;
+            tk[1] = t.y;
         }
-        const int pk[2] = {a ? pw.z : pw.x, a ? pw.w : pw.y}, tk[2] = {a ? tw.z : tw.x, a ? tw.w : tw.y};
         if (warp < NWARP)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -750,60 +809,58 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
         tile_done();
     }
     if (!failed && bc == APR_BC_REFLECT && h.nflag > 0) {
-        const int total = prefix_rows(S, tid < h.nflag ? image_rows(rec[tid].edge) : 0);
-        for (int k0 = 0; k0 < total && !failed; k0 += TILE) {
+        const int total = prefix_rows(M.list, tid < h.nflag ? image_rows(M.edge[tid]) : 0);
+        for (int k0 = 0; k0 < total && !failed; k0 += IMAGE_ROWS) {
+            const int k1 = min(k0 + IMAGE_ROWS, total);
             if (tid < TILE) {
                 const int k = k0 + tid;
-                if (k < total) {
-                    const int i = row_owner(S, h.nflag, k);
-                    put_image_row(S.rows, tid, rec + i, image_row(rec[i].edge, k - S.first[i]));
+                if (k < k1) {
+                    const int i = row_owner(M.list, h.nflag, k);
+                    put_image_row(S.rows, tid, i, image_row(M.edge[i], k - M.list.first[i]));
                 } else {
                     S.rows.mask[tid] = 0;
                 }
             }
             tile_ready();
-            const uint32_t D = S.tmem;
-            failed = tile_gemm(S, gout, gout, wide, D, phase, err);
+            failed = tile_gemm<false>(S, 0, gout, gout, wide, D, phase, err);
             if (failed) break;
-            // source children of half a (64 columns) through shared memory; one
-            // thread per (record, child place (b, e), four channels) adds the rows' sums in order
-            const int i0 = row_owner(S, h.nflag, k0), i1 = row_owner(S, h.nflag, min(k0 + TILE, total) - 1);
-            for (int half = 0; half < 2; ++half) {
-                if (warp < NWARP)
+            // source children through shared memory; one thread per (record, child, four channels) adds the
+            // sums of the record's rows in order, then adds them to the child
+            if (warp < NWARP && 32 * q < IMAGE_ROWS)
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
+                for (int c = 0; c < 4; ++c) {
                     float v[16];
-                    const int col = 32 * a + 16 * c, r = 32 * q + lane;
-                    tmem_ld16(D + (uint32_t(32 * q) << 16) + 64 * half + col, v);
+                    tmem_ld16(D + (uint32_t(32 * q) << 16) + 64 * a + 16 * c, v);
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        *image_chunk(S, r, col / 4 + k) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+                        *image_chunk(M, 32 * q + lane, 16 * a + 4 * c + k) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
                 }
-                block_sync();
-                for (int w = tid; w < (i1 - i0 + 1) * 16; w += TNT) {
-                    const int i = i0 + (w >> 4), place = (w >> 2) & 3, ch = w & 3;
-                    const unsigned edge = rec[i].edge, miss = missing_children(edge);
-                    const TreeNodePlan &m = U.nplan[rec[i].node];
-                    for (int k = max(S.first[i], k0); k < min(S.first[i + 1], k0 + TILE); ++k) {
-                        const int t = image_row(edge, k - S.first[i]);
-                        const unsigned mir = (t >> 4 ? 4u : 0u) | ((t >> 2) & 3 ? 2u : 0u) | (t & 3 ? 1u : 0u);
-                        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-                        unsigned to = 8u;   // the target child (the same for every source found)
-                        for (int src = 0; src < 4; ++src) {
-                            const unsigned full = (4u * half + src) ^ mir;   // before a missing child is folded
-                            if ((t == 0 && !(full & miss)) || int((full & ~miss) & 3u) != place) continue;
-                            to = full & ~miss;
-                            const float4 v = *image_chunk(S, k - k0, src * 4 + ch);
+            block_sync();
+            const int i0 = row_owner(M.list, h.nflag, k0), i1 = row_owner(M.list, h.nflag, k1 - 1);
+            for (int w = tid; w < (i1 - i0 + 1) * 32; w += TNT) {
+                const int i = i0 + (w >> 5), ch = w & 3;
+                const unsigned to = (w >> 2) & 7, edge = M.edge[i], miss = missing_children(edge);
+                const unsigned p = unsigned(reinterpret_cast<const int *>(S.children + i)[to >> 1]), pm = p >> 30;
+                const unsigned t = unsigned(reinterpret_cast<const int *>(M.nodes + i)[to >> 1]), tm = t >> 30;
+                const int e = int(to & 1u);
+                float *dst;
+                if ((pm >> e) & 1u) dst = gp + (size_t(p & TNP_INDEX) + (e ? pm & 1u : 0u)) * MC + 4 * ch;
+                else if ((tm >> e) & 1u) dst = gt + (size_t(t & TNP_INDEX) + (e ? tm & 1u : 0u)) * MC + 4 * ch;
+                else continue;
+                float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int k = max(M.list.first[i], k0); k < min(M.list.first[i + 1], k1); ++k) {
+                    const int sh = image_row(edge, k - M.list.first[i]);
+                    const unsigned mir = (sh >> 4 ? 4u : 0u) | ((sh >> 2) & 3 ? 2u : 0u) | (sh & 3 ? 1u : 0u);
+                    unsigned f = 0;   // the child itself, then the missing ones that it stands for
+                    do {
+                        if (sh != 0 || f != 0) {
+                            const float4 v = *image_chunk(M, k - k0, int((to | f) ^ mir) * 4 + ch);
                             s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
                         }
-                        if (to == 8u) continue;
-                        const unsigned p = unsigned(m.p[to >> 1]), tt = unsigned(m.t[to >> 1]), pm = p >> 30, tm = tt >> 30;
-                        const int e = int(to & 1u);
-                        if ((pm >> e) & 1u) add4(gp + (size_t(p & TNP_INDEX) + (e ? pm & 1u : 0u)) * MC + 4 * ch, s);
-                        else if ((tm >> e) & 1u) add4(gt + (size_t(tt & TNP_INDEX) + (e ? tm & 1u : 0u)) * MC + 4 * ch, s);
-                    }
+                        f = (f - miss) & miss;
+                    } while (f != 0);
                 }
-                block_sync();
+                add4(dst, s);
             }
             tile_done();
         }
@@ -817,55 +874,76 @@ __global__ void __launch_bounds__(TNT, 2) mc_leaf_adjoint_kernel(const UnitView 
                                                                 const uint4 *__restrict__ gout, float *__restrict__ gp,
                                                                 unsigned *err) {
     extern __shared__ __align__(128) unsigned char smraw[];
-    McSmem &S = *reinterpret_cast<McSmem *>(smraw);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    McLeafSmem &M = *reinterpret_cast<McLeafSmem *>(smraw);
+    McSmem &S = M.s;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.lhdr[blockIdx.x];
-    const LeafRec *rec = U.lrec + h.rec0;
     const bool reflect = bc == APR_BC_REFLECT;
+    // thread i keeps record i from its header to the staging
+    uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
+    if (tid < h.nrec) {
+        const uint4 *r = reinterpret_cast<const uint4 *>(U.lrec + h.rec0 + tid);
+        q0 = __ldg(r);
+        q1 = __ldg(r + 1);
+    }
     stage_codes<false>(U, h, true, false, S.code);
+    const unsigned edge = q0.z & 0xffffu;
+    if (tid < UNIT_RECS) {
+        unsigned b[9];
+        unpack_bases(q0.z, make_uint2(q0.w, q1.x), make_uint2(q1.y, q1.z), b);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) S.rows.base[k][tid] = uint16_t(b[k]);
+        M.particle[tid] = int(q0.x);
+        M.mask[tid] = q0.y;
+        M.edge[tid] = uint16_t(edge);
+    }
     tile_setup(S, W, h.lev);
     const bool wide = (reinterpret_cast<uintptr_t>(gout) & 31u) == 0;
     uint32_t phase = 0;
-    const int total = prefix_rows(S, tid < h.nrec ? (reflect ? __popcll(edge_shifts<1>(rec[tid].edge)) : 1) : 0);
+    const int total = prefix_rows(M.list, tid < h.nrec ? (reflect ? __popcll(edge_shifts<1>(edge)) : 1) : 0);
     for (int k0 = 0; k0 < total; k0 += TILE) {
-        unsigned skip = 0;   // cells outside the grid are no part of the source (zero boundary)
         if (tid < TILE) {
             const int k = k0 + tid;
             if (k < total) {
-                const int i = row_owner(S, h.nrec, k);
-                put_leaf_row(S.rows, tid, rec + i, reflect ? nth_bit(edge_shifts<1>(rec[i].edge), k - S.first[i]) : 0);
-                if (!reflect) skip = missing_children(rec[i].edge);
+                const int i = total == h.nrec ? k : row_owner(M.list, h.nrec, k);
+                put_leaf_row(S.rows, tid, i, M.mask[i], reflect ? nth_bit(edge_shifts<1>(M.edge[i]), k - M.list.first[i]) : 0);
+                M.skip[tid] = uint8_t(reflect ? 0u : missing_children(M.edge[i]));
             } else {
                 S.rows.mask[tid] = 0;
+                M.skip[tid] = 0;
             }
         }
         tile_ready();
         const uint32_t D = S.tmem;
-        if (tile_gemm(S, gout, gout, wide, D, phase, err)) break;
-        if (warp < 4) {   // thread = row
+        if (tile_gemm<false>(S, 0, gout, gout, wide, D, phase, err)) break;
+        if (warp < NWARP) {   // lane = row, half of the cells
+            const int q = warp & 3, a = warp >> 2, r = 32 * q + lane;
             float s[16];
 #pragma unroll
             for (int k = 0; k < 16; ++k) s[k] = 0.f;
-            for (unsigned c = 0; c < 8; ++c) {
+            for (unsigned c = 0; c < 4; ++c) {
                 float v[16];
-                tmem_ld16(D + (uint32_t(32 * warp) << 16) + 16 * c, v);
-                if (!(c & skip))
+                tmem_ld16(D + (uint32_t(32 * q) << 16) + 64 * a + 16 * c, v);
+                if (!((4u * a + c) & M.skip[r]))
 #pragma unroll
                     for (int k = 0; k < 16; ++k) s[k] += v[k];
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) *image_chunk(S, tid, k) = make_float4(s[4 * k], s[4 * k + 1], s[4 * k + 2], s[4 * k + 3]);
+            for (int k = 0; k < 4; ++k)
+                M.sums[a][r * 4 + (k ^ (r & 3))] = make_float4(s[4 * k], s[4 * k + 1], s[4 * k + 2], s[4 * k + 3]);
         }
         block_sync();
-        const int i0 = row_owner(S, h.nrec, k0), i1 = row_owner(S, h.nrec, min(k0 + TILE, total) - 1);
+        const int k1 = min(k0 + TILE, total);
+        const int i0 = total == h.nrec ? k0 : row_owner(M.list, h.nrec, k0), i1 = total == h.nrec ? k1 - 1 : row_owner(M.list, h.nrec, k1 - 1);
         for (int w = tid; w < (i1 - i0 + 1) * 4; w += TNT) {
             const int i = i0 + (w >> 2), ch = w & 3;
             float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int k = max(S.first[i], k0); k < min(S.first[i + 1], k0 + TILE); ++k) {
-                const float4 v = *image_chunk(S, k - k0, ch);
-                s = make_float4(s.x + v.x, s.y + v.y, s.z + v.z, s.w + v.w);
+            for (int k = max(M.list.first[i], k0); k < min(M.list.first[i + 1], k1); ++k) {
+                const int j = (k - k0) * 4 + (ch ^ ((k - k0) & 3));
+                const float4 u = M.sums[0][j], v = M.sums[1][j];
+                s = make_float4(s.x + (u.x + v.x), s.y + (u.y + v.y), s.z + (u.z + v.z), s.w + (u.w + v.w));
             }
-            add4(gp + size_t(rec[i].particle) * MC + 4 * ch, s);
+            add4(gp + size_t(M.particle[i]) * MC + 4 * ch, s);
         }
         tile_done();
     }
@@ -1048,7 +1126,11 @@ __global__ void mc_wgrad_reduce_kernel(const float *__restrict__ partial, const 
 
 // The tile kernels' shared memory admits two blocks per SM (228 KB per SM, 1 KB reserved per block), each
 // with half of the SM's 512 tensor-memory columns; the weight gradient takes an SM to itself.
-static_assert(2 * (sizeof(McSmem) + 1024) <= 228 * 1024, "tile kernels: two blocks per SM");
+// A third block would wait for tensor memory with its SM's other resources in hand (leaf adjoint of 1 M particles: 95
+// instead of 76 us): the leaf kernel, whose registers admit three, takes more than a third of the shared memory.
+constexpr size_t TWO_BLOCKS = 228 * 1024 / 3;
+static_assert(sizeof(McLeafSmem) <= 113 * 1024, "leaf units: two blocks per SM");
+static_assert(2 * (sizeof(McAdjSmem) + 1024) <= 228 * 1024, "tile kernels: two blocks per SM");
 static_assert(sizeof(WgradSmem) <= 227 * 1024, "weight gradient: one block per SM");
 static_assert(offsetof(McSmem, W) % 128 == 0 && offsetof(McSmem, bar) % 8 == 0, "alignment");
 static_assert(offsetof(WgradSmem, A) % 128 == 0 && offsetof(WgradSmem, g) % 128 == 0 && offsetof(WgradSmem, bar) % 8 == 0, "alignment");
@@ -1069,7 +1151,10 @@ int wgrad_ctas(int n_units) {
 template <typename... KArgs, typename... Args>
 cudaError_t launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl, Args &&...args) {
     if (grid <= 0) return cudaSuccess;
-    const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void *>(kernel), smem);
+    // two tile kernels' blocks on a multiprocessor (tensor memory admits no more), one of the weight gradient. Left to
+    // itself the split leaves 28 or 60 KB of L1 cache
+    const int blocks = 2 * (smem + 1024) <= 228 * 1024 ? 2 : 1;
+    const cudaError_t e = set_max_dynamic_smem(reinterpret_cast<const void *>(kernel), smem, blocks);
     if (e != cudaSuccess) return e;
     return launch_pdl(kernel, dim3(grid), dim3(block), smem, s, pdl, std::forward<Args>(args)...);
 }
@@ -1191,9 +1276,9 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
         const uint4 *g4 = reinterpret_cast<const uint4 *>(grad_out);
         if (e == cudaSuccess) e = layout_weights(weights, n_levels, 1, wt, stream);
         if (e == cudaSuccess)
-            e = launch(mc_adjoint_kernel, h->U.n, TNT, sizeof(McSmem), stream, true, h->U, wt, bc, g4, grad_particles, gt, h->d_err);
+            e = launch(mc_adjoint_kernel, h->U.n, TNT, sizeof(McAdjSmem), stream, true, h->U, wt, bc, g4, grad_particles, gt, h->d_err);
         if (e == cudaSuccess)
-            e = launch(mc_leaf_adjoint_kernel, h->U.nl, TNT, sizeof(McSmem), stream, false, h->U, wt, bc, g4, grad_particles, h->d_err);
+            e = launch(mc_leaf_adjoint_kernel, h->U.nl, TNT, std::max(sizeof(McLeafSmem), TWO_BLOCKS), stream, false, h->U, wt, bc, g4, grad_particles, h->d_err);
         bool chained = false;   // the launches after the first start early (programmatic dependent launch)
         const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
         for (int i = 0; i < T.n && e == cudaSuccess; ++i) {

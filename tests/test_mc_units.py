@@ -101,3 +101,25 @@ def test_element_wise_layers_at_every_alignment(n, offset):
     assert torch.equal(G.apr_mc_relu_bf16(c.view(-1)[:n * C - 5], buf((n * C - 5,), torch.bfloat16)), ref.view(-1)[:n * C - 5])
     ref = torch.where(c > 0, g, torch.zeros_like(g)).to(torch.bfloat16)
     assert torch.equal(G.apr_mc_relu_backward_bf16(c, g, buf((n, C), torch.bfloat16)), ref)
+
+
+@pytest.mark.parametrize("bc", [0, 1])
+def test_outputs_at_16_byte_alignment_are_the_same_bits(bc):
+    """32-byte stores where the outputs allow them, 16-byte stores else: the same numbers."""
+    apr = CASES["odd_ends"]()
+    rng = np.random.default_rng(9)
+    lay = G.AprLayout.from_apr(apr, FLAGS)
+    x, g = (bf16(rng.integers(-64, 65, size=(apr.n_particles, C)) / 8.0, 0) for _ in range(2))
+    w = bf16(rng.integers(-16, 17, size=(apr.n_levels, C, C, 27)) / 16.0, 0)
+    tree = G.apr_tree_restrict_bf16(lay, x)
+
+    def at(offset, dtype):
+        return torch.empty(apr.n_particles * C + offset, dtype=dtype, device="cuda")[offset:].view(apr.n_particles, C)
+
+    res = []
+    for o32, o16 in ((0, 0), (4, 8)):
+        res.append((G.apr_convolve_mc(lay, x, tree, w, bc, out=at(o32, torch.float32)),
+                    G.apr_convolve_mc_relu_bf16(lay, x, tree, w, bc, out=at(o16, torch.bfloat16)),
+                    G.apr_convolve_mc_backward(lay, x, tree, w, g, bc, need_weights=False, grad_particles=at(o32, torch.float32))[0]))
+    for a, b in zip(*res):
+        assert torch.equal(a, b)

@@ -275,7 +275,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
                 e = cudaMemcpyAsync(static_cast<char *>(p) + nb, X.vplan.data(), vb, cudaMemcpyHostToDevice, cs);
         }
         const UnitPlan &UP = X.units;
-        UnitHdr *d_hdr = nullptr, *d_lhdr = nullptr, *d_work = nullptr;
+        UnitHdr *d_hdr = nullptr, *d_lhdr = nullptr, *d_work = nullptr, *d_adj = nullptr;
         uint4 *d_pure = nullptr, *d_lpure = nullptr;
         TreeNodePlan *d_nmap = nullptr, *d_lnmap = nullptr;
         uint32_t *d_ninfo = nullptr, *d_lninfo = nullptr;
@@ -286,6 +286,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         if (e == cudaSuccess) e = upload(h, &d_hdr, UP.hdr.data(), UP.hdr.size());
         if (e == cudaSuccess) e = upload(h, &d_lhdr, UP.lhdr.data(), UP.lhdr.size());
         if (e == cudaSuccess) e = upload(h, &d_work, UP.work.data(), UP.work.size());
+        if (e == cudaSuccess) e = upload(h, &d_adj, UP.work_adj.data(), UP.work_adj.size());
         if (e == cudaSuccess) e = upload(h, &d_pure, UP.pure.data(), UP.pure.size());
         if (e == cudaSuccess) e = upload(h, &d_lpure, UP.lpure.data(), UP.lpure.size());
         if (e == cudaSuccess) e = upload(h, &d_nmap, UP.nmap.data(), UP.nmap.size());
@@ -298,7 +299,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         if (e == cudaSuccess) e = upload(h, &d_tf, UP.tile_f.data(), UP.tile_f.size());
         if (e == cudaSuccess) e = upload(h, &d_tb, UP.tile_b.data(), UP.tile_b.size());
         if (e == cudaSuccess) e = upload(h, &d_ltb, UP.ltile_b.data(), UP.ltile_b.size());
-        h->U = UnitView{d_hdr, d_lhdr, d_work, d_pure, d_lpure, d_nmap, d_lnmap, d_ninfo, d_lninfo, d_oth, d_rec, d_lrec, d_tf, d_tb, d_ltb, h->d_tnplan,
+        h->U = UnitView{d_hdr, d_lhdr, d_work, d_adj, d_pure, d_lpure, d_nmap, d_lnmap, d_ninfo, d_lninfo, d_oth, d_rec, d_lrec, d_tf, d_tb, d_ltb, h->d_tnplan,
                         int32_t(UP.hdr.size()), int32_t(UP.lhdr.size())};
         h->n_fwd_units = UP.n_forward;
         for (int i = X.l_max - X.l_min; i >= 0; --i) {   // finest first

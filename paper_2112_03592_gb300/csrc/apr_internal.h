@@ -99,7 +99,7 @@ struct alignas(16) LeafRec {
 static_assert(sizeof(LeafRec) == 32, "leaf records are two 16-byte words");
 struct UnitPlan {                          // host
     std::vector<UnitHdr> hdr, lhdr;        // node units (finest level first), leaf units (longest first)
-    std::vector<UnitHdr> work;             // the node units again: those of the forward pass, then the rest, longest first
+    std::vector<UnitHdr> work, work_adj;   // the node units again, longest first: those of the forward pass, then the rest; all
     int32_t n_forward = 0;                 // node units of the levels down to the coarsest that holds particles
     std::vector<uint4> pure, lpure;        // entries: pure slots, other nodes, the rest
     std::vector<TreeNodePlan> nmap, lnmap;
@@ -123,7 +123,7 @@ struct UnitRanges {                // partials of level l_min + i: first[i] .. l
     int first[MAXL], last[MAXL];
 };
 struct UnitView {                          // device
-    const UnitHdr *hdr, *lhdr, *work;
+    const UnitHdr *hdr, *lhdr, *work, *work_adj;
     const uint4 *pure, *lpure;
     const TreeNodePlan *nmap, *lnmap;
     const uint32_t *ninfo, *lninfo;

@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
     McAdjSmem &M = *reinterpret_cast<McAdjSmem *>(smraw);
     McSmem &S = M.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const UnitHdr h = U.work[blockIdx.x];
+    const UnitHdr h = U.work_adj[blockIdx.x];
     const NodeRec *rec = U.rec + h.rec0;
     NodeRow row;
     row.load(U, h, true);

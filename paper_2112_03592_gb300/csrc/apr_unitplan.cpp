@@ -481,10 +481,11 @@ void virtual_parents(HostIndex &X) {
 // level first, along the curve) the long blocks of the second finest level still start in the last of two or
 // three waves. Measured: 20 Richardson-Lucy iterations of 2.8 M particles (3 waves) 2717 -> 2506 us, gradient
 // magnitude of 1.2 M 39 -> 35 us, 16-channel leaf adjoint of 1 M 90 -> 75 us and of the FP32 one of 8 M 84 -> 72 us.
-// The lost neighbourhood of units that run together costs up to 5 us of the 8 M particles' 124 us node adjoint.
+// flag: what an edge record's images cost on top (16-channel data adjoint of 1 M particles, whose images take tiles of
+// their own: 106 -> 96 us; FP32 of 8 M 129 -> 124 us, which makes up for the lost neighbourhood).
 template <typename It>
-void sort_by_work(It first, It last) {
-    auto work = [](const UnitHdr &h) { return 4 * int(h.nrec) + int(h.npure) + 2 * (int(h.nnode) + int(h.noth)); };
+void sort_by_work(It first, It last, int flag = 0) {
+    auto work = [flag](const UnitHdr &h) { return (4 * int(h.nrec) + int(h.npure) + 2 * (int(h.nnode) + int(h.noth))) + flag * int(h.nflag); };
     std::stable_sort(first, last, [&](const UnitHdr &a, const UnitHdr &b) { return work(a) > work(b); });
 }
 
@@ -639,6 +640,8 @@ void build_units(HostIndex &X) {
     const auto forward = U.work.begin() + U.n_forward;
     sort_by_work(U.work.begin(), forward);
     sort_by_work(forward, U.work.end());
+    U.work_adj = U.hdr;
+    sort_by_work(U.work_adj.begin(), U.work_adj.end(), 20);
     // whether every particle and tree node is some parent's child (each then has its own gradient
     // written by exactly one record)
     int64_t child_p = 0, child_t = 0;

@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(UT, 4) unit_adjoint_kernel(const UnitView U, c
                                                              const TileRange tr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AdjSmem &S = *reinterpret_cast<AdjSmem *>(smem_raw);
-    const UnitHdr h = U.work[blockIdx.x];
+    const UnitHdr h = U.work_adj[blockIdx.x];
     const int tid = threadIdx.x;
     Rec rec{};
     const bool live = tid < h.nrec && tr.has(U.tile_b, h.rec0 + tid);

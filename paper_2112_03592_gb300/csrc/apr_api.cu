@@ -105,11 +105,9 @@ apr_status_t pushdown_levels(apr_handle_t h, float *grad_tree, float *grad_parti
     if (l0 < X.l_min) l0 = X.l_min;
     if (l1 > X.l_max - 1) l1 = X.l_max - 1;
     cudaError_t e = cudaSuccess;
-    bool chained = false;   // the launches after the first start early (programmatic dependent launch)
     const TreeGroups T = tree_groups(X, l0, l1, 4);
     for (int i = 0; i < T.n && e == cudaSuccess; ++i) {
-        e = launch_tree_pushdown(h->d_tnplan, T.g[i], grad_particles, grad_tree, s, chained);
-        chained = true;
+        e = launch_tree_pushdown(h->d_tnplan, T.g[i], grad_particles, grad_tree, s, true);
     }
     return cuda_status(e);
 }
@@ -506,12 +504,10 @@ apr_status_t apr_tree_restrict(apr_handle_t h, const float *particles, float *tr
     if (channels < 1 || channels > 64) return APR_ERR_INVALID_ARG;
     if ((!particles && h->X.np) || (!tree && h->X.nt)) return APR_ERR_INVALID_ARG;
     const HostIndex &X = h->X;
-    bool chained = false;   // the launches after the first start early (programmatic dependent launch)
     const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 4);
     for (int i = T.n - 1; i >= 0; --i) {   // the finest group first
         for (int c = 0; c < channels; ++c) {  // channels-last values: one strided pass per channel
-            const cudaError_t e = launch_tree_restrict(h->d_tnplan, T.g[i], particles, tree, stream, channels, c, chained);
-            chained = true;
+            const cudaError_t e = launch_tree_restrict(h->d_tnplan, T.g[i], particles, tree, stream, channels, c, true);
             if (e != cudaSuccess) return cuda_status(e);
         }
     }

@@ -65,6 +65,13 @@ __host__ __device__ __forceinline__ void row_range(const uint32_t *rp, const uin
 // attribute both are no-ops.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// What an earlier launch may write while this kernel already runs (all but the handle's own arrays) is read after
+// pdl_wait, and not through the read-only path, which assumes that it stays as it is for the kernel's lifetime.
+__device__ __forceinline__ float load_after_wait(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 
 }  // namespace dev
 }  // namespace aprk

@@ -155,13 +155,16 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint4 &a, const u
                  : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// 32 bytes at a 32-byte aligned address.
+// 32 bytes at a 32-byte aligned address (16 below); not through the read-only path, as load_after_wait.
 __device__ __forceinline__ void load32(const uint4 *p, uint4 &a, uint4 &b) {
-    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
                  : "l"(p));
 }
 
+__device__ __forceinline__ void load16(const uint4 *p, uint4 &a) {
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "l"(p));
+}
 // 32 bytes to a 32-byte aligned address.
 __device__ __forceinline__ void store32(void *p, const uint4 &a, const uint4 &b) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
@@ -256,9 +259,10 @@ __device__ __forceinline__ void weight_block(int blk, int &tz, int &tx, int &ty)
 }
 
 // out[lev][block][...] from W[lev][co][ci][e]. adjoint: N = ci, K = co, taps flipped; else N = co, K = ci.
-__global__ void mc_weight_layout_kernel(const uint16_t *__restrict__ W, int n_levels, int adjoint,
+__global__ void mc_weight_layout_kernel(const uint16_t *W, int n_levels, int adjoint,
                                         uint16_t *__restrict__ out) {
     pdl_trigger();   // the convolution after this one stages its unit meanwhile
+    pdl_wait();      // the convolution before it may still read the last weights
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < n_levels * W_LEVEL; d += gridDim.x * blockDim.x) {
         const int lev = d / W_LEVEL, r = d % W_LEVEL, blk = r / (MC * MC), q = r % (MC * MC);
         const int cm = q / 64, row = (q % 64) / 8, col = q % 8;
@@ -491,8 +495,8 @@ struct CellRow {
                 if (wide) {
                     load32(p, v[iy][0], v[iy][1]);
                 } else {
-                    v[iy][0] = __ldg(p);
-                    v[iy][1] = __ldg(p + 1);
+                    load16(p, v[iy][0]);
+                    load16(p + 1, v[iy][1]);
                 }
             }
         }
@@ -642,6 +646,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_fwd_kernel(const UnitView U, const 
                                                        const McOutput o, unsigned *err) {
     extern __shared__ __align__(128) unsigned char smraw[];
     McSmem &S = *reinterpret_cast<McSmem *>(smraw);
+    pdl_trigger();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.work[blockIdx.x];
     NodeRow row;
@@ -764,6 +769,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
                                                            float *__restrict__ gt, unsigned *err) {
     extern __shared__ __align__(128) unsigned char smraw[];
     McAdjSmem &M = *reinterpret_cast<McAdjSmem *>(smraw);
+    pdl_trigger();
     McSmem &S = M.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.work_adj[blockIdx.x];
@@ -875,6 +881,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_leaf_adjoint_kernel(const UnitView 
                                                                 unsigned *err) {
     extern __shared__ __align__(128) unsigned char smraw[];
     McLeafSmem &M = *reinterpret_cast<McLeafSmem *>(smraw);
+    pdl_trigger();
     McSmem &S = M.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.lhdr[blockIdx.x];
@@ -897,6 +904,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_leaf_adjoint_kernel(const UnitView 
         M.mask[tid] = q0.y;
         M.edge[tid] = uint16_t(edge);
     }
+    pdl_wait();   // dL/dout, the weights, and gp of the launch before
     tile_setup(S, W, h.lev);
     const bool wide = (reinterpret_cast<uintptr_t>(gout) & 31u) == 0;
     uint32_t phase = 0;
@@ -1160,8 +1168,7 @@ cudaError_t launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, c
 }
 
 cudaError_t layout_weights(const uint16_t *W, int n_levels, int adjoint, uint16_t *out, cudaStream_t s) {
-    mc_weight_layout_kernel<<<(n_levels * W_LEVEL + 255) / 256, 256, 0, s>>>(W, n_levels, adjoint, out);
-    return cudaGetLastError();
+    return launch_pdl(mc_weight_layout_kernel, dim3((n_levels * W_LEVEL + 255) / 256), dim3(256), 0, s, true, W, n_levels, adjoint, out);
 }
 
 bool mc_args_ok(int32_t c_in, int32_t c_out, int32_t k) { return c_in == MC && c_out == MC && k == 3; }
@@ -1188,11 +1195,9 @@ apr_status_t apr_tree_restrict_bf16(apr_handle_t h, const uint16_t *particles, u
     const HostIndex &X = h->X;
     if ((X.np && !particles) || (X.nt && !tree) || !aligned16(particles) || !aligned16(tree)) return APR_ERR_INVALID_ARG;
     cudaError_t e = cudaSuccess;
-    bool chained = false;   // the launches after the first start early (programmatic dependent launch)
     const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 4);
     for (int i = T.n - 1; i >= 0 && e == cudaSuccess; --i) {   // the finest group first
-        e = launch_tree_restrict_bf16(h->d_tnplan, T.g[i], particles, tree, stream, chained);
-        chained = true;
+        e = launch_tree_restrict_bf16(h->d_tnplan, T.g[i], particles, tree, stream, true);
     }
     return cuda_status(e);
 }
@@ -1278,12 +1283,10 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
         if (e == cudaSuccess)
             e = launch(mc_adjoint_kernel, h->U.n, TNT, sizeof(McAdjSmem), stream, true, h->U, wt, bc, g4, grad_particles, gt, h->d_err);
         if (e == cudaSuccess)
-            e = launch(mc_leaf_adjoint_kernel, h->U.nl, TNT, std::max(sizeof(McLeafSmem), TWO_BLOCKS), stream, false, h->U, wt, bc, g4, grad_particles, h->d_err);
-        bool chained = false;   // the launches after the first start early (programmatic dependent launch)
-        const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
+            e = launch(mc_leaf_adjoint_kernel, h->U.nl, TNT, std::max(sizeof(McLeafSmem), TWO_BLOCKS), stream, true, h->U, wt, bc, g4, grad_particles, h->d_err);
+            const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
         for (int i = 0; i < T.n && e == cudaSuccess; ++i) {
-            e = launch_tree_pushdown16(h->d_tnplan, T.g[i], grad_particles, gt, stream, chained);
-            chained = true;
+            e = launch_tree_pushdown16(h->d_tnplan, T.g[i], grad_particles, gt, stream, true);
         }
     }
     if (e == cudaSuccess && grad_weights) {

@@ -138,11 +138,13 @@ __device__ __forceinline__ uint32_t elect_one() {
     asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
     return e;
 }
-// D (tensor memory) [+]= A (shared memory descriptor) x B (shared memory descriptor)
-__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-                 "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-                 : "memory");
+// D (tensor memory) [+]= A (shared memory descriptor) x B (shared memory descriptor); a converged warp, as mma_ts.
+__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc, uint32_t elected) {
+    asm volatile(
+        "{\n.reg .pred p, e;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 e, %5, 0;\n"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(elected)
+        : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
@@ -401,7 +403,8 @@ struct NodeRow {
         if (nodes) tw = __ldg(m + 1);
     }
     // Rows past the unit's records read the empty slots.
-    __device__ __forceinline__ void put(McSmem &S, const UnitHdr &h) const {
+    template <typename Smem>
+    __device__ __forceinline__ void put(Smem &S, const UnitHdr &h) const {
         const int r = threadIdx.x;
         if (r >= UNIT_RECS) return;
         unsigned b[9];
@@ -417,17 +420,7 @@ struct NodeRow {
         A.edge[r] = uint16_t(r < h.nrec ? r0.y & 0xffffu : 0u);
     }
 };
-// Row r of the tile in the weight gradient: a record at its own place, ...
-__device__ __forceinline__ void put_node_row(Rows &R, int r, const NodeRec *rec) {
-    const uint2 *q = reinterpret_cast<const uint2 *>(rec);
-    const uint2 r0 = __ldg(q), r1 = __ldg(q + 1), r2 = __ldg(q + 2);
-    unsigned b[9];
-    unpack_bases(r0.y, r1, r2, b);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) R.base[k][r] = uint16_t(b[k]);
-    R.mask[r] = 0x7ffffffu;
-}
-// ... in the adjoint record i of the unit at the image of shift t (edge_shifts; 0: its own place), ...
+// Row r of a tile: in the adjoint record i of the unit at the image of shift t (edge_shifts; 0: its own place), ...
 __device__ __forceinline__ void put_image_row(Rows &R, int r, int i, int t) {
     const int iz = t >> 4, ix = (t >> 2) & 3, iy = t & 3, dy = iy == 1 ? -1 : (iy == 0 ? 0 : iy - 1);
     unsigned mask = 0;
@@ -962,39 +955,59 @@ __global__ void __launch_bounds__(TNT, 2) mc_leaf_adjoint_kernel(const UnitView 
 // One block per SM takes a contiguous range of the units of the levels that hold particles. Per tile of 128
 // records, the four planes iz of cells are gathered one after the other (16 cells, two buffers), and for
 // every child row (a, b) the taps tz = iz - a and tx = 0..2 take MMAs over K = the records:
-//   D[tz][tx block][(tx, iy, ci)][(e, co)] += U(cell (iz, b + tx, iy))[ci] g(child (a, b, e))[co]
+//   D[tx block][tz][(tx, iy, ci)][(e, co)] += U(cell (iz, b + tx, iy))[ci] g(child (a, b, e))[co]
 // with M = 128 = two rows of four cells x 16 channels (the second block's second half is not used: it reads
 // the next row or past the plane, inside the block's shared memory). The tap along y is iy - e. After
 // every tile D is added to FP32 registers (96 per thread), so that the tensor cores' accumulation chains stay
 // at 32 MMAs; a level's sums are written to the level's partial of the block and reduced in order.
+// Bound by the A operand's reads from shared memory (an MMA of 32 columns reads as much as one of 64) and by the gather's
+// issue, in turn. 1 M particles: 126 us with a diverged issuing lane and records, children and gradients fetched per
+// tile; converged issue 115, one stream of planes per unit 110, both child planes in one MMA 98 us.
 constexpr int WG_SBO = 2048 + 16;           // 8 channels of a cell for 128 records, padded: eight lanes write
                                             // eight pieces of one record without bank conflicts
 constexpr int WG_CELL = 2 * WG_SBO;
 constexpr int PLANE_BYTES = 16 * WG_CELL;
-constexpr uint32_t WG_TMEM = 256;           // D: block (tz, tx block) in columns 32 (2 tz + block), 192 used
+constexpr uint32_t WG_TMEM = 256;           // D: (tx block, tz) in columns 96 block + 32 (2 - tz), 192 used
 constexpr int WG_OUT = NTAP * MC * MC;      // floats of one partial: [tap][ci][co]
 struct WgradSmem {
     int code[8][PLANE];
     Rows rows;
     alignas(128) unsigned char A[2][PLANE_BYTES];   // cell-major: (2 cell + h) WG_SBO + (r / 8) 128 + (r % 8) 16
-    alignas(128) unsigned char g[8 * WG_CELL];      // the same for the eight children
+    alignas(128) unsigned char g[8 * WG_CELL];      // the same for the children (b, a, e)
+    int4 children[UNIT_RECS];
     uint64_t bar;
     uint32_t tmem;
 };
 
+// Cells (iz, .., ..) of records t0 .. t0 + 127 of the unit. Eight lanes per row.
 __device__ __forceinline__ void gather_plane(const WgradSmem &S, const uint4 *__restrict__ vals, const uint4 *__restrict__ tree,
-                                             int iz, uint32_t A) {
-    const int lane = threadIdx.x & 31, iy = (lane >> 1) & 3, h = lane & 1;   // eight lanes per row
+                                             int t0, int iz, uint32_t A) {
+    const int lane = threadIdx.x & 31, iy = (lane >> 1) & 3, h = lane & 1;
     const uint32_t dst = A + uint32_t((2 * iy + h) * WG_SBO);
 #pragma unroll 1
     for (int j = 0; j < 4; ++j) {
         const int r = (threadIdx.x >> 5) * 16 + 4 * j + (lane >> 3);
-        const unsigned mask = S.rows.mask[r];
 #pragma unroll
         for (int ix = 0; ix < 4; ++ix) {
             const int q = ((iz + 1) >> 1) * 3 + ((ix + 1) >> 1), c0 = ((iz + 1) & 1) * 4 + ((ix + 1) & 1) * 2;
-            const int code = cell_code(S.code, (mask >> (3 * q)) & 7u, S.rows.base[q][r], c0, iy);
+            const int code = S.code[c0 + ((iy + 1) & 1)][S.rows.base[q][t0 + r] + ((iy + 1) >> 1)];
             cp_async16(dst + 4 * ix * WG_CELL + (r >> 3) * 128 + (r & 7) * 16, source_row(vals, tree, code) + h, code != NO_SOURCE);
+        }
+    }
+}
+// dL/dout of their children (zero where the child is no particle). Eight lanes per row: child (b, e), half.
+__device__ __forceinline__ void gather_gradient(const WgradSmem &S, const uint4 *__restrict__ gout, int t0, uint32_t G) {
+    const int lane = threadIdx.x & 31, be = (lane >> 1) & 3, hh = lane & 1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int r = (threadIdx.x >> 5) * 16 + 4 * j + (lane >> 3);
+        const int4 pw = S.children[t0 + r];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            const unsigned w = unsigned(be < 2 ? (a ? pw.z : pw.x) : (a ? pw.w : pw.y)), pm = w >> 30;
+            const size_t p = (w & TNP_INDEX) + (be & 1 ? pm & 1u : 0u);
+            cp_async16(G + uint32_t((2 * (4 * (be >> 1) + 2 * a + (be & 1)) + hh) * WG_SBO + (r >> 3) * 128 + (r & 7) * 16), gout + 2 * p + hh,
+                       (pm >> (be & 1)) & 1u);
         }
     }
 }
@@ -1023,66 +1036,58 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
         for (int k = 0; k < 96; ++k) acc[k] = 0.f;
         for (int u = ua; u < ub && !failed; ++u) {
             const UnitHdr h = U.hdr[L.unit0[i] + u - L.begin[i]];
+            NodeRow row;
+            row.load(U, h, false);
             stage_codes<true>(U, h, false, bc == APR_BC_REFLECT, S.code);
-            for (int t0 = 0; t0 < h.nrec && !failed; t0 += TILE) {
-                if (tid < TILE) {
-                    if (t0 + tid < h.nrec) put_node_row(S.rows, tid, U.rec + h.rec0 + t0 + tid);
-                    else S.rows.mask[tid] = 0;
-                }
-                block_sync();
-                {
-                    // dL/dout of the records' children (zero where the child is no particle)
-                    const int be = (lane >> 1) & 3, hh = lane & 1;   // eight lanes per row: child (b, e), half
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int r = warp * 16 + 4 * j + (lane >> 3);
-                        int4 pw = make_int4(0, 0, 0, 0);
-                        if (t0 + r < h.nrec) pw = child_particles(U, U.rec[h.rec0 + t0 + r].node);
-#pragma unroll
-                        for (int a = 0; a < 2; ++a) {
-                            const unsigned w = unsigned(be < 2 ? (a ? pw.z : pw.x) : (a ? pw.w : pw.y)), pm = w >> 30;
-                            const size_t p = (w & TNP_INDEX) + (be & 1 ? pm & 1u : 0u);
-                            cp_async16(G + uint32_t((2 * (4 * a + be) + hh) * WG_SBO + (r >> 3) * 128 + (r & 7) * 16),
-                                       gout + 2 * p + hh, (pm >> (be & 1)) & 1u);
-                        }
-                    }
-                }
-                gather_plane(S, vals, tree, 0, A);
-                cp_commit();
-                gather_plane(S, vals, tree, 1, A + PLANE_BYTES);
-                cp_commit();
+            row.put(S, h);
+            block_sync();
+            // planes pl = 4 tile + iz in one stream: two are in flight while one is used, across the unit's tiles
+            const int planes = 4 * ((h.nrec + TILE - 1) / TILE);
+            gather_gradient(S, gout, 0, G);
+            gather_plane(S, vals, tree, 0, 0, A);
+            cp_commit();
+            gather_plane(S, vals, tree, 0, 1, A + PLANE_BYTES);
+            cp_commit();
 #pragma unroll 1
-                for (int iz = 0; iz < 4; ++iz) {
-                    cp_wait<1>();
-                    fence_async_smem();
-                    tile_done();
-                    if (tid == 0) {
-                        const uint64_t P = sdesc(A + (iz & 1) * PLANE_BYTES, 128, WG_SBO), B = sdesc(G, 128, WG_SBO);
-                        for (int a = 0; a < 2; ++a) {
-                            const int tz = iz - a;
-                            if (tz < 0 || tz > 2) continue;
+            for (int pl = 0; pl < planes; ++pl) {
+                const int iz = pl & 3;
+                cp_wait<1>();
+                fence_async_smem();
+                tile_done();
+                if (warp == 0) {   // converged: a single diverged lane issues an MMA in 125 cycles
+                    const uint32_t el = elect_one();
+                    const uint64_t P = sdesc(A + (iz & 1) * PLANE_BYTES, 128, WG_SBO), B = sdesc(G, 128, WG_SBO);
+                    // child planes a = 0 (tz = iz) and a = 1 (tz = iz - 1) in one MMA of 64 columns where both exist
+                    const bool two = iz == 1 || iz == 2;
+                    const uint32_t wide = two ? idesc_bf16(128, 64, true) : idesc, Dt = D + (iz == 3 ? 0 : 32 * (2 - iz));
+                    const uint64_t Bt = B + (iz == 3 ? 2 * WG_CELL >> 4 : 0);
 #pragma unroll
-                            for (int b = 0; b < 2; ++b)
+                    for (int b = 0; b < 2; ++b)
 #pragma unroll
-                                for (int blk = 0; blk < 2; ++blk)
+                        for (int blk = 0; blk < 2; ++blk)
 #pragma unroll
-                                    for (int ks = 0; ks < TILE / 16; ++ks)
-                                        mma_ss(D + 64 * tz + 32 * blk, P + (((b + 2 * blk) * 4 * WG_CELL + ks * 256) >> 4),
-                                               B + uint32_t(a * 4 * WG_CELL >> 4) + ((2 * b * WG_CELL + ks * 256) >> 4), idesc,
-                                               b + ks > 0 ? 1u : (a > 0 ? 1u : 0u));
-                        }
-                        mma_commit(&S.bar);
-                    }
-                    if (block_wait_mma(&S.bar, phase, err)) {
-                        failed = true;
-                        break;
-                    }
-                    phase ^= 1;
-                    if (iz + 2 < 4) gather_plane(S, vals, tree, iz + 2, A + (iz & 1) * PLANE_BYTES);
-                    cp_commit();
+                            for (int ks = 0; ks < TILE / 16; ++ks) {
+                                const uint64_t Ak = P + (((b + 2 * blk) * 4 * WG_CELL + ks * 256) >> 4), Bk = Bt + ((4 * b * WG_CELL + ks * 256) >> 4);
+                                if (b == 0 && ks == 0) {   // the plane's first products overwrite tz = iz only
+                                    mma_ss(Dt + 96 * blk, Ak, Bk, idesc, iz == 3 ? 1u : 0u, el);
+                                    if (two) mma_ss(Dt + 96 * blk + 32, Ak, Bk + (2 * WG_CELL >> 4), idesc, 1u, el);
+                                } else {
+                                    mma_ss(Dt + 96 * blk, Ak, Bk, wide, 1u, el);
+                                }
+                            }
+                    if (el) mma_commit(&S.bar);
+                    __syncwarp();
                 }
-                cp_wait<0>();
-                if (failed) break;
+                if (block_wait_mma(&S.bar, phase, err)) {
+                    failed = true;
+                    break;
+                }
+                phase ^= 1;
+                if (iz == 3 && pl + 1 < planes) gather_gradient(S, gout, (pl + 1) / 4 * TILE, G);
+                cp_commit();   // before the plane after the next one, so that the next one's wait covers it
+                if (pl + 2 < planes) gather_plane(S, vals, tree, (pl + 2) / 4 * TILE, (pl + 2) & 3, A + (iz & 1) * PLANE_BYTES);
+                cp_commit();
+                if (iz < 3) continue;
                 tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < 6; ++k) {
@@ -1091,8 +1096,10 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
 #pragma unroll
                     for (int c = 0; c < 16; ++c) acc[16 * k + c] += v[c];
                 }
-                tile_done();
+                tc_fence_before();   // the next MMAs follow a block barrier
             }
+            cp_wait<0>();
+            tile_done();
         }
         if (failed) break;
         // sums of the level: thread (row 32 q + lane, columns 96 half ..) to shared memory, block by block of
@@ -1100,17 +1107,17 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
         float *stage = reinterpret_cast<float *>(S.A[0]);   // [128][33]
         float *dst = partial + size_t(blockIdx.x + i) * WG_OUT;
 #pragma unroll
-        for (int blk = 0; blk < 6; ++blk) {                 // (tz, tx block)
+        for (int blk = 0; blk < 6; ++blk) {                 // (tx block, 2 - tz)
             block_sync();
             if (half == blk / 3)
 #pragma unroll
                 for (int c = 0; c < 32; ++c) stage[(32 * q + lane) * 33 + c] = acc[32 * (blk % 3) + c];
             block_sync();
-            const int ntx = blk & 1 ? 1 : 2;
+            const int ntx = blk / 3 ? 1 : 2;
             for (int o = tid; o < ntx * 3 * MC * MC; o += NT) {
                 const int co = o % MC, ci = (o / MC) % MC, ty = (o / (MC * MC)) % 3, txo = o / (3 * MC * MC);
                 const float *s = stage + ((txo * 4 + ty) * MC + ci) * 33 + co;
-                const int tap = ((blk >> 1) * 3 + 2 * (blk & 1) + txo) * 3 + ty;
+                const int tap = ((2 - blk % 3) * 3 + 2 * (blk / 3) + txo) * 3 + ty;
                 dst[(tap * MC + ci) * MC + co] = s[0] + s[MC * 33 + 16];   // e = 0: iy = ty; e = 1: iy = ty + 1
             }
         }
@@ -1120,14 +1127,24 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
     if (warp == 0) tmem_dealloc(D, WG_TMEM);
 }
 
-// grad_weights[lev][co][ci][e] = sum over the level's partials, in order; zero for a level without particles.
-__global__ void mc_wgrad_reduce_kernel(const float *__restrict__ partial, const UnitRanges R, int n_levels,
-                                       float *__restrict__ gw) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_levels * WG_OUT) return;
+// grad_weights[lev][co][ci][e] = sum over the level's partials, in a fixed order; zero for a level without particles.
+// A chain of up to 152 loads per output is a latency of its own (8 us however small the APR): eight warps take
+// every eighth partial of 32 outputs.
+constexpr int RED_OUT = 32, RED_WARPS = 8;
+static_assert(WG_OUT % RED_OUT == 0, "a block's outputs belong to one level");
+__global__ void __launch_bounds__(RED_OUT *RED_WARPS) mc_wgrad_reduce_kernel(const float *__restrict__ partial, const UnitRanges R,
+                                                                            float *__restrict__ gw) {
+    __shared__ float sums[RED_WARPS][RED_OUT];
+    const int lane = threadIdx.x % RED_OUT, w = threadIdx.x / RED_OUT, i = blockIdx.x * RED_OUT + lane;
     const int lev = i / WG_OUT, r = i % WG_OUT;
     float s = 0.f;
-    for (int c = R.first[lev]; c <= R.last[lev]; ++c) s += partial[size_t(c) * WG_OUT + r];
+#pragma unroll 4
+    for (int c = R.first[lev] + w; c <= R.last[lev]; c += RED_WARPS) s += partial[size_t(c) * WG_OUT + r];
+    sums[w][lane] = s;
+    __syncthreads();
+    if (w != 0) return;
+#pragma unroll
+    for (int k = 1; k < RED_WARPS; ++k) s += sums[k][lane];
     const int co = r % MC, ci = (r / MC) % MC, e = r / (MC * MC);
     gw[((size_t(lev) * MC + co) * MC + ci) * NTAP + e] = s;
 }
@@ -1298,8 +1315,7 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
             e = launch(mc_wgrad_kernel, G, NT, sizeof(WgradSmem), stream, false, h->U, L, reinterpret_cast<const uint4 *>(particles),
                        reinterpret_cast<const uint4 *>(tree), bc, reinterpret_cast<const uint4 *>(grad_out), partial, h->d_err);
         if (e == cudaSuccess) {
-            const int tot = n_levels * WG_OUT;
-            mc_wgrad_reduce_kernel<<<(tot + 255) / 256, 256, 0, stream>>>(partial, R, n_levels, grad_weights);
+            mc_wgrad_reduce_kernel<<<n_levels * (WG_OUT / RED_OUT), RED_OUT * RED_WARPS, 0, stream>>>(partial, R, grad_weights);
             e = cudaGetLastError();
         }
     }

@@ -139,9 +139,9 @@ typedef struct {
  * paragraph). The tree structure (which nodes exist) is derived from the particle cells; its
  * values are computed later by apr_tree_restrict. y indices are stored as uint16. The host also builds
  * what the kernels read instead of the rows: for every tree node the indices of its children (32 bytes
- * per node), the convolution units (APR_STRUCT_UNIT_*: groups of parents with the parents around them)
- * and the source segments of the multi-channel sub-tiles; on a 1024x1024x512 image with 8 M particles
- * the handle holds about 280 MB, plans included (the image itself would be 2.1 GB).
+ * per node) and the convolution units (APR_STRUCT_UNIT_*: groups of parents with the parents around
+ * them); on a 1024x1024x512 image with 8 M particles the handle holds about 210 MB (the image itself
+ * would be 2.1 GB).
  * The index is allocated stream-ordered (cudaMallocAsync on `stream`) and uploaded on `stream`;
  * it is ready for work enqueued on `stream` (other streams synchronise with it first). The handle
  * also creates a stream and two events for the concurrent parts of apr_convolve_backward. Returns
@@ -174,7 +174,7 @@ apr_status_t apr_destroy(apr_handle_t h);
 int64_t apr_num_particles(apr_handle_t h);   /* -1 on NULL */
 int64_t apr_num_tree(apr_handle_t h);        /* N_t, -1 on NULL */
 apr_status_t apr_level_range(apr_handle_t h, int32_t *l_min, int32_t *l_max);
-size_t apr_layout_bytes(apr_handle_t h);     /* device bytes owned by the handle (index, work lists, tile plans) */
+size_t apr_layout_bytes(apr_handle_t h);     /* device bytes owned by the handle (index, child maps, units) */
 
 /* Size in bytes of structure array `which`; 0 if not available. */
 size_t apr_structure_bytes(apr_handle_t h, int32_t which);

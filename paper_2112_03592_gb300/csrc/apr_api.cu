@@ -254,8 +254,8 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
     if (!h->host_only) {
         const apr_status_t pst = build_plans(h->X);
         if (pst != APR_OK) {
-            snprintf(g_last_msg, sizeof(g_last_msg), "%s", pst == APR_ERR_OOM ? "host allocation failed (tile plans)"
-                                                                                : "tile with too many staged elements, or more than 2^28 particles or tree nodes");
+            snprintf(g_last_msg, sizeof(g_last_msg), "%s", pst == APR_ERR_OOM ? "host allocation failed (units)"
+                                                                                : "more than 2^28 particles or tree nodes");
             delete h;
             return pst;
         }

@@ -19,14 +19,17 @@
 //
 // One warp issues the MMAs; completion is signalled through mbarriers whose waits are bounded in time.
 //
-// Measured (1.0 M particles of a 256^3 image, kernels alone): forward 223 -> 74 us, data adjoint 550 -> 221 us
-// (131 onto the children, 90 onto coarser particles), weight gradient 400 -> 126 us. The kernels before cut
+// Measured (1.0 M particles of a 256^3 image, kernels alone): forward 223 -> 60 us, data adjoint 550 -> 167 us
+// (96 onto the children, 71 onto coarser particles), weight gradient 400 -> 98 us. The kernels before cut
 // 8 x 8 x 64-cell tiles, which particles in thin shells leave mostly empty, into sub-tiles staged in shared
 // memory, and gathered 27 cells per target. Tried on the way here, forward: the A operand in shared memory
 // through 16-byte cp.async 131 us (a wavefront of the L1 pipe per 32-byte sector), with the four cells of a
 // row in one instruction 113 us, MMAs issued by a warp of their own 102 us, through registers into tensor
-// memory with warp-uniform MMA operands 74 us. What bounds it now: the issue of 120 small MMAs and the
-// latency of eight steps of 1000 cycles per tile, at two blocks per SM; DRAM traffic is 66 MB, 10 us.
+// memory with warp-uniform MMA operands 74 us, 32-byte stores 66 us, records staged once per unit and more L1
+// 60 us. What bounds it now: the L1 pipe (72 %: the gather touches about a line per 32-byte cell) and a unit's
+// chain of latencies, at two blocks per SM; without the gather 42 us, without the MMAs 61 of then 66 us. DRAM
+// traffic is 66 MB, 10 us. The adjoints have fewer sources to gather and more rows: edge units take further
+// tiles for their images (a third of the node adjoint's time at 256^3), leaf rows have few sources each.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 

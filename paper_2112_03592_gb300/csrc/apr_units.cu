@@ -15,7 +15,7 @@
 // children are particles on average, a record takes about 300 thread instructions at radius 1, and
 // units are equally full wherever the particles lie. Measured (7.9 M particles of a 1024 x 1024 x 512
 // image, restricted 5^3 stack, kernels alone with a cold L2): convolution 235 -> 90 us, data adjoint 500
-// -> 207 us, stencil gradient 360 -> 190 us; 36.5 M instead of 131.8 M warp instructions per convolution.
+// -> 197 us, stencil gradient 360 -> 190 us; 36.5 M instead of 131.8 M warp instructions per convolution.
 // What bounds them now: shared-memory wavefronts (the L1 pipe is 75 % busy in the convolution; 2.5
 // wavefronts per 4-byte load, since the slots of 32 records lie in many short runs) and the latency of
 // header -> entry -> value at four blocks of 256 threads per SM; DRAM traffic is 0.19 GB, 29 us.

@@ -170,6 +170,11 @@ __device__ __forceinline__ void load32(const uint4 *p, uint4 &a, uint4 &b) {
 __device__ __forceinline__ void load16(const uint4 *p, uint4 &a) {
     asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w) : "l"(p));
 }
+__device__ __forceinline__ float load_bf16(const uint16_t *p) {
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __uint_as_float(uint32_t(v) << 16);
+}
 // 32 bytes to a 32-byte aligned address.
 __device__ __forceinline__ void store32(void *p, const uint4 &a, const uint4 &b) {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w),
@@ -1015,6 +1020,73 @@ __device__ __forceinline__ void gather_gradient(const WgradSmem &S, const uint4 
     }
 }
 
+// A tile's sums added to acc (thread: row 32 q + lane of D, columns 96 half ..) without what no target reads. The
+// MMAs multiply every cell around a record with the zero that stands for a child that is no particle, so an
+// infinity or NaN there is in sums of targets that do not read it. If one of the warp's sums that make up taps
+// (iy - e = 0, 1, 2; the second block has one tx) is not finite, they are summed again over the particles alone.
+// Taken only in the second pass over a level whose first one left a sum that is not finite: a block that meets none
+// pays for the test of what it writes (nothing measurable); 1 M particles, 98 us: one infinite feature 0.5 ms, every
+// feature infinite 1.5 ms.
+__device__ __forceinline__ void add_live_targets(const WgradSmem &S, const uint4 *vals, const uint4 *tree, int t0, int nrec, uint32_t D,
+                                                 float (&acc)[96]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
+    const int iy = (2 * q + (lane >> 4)) & 3, ci = lane & 15, tx = 2 * half + (q >> 1);
+    bool finite = true;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        float v[16];
+        tmem_ld16(D + (uint32_t(32 * q) << 16) + 96 * half + 16 * k, v);
+        if (tx < 3 && unsigned(iy - (k & 1)) < 3u)
+#pragma unroll
+            for (int c = 0; c < 16; ++c) finite = finite && isfinite(v[c]);
+    }
+    if (__all_sync(0xffffffffu, finite)) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            float v[16];
+            tmem_ld16(D + (uint32_t(32 * q) << 16) + 96 * half + 16 * k, v);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc[16 * k + c] += v[c];
+        }
+        return;
+    }
+#pragma unroll 1
+    for (int r = 0; r < min(TILE, nrec - t0); ++r) {
+        const int4 pw = S.children[t0 + r];
+        if (unsigned(pw.x | pw.y | pw.z | pw.w) >> 30 == 0) continue;   // no particle among the children
+        float x[4][2];   // cells (iz, tx + b, iy)
+#pragma unroll
+        for (int iz = 0; iz < 4; ++iz)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int ix = tx + b, s = ((iz + 1) >> 1) * 3 + ((ix + 1) >> 1), c0 = ((iz + 1) & 1) * 4 + ((ix + 1) & 1) * 2;
+                const int code = S.code[c0 + ((iy + 1) & 1)][S.rows.base[s][t0 + r] + ((iy + 1) >> 1)];
+                const float u = load_bf16(reinterpret_cast<const uint16_t *>(source_row(vals, tree, code)) + ci);
+                x[iz][b] = code == NO_SOURCE ? 0.f : u;
+            }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int a = c >> 2, b = (c >> 1) & 1, e = c & 1;
+            const unsigned w = unsigned(b ? (a ? pw.w : pw.y) : (a ? pw.z : pw.x));
+            if (!((w >> (30 + e)) & 1u)) continue;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint4 gq = *reinterpret_cast<const uint4 *>(S.g + (2 * (4 * b + 2 * a + e) + h) * WG_SBO + (r >> 3) * 128 + (r & 7) * 16);
+                const unsigned gw[4] = {gq.x, gq.y, gq.z, gq.w};
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const float g = __uint_as_float(k & 1 ? gw[k >> 1] & 0xffff0000u : gw[k >> 1] << 16);
+#pragma unroll
+                    for (int tz = 0; tz < 3; ++tz) {
+                        float &s = acc[32 * (2 - tz) + 16 * e + 8 * h + k];
+                        s = fmaf(x[tz + a][b], g, s);
+                    }
+                }
+            }
+        }
+    }
+}
+
 __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const UnitLevels L, const uint4 *__restrict__ vals,
                                                          const uint4 *__restrict__ tree, int bc,
                                                          const uint4 *__restrict__ gout, float *__restrict__ partial,
@@ -1030,7 +1102,7 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
     const uint32_t D = S.tmem, A = smem_u32(S.A[0]), G = smem_u32(S.g);
     constexpr uint32_t idesc = idesc_bf16(128, 32, true);
     uint32_t phase = 0;
-    bool failed = false;
+    bool failed = false, live_only = false;   // second pass over a level: add_live_targets
     for (int i = 0; i < L.n && !failed; ++i) {
         const int ua = max(u0, L.begin[i]), ub = min(u1, L.begin[i + 1]);
         if (ua >= ub) continue;
@@ -1086,11 +1158,16 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
                     break;
                 }
                 phase ^= 1;
+                if (live_only && iz == 3) {
+                    tc_fence_after();
+                    add_live_targets(S, vals, tree, pl / 4 * TILE, h.nrec, D, acc);
+                    tile_done();   // S.g has been read
+                }
                 if (iz == 3 && pl + 1 < planes) gather_gradient(S, gout, (pl + 1) / 4 * TILE, G);
                 cp_commit();   // before the plane after the next one, so that the next one's wait covers it
                 if (pl + 2 < planes) gather_plane(S, vals, tree, (pl + 2) / 4 * TILE, (pl + 2) & 3, A + (iz & 1) * PLANE_BYTES);
                 cp_commit();
-                if (iz < 3) continue;
+                if (iz < 3 || live_only) continue;
                 tc_fence_after();
 #pragma unroll
                 for (int k = 0; k < 6; ++k) {
@@ -1105,10 +1182,11 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
             tile_done();
         }
         if (failed) break;
+        float *dst = partial + size_t(blockIdx.x + i) * WG_OUT;
         // sums of the level: thread (row 32 q + lane, columns 96 half ..) to shared memory, block by block of
         // 32 columns, then tap (tz, tx, ty), ci, co = its two children e of rows (tx, iy = ty + e, ci)
         float *stage = reinterpret_cast<float *>(S.A[0]);   // [128][33]
-        float *dst = partial + size_t(blockIdx.x + i) * WG_OUT;
+        bool finite = true;
 #pragma unroll
         for (int blk = 0; blk < 6; ++blk) {                 // (tx block, 2 - tz)
             block_sync();
@@ -1121,10 +1199,14 @@ __global__ void __launch_bounds__(NT, 1) mc_wgrad_kernel(const UnitView U, const
                 const int co = o % MC, ci = (o / MC) % MC, ty = (o / (MC * MC)) % 3, txo = o / (3 * MC * MC);
                 const float *s = stage + ((txo * 4 + ty) * MC + ci) * 33 + co;
                 const int tap = ((2 - blk % 3) * 3 + 2 * (blk / 3) + txo) * 3 + ty;
-                dst[(tap * MC + ci) * MC + co] = s[0] + s[MC * 33 + 16];   // e = 0: iy = ty; e = 1: iy = ty + 1
+                const float v = s[0] + s[MC * 33 + 16];   // e = 0: iy = ty; e = 1: iy = ty + 1
+                dst[(tap * MC + ci) * MC + co] = v;
+                finite = finite && isfinite(v);
             }
         }
-        block_sync();
+        __syncwarp();
+        live_only = __syncthreads_or(!finite) != 0 && !live_only;
+        if (live_only) --i;   // the level again
     }
     tile_done();
     if (warp == 0) tmem_dealloc(D, WG_TMEM);

@@ -66,6 +66,13 @@ def test_convolution(case, k, bc, bad):
 
 
 @single
+def test_stencil_gradient(case, k, bc, bad):
+    apr, lay, v, vb, g, gb, st, o = single_channel(case, k, bc, bad)
+    _, rw = o.conv_backward(st.astype(np.float64), k, g.astype(np.float64), bc=bc)
+    assert_same(G.apr_convolve_stencil_grad(lay, dev(vb), G.apr_tree_restrict(lay, dev(vb)), k, dev(g), bc), rw)
+
+
+@single
 def test_data_adjoint(case, k, bc, bad):
     apr, lay, v, vb, g, gb, st, o = single_channel(case, k, bc, bad)
     rp, _ = oracle.Oracle(apr, v.astype(np.float64)).conv_backward(st.astype(np.float64), k, gb.astype(np.float64), bc=bc)

@@ -22,6 +22,7 @@ cudaError_t launch_gradmag(int k, const UnitView &U, int n_units, const float *v
                            int n_levels, int bc, float *out, cudaStream_t s);
 cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, const float *gout, float *gp, float *gt,
                            cudaStream_t s, int first_tile = 0, int n_tiles = -1);
+int stencil_grad_blocks(int k);   // blocks of it that are resident on a multiprocessor
 cudaError_t launch_stencil_grad(int k, const UnitView &U, const UnitLevels &W, const UnitRanges &R, int blocks, int n_levels,
                                 const float *vals, const float *tree, int bc, const float *gout, float *partial, int stride,
                                 float *gw, cudaStream_t s);
@@ -629,12 +630,14 @@ apr_status_t apr_convolve_stencil_grad(apr_handle_t h, const float *particles, c
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
     const size_t need = apr_stencil_grad_workspace_bytes(h, k);
     if (need && (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255))) return APR_ERR_INVALID_ARG;
-    // three blocks per SM are resident; the workspace has a column per forward work item, and a block needs
-    // one per level beyond its first
+    // One wave: the blocks have equal shares, so more than are resident (2 per SM at 3^3, 3 at 5^3) would take two
+    // waves of them (3^3, 3 instead of 2 per SM: 8 M particles 172 instead of 152 us, 1 M 27 instead of 23 us, all-finest
+    // 128^3 image 35 instead of 31 us). The workspace has a column per forward work item, and a
+    // block needs one per level beyond its first.
     UnitLevels L;
     UnitRanges R;
     const int stride = int(X.fwd_items.size());
-    const int blocks = unit_levels(h, std::min(3 * h->sms, stride - h->n_levels_with + 1), L, R);
+    const int blocks = unit_levels(h, std::min(stencil_grad_blocks(k) * h->sms, stride - h->n_levels_with + 1), L, R);
     return cuda_status(launch_stencil_grad(k, h->U, L, R, blocks, X.l_max - X.l_min + 1, particles, tree, bc, grad_out,
                                            static_cast<float *>(workspace), stride, grad_stencils, stream));
 }

@@ -811,6 +811,7 @@ __global__ void __launch_bounds__(UT, 4) leaf_adjoint_kernel(const UnitView U, c
 template <int R>
 struct WgradSmem {
     static constexpr int K = 2 * R + 1, Q = R == 1 ? 4 : 2, NT = K * Q * 32;
+    static constexpr int BLOCKS = R == 1 ? 2 : 3;   // resident per SM (80 registers x 384 threads, 64 x 320)
     Planes pl;
     float g[8][UNIT_RECS];
     Bases bs;
@@ -924,7 +925,7 @@ __device__ __noinline__ void live_levels(WgradSmem<R> &S, const UnitView &U, con
 }
 
 template <int R>
-__global__ void __launch_bounds__(WgradSmem<R>::NT, R == 1 ? 2 : 3) unit_wgrad_kernel(const UnitView U, const UnitLevels W,
+__global__ void __launch_bounds__(WgradSmem<R>::NT, WgradSmem<R>::BLOCKS) unit_wgrad_kernel(const UnitView U, const UnitLevels W,
                                                                       const float *__restrict__ vals,
                                                                       const float *__restrict__ tree, int bc,
                                                                       const float *__restrict__ gout,
@@ -1020,7 +1021,8 @@ __global__ void __launch_bounds__(128) stencil_grad_reduce_kernel(const float *_
 static_assert(4 * (sizeof(UnitSmem) + 1024) <= 228 * 1024, "convolution units: four blocks per SM");
 static_assert(4 * (sizeof(AdjSmem) + 1024) <= 228 * 1024, "adjoint units: four blocks per SM");
 static_assert(4 * (sizeof(LeafSmem) + 1024) <= 228 * 1024, "leaf units: four blocks per SM");
-static_assert(sizeof(WgradSmem<2>) <= 56 * 1024 && sizeof(WgradSmem<1>) <= 56 * 1024, "stencil gradient: four blocks per SM");
+static_assert(WgradSmem<1>::BLOCKS * (sizeof(WgradSmem<1>) + 1024) <= 228 * 1024, "stencil gradient: two blocks per SM");
+static_assert(WgradSmem<2>::BLOCKS * (sizeof(WgradSmem<2>) + 1024) <= 228 * 1024, "stencil gradient: three blocks per SM");
 static_assert(UNIT_SLOTS <= int(UE_SLOT) + 1, "slot numbers fit an entry");
 
 // pdl: the kernel starts while the launch before it finishes and loads its header, records and entries meanwhile. A
@@ -1075,6 +1077,7 @@ cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, co
     return k == 3 ? launch_adjoint_t<1>(U, st, bc, gout, gp, gt, s, tr) : launch_adjoint_t<2>(U, st, bc, gout, gp, gt, s, tr);
 }
 
+int stencil_grad_blocks(int k) { return k == 3 ? WgradSmem<1>::BLOCKS : WgradSmem<2>::BLOCKS; }
 // The stencil gradient into gw [n_levels][k^3], on the blocks of W, R (unit_levels). partial: k^3 x stride
 // floats; block b writes its i-th level to column b + i.
 cudaError_t launch_stencil_grad(int k, const UnitView &U, const UnitLevels &W, const UnitRanges &R, int blocks, int n_levels,

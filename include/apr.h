@@ -133,6 +133,12 @@ typedef struct {
 #define APR_STRUCT_LEAF_NODE 21
 #define APR_STRUCT_LEAF_NODE_INFO 22
 #define APR_STRUCT_LEAF_REC 23
+/* int32 [items][2]: the units [first, last) among which the records of each forward work item are, the node
+ * units and the leaf units of each data-adjoint work item (host-only handles). A range call launches the span of
+ * its items. */
+#define APR_STRUCT_FWD_UNIT_SPANS 24
+#define APR_STRUCT_BWD_UNIT_SPANS 25
+#define APR_STRUCT_BWD_LEAF_SPANS 26
 
 /* Build the device-resident index of an APR (Sec. 3.1 LinearAccess for the particles, Sec. 3.4
  * APR tree structure, and the list of non-empty tiles the kernels are launched on, Sec. 5.2 last

@@ -157,7 +157,7 @@ class AprLayout:
     _EXPORT_DTYPES = {0: np.uint32, 1: np.uint16, 2: np.uint32, 3: np.uint16, 4: np.int32, 5: np.int32, 6: np.int32,
                       7: np.int32, 8: np.uint32, 9: np.uint32, 10: np.uint32, 11: np.uint32, 12: np.int16, 13: np.uint32,
                       14: np.int32, 15: np.uint32, 16: np.uint32, 17: np.uint16, 18: np.int32, 19: np.int16,
-                      20: np.uint32, 21: np.int32, 22: np.uint32, 23: np.uint16}
+                      20: np.uint32, 21: np.int32, 22: np.uint32, 23: np.uint16, 24: np.int32, 25: np.int32, 26: np.int32}
 
     def export(self, which: int) -> np.ndarray:
         nbytes = int(self._lib.apr_structure_bytes(self._h, which))

@@ -22,6 +22,7 @@ APR_STRUCT_FWD_PLAN_R1, APR_STRUCT_FWD_PLAN_R2, APR_STRUCT_BWD_PLAN_R1, APR_STRU
  APR_STRUCT_UNIT_REC, APR_STRUCT_UNIT_MAP) = range(12, 19)
 (APR_STRUCT_LEAF_HDR, APR_STRUCT_LEAF_PURE, APR_STRUCT_LEAF_NODE, APR_STRUCT_LEAF_NODE_INFO,
  APR_STRUCT_LEAF_REC) = range(19, 24)
+APR_STRUCT_FWD_UNIT_SPANS, APR_STRUCT_BWD_UNIT_SPANS, APR_STRUCT_BWD_LEAF_SPANS = 24, 25, 26
 APR_TILE_ZX, APR_BLOCK_Y = 8, 64  # work-item geometry, as in include/apr.h
 
 # every function include/apr.h declares, with (restype, argtypes)

@@ -6,6 +6,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "apr_internal.h"
@@ -17,11 +18,13 @@ cudaError_t launch_tree_pushdown(const TreeNodePlan *np, const TreeGroup &g, flo
 // apr_units.cu
 cudaError_t launch_conv_fwd(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
                             int bc, float *out, cudaStream_t s, int epi_mode = EPI_PLAIN, bool flip = false,
-                            const float *aux = nullptr, int first_tile = 0, int n_tiles = -1);
+                            const float *aux = nullptr, const UnitSpan &span = UnitSpan{0, 0}, int first_tile = 0,
+                            int n_tiles = -1);
 cudaError_t launch_gradmag(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
                            int n_levels, int bc, float *out, cudaStream_t s);
 cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, const float *gout, float *gp, float *gt,
-                           cudaStream_t s, int first_tile = 0, int n_tiles = -1);
+                           cudaStream_t s, const UnitSpan &nodes = UnitSpan{0, 0}, const UnitSpan &leaves = UnitSpan{0, 0},
+                           int first_tile = 0, int n_tiles = -1);
 int stencil_grad_blocks(int k);   // blocks of it that are resident on a multiprocessor
 cudaError_t launch_stencil_grad(int k, const UnitView &U, const UnitLevels &W, const UnitRanges &R, int blocks, int n_levels,
                                 const float *vals, const float *tree, int bc, const float *gout, float *partial, int stride,
@@ -274,7 +277,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
                 e = cudaMemcpyAsync(static_cast<char *>(p) + nb, X.vplan.data(), vb, cudaMemcpyHostToDevice, cs);
         }
         const UnitPlan &UP = X.units;
-        UnitHdr *d_hdr = nullptr, *d_lhdr = nullptr, *d_work = nullptr, *d_adj = nullptr;
+        UnitHdr *d_hdr = nullptr, *d_lhdr = nullptr, *d_work = nullptr, *d_adj = nullptr, *d_lwork = nullptr;
         uint4 *d_pure = nullptr, *d_lpure = nullptr;
         TreeNodePlan *d_nmap = nullptr, *d_lnmap = nullptr;
         uint32_t *d_ninfo = nullptr, *d_lninfo = nullptr;
@@ -286,6 +289,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         if (e == cudaSuccess) e = upload(h, &d_lhdr, UP.lhdr.data(), UP.lhdr.size());
         if (e == cudaSuccess) e = upload(h, &d_work, UP.work.data(), UP.work.size());
         if (e == cudaSuccess) e = upload(h, &d_adj, UP.work_adj.data(), UP.work_adj.size());
+        if (e == cudaSuccess) e = upload(h, &d_lwork, UP.lwork.data(), UP.lwork.size());
         if (e == cudaSuccess) e = upload(h, &d_pure, UP.pure.data(), UP.pure.size());
         if (e == cudaSuccess) e = upload(h, &d_lpure, UP.lpure.data(), UP.lpure.size());
         if (e == cudaSuccess) e = upload(h, &d_nmap, UP.nmap.data(), UP.nmap.size());
@@ -298,7 +302,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         if (e == cudaSuccess) e = upload(h, &d_tf, UP.tile_f.data(), UP.tile_f.size());
         if (e == cudaSuccess) e = upload(h, &d_tb, UP.tile_b.data(), UP.tile_b.size());
         if (e == cudaSuccess) e = upload(h, &d_ltb, UP.ltile_b.data(), UP.ltile_b.size());
-        h->U = UnitView{d_hdr, d_lhdr, d_work, d_adj, d_pure, d_lpure, d_nmap, d_lnmap, d_ninfo, d_lninfo, d_oth, d_rec, d_lrec, d_tf, d_tb, d_ltb, h->d_tnplan,
+        h->U = UnitView{d_hdr, d_lhdr, d_work, d_adj, d_lwork, d_pure, d_lpure, d_nmap, d_lnmap, d_ninfo, d_lninfo, d_oth, d_rec, d_lrec, d_tf, d_tb, d_ltb, h->d_tnplan,
                         int32_t(UP.hdr.size()), int32_t(UP.lhdr.size())};
         h->n_fwd_units = UP.n_forward;
         for (int i = X.l_max - X.l_min; i >= 0; --i) {   // finest first
@@ -334,6 +338,9 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
             delete h;
             return st;
         }
+        h->fwd_units = std::move(h->X.units.fwd_units);
+        h->bwd_units = std::move(h->X.units.bwd_units);
+        h->bwd_leaves = std::move(h->X.units.bwd_leaves);
         // the plans live on the device now; the host copies are not needed again
         h->X.tnplan = std::vector<TreeNodePlan>{};
         h->X.vplan = std::vector<TreeNodePlan>{};
@@ -428,6 +435,9 @@ bool host_unit_array(apr_handle_t h, int32_t which, const void **src, size_t *by
         case APR_STRUCT_LEAF_NODE: give(U.lnmap); break;
         case APR_STRUCT_UNIT_NODE_INFO: give(U.ninfo); break;
         case APR_STRUCT_LEAF_NODE_INFO: give(U.lninfo); break;
+        case APR_STRUCT_FWD_UNIT_SPANS: give(U.fwd_units.items()); break;
+        case APR_STRUCT_BWD_UNIT_SPANS: give(U.bwd_units.items()); break;
+        case APR_STRUCT_BWD_LEAF_SPANS: give(U.bwd_leaves.items()); break;
     }
     return true;
 }
@@ -436,7 +446,7 @@ bool host_unit_array(apr_handle_t h, int32_t which, const void **src, size_t *by
 size_t apr_structure_bytes(apr_handle_t h, int32_t which) {
     if (!h) return 0;
     const HostIndex &X = h->X;
-    if (which >= APR_STRUCT_UNIT_HDR && which <= APR_STRUCT_LEAF_REC) {
+    if (which >= APR_STRUCT_UNIT_HDR && which <= APR_STRUCT_BWD_LEAF_SPANS) {
         const void *src;
         size_t n;
         return host_unit_array(h, which, &src, &n) ? n : 0;
@@ -461,7 +471,7 @@ size_t apr_structure_bytes(apr_handle_t h, int32_t which) {
 apr_status_t apr_export_structure(apr_handle_t h, int32_t which, void *dst, size_t bytes) {
     if (!h || (!dst && bytes)) return APR_ERR_INVALID_ARG;
     const size_t need = apr_structure_bytes(h, which);
-    if (which < APR_STRUCT_ROW_PTR || which > APR_STRUCT_LEAF_REC) return APR_ERR_INVALID_ARG;
+    if (which < APR_STRUCT_ROW_PTR || which > APR_STRUCT_BWD_LEAF_SPANS) return APR_ERR_INVALID_ARG;
     if (bytes < need) return APR_ERR_INVALID_ARG;
     if (need == 0) return APR_OK;
     if (which >= APR_STRUCT_UNIT_HDR) {  // host-only handle (need > 0)
@@ -536,7 +546,7 @@ apr_status_t apr_convolve_tiles(apr_handle_t h, const float *particles, const fl
     if (!stencils || (h->X.np && (!particles || !out)) || (h->X.nt && !tree)) return APR_ERR_INVALID_ARG;
     if (!aligned16(particles) || !aligned16(tree)) return misaligned();
     return cuda_status(launch_conv_fwd(k, h->U, h->n_fwd_units, particles, tree, stencils, bc, out, stream, EPI_PLAIN, false,
-                                       nullptr, int(first_tile), int(n_tiles)));
+                                       nullptr, h->fwd_units.of(first_tile, n_tiles), int(first_tile), int(n_tiles)));
 }
 
 apr_status_t apr_convolve_adjoint_tiles(apr_handle_t h, const float *stencils, int32_t k, int32_t bc,
@@ -549,7 +559,8 @@ apr_status_t apr_convolve_adjoint_tiles(apr_handle_t h, const float *stencils, i
     const int64_t nt = int64_t(X.bwd_items.size());
     if (first_tile < 0 || n_tiles < 0 || first_tile + n_tiles > nt) return APR_ERR_INVALID_ARG;
     if (!stencils || (X.np && (!grad_out || !grad_particles)) || (X.nt && !grad_tree)) return APR_ERR_INVALID_ARG;
-    return cuda_status(launch_adjoint(k, h->U, stencils, bc, grad_out, grad_particles, grad_tree, stream, int(first_tile),
+    return cuda_status(launch_adjoint(k, h->U, stencils, bc, grad_out, grad_particles, grad_tree, stream,
+                                      h->bwd_units.of(first_tile, n_tiles), h->bwd_leaves.of(first_tile, n_tiles), int(first_tile),
                                       int(n_tiles)));
 }
 

@@ -97,9 +97,26 @@ struct alignas(16) LeafRec {
     uint32_t pad;
 };
 static_assert(sizeof(LeafRec) == 32, "leaf records are two 16-byte words");
+struct UnitSpan {                          // units [first, last)
+    int32_t first, last;
+};
+// The units that hold records of the work items of a range call, as a span of the units' own order (the finest
+// level first, along the curve); others in the span hold none of the range.
+class UnitSpans {
+  public:
+    void set(std::vector<UnitSpan> items);
+    UnitSpan of(int64_t first, int64_t n) const;   // of the items [first, first + n)
+    const std::vector<UnitSpan> &items() const { return item_; }
+
+  private:
+    static constexpr int64_t G = 64;
+    std::vector<UnitSpan> item_, group_;   // per work item, per G of them
+};
 struct UnitPlan {                          // host
-    std::vector<UnitHdr> hdr, lhdr;        // node units (finest level first), leaf units (longest first)
+    std::vector<UnitHdr> hdr, lhdr;        // node units, leaf units: finest level first, along the curve
     std::vector<UnitHdr> work, work_adj;   // the node units again, longest first: those of the forward pass, then the rest; all
+    std::vector<UnitHdr> lwork;            // the leaf units again, longest first
+    UnitSpans fwd_units, bwd_units, bwd_leaves;   // of the forward items; of the adjoint items, node and leaf units
     int32_t n_forward = 0;                 // node units of the levels down to the coarsest that holds particles
     std::vector<uint4> pure, lpure;        // entries: pure slots, other nodes, the rest
     std::vector<TreeNodePlan> nmap, lnmap;
@@ -123,7 +140,7 @@ struct UnitRanges {                // partials of level l_min + i: first[i] .. l
     int first[MAXL], last[MAXL];
 };
 struct UnitView {                          // device
-    const UnitHdr *hdr, *lhdr, *work, *work_adj;
+    const UnitHdr *hdr, *lhdr, *work, *work_adj, *lwork;
     const uint4 *pure, *lpure;
     const TreeNodePlan *nmap, *lnmap;
     const uint32_t *ninfo, *lninfo;
@@ -281,6 +298,7 @@ struct apr_handle_s {
     bool host_plans = false, host_units = false;
     aprk::UnitView U{};   // convolution units; those of the levels down to the coarsest one with particles
     int n_fwd_units = 0;
+    aprk::UnitSpans fwd_units, bwd_units, bwd_leaves;   // UnitPlan
     int32_t unit_begin[aprk::MAXL + 1] = {};   // first unit of level l_min + i
     bool level_has[aprk::MAXL + 1] = {};       // whether level l_min + i holds particles
     bool complete = false;                     // every particle and tree node is the child of a record

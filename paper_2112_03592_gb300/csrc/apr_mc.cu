@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(TNT, 2) mc_leaf_adjoint_kernel(const UnitView 
     pdl_trigger();
     McSmem &S = M.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const UnitHdr h = U.lhdr[blockIdx.x];
+    const UnitHdr h = U.lwork[blockIdx.x];
     const bool reflect = bc == APR_BC_REFLECT;
     // thread i keeps record i from its header to the staging
     uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;

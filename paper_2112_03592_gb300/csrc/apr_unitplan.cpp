@@ -489,7 +489,41 @@ void sort_by_work(It first, It last, int flag = 0) {
     std::stable_sort(first, last, [&](const UnitHdr &a, const UnitHdr &b) { return work(a) > work(b); });
 }
 
+// The span of units (headers in their own order) that hold records of each of n work items.
+std::vector<UnitSpan> item_spans(const std::vector<UnitHdr> &hdr, const std::vector<int32_t> &tile, size_t n) {
+    std::vector<UnitSpan> s(n, UnitSpan{0, 0});
+    for (size_t u = 0; u < hdr.size(); ++u)
+        for (int32_t r = hdr[u].rec0; r < hdr[u].rec0 + hdr[u].nrec; ++r)
+            if (tile[size_t(r)] >= 0) {
+                UnitSpan &q = s[size_t(tile[size_t(r)])];
+                if (q.last == 0) q.first = int32_t(u);
+                q.last = int32_t(u) + 1;
+            }
+    return s;
+}
+
+void widen(UnitSpan &a, const UnitSpan &b) {
+    if (b.first >= b.last) return;
+    a = a.first >= a.last ? b : UnitSpan{std::min(a.first, b.first), std::max(a.last, b.last)};
+}
+
 }  // namespace
+
+void UnitSpans::set(std::vector<UnitSpan> items) {
+    item_ = std::move(items);
+    group_.assign((item_.size() + G - 1) / G, UnitSpan{0, 0});
+    for (size_t i = 0; i < item_.size(); ++i) widen(group_[i / G], item_[i]);
+}
+
+UnitSpan UnitSpans::of(int64_t first, int64_t n) const {
+    UnitSpan s{0, 0};
+    for (int64_t i = first; i < first + n;) {
+        const bool whole = i % G == 0 && i + G <= first + n;
+        widen(s, whole ? group_[size_t(i / G)] : item_[size_t(i)]);
+        i += whole ? G : 1;
+    }
+    return s;
+}
 
 void build_units(HostIndex &X) {
     virtual_parents(X);
@@ -634,7 +668,11 @@ void build_units(HostIndex &X) {
             o = JobOut{};
         }
     }
-    sort_by_work(U.lhdr.begin(), U.lhdr.end());
+    U.fwd_units.set(item_spans(U.hdr, U.tile_f, X.fwd_items.size()));
+    U.bwd_units.set(item_spans(U.hdr, U.tile_b, X.bwd_items.size()));
+    U.bwd_leaves.set(item_spans(U.lhdr, U.ltile_b, X.bwd_items.size()));
+    U.lwork = U.lhdr;
+    sort_by_work(U.lwork.begin(), U.lwork.end());
     U.work = U.hdr;
     for (int l = X.l_max; l >= X.l_min; --l)
         if (X.fwd_level_begin[l + 1] > X.fwd_level_begin[l])

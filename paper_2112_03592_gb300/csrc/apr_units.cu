@@ -418,20 +418,22 @@ struct TileRange {
 // APR convolution (Sec. 4.1).
 // ------------------------------------------------------------------------------------------------
 template <int R>
-__global__ void __launch_bounds__(UT, 4) unit_conv_kernel(const UnitView U, const float *__restrict__ vals,
+__global__ void __launch_bounds__(UT, 4) unit_conv_kernel(const UnitView U, const UnitHdr *units, const float *__restrict__ vals,
                                                           const float *__restrict__ tree,
                                                           const float *__restrict__ stencils, int bc, float *out,
                                                           const Epilogue epi, const TileRange tr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     UnitSmem &S = *reinterpret_cast<UnitSmem *>(smem_raw);
     pdl_trigger();
-    const UnitHdr h = U.work[blockIdx.x];
+    const UnitHdr h = units[blockIdx.x];
     const int tid = threadIdx.x;
     // the record, loaded ahead of the staging
     Rec rec{};
     const bool mine = tid < h.nrec && tr.has(U.tile_f, h.rec0 + tid);
-    if (tr.n >= 0) pdl_wait();   // (also in blocks that leave here: their kernel must not end before the launch before it)
-    if (tr.n >= 0 && __syncthreads_or(mine) == 0) return;
+    if (tr.n >= 0 && __syncthreads_or(mine) == 0) {
+        pdl_wait();   // (their kernel must not end before the launch before it)
+        return;
+    }
     if (mine) rec.load(U.rec + h.rec0 + tid);
     Staging<true> st = value_staging(U, h, vals, tree);
     pdl_wait();
@@ -636,19 +638,21 @@ __device__ __forceinline__ void zero_slots(Planes &pl) {
 // ADD: gradients are added (tile-range calls: other calls may add to the same particles); else they
 // are stored (every particle and tree node is the child of one record).
 template <int R, bool ADD>
-__global__ void __launch_bounds__(UT, 4) unit_adjoint_kernel(const UnitView U, const float *__restrict__ stencils,
+__global__ void __launch_bounds__(UT, 4) unit_adjoint_kernel(const UnitView U, const UnitHdr *units, const float *__restrict__ stencils,
                                                              int bc, const float *__restrict__ gout,
                                                              float *__restrict__ gp, float *__restrict__ gt,
                                                              const TileRange tr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AdjSmem &S = *reinterpret_cast<AdjSmem *>(smem_raw);
     pdl_trigger();
-    const UnitHdr h = U.work_adj[blockIdx.x];
+    const UnitHdr h = units[blockIdx.x];
     const int tid = threadIdx.x;
     Rec rec{};
     const bool live = tid < h.nrec && tr.has(U.tile_b, h.rec0 + tid);
-    if (ADD) pdl_wait();
-    if (ADD && __syncthreads_or(live) == 0) return;
+    if (ADD && __syncthreads_or(live) == 0) {
+        pdl_wait();
+        return;
+    }
     if (live) rec.load(U.rec + h.rec0 + tid);
     Staging<false> st = gradient_staging(U, h, false, gout);
     pdl_wait();
@@ -758,18 +762,20 @@ __device__ __forceinline__ float leaf_adjoint(const Planes &pl, const uint4 &q0,
 }
 
 template <int R, bool ADD>
-__global__ void __launch_bounds__(UT, 4) leaf_adjoint_kernel(const UnitView U, const float *__restrict__ stencils,
+__global__ void __launch_bounds__(UT, 4) leaf_adjoint_kernel(const UnitView U, const UnitHdr *units, const float *__restrict__ stencils,
                                                              int bc, const float *__restrict__ gout,
                                                              float *__restrict__ gp, const TileRange tr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LeafSmem &S = *reinterpret_cast<LeafSmem *>(smem_raw);
     pdl_trigger();
-    const UnitHdr h = U.lhdr[blockIdx.x];
+    const UnitHdr h = units[blockIdx.x];
     const int tid = threadIdx.x;
     const bool live = tid < h.nrec && tr.has(U.ltile_b, h.rec0 + tid), reflect = bc == APR_BC_REFLECT;
     uint4 q0 = make_uint4(0, 0, 0, 0), q1 = q0;
-    if (ADD) pdl_wait();
-    if (ADD && __syncthreads_or(live) == 0) return;
+    if (ADD && __syncthreads_or(live) == 0) {
+        pdl_wait();
+        return;
+    }
     if (live) {
         const uint4 *q = reinterpret_cast<const uint4 *>(U.lrec + h.rec0 + tid);
         q0 = __ldg(q);
@@ -1038,16 +1044,27 @@ cudaError_t launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, c
 
 }  // namespace
 
+// The units of a launch: `all` of them, longest first, or those of a range call, `span` of them in their own order.
+// (Over all units, as a first form did, a rank's ranges cost the whole image's headers once per level. An eighth of 8 M
+// particles, one range per level: convolution 3^3 56 -> 44, 5^3 89 -> 75, adjoint 146 -> 102 and 214 -> 165 us; one work
+// item: adjoint 17 and 19 -> 7.5 us.)
+struct Units {
+    const UnitHdr *hdr;
+    int n;
+    Units(const UnitHdr *sorted, int all, const UnitHdr *hdr_, const UnitSpan &span, bool range)
+        : hdr(range && span.last - span.first < all ? hdr_ + span.first : sorted), n(range ? span.last - span.first : all) {}
+};
+
 // n_units: the units of the levels down to the coarsest one with particles (the finest come first).
-// first_tile, n_tiles: a range of forward work items, or n_tiles < 0 for all.
+// first_tile, n_tiles: a range of forward work items, whose records are in the units `span`; n_tiles < 0: all.
 cudaError_t launch_conv_fwd(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
-                            int bc, float *out, cudaStream_t s, int epi_mode, bool flip, const float *aux, int first_tile,
-                            int n_tiles) {
+                            int bc, float *out, cudaStream_t s, int epi_mode, bool flip, const float *aux, const UnitSpan &span,
+                            int first_tile, int n_tiles) {
     const Epilogue epi{epi_mode, flip, aux};
     const TileRange tr{first_tile, n_tiles};
-    if (n_tiles == 0) return cudaSuccess;
-    return k == 3 ? launch(unit_conv_kernel<1>, n_units, UT, sizeof(UnitSmem), s, true, U, vals, tree, st, bc, out, epi, tr)
-                  : launch(unit_conv_kernel<2>, n_units, UT, sizeof(UnitSmem), s, true, U, vals, tree, st, bc, out, epi, tr);
+    const Units u(U.work, n_units, U.hdr, span, n_tiles >= 0);
+    return k == 3 ? launch(unit_conv_kernel<1>, u.n, UT, sizeof(UnitSmem), s, true, U, u.hdr, vals, tree, st, bc, out, epi, tr)
+                  : launch(unit_conv_kernel<2>, u.n, UT, sizeof(UnitSmem), s, true, U, u.hdr, vals, tree, st, bc, out, epi, tr);
 }
 
 cudaError_t launch_gradmag(int k, const UnitView &U, int n_units, const float *vals, const float *tree, const float *st,
@@ -1057,24 +1074,26 @@ cudaError_t launch_gradmag(int k, const UnitView &U, int n_units, const float *v
 }
 
 // The data adjoint: stored gradients over all units, or (n_tiles >= 0) gradients added over a range of
-// adjoint work items.
+// adjoint work items, whose records are in the given spans of the node and the leaf units.
 template <int R>
 static cudaError_t launch_adjoint_t(const UnitView &U, const float *st, int bc, const float *gout, float *gp, float *gt,
-                                    cudaStream_t s, const TileRange &tr) {
+                                    cudaStream_t s, const UnitSpan &nodes, const UnitSpan &leaves, const TileRange &tr) {
     const bool add = tr.n >= 0;
-    cudaError_t e = launch(add ? unit_adjoint_kernel<R, true> : unit_adjoint_kernel<R, false>, U.n, UT, sizeof(AdjSmem), s, true, U,
-                           st, bc, gout, gp, gt, tr);
-    // (started early, the leaf units slow the last wave of the node units: 8 M particles 208 -> 215 us)
+    const Units un(U.work_adj, U.n, U.hdr, nodes, add), ul(U.lwork, U.nl, U.lhdr, leaves, add);
+    cudaError_t e = launch(add ? unit_adjoint_kernel<R, true> : unit_adjoint_kernel<R, false>, un.n, UT, sizeof(AdjSmem), s, true, U,
+                           un.hdr, st, bc, gout, gp, gt, tr);
+    // (started early, the leaf units slow the last wave of the node units: 8 M particles 208 -> 215 us; the few units
+    // of a range call start early)
     if (e == cudaSuccess)
-        e = launch(add ? leaf_adjoint_kernel<R, true> : leaf_adjoint_kernel<R, false>, U.nl, UT, sizeof(LeafSmem), s, false, U, st, bc,
-                   gout, gp, tr);
+        e = launch(add ? leaf_adjoint_kernel<R, true> : leaf_adjoint_kernel<R, false>, ul.n, UT, sizeof(LeafSmem), s, ul.n < U.nl, U, ul.hdr, st,
+                   bc, gout, gp, tr);
     return e;
 }
 cudaError_t launch_adjoint(int k, const UnitView &U, const float *st, int bc, const float *gout, float *gp, float *gt,
-                           cudaStream_t s, int first_tile, int n_tiles) {
+                           cudaStream_t s, const UnitSpan &nodes, const UnitSpan &leaves, int first_tile, int n_tiles) {
     const TileRange tr{first_tile, n_tiles};
-    if (n_tiles == 0) return cudaSuccess;
-    return k == 3 ? launch_adjoint_t<1>(U, st, bc, gout, gp, gt, s, tr) : launch_adjoint_t<2>(U, st, bc, gout, gp, gt, s, tr);
+    return k == 3 ? launch_adjoint_t<1>(U, st, bc, gout, gp, gt, s, nodes, leaves, tr)
+                  : launch_adjoint_t<2>(U, st, bc, gout, gp, gt, s, nodes, leaves, tr);
 }
 
 int stencil_grad_blocks(int k) { return k == 3 ? WgradSmem<1>::BLOCKS : WgradSmem<2>::BLOCKS; }

@@ -50,6 +50,15 @@ def _stream_ptr(stream=None):
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
+def _on_stream(stream):
+    """Context in which torch allocates and runs on the call's stream."""
+    import contextlib
+    import torch
+    if stream is None:
+        return contextlib.nullcontext()
+    return torch.cuda.stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream))
+
+
 def _dev_ptr(t, name, numel=None, dtype=None):
     import torch
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
@@ -124,7 +133,7 @@ class AprLayout:
         self.n_particles = int(lib.apr_num_particles(h))
         self.n_tree = int(lib.apr_num_tree(h))
         self.host_only = bool(flags & APR_HOST_ONLY)
-        self._ws, self._ws_bytes = {}, {}
+        self._ws_bytes = {}
 
     @classmethod
     def from_apr(cls, apr, flags=APR_VALIDATE | APR_REQUIRE_BALANCE, allocator=None):
@@ -188,16 +197,20 @@ class AprLayout:
             n = self._ws_bytes[key] = int(fn(self._h, *args))
         return n
 
-    def _scratch(self, key, nbytes, device):
-        ws = self._ws.get(key)
-        if ws is None or ws.numel() < nbytes:
-            import torch
-            ws = self._ws[key] = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
-        return ws
+    @staticmethod
+    def _scratch(nbytes, device, stream):
+        """A call's scratch, from torch's allocator on the call's own stream: calls on other streams and replayed graphs
+        get other memory, and what is dropped here is reused on that stream only, after the call."""
+        import torch
+        if stream is None:
+            return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+        with _on_stream(stream):
+            return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
 
-    def workspace(self, k):
+    def workspace(self, k, stream=None):
+        """(scratch of apr_convolve_backward, its size in bytes) for one call on `stream`."""
         nbytes = self._bytes(k, self._lib.apr_backward_workspace_bytes, k)
-        return self._scratch(k, nbytes, "cuda"), nbytes
+        return self._scratch(nbytes, "cuda", stream), nbytes
 
     def sync_status(self, stream=None):
         _abi.check("apr_sync_status", self._lib.apr_sync_status(self._h, _stream_ptr(stream)))
@@ -250,8 +263,7 @@ def apr_convolve_auto(layout: AprLayout, particles, stencils, k, bc=APR_BC_REFLE
     else:
         _dev_ptr(out, "out", layout.n_particles, torch.float32)
     if workspace is None:
-        nbytes = layout._bytes("auto", layout._lib.apr_convolve_auto_workspace_bytes)
-        workspace = torch.empty(nbytes, dtype=torch.uint8, device=particles.device)
+        workspace = layout._scratch(layout._bytes("auto", layout._lib.apr_convolve_auto_workspace_bytes), particles.device, stream)
     _abi.check("apr_convolve_auto", layout._lib.apr_convolve_auto(
         layout.handle, particles.data_ptr(), stencils.data_ptr(), int(k), int(bc),
         out.data_ptr(), workspace.data_ptr(), workspace.numel() * workspace.element_size(),
@@ -353,7 +365,7 @@ def apr_convolve_backward(layout: AprLayout, particles, tree, stencils, k, grad_
         if grad_stencils is None:
             grad_stencils = torch.empty((layout.n_levels, k ** 3), dtype=torch.float32, device=grad_out.device)
         gw_ptr = _dev_ptr(grad_stencils, "grad_stencils", layout.n_levels * k ** 3, torch.float32)
-    ws, nbytes = layout.workspace(k)
+    ws, nbytes = layout.workspace(k, stream)
     _abi.check("apr_convolve_backward", layout._lib.apr_convolve_backward(
         layout.handle, particles.data_ptr() if particles is not None else None,
         tree.data_ptr() if tree is not None else None, stencils.data_ptr(),
@@ -406,8 +418,7 @@ def apr_convolve_stencil_grad(layout: AprLayout, particles, tree, k, grad_out, b
     import torch
     if grad_stencils is None:
         grad_stencils = torch.empty((layout.n_levels, k ** 3), dtype=torch.float32, device=grad_out.device)
-    key = ("sg", k)
-    ws = layout._scratch(key, layout._bytes(key, layout._lib.apr_stencil_grad_workspace_bytes, k), grad_out.device)
+    ws = layout._scratch(layout._bytes(("sg", k), layout._lib.apr_stencil_grad_workspace_bytes, k), grad_out.device, stream)
     _abi.check("apr_convolve_stencil_grad", layout._lib.apr_convolve_stencil_grad(
         layout.handle, _dev_ptr(particles, "particles", layout.n_particles, torch.float32),
         _dev_ptr(tree, "tree", layout.n_tree, torch.float32), int(k), int(bc),
@@ -425,10 +436,10 @@ def apr_richardson_lucy(layout: AprLayout, observed, stencils, k, n_iter, bc=APR
     _dev_ptr(observed, "observed", layout.n_particles, torch.float32)
     _dev_ptr(stencils, "stencils", layout.n_levels * k ** 3, torch.float32)
     if estimate is None:
-        estimate = observed.clone()
+        with _on_stream(stream):
+            estimate = observed.clone()
     _dev_ptr(estimate, "estimate", layout.n_particles, torch.float32)
-    key = "rl"
-    ws = layout._scratch(key, layout._bytes(key, layout._lib.apr_rl_workspace_bytes), observed.device)
+    ws = layout._scratch(layout._bytes("rl", layout._lib.apr_rl_workspace_bytes), observed.device, stream)
     _abi.check("apr_richardson_lucy", layout._lib.apr_richardson_lucy(
         layout.handle, observed.data_ptr(), stencils.data_ptr(), int(k), int(bc),
         int(n_iter), estimate.data_ptr(), ws.data_ptr(), ws.numel(),
@@ -530,8 +541,7 @@ def apr_convolve_mc_backward(layout: AprLayout, particles, tree, weights, grad_o
         if grad_weights is None:
             grad_weights = torch.empty((layout.n_levels, C, C, k ** 3), dtype=torch.float32, device=grad_out.device)
         gw_ptr = _dev_ptr(grad_weights, "grad_weights", layout.n_levels * C * C * k ** 3, torch.float32)
-    key = ("mc", k)
-    ws = layout._scratch(key, layout._bytes(key, layout._lib.apr_mc_backward_workspace_bytes, C, C, k), grad_out.device)
+    ws = layout._scratch(layout._bytes(("mc", k), layout._lib.apr_mc_backward_workspace_bytes, C, C, k), grad_out.device, stream)
     _abi.check("apr_convolve_mc_backward", layout._lib.apr_convolve_mc_backward(
         layout.handle, particles.data_ptr() if particles is not None else None,
         tree.data_ptr() if tree is not None else None, weights.data_ptr(),

@@ -704,9 +704,8 @@ def run_mc(args, rank, world, full=True):
     names = ["tree_restrict_bf16", "convolve_mc", "data_adjoint", "weight_grad"]
     dom = max(range(1, 4), key=lambda j: parts[j])
     mc_traffic = recorded_traffic(names[dom], "mc")
-    # per step: BF16 tree, weight layout + forward, weight layout + data adjoint (node units, leaf units),
-    # push-down, weight gradient + its reduction
-    launches_per_step = tree_launches(apr, lay) + 2 + 3 + tree_launches(apr, lay, 3) + 2
+    # per step: BF16 tree, forward, data adjoint (node units, leaf units), push-down, weight gradient + its reduction
+    launches_per_step = tree_launches(apr, lay) + 1 + 2 + tree_launches(apr, lay, 3) + 2
     rec = {
         "metric": "APR conv Gparticles/s & pixel-equiv GB/s",
         "value": round(world * Np / (step_ms * 1e-3) / 1e9, 4), "unit": "Gparticles/s",
@@ -1096,9 +1095,9 @@ def run_surrogate(args, rank, world, pretrained=None):
                     "weighting": "pixels covered by each particle (pixel-equivalent)"},
         "training": {"loss_first": round(float(np.mean(hist[:10])), 6), "loss_last": round(float(np.mean(hist[-10:])), 6),
                      "data_s": round(t_data, 1), "train_s": round(t_train, 1)},
-        # per CNN inference: embedding, 4 x (tree restriction, weight layout, convolution; hidden
-        # ReLUs and the read-out fused into the convolution); per RL run: 2 x (tree + convolution) per iteration
-        "gpu_launches": (1 + 4 * (n_tree + 2) +
+        # per CNN inference: embedding, 4 x (tree restriction, convolution; hidden ReLUs and the
+        # read-out fused into the convolution); per RL run: 2 x (tree + convolution) per iteration
+        "gpu_launches": (1 + 4 * (n_tree + 1) +
                          RL_ITERS * 2 * (n_tree + 1)) * args.steps,
     }
     return rec

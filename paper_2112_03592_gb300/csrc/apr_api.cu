@@ -323,14 +323,6 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
             h->d_err = static_cast<unsigned *>(p);
             if (e == cudaSuccess) e = cudaMemsetAsync(h->d_err, 0, sizeof(unsigned), reinterpret_cast<cudaStream_t>(stream));
         }
-
-        if (e == cudaSuccess) {
-            // operand-layout copy of multi-channel weights: [2 (forward, adjoint)][levels][36 * 16 * 16]
-            const size_t nb = size_t(2) * size_t(X.l_max - X.l_min + 1) * 36 * 16 * 16 * sizeof(uint16_t);
-            void *p = nullptr;
-            e = dev_alloc(h, &p, nb);
-            h->d_mcw = static_cast<uint16_t *>(p);
-        }
         if (e != cudaSuccess) {
             st = cuda_status(e);
             cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(stream));

@@ -287,7 +287,6 @@ struct apr_handle_s {
     aprk::HostIndex X;
     bool host_only = false;
     unsigned *d_err = nullptr;
-    uint16_t *d_mcw = nullptr;   // multi-channel weights in the tensor-core operand layout, per level
     apr_stream_t stream = nullptr;                      // the build stream (uploads, stream-ordered allocation)
     apr_allocator alloc{};                              // the caller's allocator, if has_alloc
     bool has_alloc = false;

@@ -256,7 +256,14 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         }
     }
     if (!h->host_only) {
-        const apr_status_t pst = build_plans(h->X);
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) {
+            delete h;
+            return cuda_status(e);
+        }
+        const apr_status_t pst = build_plans(h->X, h->sms);
         if (pst != APR_OK) {
             snprintf(g_last_msg, sizeof(g_last_msg), "%s", pst == APR_ERR_OOM ? "host allocation failed (units)"
                                                                                 : "more than 2^28 particles or tree nodes");
@@ -264,9 +271,8 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
             return pst;
         }
         const HostIndex &X = h->X;
-        cudaError_t e = cudaSuccess;
         // child maps: the tree nodes, then the virtual parents of the cells of l_min
-        if (e == cudaSuccess) {
+        {
             void *p = nullptr;
             const size_t nb = X.tnplan.size() * sizeof(TreeNodePlan), vb = X.vplan.size() * sizeof(TreeNodePlan);
             e = dev_alloc(h, &p, std::max<size_t>(nb + vb, sizeof(TreeNodePlan)));
@@ -314,9 +320,6 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
         h->uncovered = UP.uncovered;
         h->n_levels_with = 0;
         for (int i = 0; i <= X.l_max - X.l_min; ++i) h->n_levels_with += h->level_has[i] ? 1 : 0;
-        int dev = 0;
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess) {
             void *p = nullptr;
             e = dev_alloc(h, &p, sizeof(unsigned));
@@ -402,7 +405,7 @@ bool host_unit_array(apr_handle_t h, int32_t which, const void **src, size_t *by
         std::lock_guard<std::mutex> lk(h->plan_mu);
         if (!h->host_units) {
             try {
-                build_units(h->X);
+                build_units(h->X, HOST_ONLY_SMS);
             } catch (const std::bad_alloc &) {
                 return false;
             }

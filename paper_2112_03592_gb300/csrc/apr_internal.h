@@ -219,12 +219,13 @@ TreeGroups tree_groups(const HostIndex &X, int l0, int l1, int max_levels);
 // receives a short reason on failure.
 apr_status_t build_index(const apr_host_layout &L, uint32_t flags, HostIndex &out, const char **msg);
 
-// Builds what a device handle's kernels read (apr_plan.cu): the child maps and the convolution units. Returns APR_OK, APR_ERR_OOM (host allocation) or APR_ERR_UNSUPPORTED.
-apr_status_t build_plans(HostIndex &X);
+// Builds what the kernels read on a device of `sms` multiprocessors (apr_plan.cu): the child maps and the units. Returns APR_OK, APR_ERR_OOM (host allocation) or APR_ERR_UNSUPPORTED.
+apr_status_t build_plans(HostIndex &X, int sms);
 // Builds the tile plans of X's forward and data-adjoint work items (apr_export_structure).
 apr_status_t build_tile_plans(HostIndex &X);
-// The convolution units of X (after tree_node_plan); throws std::bad_alloc.
-void build_units(HostIndex &X);
+// The convolution units of X (after tree_node_plan) for a device of `sms` multiprocessors; throws std::bad_alloc.
+void build_units(HostIndex &X, int sms);
+constexpr int HOST_ONLY_SMS = 152;   // the units of a host-only handle are a GB300's
 // The child map of every tree node (TreeNodePlan), by one merge of each tree row with its child rows.
 // In a complete index every in-grid child cell of a node is a particle or a node of the next level.
 bool tree_node_plan(const DevLayout &L, const HostIndex &X, std::vector<TreeNodePlan> &P);

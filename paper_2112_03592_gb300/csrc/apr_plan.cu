@@ -201,12 +201,12 @@ apr_status_t run_jobs(std::vector<std::function<bool()>> jobs) {
 
 }  // namespace
 
-apr_status_t build_plans(HostIndex &X) {
+apr_status_t build_plans(HostIndex &X, int sms) {
     const DevLayout L = host_layout_view(X);
     if (X.np >= FPLAN_MAX_INDEX || X.nt >= FPLAN_MAX_INDEX) return APR_ERR_UNSUPPORTED;
     try {
         if (!tree_node_plan(L, X, X.tnplan)) return APR_ERR_UNSUPPORTED;
-        build_units(X);
+        build_units(X, sms);
     } catch (...) {  // host allocation failure
         return APR_ERR_OOM;
     }

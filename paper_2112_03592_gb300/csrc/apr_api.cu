@@ -58,25 +58,22 @@ cudaError_t dev_alloc(apr_handle_s *h, void **p, size_t bytes) {
     return cudaSuccess;
 }
 
-// Device copy of n elements on the build stream, the allocation rounded up to a multiple of `pad`
-// elements (zeroed tail): the y arrays are read in aligned 8-element packets. The host arrays are
-// pageable, so cudaMemcpyAsync has staged them when it returns; the caller may free them.
+// Device copy of n elements on the build stream (an empty array gets one element's space, so that its pointer is one).
+// The host arrays are pageable, so cudaMemcpyAsync has staged them when it returns; the caller may free them.
 template <typename T>
-cudaError_t upload(apr_handle_s *h, T **dst, const T *src, size_t n, size_t pad = 1) {
+cudaError_t upload(apr_handle_s *h, T **dst, const T *src, size_t n) {
     *dst = nullptr;
-    const size_t na = ((n ? n : 1) + pad - 1) / pad * pad;
     void *p = nullptr;
-    cudaError_t e = dev_alloc(h, &p, na * sizeof(T));
+    cudaError_t e = dev_alloc(h, &p, std::max<size_t>(n, 1) * sizeof(T));
     if (e != cudaSuccess) return e;
     *dst = static_cast<T *>(p);
-    const cudaStream_t s = reinterpret_cast<cudaStream_t>(h->stream);
-    if (n) e = cudaMemcpyAsync(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && na > n) e = cudaMemsetAsync(*dst + n, 0, (na - n) * sizeof(T), s);
+    if (n) e = cudaMemcpyAsync(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice, reinterpret_cast<cudaStream_t>(h->stream));
     return e;
 }
 
-// Staged value arrays (particles and tree values of the forward-type calls) are read in 16-byte
-// vectors: their base addresses must be 16-byte aligned.
+// The value arrays of the forward-type calls (particles and tree values) must be 16-byte aligned. The multi-channel
+// kernels load 16 and 32 bytes; the single-channel ones load single floats, and for them the rule stands as
+// part of the interface, which has always refused other addresses.
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Releases every device block of the handle (the caller has synchronised the device).

@@ -11,7 +11,7 @@
 namespace aprk {
 namespace dev {
 
-constexpr int NT = 256;                // threads per block of every kernel below
+constexpr int NT = 256;                // threads of the multi-channel weight gradient and of the other tile kernels' gathering warps
 constexpr int NWARP = NT / 32;
 static_assert(TZ % 2 == 0 && TX % 2 == 0, "tiles must be even-aligned (coarse cells)");
 
@@ -34,6 +34,7 @@ __host__ __device__ __forceinline__ int reflect_idx(int i, int d) {
     return m >= d ? p - 1 - m : m;
 }
 
+// The rows' y-block offsets: blk_start and row_range serve the exported tile plans (apr_tile.cuh), no kernel.
 // First element of y-block j of a row (particles or tree); j >= nb gives the row end.
 __host__ __device__ __forceinline__ uint32_t blk_start(const uint32_t *rp, const uint16_t *off, int row0, int off0,
                                                        int nb, int rr, int j) {

@@ -19,16 +19,16 @@
 //
 // One warp issues the MMAs; completion is signalled through mbarriers whose waits are bounded in time.
 //
-// Measured (1.0 M particles of a 256^3 image, kernels alone): forward 223 -> 60 us, data adjoint 550 -> 167 us
-// (96 onto the children, 71 onto coarser particles), weight gradient 400 -> 98 us. The kernels before cut
+// Measured (1.0 M particles of a 256^3 image, kernels alone): forward 223 -> 63 us, data adjoint 550 -> 173 us
+// (97 onto the children, 76 onto coarser particles), weight gradient 400 -> 100 us. The kernels before cut
 // 8 x 8 x 64-cell tiles, which particles in thin shells leave mostly empty, into sub-tiles staged in shared
 // memory, and gathered 27 cells per target. Tried on the way here, forward: the A operand in shared memory
 // through 16-byte cp.async 131 us (a wavefront of the L1 pipe per 32-byte sector), with the four cells of a
 // row in one instruction 113 us, MMAs issued by a warp of their own 102 us, through registers into tensor
 // memory with warp-uniform MMA operands 74 us, 32-byte stores 66 us, records staged once per unit and more L1
-// 60 us. What bounds it now: the L1 pipe (72 %: the gather touches about a line per 32-byte cell) and a unit's
+// 60 us (63 with the weights laid out by every block, stage_weights). What bounds it now: the L1 pipe (68 %: the gather touches about a line per 32-byte cell) and a unit's
 // chain of latencies, at two blocks per SM; without the gather 42 us, without the MMAs 61 of then 66 us. DRAM
-// traffic is 66 MB, 10 us. The adjoints have fewer sources to gather and more rows: edge units take further
+// traffic is 73 MB, 11 us. The adjoints have fewer sources to gather and more rows: edge units take further
 // tiles for their images (a third of the node adjoint's time at 256^3), leaf rows have few sources each.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -791,7 +791,6 @@ __global__ void __launch_bounds__(TNT, 2) mc_adjoint_kernel(const UnitView U, co
     McSmem &S = M.s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const UnitHdr h = U.work_adj[blockIdx.x];
-    const NodeRec *rec = U.rec + h.rec0;
     NodeRow row;
     row.load(U, h, true);
     stage_codes<false>(U, h, false, false, S.code);
@@ -1390,7 +1389,7 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
             e = launch(mc_adjoint_kernel, h->U.n, TNT, sizeof(McAdjSmem), stream, true, h->U, weights, bc, g4, grad_particles, gt, h->d_err);
         if (e == cudaSuccess)
             e = launch(mc_leaf_adjoint_kernel, h->U.nl, TNT, std::max(sizeof(McLeafSmem), TWO_BLOCKS), stream, true, h->U, weights, bc, g4, grad_particles, h->d_err);
-            const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
+        const TreeGroups T = tree_groups(X, X.l_min, X.l_max - 1, 3);
         for (int i = 0; i < T.n && e == cudaSuccess; ++i) {
             e = launch_tree_pushdown16(h->d_tnplan, T.g[i], grad_particles, gt, stream, true);
         }

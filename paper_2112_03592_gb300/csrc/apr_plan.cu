@@ -1,7 +1,7 @@
 // Host builders of what the kernels read: the child maps of the tree nodes (tree_node_plan) and, through
-// build_units (apr_unitplan.cpp), the convolution units. Also the tile plans that apr_export_structure gives: for every forward and data-adjoint
-// work item and both stencil radii the non-empty source segments of the item's patch (fwd_segment,
-// bwd_segment in apr_tile.cuh), with the prefix of their 8-element packets.
+// build_units (apr_unitplan.cpp), the convolution units. Also the tile plans that apr_export_structure gives, and
+// that nothing else reads: for every forward and data-adjoint work item and both stencil radii the non-empty source
+// segments of the item's patch (fwd_segment, bwd_segment in apr_tile.cuh), with the prefix of their 8-element packets.
 #include <functional>
 #include <thread>
 #include <vector>

@@ -1,5 +1,5 @@
 // Geometry of an 8 x 8 x 64-cell work item and the source segments of its patch, as the tile plans that
-// apr_export_structure gives list them (apr_plan.cu).
+// apr_export_structure gives list them (apr_plan.cu). Host code; no kernel reads the plans.
 #pragma once
 
 #include "apr_device.cuh"

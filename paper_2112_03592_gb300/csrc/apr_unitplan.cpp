@@ -590,7 +590,7 @@ void build_units(HostIndex &X, int sms) {
     // Records per unit: 256 where that fills the chip (4 resident units of 128 and more per multiprocessor), fewer for small
     // APRs, whose calls are bound by the latency of one unit, not by throughput. Measured with 256, 128 and 64: 142 k
     // parents, 16-channel training step 401, 424 and 586 us, gradient magnitude (174 k) 38, 43 and 51 us; 6 k parents, 16-channel
-    // training step 128, 96 and 94 us, 20 Richardson-Lucy iterations 301, 284 and 278 us.
+    // training step 128, 96 and 94 us, ten Richardson-Lucy iterations 301, 284 and 278 us.
     const int UN = parents >= int64_t(sms) * 4 * 128 ? 256 : parents >= int64_t(sms) * 64 ? 128 : 64;
     std::vector<ParentLevel> levels;
     std::vector<std::vector<int32_t>> tf, tb;

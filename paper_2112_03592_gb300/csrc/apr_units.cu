@@ -18,7 +18,7 @@
 // -> 197 us, stencil gradient 360 -> 190 us; 36.5 M instead of 131.8 M warp instructions per convolution.
 // What bounds them now: shared-memory wavefronts (the L1 pipe is 75 % busy in the convolution; 2.5
 // wavefronts per 4-byte load, since the slots of 32 records lie in many short runs) and the latency of
-// header -> entry -> value at four blocks of 256 threads per SM; DRAM traffic is 0.19 GB, 29 us.
+// header -> entry -> value at four blocks of 256 threads per SM; DRAM traffic is 0.23 GB, 34 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1032,7 +1032,7 @@ static_assert(WgradSmem<2>::BLOCKS * (sizeof(WgradSmem<2>) + 1024) <= 228 * 1024
 static_assert(UNIT_SLOTS <= int(UE_SLOT) + 1, "slot numbers fit an entry");
 
 // pdl: the kernel starts while the launch before it finishes and loads its header, records and entries meanwhile. A
-// chain of small launches is bound by these: 20 Richardson-Lucy iterations of 40 k particles 409 -> 272 us, of 2.8 M
+// chain of small launches is bound by these: ten Richardson-Lucy iterations of 40 k particles 409 -> 272 us, 20 of 2.8 M
 // 2506 -> 2354 us; restriction and 5^3 convolution of 1 M 30 -> 27 us; gradient magnitude of 1.2 M 35 -> 31 us.
 template <typename... KArgs, typename... Args>
 cudaError_t launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl, Args &&...args) {

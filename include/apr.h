@@ -18,8 +18,10 @@
  *   - Work is enqueued asynchronously on the given stream (NULL = the legacy default stream); the
  *     caller synchronises. Launch failures return APR_ERR_CUDA. Device-side checks record into an
  *     error word read by apr_sync_status().
- *   - Not thread-safe per handle: calls on one handle must not run concurrently on different
- *     streams when they share output buffers or the handle's scratch.
+ *   - Calls on one handle may run at the same time on different streams, and be made by different
+ *     threads, as long as no buffer that one of them writes (outputs, workspaces) is used by another:
+ *     they share the read-only index. apr_convolve_backward's two-stream part is ordered by a mutex while it
+ *     enqueues; apr_convolve_backward_noalloc shares the library's scratch array (see there).
  */
 #ifndef APR_H
 #define APR_H

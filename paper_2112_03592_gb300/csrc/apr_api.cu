@@ -123,6 +123,7 @@ apr_status_t misaligned() {
 namespace aprk {
 TreeGroups tree_groups(const HostIndex &X, int l0, int l1, int max_levels) {
     TreeGroups out;
+    if (!X.complete) max_levels = 1;
     for (int l = l0; l <= l1;) {
         int64_t b = 0, n = 0;
         tree_level_nodes(X, l, b, n);
@@ -313,7 +314,7 @@ apr_status_t apr_build_device_ex(const apr_host_layout *layout, uint32_t flags, 
             h->level_has[i] = X.fwd_level_begin[l + 1] > X.fwd_level_begin[l];
             h->unit_begin[i] = UP.level_begin[i];
         }
-        h->complete = UP.complete;
+        h->X.complete = UP.complete;
         h->uncovered = UP.uncovered;
         h->n_levels_with = 0;
         for (int i = 0; i <= X.l_max - X.l_min; ++i) h->n_levels_with += h->level_has[i] ? 1 : 0;
@@ -600,8 +601,8 @@ apr_status_t apr_convolve_adjoint(apr_handle_t h, const float *stencils, int32_t
     // the units store the gradient of every particle and tree node; only in an index in which some have
     // no record (a layout that was not validated) are the arrays cleared first
     cudaError_t e = cudaSuccess;
-    if (!h->complete && X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * sizeof(float), stream);
-    if (!h->complete && e == cudaSuccess && X.nt) e = cudaMemsetAsync(grad_tree, 0, size_t(X.nt) * sizeof(float), stream);
+    if (!X.complete && X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * sizeof(float), stream);
+    if (!X.complete && e == cudaSuccess && X.nt) e = cudaMemsetAsync(grad_tree, 0, size_t(X.nt) * sizeof(float), stream);
     if (e == cudaSuccess) e = launch_adjoint(k, h->U, stencils, bc, grad_out, grad_particles, grad_tree, stream);
     return cuda_status(e);
 }

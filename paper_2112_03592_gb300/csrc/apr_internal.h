@@ -190,6 +190,7 @@ struct HostIndex {
     std::vector<uint16_t> vy;
     std::vector<TreeNodePlan> vplan;
     UnitPlan units;                           // convolution units (build_units)
+    bool complete = false;                    // every particle and tree node is the child of a record (kept from units)
 };
 
 // The tree nodes of level l (l_min <= l < l_max): [b, b + n) in tree order.
@@ -208,6 +209,8 @@ struct TreeGroup {
 // levels (at most max_levels) as keep its deepest level at or below tree_group_threads entries.
 // 2^17 entries are less than half of what is resident at once; with 2^20 a group's idle threads cost more than
 // the launches it saves (16-channel restriction of 1 M particles 28 -> 50 us, push-down of 8 M 45 -> 84 us at 2^22).
+// A group finds the nodes of its finer levels from their parents; where a cell is a particle and a node at once (a
+// layout that was not validated) the node is no parent's child, so that every level is a group of its own.
 constexpr int64_t tree_group_threads = int64_t(1) << 17;
 struct TreeGroups {
     int n = 0;
@@ -301,7 +304,6 @@ struct apr_handle_s {
     aprk::UnitSpans fwd_units, bwd_units, bwd_leaves;   // UnitPlan
     int32_t unit_begin[aprk::MAXL + 1] = {};   // first unit of level l_min + i
     bool level_has[aprk::MAXL + 1] = {};       // whether level l_min + i holds particles
-    bool complete = false;                     // every particle and tree node is the child of a record
     bool uncovered = false;                    // a cell next to a particle has no source (invalid layout)
     int n_levels_with = 0, sms = 0;            // levels with particles; multiprocessors of the device
     size_t dev_bytes = 0;

@@ -1381,8 +1381,8 @@ apr_status_t apr_convolve_mc_backward(apr_handle_t h, const uint16_t *particles,
     if (grad_particles) {
         // every particle and tree node is the child of one record, which stores its gradient; only in an
         // index in which some have no record (a layout that was not validated) are the arrays cleared first
-        if (!h->complete && X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * MC * sizeof(float), stream);
-        if (!h->complete && e == cudaSuccess && X.nt) e = cudaMemsetAsync(gt, 0, size_t(X.nt) * MC * sizeof(float), stream);
+        if (!X.complete && X.np) e = cudaMemsetAsync(grad_particles, 0, size_t(X.np) * MC * sizeof(float), stream);
+        if (!X.complete && e == cudaSuccess && X.nt) e = cudaMemsetAsync(gt, 0, size_t(X.nt) * MC * sizeof(float), stream);
         if (h->uncovered) uncovered_kernel<<<1, 1, 0, stream>>>(h->d_err);
         const uint4 *g4 = reinterpret_cast<const uint4 *>(grad_out);
         if (e == cudaSuccess)

@@ -26,7 +26,7 @@
 // through 16-byte cp.async 131 us (a wavefront of the L1 pipe per 32-byte sector), with the four cells of a
 // row in one instruction 113 us, MMAs issued by a warp of their own 102 us, through registers into tensor
 // memory with warp-uniform MMA operands 74 us, 32-byte stores 66 us, records staged once per unit and more L1
-// 60 us (63 with the weights laid out by every block, stage_weights). What bounds it now: the L1 pipe (68 %: the gather touches about a line per 32-byte cell) and a unit's
+// 60 us (63 with the weights laid out by every block, copy_weights). What bounds it now: the L1 pipe (68 %: the gather touches about a line per 32-byte cell) and a unit's
 // chain of latencies, at two blocks per SM; without the gather 42 us, without the MMAs 61 of then 66 us. DRAM
 // traffic is 73 MB, 11 us. The adjoints have fewer sources to gather and more rows: edge units take further
 // tiles for their images (a third of the node adjoint's time at 256^3), leaf rows have few sources each.
@@ -586,11 +586,10 @@ __device__ __forceinline__ bool tile_gemm(McSmem &S, int row0, const uint4 *__re
 // N = ci, K = co, taps flipped. They arrive as they lie in memory, every thread takes the 27 taps of one (n, k),
 // and the blocks are written over them. Every block does this for itself: a kernel that laid them out ahead of each
 // convolution needed a buffer in the handle, which calls on two streams overwrote for one another. Measured with that
-// kernel and without: training step of 1 M particles 390.9 and 390.0 us, of 45 k 79.8 and 78.0, four layers of 2.4 M 651.5
-// and 654.2.
-template <bool ADJ>
-__device__ __forceinline__ void stage_weights(McSmem &S, const uint16_t *__restrict__ W, int lev) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// kernel and without: training step of 1 M particles 394.7 and 393.5 us, of 45 k 80.1 and 77.5, four layers of 2.4 M 658.7
+// and 658.2 (661 with the copy behind the tensor-memory allocation).
+__device__ __forceinline__ void copy_weights(McSmem &S, const uint16_t *__restrict__ W, int lev) {
+    const int tid = threadIdx.x;
     const uint16_t *src = W + size_t(lev) * W_LEVEL;
     uint16_t *w = reinterpret_cast<uint16_t *>(S.W);
     if ((reinterpret_cast<uintptr_t>(W) & 15u) == 0) {
@@ -599,6 +598,11 @@ __device__ __forceinline__ void stage_weights(McSmem &S, const uint16_t *__restr
         for (int i = tid; i < W_LEVEL; i += TNT) w[i] = load_u16(src + i);
     }
     cp_commit();
+}
+template <bool ADJ>
+__device__ __forceinline__ void transpose_weights(McSmem &S) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint16_t *w = reinterpret_cast<uint16_t *>(S.W);
     cp_wait<0>();
     block_sync();
     // a warp's lanes: 4 n x 8 k (its 2-byte stores fill 16 banks)
@@ -622,10 +626,11 @@ __device__ __forceinline__ void stage_weights(McSmem &S, const uint16_t *__restr
 template <bool ADJ>
 __device__ __forceinline__ void tile_setup(McSmem &S, const uint16_t *W, int lev) {
     const int tid = threadIdx.x;
+    copy_weights(S, W, lev);   // (before the allocation, which its warp waits for)
     if (tid < STAGES) mbar_init(&S.bar[tid]);
     __syncwarp();
     if ((tid >> 5) == 0) tmem_alloc(smem_u32(&S.tmem), TMEM_COLS);
-    stage_weights<ADJ>(S, W, lev);
+    transpose_weights<ADJ>(S);
 }
 // Ends the set-up: weights visible to the tensor cores, rows and codes visible to the block.
 __device__ __forceinline__ void tile_ready() {
